@@ -172,13 +172,13 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
 
   if (warp == 9) {
     // ---------------- TMA producer: the K/V tiles of the key range ----------------
-    if (lane == 0) {
-      for (int t = 0; t < n_tiles; ++t) {
-        const int st = t % UA_STAGES;
-        if (t >= UA_STAGES && !mbar_wait(smem_u32(&kv_empty[st]), (uint32_t)(t / UA_STAGES - 1) & 1u, abortp)) {
-          ok = false;
-          break;
-        }
+    for (int t = 0; t < n_tiles; ++t) {
+      const int st = t % UA_STAGES;
+      if (t >= UA_STAGES && !mbar_wait_warp(smem_u32(&kv_empty[st]), (uint32_t)(t / UA_STAGES - 1) & 1u, abortp)) {
+        ok = false;
+        break;
+      }
+      if (elect_one()) {
         const uint32_t fb = smem_u32(&kv_full[st]);
         mbar_expect_tx(fb, SM::STAGE);
         const uint32_t dst = kv_s + st * SM::STAGE;
@@ -189,6 +189,7 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
           tma_load_3d(dst + SM::KV_TILE + p * (UA_KEYS * 128), &tmV, fb, kh * HD + p * 64, key0, b);
         }
       }
+      __syncwarp();
     }
   } else if (warp == 8) {
     // ---------------- MMA issuer ----------------
@@ -197,27 +198,41 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
     // and P_i are A operands in tensor memory (P_i in the columns its scores came from), so shared memory is
     // read for K and V only.  A commit covers every MMA issued before it, so when s_full[i] flips for tile t+1
     // the product O_i += P_i V of tile t has completed too: the group may then rescale O_i.
-    if (lane == 0) {
+    {
       constexpr uint32_t idesc_s = make_idesc(UA_ROWS, UA_KEYS);
       constexpr uint32_t idesc_o = make_idesc(UA_ROWS, HD) | (1u << 16);  // B operand (V) is MN-major
       auto issue_s = [&](int i, int st) {
         const uint32_t k_s = kv_s + st * SM::STAGE;
+        if (elect_one()) {
 #pragma unroll
-        for (int ks = 0; ks < HD / 16; ++ks) {
-          const uint32_t koff = (ks >> 2) * (UA_KEYS * 128) + (ks & 3) * 32;  // panel, then 32 bytes per k-step
-          // A = 16 dimensions of Q_i from tensor memory (8 columns of bf16 pairs per k-step)
-          umma_bf16_ta(tmem + SM::S_COL + (uint32_t)(i * UA_KEYS), tmem + SM::Q_COL + (uint32_t)(i * (HD / 2) + ks * 8),
-                       make_smem_desc(k_s + koff), idesc_s, ks > 0 ? 1u : 0u);
+          for (int ks = 0; ks < HD / 16; ++ks) {
+            const uint32_t koff = (ks >> 2) * (UA_KEYS * 128) + (ks & 3) * 32;  // panel, then 32 bytes per k-step
+            // A = 16 dimensions of Q_i from tensor memory (8 columns of bf16 pairs per k-step)
+            umma_bf16_ta(tmem + SM::S_COL + (uint32_t)(i * UA_KEYS), tmem + SM::Q_COL + (uint32_t)(i * (HD / 2) + ks * 8),
+                         make_smem_desc(k_s + koff), idesc_s, ks > 0 ? 1u : 0u);
+          }
+          umma_commit(smem_u32(&s_full[i]));
         }
-        umma_commit(smem_u32(&s_full[i]));
+        __syncwarp();
       };
-      ok = mbar_wait(smem_u32(&q_bar), 0u, abortp) && mbar_wait(smem_u32(&kv_full[0]), 0u, abortp);
+      // O_i += P_i V: A = 16 keys of P_i from tensor memory; V: 16 key rows of 128 bytes
+      auto issue_o = [&](int i, uint32_t v_s, bool accumulate) {
+        if (elect_one()) {
+#pragma unroll
+          for (int ks = 0; ks < UA_KEYS / 16; ++ks)
+            umma_bf16_ta(tmem + SM::O_COL + (uint32_t)(i * HD), tmem + SM::S_COL + (uint32_t)(i * UA_KEYS + ks * 8),
+                         make_smem_desc_mn(v_s + ks * (16 * 128), UA_KEYS * 128, 1024), idesc_o,
+                         (accumulate || ks > 0) ? 1u : 0u);
+        }
+        __syncwarp();
+      };
+      ok = mbar_wait_warp(smem_u32(&q_bar), 0u, abortp) && mbar_wait_warp(smem_u32(&kv_full[0]), 0u, abortp);
       if (ok && kpar) {
         // group i owns key tiles i, i + 2, ...: S_0(0), S_1(1); then per tile t (group i = t % 2):
         // O_i += P_i(t) V(t) and right behind it S_i(t + 2)
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         issue_s(0, 0);
-        ok = mbar_wait(smem_u32(&kv_full[1]), 0u, abortp);
+        ok = mbar_wait_warp(smem_u32(&kv_full[1]), 0u, abortp);
         if (ok) {
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           issue_s(1, 1);
@@ -226,24 +241,20 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
           const int i = t & 1, u = t >> 1;
           const int st = t % UA_STAGES;
           const uint32_t v_s = kv_s + st * SM::STAGE + SM::KV_TILE;
-          ok = mbar_wait(smem_u32(&p_full[i]), (uint32_t)u & 1u, abortp);
+          ok = mbar_wait_warp(smem_u32(&p_full[i]), (uint32_t)u & 1u, abortp);
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-          for (int ks = 0; ks < UA_KEYS / 16; ++ks)
-            umma_bf16_ta(tmem + SM::O_COL + (uint32_t)(i * HD), tmem + SM::S_COL + (uint32_t)(i * UA_KEYS + ks * 8),
-                         make_smem_desc_mn(v_s + ks * (16 * 128), UA_KEYS * 128, 1024), idesc_o,
-                         (u > 0 || ks > 0) ? 1u : 0u);
+          issue_o(i, v_s, u > 0);
           if (t + 2 < n_tiles) {
             const int st2 = (t + 2) % UA_STAGES;
-            ok = mbar_wait(smem_u32(&kv_full[st2]), (uint32_t)((t + 2) / UA_STAGES) & 1u, abortp);
+            ok = mbar_wait_warp(smem_u32(&kv_full[st2]), (uint32_t)((t + 2) / UA_STAGES) & 1u, abortp);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             issue_s(i, st2);
           } else {
-            umma_commit(smem_u32(&o_full[i]));  // the group's last tile: O_i is final when this fires
+            if (elect_one()) umma_commit(smem_u32(&o_full[i]));  // the group's last tile: O_i is final when this fires
           }
-          umma_commit(smem_u32(&kv_empty[st]));  // only group i reads tile t
+          if (elect_one()) umma_commit(smem_u32(&kv_empty[st]));  // only group i reads tile t
         }
       } else if (ok) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -254,27 +265,23 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
         const uint32_t v_s = kv_s + st * SM::STAGE + SM::KV_TILE;
         bool next_ready = t + 1 >= n_tiles;
         for (int i = 0; i < live && ok; ++i) {
-          ok = mbar_wait(smem_u32(&p_full[i]), (uint32_t)t & 1u, abortp);
+          ok = mbar_wait_warp(smem_u32(&p_full[i]), (uint32_t)t & 1u, abortp);
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-          for (int ks = 0; ks < UA_KEYS / 16; ++ks)   // A = 16 keys of P_i from tensor memory; V: 16 key rows of 128 bytes
-            umma_bf16_ta(tmem + SM::O_COL + (uint32_t)(i * HD), tmem + SM::S_COL + (uint32_t)(i * UA_KEYS + ks * 8),
-                         make_smem_desc_mn(v_s + ks * (16 * 128), UA_KEYS * 128, 1024), idesc_o,
-                         (t > 0 || ks > 0) ? 1u : 0u);
+          issue_o(i, v_s, t > 0);
           if (t + 1 < n_tiles) {
             if (!next_ready) {
-              ok = mbar_wait(smem_u32(&kv_full[st_next]), (uint32_t)((t + 1) / UA_STAGES) & 1u, abortp);
+              ok = mbar_wait_warp(smem_u32(&kv_full[st_next]), (uint32_t)((t + 1) / UA_STAGES) & 1u, abortp);
               if (!ok) break;
               asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
               next_ready = true;
             }
             issue_s(i, st_next);
           } else {
-            umma_commit(smem_u32(&o_full[i]));  // last tile: O_i is final when this fires
+            if (elect_one()) umma_commit(smem_u32(&o_full[i]));  // last tile: O_i is final when this fires
           }
         }
-        if (ok) umma_commit(smem_u32(&kv_empty[st]));  // the stage may be refilled once these MMAs have read it
+        if (ok && elect_one()) umma_commit(smem_u32(&kv_empty[st]));  // the stage may be refilled once these MMAs have read it
       }
     }
   } else {

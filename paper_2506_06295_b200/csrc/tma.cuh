@@ -35,6 +35,10 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+// Arrival on a barrier of another CTA of the cluster (shared::cluster address, see cluster_addr).
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
+}
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -59,6 +63,46 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
         *abort_flag = 1;
         return false;
       }
+    }
+  }
+  return true;
+}
+// One lane of a converged warp.  Code that issues TMA copies and tcgen05 instructions runs in all 32 lanes and guards
+// each group of instructions with this: behind `lane == 0` the compiler cannot tell that one thread is active and
+// moves every operand through a per-lane sequence (four MMAs and a commit took 330 cycles of the issuing thread
+// against 150 behind elect, and that thread was what bounded the GEMM main loops: 600 against 460 cycles per k-block
+// of a 256 x 128 tile).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r != 0;
+}
+// Whether the phase has completed, without waiting; the whole warp, which gets one answer.
+__device__ __forceinline__ bool mbar_peek_warp(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return __all_sync(0xffffffffu, ok != 0);
+}
+// mbar_wait by a converged warp, which gets one answer.  `ready`: an earlier mbar_peek_warp of this phase said so.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+                                               bool ready = false) {
+  if (ready || __all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const uint64_t t0 = gtime();
+  uint32_t it = 0;
+  while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+    if ((++it & 63u) == 0u) {
+      bool stop = *abort_flag != 0;
+      if (!stop && gtime() - t0 > g_wait_limit_ns) {
+        *abort_flag = 1;
+        stop = true;
+      }
+      if (__any_sync(0xffffffffu, stop)) return false;
     }
   }
   return true;
