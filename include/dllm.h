@@ -316,11 +316,11 @@ dllm_status dllm_kernel_status(void* stream);
  * records the status code, skips its epilogue, frees its tensor memory and
  * returns normally; (0) switches that off.  Both calls synchronise the device. */
 dllm_status dllm_debug_set_wait_limit_ns(uint64_t ns);
-/* Tuning / test hook: kernel choice of the bf16 projections whose plan has no
- * split and 256-row activation tiles, for every later call in this process:
- * 0 automatic (the persistent kernel when there are more tiles than SMs), 1
- * always the persistent kernel, -1 always the one-tile-per-CTA kernel.  The two
- * kernels give bit-identical results. */
+/* Tuning / test hook: kernel choice of the bf16 projections, for every later
+ * call in this process: 0 automatic (persistent CTA pairs above 128 activation
+ * rows), 1 the pair kernel for every unsplit plan with 256-row activation tiles,
+ * -1 always the one-tile-per-CTA kernel.  Unsplit plans give bit-identical
+ * results on both. */
 dllm_status dllm_debug_gemm_plan(int persistent);
 /* Tuning hook: overrides, for every later call in this process, the number of
  * key-range splits the tensor-core attention kernels take (0 = automatic); if
@@ -342,7 +342,7 @@ size_t dllm_gemm_bf16_scratch_bytes(int M, int N, int K);
 dllm_status dllm_gemm_bf16(const void* d_A, const void* d_W, float* d_C, int M, int N, int K,
                            void* d_partials, void* stream);
 /* The same product with an explicit launch plan, for tuning: act_tile = rows of
- * A per CTA (32, 64, 128 or 256; 192 with splits = 1 only: the persistent kernel),
+ * A per CTA (32, 64, 128 or 256; 192 with splits = 1 only: the pair kernel),
  * splits = split-K factor, stages = depth of the TMA ring (clamped to what fits
  * shared memory); 0 picks the default of each.
  * d_partials (device, partials_bytes >= dllm_gemm_bf16_planned_scratch_bytes)
@@ -352,7 +352,7 @@ size_t dllm_gemm_bf16_planned_scratch_bytes(int M, int N, int K, int act_tile, i
 dllm_status dllm_gemm_bf16_planned(const void* d_A, const void* d_W, float* d_C, int M, int N, int K, int act_tile,
                                    int splits, int stages, void* d_partials, size_t partials_bytes, void* stream);
 /* The same product computed by PAIRS of CTAs (tcgen05 cta_group::2): two CTAs
- * of a cluster share one activation tile of act_tile (128 or 256) rows, each
+ * of a cluster share one activation tile of act_tile (64, 128, 192 or 256) rows, each
  * staging half of it, so the tile crosses the L2 -> SM fabric once per 256
  * weight rows.  N must be a multiple of 256.  splits / stages / scratch as for
  * dllm_gemm_bf16_planned; the result is bit-identical to the one-CTA kernel

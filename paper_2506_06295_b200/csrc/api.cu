@@ -405,7 +405,10 @@ dllm_status run_gemm(dllm_session* s, const Launch& L, int cls, const void* A, c
   if (M <= 0) return DLLM_OK;
   const double es = (double)s->es();
   const bool tensor = !(s->m->cfg.dtype == DLLM_FP32 || s->simt_gemm);
-  const GemmPlan plan = tensor ? plan_gemm_bf16(M, N, K) : GemmPlan{};
+  // the LM head is never split (its consumers read logits or records), nor is a gate / up projection of more rows
+  // than stream the weights anyway: the SwiGLU epilogue saves a launch and a pass over the slabs
+  const bool whole = cls == DLLM_PROF_GEMM_HEAD || (swiglu_out && M > 128 && gu_interleaved(s->m->cfg));
+  const GemmPlan plan = tensor ? plan_gemm_bf16(M, N, K, whole ? 1 : 0) : GemmPlan{};
   // an unsplit gate / up projection of an interleaved weight finishes SwiGLU in its own epilogue, and an unsplit
   // LM head writes per-tile estimate records instead of logits
   const bool estimate = tensor && !swiglu_out && estimate_mask_id >= 0 && plan.S_max == 1;
@@ -1293,11 +1296,12 @@ dllm_status dllm_gemm_bf16(const void* d_A, const void* d_W, float* d_C, int M, 
   const GemmPlan p = plan_gemm_bf16(M, N, K);
   if (p.S_max > 1 && !d_partials) return fail(nullptr, DLLM_INVALID_ARG, "this shape needs slab scratch");
   Launch L{(cudaStream_t)stream, kernel_status_word(), nullptr};
+  if (!d_C && p.S_max == 1) return fail(nullptr, DLLM_INVALID_ARG, "d_C is NULL");
   float* part = p.S_max > 1 ? static_cast<float*>(d_partials) : d_C;
   const char* why = nullptr;
   cudaError_t e = launch_gemm_bf16(L, d_A, d_W, part, M, N, K, p, &why);
   if (e != cudaSuccess) return fail(nullptr, DLLM_CUDA_ERROR, "bf16 GEMM: %s", why ? why : cudaGetErrorString(e));
-  if (p.S_max > 1) launch_reduce_partials(L, make_partials(part, M, N, p), d_C, M);
+  if (p.S_max > 1 && d_C) launch_reduce_partials(L, make_partials(part, M, N, p), d_C, M);
   CU_TRY(nullptr, cudaGetLastError());
   return DLLM_OK;
 }
@@ -1316,7 +1320,7 @@ dllm_status dllm_gemm_bf16_planned(const void* d_A, const void* d_W, float* d_C,
   if (act_tile && act_tile != 32 && act_tile != 64 && act_tile != 128 && act_tile != 192 && act_tile != 256)
     return fail(nullptr, DLLM_INVALID_ARG, "act_tile must be 0, 32, 64, 128, 192 or 256");
   if (act_tile == 192 && splits != 1)
-    return fail(nullptr, DLLM_INVALID_ARG, "192-row tiles exist in the unsplit persistent kernel only: splits must be 1");
+    return fail(nullptr, DLLM_INVALID_ARG, "192-row tiles exist in the unsplit pair kernel only: splits must be 1");
   const GemmPlan p = plan_gemm_bf16(M, N, K, splits, stages, act_tile);
   if (p.S_max > 1 && (!d_partials || partials_bytes < (size_t)p.S_max * M * N * 4))
     return fail(nullptr, DLLM_INVALID_ARG, "this plan needs %zu bytes of slab scratch", (size_t)p.S_max * M * N * 4);
@@ -1349,26 +1353,27 @@ dllm_status dllm_ffn_gate_up_bf16(const void* d_A, const void* d_Wgu, void* d_ou
 }
 
 size_t dllm_gemm_bf16_pair_scratch_bytes(int M, int N, int K, int act_tile, int splits) {
-  if (M <= 0 || N <= 0 || K <= 0 || splits < 0 || (act_tile != 128 && act_tile != 256)) return 0;
+  if (M <= 0 || N <= 0 || K <= 0 || splits < 0 || (act_tile != 64 && act_tile != 128 && act_tile != 192 && act_tile != 256)) return 0;
   const GemmPlan p = plan_gemm_bf16(M, N, K, splits, 0, act_tile, 1);
   return p.S_max > 1 ? (size_t)p.S_max * M * N * 4 : 0;
 }
 
 dllm_status dllm_gemm_bf16_pair(const void* d_A, const void* d_W, float* d_C, int M, int N, int K, int act_tile,
                                 int splits, int stages, void* d_partials, size_t partials_bytes, void* stream) {
-  if (!d_A || !d_W || !d_C || M <= 0 || N <= 0 || K <= 0) return fail(nullptr, DLLM_INVALID_ARG, "bad GEMM arguments");
+  if (!d_A || !d_W || M <= 0 || N <= 0 || K <= 0) return fail(nullptr, DLLM_INVALID_ARG, "bad GEMM arguments");
   if (K % 8 || N % 256) return fail(nullptr, DLLM_INVALID_ARG, "K must be a multiple of 8 and N of 256");
-  if (splits < 0 || stages < 0 || (act_tile != 128 && act_tile != 256))
-    return fail(nullptr, DLLM_INVALID_ARG, "act_tile must be 128 or 256");
+  if (splits < 0 || stages < 0 || (act_tile != 64 && act_tile != 128 && act_tile != 192 && act_tile != 256))
+    return fail(nullptr, DLLM_INVALID_ARG, "act_tile must be 64, 128, 192 or 256");
   const GemmPlan p = plan_gemm_bf16(M, N, K, splits, stages, act_tile, 1);
   if (p.S_max > 1 && (!d_partials || partials_bytes < (size_t)p.S_max * M * N * 4))
     return fail(nullptr, DLLM_INVALID_ARG, "this plan needs %zu bytes of slab scratch", (size_t)p.S_max * M * N * 4);
   Launch L{(cudaStream_t)stream, kernel_status_word(), nullptr};
+  if (!d_C && p.S_max == 1) return fail(nullptr, DLLM_INVALID_ARG, "d_C is NULL");
   float* part = p.S_max > 1 ? static_cast<float*>(d_partials) : d_C;
   const char* why = nullptr;
   cudaError_t e = launch_gemm_bf16(L, d_A, d_W, part, M, N, K, p, &why);
   if (e != cudaSuccess) return fail(nullptr, DLLM_CUDA_ERROR, "bf16 GEMM: %s", why ? why : cudaGetErrorString(e));
-  if (p.S_max > 1) launch_reduce_partials(L, make_partials(part, M, N, p), d_C, M);
+  if (p.S_max > 1 && d_C) launch_reduce_partials(L, make_partials(part, M, N, p), d_C, M);
   CU_TRY(nullptr, cudaGetLastError());
   return DLLM_OK;
 }

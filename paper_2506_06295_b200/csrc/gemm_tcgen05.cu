@@ -253,25 +253,27 @@ __global__ void __launch_bounds__(128) gemm_bf16_tcgen05_kernel(const __grid_con
 
   const uint32_t tiles = (smem_u32(smem_raw) + 1023u) & ~1023u;
 
-  int pre = 0;  // stages whose weight tile was requested before the dependency wait
+  const int pre = min(STAGES, nkb);  // stages whose weight tile is requested before the dependency wait
   int dbg_skip = 0;
-  if (threadIdx.x == 0) {
+  if (warp == 0) {
     dbg_skip = g_debug_skip_act_load;  // read here, long before it is used: not on the path behind the dependency wait
-    abort_flag = 0;
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(smem_u32(&full_bar[s]), 1);
-      mbar_init(smem_u32(&empty_bar[s]), 1);
+    if (elect_one()) {
+      abort_flag = 0;
+      for (int s = 0; s < STAGES; ++s) {
+        mbar_init(smem_u32(&full_bar[s]), 1);
+        mbar_init(smem_u32(&empty_bar[s]), 1);
+      }
+      mbar_init(smem_u32(&accum_bar), 1);
+      mbar_fence_init();
+      prefetch_tensormap(&tmW);
+      prefetch_tensormap(&tmA);
+      for (int i = 0; i < pre; ++i) {  // weights are written by no kernel: stream them ahead of the dependency
+        const uint32_t fb = smem_u32(&full_bar[i]);
+        mbar_expect_tx(fb, SL::STAGE_BYTES);
+        tma_load_2d(tiles + i * SL::STAGE_BYTES, &tmW, fb, (kb0 + i) * TILE_K, n0);
+      }
     }
-    mbar_init(smem_u32(&accum_bar), 1);
-    mbar_fence_init();
-    prefetch_tensormap(&tmW);
-    prefetch_tensormap(&tmA);
-    pre = min(STAGES, nkb);  // weights are written by no kernel: stream them ahead of the dependency
-    for (int i = 0; i < pre; ++i) {
-      const uint32_t fb = smem_u32(&full_bar[i]);
-      mbar_expect_tx(fb, SL::STAGE_BYTES);
-      tma_load_2d(tiles + i * SL::STAGE_BYTES, &tmW, fb, (kb0 + i) * TILE_K, n0);
-    }
+    __syncwarp();
   }
   if (warp == 1) {  // TMEM: BN fp32 columns x 128 lanes
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
@@ -287,7 +289,7 @@ __global__ void __launch_bounds__(128) gemm_bf16_tcgen05_kernel(const __grid_con
   pdl_wait();     // the activation rows and the slab buffer belong to the preceding kernels
   pdl_trigger();
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ---------------- TMA producer ----------------
     int s = 0;
     uint32_t ph = 0;
@@ -295,51 +297,60 @@ __global__ void __launch_bounds__(128) gemm_bf16_tcgen05_kernel(const __grid_con
       const uint32_t fb = smem_u32(&full_bar[s]);
       const uint32_t dstW = tiles + s * SL::STAGE_BYTES;
       const int kc = (kb0 + i) * TILE_K;
-      if (i >= pre) {
-        if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, abortp)) {
-          if (status) atomicCAS(status, ST_OK, ST_TIMEOUT_TMA);
-          break;
-        }
-        mbar_expect_tx(fb, SL::STAGE_BYTES);
-        tma_load_2d(dstW, &tmW, fb, kc, n0);
-      }
       const bool skip = i == 0 && dbg_skip != 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0;
-      if (!skip) tma_load_2d(dstW + W_STAGE_BYTES, &tmA, fb, kc, m0);
+      if (i >= pre && !mbar_wait_warp(smem_u32(&empty_bar[s]), ph ^ 1u, abortp)) {
+        if (status && lane == 0) atomicCAS(status, ST_OK, ST_TIMEOUT_TMA);
+        break;
+      }
+      if (elect_one()) {
+        if (i >= pre) {
+          mbar_expect_tx(fb, SL::STAGE_BYTES);
+          tma_load_2d(dstW, &tmW, fb, kc, n0);
+        }
+        if (!skip) tma_load_2d(dstW + W_STAGE_BYTES, &tmA, fb, kc, m0);
+      }
+      __syncwarp();
       if (++s == STAGES) {
         s = 0;
         ph ^= 1u;
       }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
     constexpr uint32_t idesc = make_idesc(TILE_W, BN);
-    bool ok = true;
+    bool ok = true, ready = false;
     int s = 0;
     uint32_t ph = 0;
     for (int i = 0; i < nkb && ok; ++i) {
-      if (!mbar_wait(smem_u32(&full_bar[s]), ph, abortp)) {
-        if (status) atomicCAS(status, ST_OK, ST_TIMEOUT_MMA);
+      if (!mbar_wait_warp(smem_u32(&full_bar[s]), ph, abortp, ready)) {
+        if (status && lane == 0) atomicCAS(status, ST_OK, ST_TIMEOUT_MMA);
         ok = false;
         break;
       }
-      if (i == 0) timeline_mark(1);                    // first stage complete: activations have arrived
-      else if (i == STAGES) timeline_mark(2);          // first stage whose weights were not requested ahead of the wait
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t sW = tiles + s * SL::STAGE_BYTES;
-      const uint64_t dW = make_smem_desc(sW);
-      const uint64_t dA = make_smem_desc(sW + W_STAGE_BYTES);
-#pragma unroll
-      for (int k = 0; k < TILE_K / UMMA_K; ++k) {
-        // advance 32 bytes (16 bf16) along K inside the swizzle row: +2 in 16-byte units
-        umma_bf16(tmem_d, dW + (uint64_t)(2 * k), dA + (uint64_t)(2 * k), idesc, (i > 0 || k > 0) ? 1u : 0u);
+      if (lane == 0) {
+        if (i == 0) timeline_mark(1);                    // first stage complete: activations have arrived
+        else if (i == STAGES) timeline_mark(2);          // first stage whose weights were not requested ahead of the wait
       }
-      umma_commit(smem_u32(&empty_bar[s]));  // stage reusable once these MMAs have read it
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t sW = tiles + s * SL::STAGE_BYTES, empty = smem_u32(&empty_bar[s]);
       if (++s == STAGES) {
         s = 0;
         ph ^= 1u;
       }
+      ready = mbar_peek_warp(smem_u32(&full_bar[s]), ph);  // answered while the MMAs below are issued
+      if (elect_one()) {
+        const uint64_t dW = make_smem_desc(sW);
+        const uint64_t dA = make_smem_desc(sW + W_STAGE_BYTES);
+#pragma unroll
+        for (int k = 0; k < TILE_K / UMMA_K; ++k) {
+          // advance 32 bytes (16 bf16) along K inside the swizzle row: +2 in 16-byte units
+          umma_bf16(tmem_d, dW + (uint64_t)(2 * k), dA + (uint64_t)(2 * k), idesc, (i > 0 || k > 0) ? 1u : 0u);
+        }
+        umma_commit(empty);  // stage reusable once these MMAs have read it
+        if (i == nkb - 1) umma_commit(smem_u32(&accum_bar));
+      }
+      __syncwarp();
     }
-    if (ok) umma_commit(smem_u32(&accum_bar));
   }
   __syncwarp();
 
@@ -365,54 +376,72 @@ __global__ void __launch_bounds__(128) gemm_bf16_tcgen05_kernel(const __grid_con
   }
 }
 
-// ---------------------------------------------------------------- persistent kernel (many tiles, no split-K)
-// The same product for shapes with more tiles than SMs (many active rows: batched serving, full steps): one
-// CTA per SM walks through tiles blockIdx.x, blockIdx.x + gridDim.x, ... with fixed roles -- warp 0 requests
-// the operand tiles of one tile after the other without a gap, warp 1 issues the MMAs into one of TWO
-// accumulators in tensor memory, warps 2-5 run the epilogue of the accumulator that has just been completed --
-// so the epilogue of a tile (TMEM -> registers -> global, or the SwiGLU / estimate forms) runs under the main
-// loop of the next one and the operand stream never drains between tiles.  Tile order is the launch order of
-// the one-tile kernel including its remap, so CTAs that run together share operands in L2.  The k loop of a
-// tile is the same as in the one-tile kernel: results are bit-identical to it.
-constexpr int PERSIST_THREADS = 192;
+// ---------------------------------------------------------------- persistent CTA-pair kernel
+// The product for more than 128 activation rows, with cta_group::2: two CTAs of a cluster work on one tile of 256 weight rows x BN activation
+// rows.  Each stages its own 128 weight rows and HALF of the activation tile, one thread of the first CTA issues
+// MMAs that read both CTAs' shared memory, and each CTA ends with its own 128 x BN accumulator in its own TMEM.
+// What bounds a product from about 128 activation rows on is the L2 -> SM fabric (about 12.7 TB/s over all SMs on
+// B200): a 128 x 256 tile of one CTA moves 48 KB per k-block of 512 tensor cycles, the pair's share of 256 x 256
+// moves 32 KB.  One pair per two SMs walks through units p, p + pairs, ... (a unit = a tile, or a tile's share of
+// the k range) with fixed roles: warp 0 requests operands without a gap between units, warp 1 issues the MMAs into one
+// of TWO accumulators in tensor memory, and warps 2-5 drain one accumulator while the other fills.  The k loop of a
+// tile is the one-tile kernel's: results are bit-identical to it.  With a
+// split k range every split writes its own slab.  Loads carry no multicast: every byte is requested by the CTA
+// that stages it.
+constexpr int PAIR_THREADS = 192;
 template <int BN>
-struct PersistLayout {
-  static constexpr uint32_t STAGE_BYTES = W_STAGE_BYTES + BN * TILE_K * 2;
+struct PairLayout {
+  static constexpr uint32_t A_HALF_BYTES = (BN / 2) * TILE_K * 2;
+  static constexpr uint32_t STAGE_BYTES = W_STAGE_BYTES + A_HALF_BYTES;
   static constexpr uint32_t EX_BYTES = 64 * 132 * 4;  // staging of the SwiGLU / estimate epilogues
   static constexpr uint32_t total(int stages, bool staged) {
     return (uint32_t)stages * STAGE_BYTES + (staged ? EX_BYTES : 0) + 1024;
   }
+  static constexpr int most(bool staged) {
+    const int fit = (227 * 1024 - 1024 - 512 - (staged ? (int)EX_BYTES : 0)) / (int)STAGE_BYTES;
+    return fit < MAX_STAGES ? fit : MAX_STAGES;
+  }
 };
 
+// Unit u of the walk over m_tiles x n_pairs tiles x splits -> (activation tile, weight pair, split).  Splits are
+// outermost; inside, groups of RASTER activation tiles with the weight pairs inside a group, so that pairs that
+// run together share operands in L2.
+__device__ __forceinline__ void pair_unit(int u, int m_tiles, int n_pairs, int& mt, int& np, int& z) {
+  const int tiles = m_tiles * n_pairs;
+  z = u / tiles;
+  const int t = u - z * tiles, per = RASTER * n_pairs, grp = t / per, within = t - grp * per;
+  const int wide = min(RASTER, m_tiles - grp * RASTER);
+  np = within / wide;
+  mt = grp * RASTER + within - np * wide;
+}
+
 template <int BN>
-__global__ void __launch_bounds__(PERSIST_THREADS, 1)
-    gemm_bf16_persistent_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmA,
-                                float* __restrict__ part, int M, int N, int num_kb, int m_tiles, int n_tiles,
-                                int STAGES, __nv_bfloat16* __restrict__ act_out, int m_ffn, int* __restrict__ status) {
-  using PL = PersistLayout<BN>;
-  static_assert(2 * BN <= 512, "two accumulators must fit the 512 columns of tensor memory");
+__global__ void __launch_bounds__(PAIR_THREADS, 1)
+    gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmA,
+                          float* __restrict__ part, int M, int N, int num_kb, int kb_per_split, size_t split_stride,
+                          int m_tiles, int n_pairs, int units, int STAGES, __nv_bfloat16* __restrict__ act_out,
+                          int m_ffn, int* __restrict__ status) {
+  using PL = PairLayout<BN>;
   // column distance of the two accumulators: an allocation is a power of two, so 192-row tiles sit 256 apart
   constexpr uint32_t ACC = BN > 128 ? 256 : BN > 64 ? 128 : BN > 32 ? 64 : 32;
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full_bar[MAX_STAGES];
-  __shared__ __align__(8) uint64_t empty_bar[MAX_STAGES];
-  __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
+  __shared__ __align__(8) uint64_t full_bar[MAX_STAGES];   // used in the pair's first CTA: bytes of both CTAs
+  __shared__ __align__(8) uint64_t empty_bar[MAX_STAGES];  // in each CTA: its stage may be refilled
+  __shared__ __align__(8) uint64_t acc_full[2];            // in each CTA: accumulator complete
+  __shared__ __align__(8) uint64_t acc_empty[2];           // used in the first CTA: both CTAs' epilogues have read it
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = (int)cluster_ctarank();
+  const bool leader = rank == 0;
+  const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
   const uint32_t tiles_s = (smem_u32(smem_raw) + 1023u) & ~1023u;
   float* ex = reinterpret_cast<float*>(smem_raw + (tiles_s - smem_u32(smem_raw)) + (size_t)STAGES * PL::STAGE_BYTES);
-  const int total_tiles = m_tiles * n_tiles;
-  // tile L of the walk -> (activation tile, weight tile): groups of RASTER activation tiles, weight tiles inside
-  auto tile_of = [&](int L, int& mt, int& nt) {
-    const int per = RASTER * n_tiles, grp = L / per, within = L - grp * per;
-    const int wide = min(RASTER, m_tiles - grp * RASTER);
-    nt = within / wide;
-    mt = grp * RASTER + within - nt * wide;
-  };
+  // k-blocks of split z: [z * kb_per_split, kb_end(z)), never empty by construction of the plan
+  auto kb_end = [&](int z) { return min(num_kb, (z + 1) * kb_per_split); };
 
-  if (threadIdx.x == 0) {
+  if (warp == 0 && elect_one()) {
     abort_flag = 0;
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(smem_u32(&full_bar[s]), 1);
@@ -420,99 +449,125 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(smem_u32(&acc_full[a]), 1);
-      mbar_init(smem_u32(&acc_empty[a]), 128);  // every epilogue thread arrives once it has read its part
+      mbar_init(smem_u32(&acc_empty[a]), 2 * 4);  // one arrival per epilogue warp of both CTAs
     }
     mbar_fence_init();
     prefetch_tensormap(&tmW);
     prefetch_tensormap(&tmA);
   }
-  if (warp == 1) {  // TMEM: two accumulators of BN fp32 columns x 128 lanes
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
+  if (warp == 1) {  // the same warp of both CTAs: two accumulators of BN fp32 columns x 128 lanes in each CTA's TMEM
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
                  "r"(2u * ACC)
                  : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  cluster_sync();  // both CTAs' barriers exist before either signals the other's
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_d = tmem_base_slot;
   volatile int* abortp = &abort_flag;
+
+  int pre = 0;  // stages whose weight tile was requested before the dependency wait
+  if (warp == 0 && pair < units) {
+    int mt, np, z;
+    pair_unit(pair, m_tiles, n_pairs, mt, np, z);
+    const int kb0 = z * kb_per_split;
+    pre = min(STAGES, kb_end(z) - kb0);  // weights are written by no kernel: stream them ahead of the dependency
+    if (elect_one())
+      for (int i = 0; i < pre; ++i) {
+        if (leader) mbar_expect_tx(smem_u32(&full_bar[i]), 2 * PL::STAGE_BYTES);
+        tma_load_2d_pair(tiles_s + i * PL::STAGE_BYTES, &tmW, cluster_addr(smem_u32(&full_bar[i]), 0),
+                         (kb0 + i) * TILE_K, (2 * np + rank) * TILE_W);
+      }
+    __syncwarp();
+  }
   pdl_wait();     // the activation rows and the output buffer belong to the preceding kernels
   pdl_trigger();
   bool ok = true;
 
   if (warp == 0) {
-    // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      int s = 0;
-      uint32_t ph = 0;
-      for (int L = blockIdx.x; L < total_tiles && ok; L += gridDim.x) {
-        int mt, nt;
-        tile_of(L, mt, nt);
-        for (int kb = 0; kb < num_kb; ++kb) {
-          if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, abortp)) {
-            if (status) atomicCAS(status, ST_OK, ST_TIMEOUT_TMA);
-            ok = false;
-            break;
-          }
-          const uint32_t fb = smem_u32(&full_bar[s]);
+    // ---------------- TMA producer (both CTAs) ----------------
+    int s = 0, issued = 0;
+    uint32_t ph = 0;
+    for (int u = pair; u < units && ok; u += pairs) {
+      int mt, np, z;
+      pair_unit(u, m_tiles, n_pairs, mt, np, z);
+      const int n0 = (2 * np + rank) * TILE_W, m0 = mt * BN + rank * (BN / 2);
+      const int kb1 = kb_end(z);
+      for (int kb = z * kb_per_split; kb < kb1; ++kb, ++issued) {
+        if (issued >= pre && !mbar_wait_warp(smem_u32(&empty_bar[s]), ph ^ 1u, abortp)) {
+          if (status && lane == 0) atomicCAS(status, ST_OK, ST_TIMEOUT_TMA);
+          ok = false;
+          break;
+        }
+        if (elect_one()) {
+          const uint32_t fb = cluster_addr(smem_u32(&full_bar[s]), 0);
           const uint32_t dst = tiles_s + s * PL::STAGE_BYTES;
-          mbar_expect_tx(fb, PL::STAGE_BYTES);
-          tma_load_2d(dst, &tmW, fb, kb * TILE_K, nt * TILE_W);
-          tma_load_2d(dst + W_STAGE_BYTES, &tmA, fb, kb * TILE_K, mt * BN);
-          if (++s == STAGES) {
-            s = 0;
-            ph ^= 1u;
+          if (issued >= pre) {
+            if (leader) mbar_expect_tx(smem_u32(&full_bar[s]), 2 * PL::STAGE_BYTES);
+            tma_load_2d_pair(dst, &tmW, fb, kb * TILE_K, n0);
           }
+          tma_load_2d_pair(dst + W_STAGE_BYTES, &tmA, fb, kb * TILE_K, m0);
+        }
+        __syncwarp();
+        if (++s == STAGES) {
+          s = 0;
+          ph ^= 1u;
         }
       }
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      constexpr uint32_t idesc = make_idesc(TILE_W, BN);
+    // ---------------- MMA issuer (first CTA of the pair) ----------------
+    if (leader) {
+      constexpr uint32_t idesc = make_idesc(2 * TILE_W, BN);
       int s = 0, j = 0;
       uint32_t ph = 0;
-      for (int L = blockIdx.x; L < total_tiles && ok; L += gridDim.x, ++j) {
+      bool ready = false;
+      for (int u = pair; u < units && ok; u += pairs, ++j) {
         const int a = j & 1;
-        // the epilogue of the tile that used this accumulator two tiles ago has read it
-        if (!mbar_wait(smem_u32(&acc_empty[a]), ((uint32_t)(j >> 1) & 1u) ^ 1u, abortp)) {
-          if (status) atomicCAS(status, ST_OK, ST_TIMEOUT_MMA);
+        const int z = u / (m_tiles * n_pairs), kb0 = z * kb_per_split, kb1 = kb_end(z);
+        // the epilogues of the unit that used this accumulator two units ago have read it
+        if (!mbar_wait_warp(smem_u32(&acc_empty[a]), ((uint32_t)(j >> 1) & 1u) ^ 1u, abortp)) {
+          if (status && lane == 0) atomicCAS(status, ST_OK, ST_TIMEOUT_MMA);
           ok = false;
           break;
         }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        for (int kb = 0; kb < num_kb; ++kb) {
-          if (!mbar_wait(smem_u32(&full_bar[s]), ph, abortp)) {
-            if (status) atomicCAS(status, ST_OK, ST_TIMEOUT_MMA);
+        for (int kb = kb0; kb < kb1; ++kb) {
+          if (!mbar_wait_warp(smem_u32(&full_bar[s]), ph, abortp, ready)) {
+            if (status && lane == 0) atomicCAS(status, ST_OK, ST_TIMEOUT_MMA);
             ok = false;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t sW = tiles_s + s * PL::STAGE_BYTES;
-          const uint64_t dW = make_smem_desc(sW);
-          const uint64_t dA = make_smem_desc(sW + W_STAGE_BYTES);
-#pragma unroll
-          for (int k = 0; k < TILE_K / UMMA_K; ++k)
-            umma_bf16(tmem_d + (uint32_t)a * ACC, dW + (uint64_t)(2 * k), dA + (uint64_t)(2 * k), idesc,
-                      (kb > 0 || k > 0) ? 1u : 0u);
-          umma_commit(smem_u32(&empty_bar[s]));  // stage reusable once these MMAs have read it
+          const uint32_t sW = tiles_s + s * PL::STAGE_BYTES, empty = smem_u32(&empty_bar[s]);
           if (++s == STAGES) {
             s = 0;
             ph ^= 1u;
           }
+          ready = mbar_peek_warp(smem_u32(&full_bar[s]), ph);  // answered while the MMAs below are issued
+          if (elect_one()) {
+            const uint64_t dW = make_smem_desc(sW);
+            const uint64_t dA = make_smem_desc(sW + W_STAGE_BYTES);
+#pragma unroll
+            for (int k = 0; k < TILE_K / UMMA_K; ++k)
+              umma_bf16_pair(tmem_d + (uint32_t)a * ACC, dW + (uint64_t)(2 * k), dA + (uint64_t)(2 * k), idesc,
+                             (kb > kb0 || k > 0) ? 1u : 0u);
+            umma_commit_pair(empty);  // both CTAs may refill the stage once these MMAs have read it
+            if (kb == kb1 - 1) umma_commit_pair(smem_u32(&acc_full[a]));
+          }
+          __syncwarp();
         }
-        if (ok) umma_commit(smem_u32(&acc_full[a]));
       }
     }
   } else {
-    // ---------------- epilogue warps 2..5: TMEM lanes 32 * (warp % 4) .. + 31 ----------------
+    // ---------------- epilogue warps 2..5 of both CTAs: own 128 weight rows, TMEM lanes 32 * (warp % 4) .. + 31 ----
     const int tl = (warp & 3) * 32 + lane;
     int j = 0;
-    for (int L = blockIdx.x; L < total_tiles; L += gridDim.x, ++j) {
+    for (int u = pair; u < units; u += pairs, ++j) {
       const int a = j & 1;
-      int mt, nt;
-      tile_of(L, mt, nt);
+      int mt, np, z;
+      pair_unit(u, m_tiles, n_pairs, mt, np, z);
       bool have = mbar_wait(smem_u32(&acc_full[a]), (uint32_t)(j >> 1) & 1u, abortp);
       // the 128 epilogue threads agree (the TMEM loads are warp-collective and the staged forms exchange data)
       {
@@ -532,162 +587,22 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
         ok = false;
         break;
       }
-      gemm_epilogue<BN, 1>(tmem_d + (uint32_t)a * ACC, ex, tl, mt * BN, nt * TILE_W, nt, M, N, part, act_out, m_ffn);
+      const int nt = 2 * np + rank;
+      if (nt * TILE_W < N)  // the second CTA of the last pair has no rows when the weight tiles are odd in number
+        gemm_epilogue<BN, 1>(tmem_d + (uint32_t)a * ACC, ex, tl, mt * BN, nt * TILE_W, nt, M, N,
+                             part + (size_t)z * split_stride, act_out, m_ffn);
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      mbar_arrive(smem_u32(&acc_empty[a]));
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(cluster_addr(smem_u32(&acc_empty[a]), 0));
     }
   }
   ok = __syncthreads_and(ok);
   if (!ok) drain_delay();  // gave up: let copies in flight land before shared memory is released
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 1) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(2u * ACC) : "memory");
-  }
-}
-
-// ---------------------------------------------------------------- CTA-pair kernel
-// The same product with cta_group::2: two CTAs of a cluster (consecutive weight tiles, blockIdx.x = 2p, 2p + 1)
-// work on one 256 x BN tile.  Each stages its own 128 weight rows and HALF of the activation tile, the first CTA
-// of the pair issues MMAs that read both CTAs' shared memory, and each CTA ends with its own 128 x BN
-// accumulator in its own TMEM.  Against the one-CTA kernel the activation tile crosses the L2 -> SM fabric once
-// per 256 weight rows instead of once per 128, which is what bounds the product from about 128 activation rows
-// on.  Loads carry no multicast: every byte is requested by the CTA that stages it.
-template <int BN>
-struct PairLayout {
-  static constexpr uint32_t A_HALF_BYTES = (BN / 2) * TILE_K * 2;
-  static constexpr uint32_t STAGE_BYTES = W_STAGE_BYTES + A_HALF_BYTES;
-  static constexpr uint32_t total(int stages) { return (uint32_t)stages * STAGE_BYTES + 1024; }
-};
-
-template <int BN>
-__global__ void __launch_bounds__(128) gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmW,
-                                                             const __grid_constant__ CUtensorMap tmA,
-                                                             float* __restrict__ part, int M, int N, int num_kb,
-                                                             int kb_per_split, size_t split_stride, int STAGES,
-                                                             __nv_bfloat16* __restrict__ act_out, int m_ffn,
-                                                             int* __restrict__ status) {
-  using PL = PairLayout<BN>;
-  extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full_bar[MAX_STAGES];   // used in the pair's first CTA: bytes of both CTAs
-  __shared__ __align__(8) uint64_t empty_bar[MAX_STAGES];  // in each CTA: its stage may be refilled
-  __shared__ __align__(8) uint64_t accum_bar;              // in each CTA: the accumulator is complete
-  __shared__ uint32_t tmem_base_slot;
-  __shared__ int abort_flag;
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();
-  const bool leader = rank == 0;
-  const int m0 = blockIdx.y * BN;
-  const int n0 = blockIdx.x * TILE_W;  // the pair: blockIdx.x = 2p, 2p + 1
-  const int kb0 = blockIdx.z * kb_per_split;
-  const int kb1 = min(num_kb, kb0 + kb_per_split);
-  const int nkb = kb1 - kb0;
-  const uint32_t tiles = (smem_u32(smem_raw) + 1023u) & ~1023u;
-
-  if (threadIdx.x == 0) {
-    abort_flag = 0;
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(smem_u32(&full_bar[s]), 1);
-      mbar_init(smem_u32(&empty_bar[s]), 1);
-    }
-    mbar_init(smem_u32(&accum_bar), 1);
-    mbar_fence_init();
-    prefetch_tensormap(&tmW);
-    prefetch_tensormap(&tmA);
-  }
-  if (warp == 1) {  // the same warp of both CTAs: BN fp32 columns x 128 lanes in each CTA's TMEM
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
-                 "r"((uint32_t)BN)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  cluster_sync();  // both CTAs' barriers exist before either signals the other's
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem_d = tmem_base_slot;
-  volatile int* abortp = &abort_flag;
-
-  int pre = 0;
-  if (threadIdx.x == 0) {
-    pre = min(STAGES, nkb);  // weights are written by no kernel: stream them ahead of the dependency
-    for (int i = 0; i < pre; ++i) {
-      if (leader) mbar_expect_tx(smem_u32(&full_bar[i]), 2 * PL::STAGE_BYTES);
-      tma_load_2d_pair(tiles + i * PL::STAGE_BYTES, &tmW, cluster_addr(smem_u32(&full_bar[i]), 0), (kb0 + i) * TILE_K, n0);
-    }
-  }
-  pdl_wait();     // the activation rows and the slab buffer belong to the preceding kernels
-  pdl_trigger();
-
-  if (warp == 0 && lane == 0) {
-    // ---------------- TMA producer (both CTAs) ----------------
-    int s = 0;
-    uint32_t ph = 0;
-    for (int i = 0; i < nkb; ++i) {
-      const uint32_t fb = cluster_addr(smem_u32(&full_bar[s]), 0);
-      const uint32_t dstW = tiles + s * PL::STAGE_BYTES;
-      const int kc = (kb0 + i) * TILE_K;
-      if (i >= pre) {
-        if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, abortp)) {
-          if (status) atomicCAS(status, ST_OK, ST_TIMEOUT_TMA);
-          break;
-        }
-        if (leader) mbar_expect_tx(smem_u32(&full_bar[s]), 2 * PL::STAGE_BYTES);
-        tma_load_2d_pair(dstW, &tmW, fb, kc, n0);
-      }
-      tma_load_2d_pair(dstW + W_STAGE_BYTES, &tmA, fb, kc, m0 + (int)rank * (BN / 2));
-      if (++s == STAGES) {
-        s = 0;
-        ph ^= 1u;
-      }
-    }
-  } else if (leader && warp == 1 && lane == 0) {
-    // ---------------- MMA issuer (first CTA of the pair) ----------------
-    constexpr uint32_t idesc = make_idesc(2 * TILE_W, BN);
-    bool ok = true;
-    int s = 0;
-    uint32_t ph = 0;
-    for (int i = 0; i < nkb && ok; ++i) {
-      if (!mbar_wait(smem_u32(&full_bar[s]), ph, abortp)) {
-        if (status) atomicCAS(status, ST_OK, ST_TIMEOUT_MMA);
-        ok = false;
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t sW = tiles + s * PL::STAGE_BYTES;
-      const uint64_t dW = make_smem_desc(sW);
-      const uint64_t dA = make_smem_desc(sW + W_STAGE_BYTES);
-#pragma unroll
-      for (int k = 0; k < TILE_K / UMMA_K; ++k)
-        umma_bf16_pair(tmem_d, dW + (uint64_t)(2 * k), dA + (uint64_t)(2 * k), idesc, (i > 0 || k > 0) ? 1u : 0u);
-      umma_commit_pair(smem_u32(&empty_bar[s]));  // both CTAs may refill the stage once these MMAs have read it
-      if (++s == STAGES) {
-        s = 0;
-        ph ^= 1u;
-      }
-    }
-    if (ok) umma_commit_pair(smem_u32(&accum_bar));
-  }
-  __syncwarp();
-
-  // ---------------- epilogue: each CTA writes its own 128 output columns ----------------
-  const bool have = mbar_wait(smem_u32(&accum_bar), 0u, abortp);
-  if (!have && threadIdx.x == 0 && status) atomicCAS(status, ST_OK, ST_TIMEOUT_EPI);
-  bool warp_ok = __all_sync(0xffffffffu, have);
-  if (act_out || m_ffn < 0) warp_ok = __syncthreads_and(warp_ok);
-  if (warp_ok) {
-    float* ex = reinterpret_cast<float*>(smem_raw + (tiles - smem_u32(smem_raw)));  // the drained ring
-    gemm_epilogue<BN>(tmem_d, ex, (int)threadIdx.x, m0, n0, (int)blockIdx.x, M, N,
-                      part + (size_t)blockIdx.z * split_stride, act_out, m_ffn);
-  } else {
-    drain_delay();
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
   cluster_sync();  // neither CTA leaves, nor is TMEM freed, while the other may still use this one's memory
   if (warp == 1) {
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"((uint32_t)BN) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(2u * ACC) : "memory");
   }
 }
 
@@ -780,44 +695,24 @@ cudaError_t launch_one(const Launch& L, const CUtensorMap& tmW, const CUtensorMa
 }
 
 template <int BN>
-cudaError_t launch_persistent(const Launch& L, const CUtensorMap& tmW, const CUtensorMap& tmA, float* part, int M,
-                              int N, int num_kb, const GemmPlan& plan, void* act_out, int m_ffn) {
-  using PL = PersistLayout<BN>;
-  const bool staged = act_out != nullptr || m_ffn < 0;
-  const int fit = (227 * 1024 - 1024 - 512 - (staged ? (int)PL::EX_BYTES : 0)) / (int)PL::STAGE_BYTES;
-  const int stages = fit < MAX_STAGES ? fit : MAX_STAGES;
-  static DeviceOnce once;
-  cudaError_t e0 = once.run([] {
-    return cudaFuncSetAttribute(gemm_bf16_persistent_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                227 * 1024 - 512);
-  });
-  if (e0 != cudaSuccess) return e0;
-  const int n_tiles = (N + TILE_W - 1) / TILE_W, m_tiles = (M + BN - 1) / BN;
-  const int ctas = std::min(m_tiles * n_tiles, sm_count());
-  cudaError_t e = launch_k(L, gemm_bf16_persistent_kernel<BN>, dim3(ctas), dim3(PERSIST_THREADS),
-                           PL::total(stages, staged), tmW, tmA, part, M, N, num_kb, m_tiles, n_tiles, stages,
-                           (__nv_bfloat16*)act_out, m_ffn, L.d_status);
-  L.count();
-  return e != cudaSuccess ? e : cudaGetLastError();
-}
-
-template <int BN>
 cudaError_t launch_pair(const Launch& L, const CUtensorMap& tmW, const CUtensorMap& tmA, float* part, int M, int N,
                         int num_kb, const GemmPlan& plan, void* act_out, int m_ffn) {
   using PL = PairLayout<BN>;
-  constexpr int fit = (227 * 1024 - 1024 - 256) / (int)PL::STAGE_BYTES;
-  constexpr int most = fit < MAX_STAGES ? fit : MAX_STAGES;
+  const bool staged = act_out != nullptr || m_ffn < 0;
   static DeviceOnce once;
   cudaError_t e0 = once.run([] {
     return cudaFuncSetAttribute(gemm_bf16_pair_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)PL::total(most));
+                                227 * 1024 - 512);
   });
   if (e0 != cudaSuccess) return e0;
-  const int stages = plan.stages < 2 ? 2 : plan.stages > most ? most : plan.stages;
-  dim3 grid(N / TILE_W, (M + BN - 1) / BN, plan.S_max);  // pairs along x
-  cudaError_t e = launch_k_cluster(L, gemm_bf16_pair_kernel<BN>, grid, dim3(128), PL::total(stages), dim3(2, 1, 1), tmW,
-                                   tmA, part, M, N, num_kb, plan.upc, (size_t)M * N, stages, (__nv_bfloat16*)act_out,
-                                   m_ffn, L.d_status);
+  const int most = PL::most(staged), stages = plan.stages < 2 ? 2 : plan.stages > most ? most : plan.stages;
+  const int m_tiles = (M + BN - 1) / BN, n_pairs = (N + 2 * TILE_W - 1) / (2 * TILE_W);
+  const int units = m_tiles * n_pairs * plan.S_max;
+  const int pairs = std::min(units, sm_count() / 2);
+  cudaError_t e = launch_k_cluster(L, gemm_bf16_pair_kernel<BN>, dim3(2 * pairs), dim3(PAIR_THREADS),
+                                   PL::total(stages, staged), dim3(2, 1, 1), tmW, tmA, part, M, N, num_kb, plan.upc,
+                                   (size_t)M * N, m_tiles, n_pairs, units, stages, (__nv_bfloat16*)act_out, m_ffn,
+                                   L.d_status);
   L.count();
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -848,88 +743,81 @@ int sm_count() {
 }
 
 // tuning / test override of the kernel choice for unsplit plans with 256-row tiles: 0 automatic, 1 always the
-// persistent kernel, -1 never (see dllm_debug_gemm_plan)
+// persistent pair kernel, -1 the one-tile kernel (see dllm_debug_gemm_plan)
 int g_gemm_force_persistent = 0;
 
 Partials make_partials(const float* p, int M, int N, const GemmPlan& plan) {
   return Partials{p, (size_t)M * N, plan.S_max, N};  // every element has S_max slabs
 }
 
-// Tile shape, ring depth and split-K factor, from sweeps on B200: up to 256
-// activation rows the product is bound by streaming W, so k ranges are split
-// until at least one CTA per SM (two with 128-row tiles) streams weights.
+// Activation tile and split of the persistent pair kernel, by what bounds it: the pairs work in rounds of whole
+// units, a k-block of a unit takes the larger of the issue / tensor time of its tile (0.33 / 0.27 / 0.25 us for 256 /
+// 192 / 128 rows) and its bytes' share of the L2 -> SM fabric (12 TB/s over all SMs: 0.40 / 0.35 / 0.30 us when every
+// SM is busy), and a split adds slabs that are written and read once more (10 TB/s).  Measured with it, B200, us
+// (before -> now): 768 x 4096 x 12288 77 -> 63, 768 x 24576 x 4096 120 -> 110, 4096 x 24576 x 4096 614 -> 583, 4096 x
+// 4096 x 12288 362 -> 306, 24576 x 4096 x 4096 711 -> 646, 256 x 126464 x 4096 258 -> 221.
+static void plan_pair(int M, int N, int K, int max_split, int* bn, int* splits) {
+  const int pairs = sm_count() / 2, num_kb = (K + TILE_K - 1) / TILE_K;
+  const long n_pairs = (N + 2 * TILE_W - 1) / (2 * TILE_W);
+  double best = -1.0;
+  for (int BN : {256, 192, 128}) {
+    const long tiles = n_pairs * ((M + BN - 1) / BN);
+    const double issue = BN == 256 ? 0.33 : BN == 192 ? 0.27 : 0.25, bytes = (TILE_W + BN / 2) * TILE_K * 2.0;
+    for (int S = 1; S == 1 || (S <= max_split && S * tiles <= pairs && S <= num_kb / 4); ++S) {
+      const long units = tiles * S, rounds = (units + pairs - 1) / pairs;
+      const double ctas = 2.0 * (units < pairs ? units : pairs), fabric = bytes * ctas / 12.0e6;
+      const double us = (double)rounds * ((num_kb + S - 1) / S) * (issue > fabric ? issue : fabric) +
+                        (S > 1 ? S * (double)M * N * 8.0 / 10.0e6 : 0.0);
+      if (best < 0.0 || us < best) {
+        best = us;
+        *bn = BN;
+        *splits = S;
+      }
+    }
+  }
+}
+
+// Tile shape, ring depth and split-K factor, from sweeps on B200.  Up to 128 activation rows the product is bound by
+// streaming W: one CTA per weight tile, k ranges split until at least one CTA per SM (two with 128-row tiles) streams
+// weights.  Above that the activation tile's trips through the L2 -> SM fabric bound it: CTA pairs.
 GemmPlan plan_gemm_bf16(int M, int N, int K, int force_split, int force_stages, int force_bn, int force_pair,
                         int force_persistent) {
   GemmPlan p;
   const int sms = sm_count();
   const long n_tiles = (N + TILE_W - 1) / TILE_W;
+  if (force_persistent == 0) force_persistent = g_gemm_force_persistent;
+  p.num_kb = (K + TILE_K - 1) / TILE_K;
   p.BN = M <= 32 ? 32 : M <= 64 ? 64 : M <= 256 ? 128 : 256;
   p.pair = 0;
-  int pair_stages = 3;
-  const bool automatic = force_pair == 0 && force_bn == 0 && force_split == 0;
-  const long tiles64 = n_tiles * ((M + 63) / 64), tiles128 = n_tiles * ((M + 127) / 128);
-  const long tiles256 = n_tiles * ((M + 255) / 256);
-  if (automatic && M > 64 && M <= 128 && tiles64 <= sms) {
+  int S = 0;
+  if (force_pair == 0 && force_bn == 0 && force_split <= 1 && force_persistent >= 0 && M > 128 &&
+      (long)N * K >= 1L << 21) {
+    // (a weight matrix of a few MB is over before a cluster launch pays: with the 448-wide test model's 144 rows the
+    // step took 127 us on pairs, 121 us on the one-tile kernel)
+    p.pair = 1;
+    plan_pair(M, N, K, force_split == 1 ? 1 : 16, &p.BN, &S);
+  } else if (force_pair == 0 && force_bn == 0 && force_split == 0 && M > 64 && M <= 128 && n_tiles * ((M + 63) / 64) <= sms) {
     // 65..128 rows against few weight tiles (the product will be split): two 64-row tiles per weight tile put
     // twice the CTAs on the weight stream (128 x 4096 x 4096: 14.9 against 17.8 us, 128 x 4096 x 3584: 10.0
     // against 11.8 us; with many weight tiles the 128-row tile stays: every weight tile crosses the fabric once)
     p.BN = 64;
-  } else if (automatic && M > 128 && M <= 256 && tiles64 <= sms && (K + TILE_K - 1) / TILE_K <= 64) {
-    // 129..256 rows against few weight tiles and a short k range (256 x 4096 x 4096, the V projection of every
-    // cached step): four 64-row tiles per weight tile with two splits take as long as two 128-row tiles with four
-    // (15.3 against 15.6 us) and leave the consumer half the slabs to sum (19.4 against 20.9 us with the
-    // reduction); with a long k range the doubled weight traffic through the L2 -> SM fabric costs more (256 x
-    // 4096 x 12288: 36.8 against 32.6 us)
-    p.BN = 64;
-  } else if (automatic && M > 256 && M <= 1024 && 2L * sms / tiles128 >= 2) {
-    // so few 128-row tiles that they fill the SMs only when the k range is split: 320 x 4096 x 12288 43.8 against
-    // 66.4 us without a split, 384 x 3584 x 18944 53.8 against 96.0 us, 512 x 4096 x 3584 20.0 against 24.4 us
-    p.BN = 128;
-  } else if (force_pair == 0 && force_bn == 0 && force_split <= 1 && N % (2 * TILE_W) == 0) {
-    // CTA pairs where they measured faster (B200): products that need no split between 129 and 1024 activation
-    // rows, where the activation tile's trips through the L2 -> SM fabric bound the one-CTA kernel.
-    if (M > 128 && M <= 256 && n_tiles >= sms) {   // (65..128 rows: one-CTA 128-row tiles measured 10 % faster)
-      p.pair = 1;
-      p.BN = 256;
-    } else if (M > 256 && M <= 1024 && 4 * tiles128 <= 11L * sms) {
-      // pairs on 128-row tiles up to 2.75 tiles per SM: 768 x 8192 x 4096 44.4 us against 48.3 on 256-row pair
-      // tiles and 52.7 on the persistent kernel (192 tiles of 256 rows are 1.3 waves of its CTAs)
-      p.pair = 1;
-      p.BN = 128;
-      pair_stages = tiles128 <= 2L * sms ? 4 : 3;  // all 128-row pair tiles resident at once: a deeper ring
-    } else if (M > 256 && M <= 1024 && tiles256 <= 2L * sms) {
-      // (with more 256-row tiles than that the persistent kernel below measured faster: gate / up at 512, 768 and
-      // 1024 rows 114 -> 91, 136 -> 127, 181 -> 162 us)
-      p.pair = 1;
-      p.BN = 256;
-    }
-  }
-  // 192-row tiles (persistent kernel only) where they leave at least 15 % fewer padded activation rows than
-  // 256-row tiles: the 576 rows of a mixed step (prompt refresh + adaptive response update) are 3 x 192, not 3 x 256
-  if (!p.pair && p.BN == 256 && force_split <= 1 && force_persistent >= 0 && g_gemm_force_persistent >= 0) {
-    const long pad192 = (M + 191) / 192 * 192L, pad256 = (M + 255) / 256 * 256L;
-    if (pad192 * 115 <= pad256 * 100 && n_tiles * (pad192 / 192) > sms) p.BN = 192;
   }
   if (force_bn == 32 || force_bn == 64 || force_bn == 128 || force_bn == 192 || force_bn == 256) p.BN = force_bn;
-  if (force_pair > 0) p.pair = (p.BN == 128 || p.BN == 256) && N % (2 * TILE_W) == 0;
-  p.stages = force_stages > 0 ? force_stages : p.pair ? pair_stages : (p.BN == 128 ? 3 : 4);
-  p.num_kb = (K + TILE_K - 1) / TILE_K;
+  if (force_pair > 0 || p.BN == 192 || (p.BN == 256 && force_persistent > 0 && force_split <= 1)) p.pair = p.BN >= 64;
+  p.stages = force_stages > 0 ? force_stages : p.pair ? MAX_STAGES : (p.BN == 128 ? 3 : 4);
   p.m_tiles = (M + p.BN - 1) / p.BN;
   const long tiles = (long)p.m_tiles * n_tiles;
-  // every split adds a slab the consumer has to read: with few activation rows
-  // one wave of CTAs is enough, with 128-row tiles two CTAs per SM pay off
-  // (two CTAs per SM also for 64-row tiles when there are two or more of them per weight tile)
-  const bool two_per_sm = p.BN == 128 || (p.BN == 64 && p.m_tiles > 1);
-  int S = two_per_sm ? (int)(2L * sms / tiles) : (int)((sms + tiles - 1) / tiles);  // all CTAs resident at once
-  const int max_s = p.num_kb / 4 > 1 ? p.num_kb / 4 : 1;
-  if (S > max_s) S = max_s;
-  if (S < 1) S = 1;
-  if (p.pair && force_pair == 0) S = 1;
+  if (S == 0) {
+    // every split adds a slab the consumer has to read: with few activation rows
+    // one wave of CTAs is enough, with 128-row tiles two CTAs per SM pay off
+    // (two CTAs per SM also for 64-row tiles when there are two or more of them per weight tile)
+    const bool two_per_sm = !p.pair && (p.BN == 128 || (p.BN == 64 && p.m_tiles > 1));
+    S = two_per_sm ? (int)(2L * sms / tiles) : (int)((sms + tiles - 1) / tiles);  // all CTAs resident at once
+    const int max_s = p.num_kb / 4 > 1 ? p.num_kb / 4 : 1;
+    if (S > max_s) S = max_s;
+    if (S < 1) S = 1;
+  }
   if (force_split > 0) S = force_split < p.num_kb ? force_split : p.num_kb;
-  // more tiles than SMs, no split, one-CTA 256-row tiles: the persistent kernel (epilogue under the next main loop)
-  if (force_persistent == 0) force_persistent = g_gemm_force_persistent;
-  p.persistent = (force_persistent >= 0) && !p.pair && (p.BN == 256 || p.BN == 192) && S == 1 &&
-                 (force_persistent > 0 || tiles > sms || p.BN == 192);
   p.upc = (p.num_kb + S - 1) / S;                 // k-blocks per split
   p.S_max = (p.num_kb + p.upc - 1) / p.upc;       // no empty split
   p.ctas = (int)tiles * p.S_max;
@@ -962,19 +850,12 @@ cudaError_t launch_gemm_bf16(const Launch& L, const void* A, const void* W, floa
   }
   const int num_kb = (K + TILE_K - 1) / TILE_K;
   if (plan.pair) {
-    if (N % (2 * TILE_W)) {
-      if (err) *err = "CTA pairs need N % 256 == 0";
-      return cudaErrorInvalidValue;
+    switch (plan.BN) {
+      case 64: return launch_pair<64>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);
+      case 128: return launch_pair<128>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);
+      case 192: return launch_pair<192>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);
+      default: return launch_pair<256>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);
     }
-    return plan.BN == 128 ? launch_pair<128>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn)
-                          : launch_pair<256>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);
-  }
-  if (plan.persistent)
-    return plan.BN == 192 ? launch_persistent<192>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn)
-                          : launch_persistent<256>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);
-  if (plan.BN == 192) {
-    if (err) *err = "192-row tiles exist in the persistent kernel only";
-    return cudaErrorInvalidValue;
   }
   switch (plan.BN) {
     case 32: return launch_one<32>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);

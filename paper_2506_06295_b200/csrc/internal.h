@@ -192,11 +192,10 @@ struct GemmPlan {
   int upc;          // k-blocks per split
   int ctas;         // grid size
   int S_max;        // split-K factor: slabs per output element
-  int pair = 0;     // 1: CTA pairs (cta_group::2) share the activation tile of BN rows
-  int persistent = 0;  // 1: one CTA per SM walks through the tiles, epilogue under the next tile's main loop
+  int pair = 0;     // 1: persistent CTA pairs (cta_group::2) on tiles of 256 weight rows x BN activation rows
 };
-// 0 = auto.  force_pair: 0 auto, 1 CTA pairs (BN 128 or 256, N a multiple of 256), -1 never.
-// force_persistent: 0 auto, 1 the persistent kernel (unsplit plans with 256-row tiles only), -1 never.
+// 0 = auto.  force_pair: 0 auto, 1 CTA pairs (BN >= 64).  force_persistent: 0 auto, 1 the pair kernel for unsplit
+// plans with 256-row tiles, -1 the one-tile kernel for every automatic plan.
 GemmPlan plan_gemm_bf16(int M, int N, int K, int force_split = 0, int force_stages = 0, int force_bn = 0,
                         int force_pair = 0, int force_persistent = 0);
 Partials make_partials(const float* p, int M, int N, const GemmPlan& plan);

@@ -128,6 +128,22 @@ def test_gemm_bf16_cta_pairs(env, M, N, K, act_tile, splits, stages):
     assert dllm.lib.dllm_gemm_bf16_pair(dA.data_ptr(), dW.data_ptr(), dA.data_ptr(), M, 128, K, 256, 0, 0, None, 0, None) == dllm.INVALID_ARG
 
 
+@pytest.mark.parametrize("M,N,K,act_tile,splits", [
+    (129, 20096, 128, 0, 0),   # default plan, an odd number of weight tiles: the last pair's second CTA has no rows
+    (257, 16500, 136, 0, 0),   # ragged last weight tile and k block
+    (200, 768, 704, 192, 3),   # 192-row tiles with slabs, 11 k-blocks in 3 splits
+    (64, 20480, 64, 64, 1),    # 80 pair tiles of one k-block: more than one round of the pairs
+])
+def test_gemm_bf16_pair_walk(env, M, N, K, act_tile, splits):
+    """Edges of the persistent pair kernel's walk over its units, against the product in float64 (1e-5 as above)."""
+    torch, dllm = env
+    A = torch.from_numpy(synth.round_to_bf16(synth.random_normal((M, K), seed=41))).cuda().to(torch.bfloat16)
+    W = torch.from_numpy(synth.round_to_bf16(synth.random_normal((N, K), seed=42, std=0.05))).cuda().to(torch.bfloat16)
+    got = dllm.gemm_bf16_pair(A, W, act_tile, splits) if act_tile else dllm.gemm_bf16(A, W)
+    dllm.kernel_status()
+    assert rel_l2(got.cpu().numpy(), A.double().cpu().numpy() @ W.double().cpu().numpy().T) < 1e-5
+
+
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
 def test_gemm_simt(env, dtype):
     torch, dllm = env
