@@ -111,6 +111,137 @@ __global__ void __launch_bounds__(128) attn_simt_kernel(const T* __restrict__ q,
 }
 
 
+// The same arithmetic where the grid of attn_simt_kernel would leave the chip empty (few rows: the step of a small
+// model): a CTA takes four queries of one head and its eight warps take DIFFERENT chunks of 32 keys (warp w the chunks
+// w, w + 8, ...), so 96 keys are one chunk deep instead of three with a block barrier each; the warps' results are merged
+// in warp order.  lane = key for the scores (K straight from memory, q broadcast from shared memory), lane = output
+// column for P V.
+template <typename T, int ND>
+__global__ void __launch_bounds__(256, 1) attn_simt_few_kernel(const T* __restrict__ q, const T* __restrict__ Kc,
+                                                            const T* __restrict__ Vc, T* __restrict__ o, int a_seq, int n,
+                                                            int H, int Hkv, float scale) {
+  constexpr int HD = 32 * ND, NQ = 4, NW = 8;
+  __shared__ __align__(16) float qs[NQ][HD];
+  __shared__ float part[NW][NQ][HD], pm[NW][NQ], pl[NW][NQ];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int q0 = blockIdx.x * NQ, h = blockIdx.y, b = blockIdx.z, kh = h / (H / Hkv);
+  const int dq = H * HD, dkv = Hkv * HD;
+  pdl_wait();
+  pdl_trigger();
+  const T* Kb = Kc + (size_t)b * n * dkv + kh * HD;
+  const T* Vb = Vc + (size_t)b * n * dkv + kh * HD;
+  float m_run[NQ], l_run[NQ], acc[NQ][ND] = {};
+#pragma unroll
+  for (int t = 0; t < NQ; ++t) m_run[t] = -INFINITY, l_run[t] = 0.f;
+  constexpr int VB = ND <= 2 ? 32 : 16;   // V rows in flight (registers)
+  bool staged = false;
+  for (int k0 = warp * 32; k0 < n || !staged; k0 += NW * 32) {
+    // K row of this lane's key, the first V rows and (first trip) the queries are requested together
+    const int keys = min(32, n - k0);     // <= 0: this warp has no keys and only takes part in the staging
+    const bool valid = lane < keys;
+    float kv[HD], v[VB][ND];
+    auto load_v = [&](int j0) {
+#pragma unroll
+      for (int j = 0; j < VB; ++j)
+#pragma unroll
+        for (int d = 0; d < ND; ++d) v[j][d] = to_f32<T>(Vb[(size_t)(k0 + min(j0 + j, keys - 1)) * dkv + lane + 32 * d]);
+    };
+    if (keys > 0) {
+      const T* krow = Kb + (size_t)(k0 + (valid ? lane : 0)) * dkv;
+#pragma unroll
+      for (int c = 0; c < HD; c += 8) Vec8<T>::load(krow + c, *reinterpret_cast<float(*)[8]>(kv + c));
+      load_v(0);
+    }
+    if (!staged) {
+      for (int e = threadIdx.x; e < NQ * HD; e += 256) {
+        const int r = e / HD, c = e % HD;
+        qs[r][c] = q0 + r < a_seq ? to_f32<T>(q[((size_t)b * a_seq + q0 + r) * dq + h * HD + c]) * scale : 0.f;
+      }
+      __syncthreads();
+      staged = true;
+      if (keys <= 0) break;
+    }
+    float s[NQ] = {};
+#pragma unroll
+    for (int c = 0; c < HD; c += 4)
+#pragma unroll
+      for (int t = 0; t < NQ; ++t) {
+        const float4 f = *reinterpret_cast<const float4*>(&qs[t][c]);
+        s[t] = fmaf(f.x, kv[c], fmaf(f.y, kv[c + 1], fmaf(f.z, kv[c + 2], fmaf(f.w, kv[c + 3], s[t]))));
+      }
+    float p[NQ];
+#pragma unroll
+    for (int t = 0; t < NQ; ++t) {
+      const float sv = valid ? s[t] : -INFINITY;
+      const float m_new = fmaxf(m_run[t], warp_max(sv)), corr = expf(m_run[t] - m_new);  // first chunk: exp(-inf) = 0
+      p[t] = valid ? expf(sv - m_new) : 0.f;
+      l_run[t] = l_run[t] * corr + warp_sum(p[t]);
+      m_run[t] = m_new;
+#pragma unroll
+      for (int d = 0; d < ND; ++d) acc[t][d] *= corr;
+    }
+#pragma unroll
+    for (int j0 = 0; j0 < 32; j0 += VB) {
+      if (j0 > 0) {
+        if (j0 >= keys) break;
+        load_v(j0);
+      }
+#pragma unroll
+      for (int j = 0; j < VB; ++j)
+#pragma unroll
+        for (int t = 0; t < NQ; ++t) {
+          const float pj = __shfl_sync(0xffffffffu, p[t], j0 + j);   // keys past the end: p = 0
+#pragma unroll
+          for (int d = 0; d < ND; ++d) acc[t][d] = fmaf(pj, v[j][d], acc[t][d]);
+        }
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < NQ; ++t) {
+#pragma unroll
+    for (int d = 0; d < ND; ++d) part[warp][t][lane + 32 * d] = acc[t][d];
+    if (lane == 0) pm[warp][t] = m_run[t], pl[warp][t] = l_run[t];
+  }
+  __syncthreads();
+  const int used = min(NW, (n + 31) / 32);   // warps that had keys
+  for (int e = threadIdx.x; e < NQ * HD; e += 256) {
+    const int t = e / HD, c = e % HD;
+    if (q0 + t >= a_seq) continue;
+    float m = -INFINITY, l = 0.f, x = 0.f;
+    for (int w = 0; w < used; ++w) m = fmaxf(m, pm[w][t]);
+    for (int w = 0; w < used; ++w) {
+      const float f = expf(pm[w][t] - m);
+      l += f * pl[w][t];
+      x += f * part[w][t][c];
+    }
+    o[((size_t)b * a_seq + q0 + t) * dq + h * HD + c] = from_f32<T>(x / l);
+  }
+}
+
+template <typename T>
+void launch_simt(const Launch& L, const void* q, const void* Kc, const void* Vc, void* o, int B, int a_seq, int n, int H,
+                 int Hkv, int hd) {
+  const float scale = 1.0f / sqrtf((float)hd);
+  const long ctas = (long)((a_seq + TQ - 1) / TQ) * H * B;
+  // below two CTAs of 16 queries per SM the warps share the keys instead of the queries (four times the CTAs); above, the
+  // 16 queries of a CTA share each key's trip into shared memory
+  const bool aligned = (((uintptr_t)Kc) & 15) == 0 && (Hkv * hd * sizeof(T)) % 16 == 0;
+  if (ctas < 2L * sm_count() && aligned) {
+    const dim3 grid((a_seq + 3) / 4, H, B);
+    auto go = [&](auto* kernel) {
+      launch_k(L, kernel, grid, dim3(256), 0, (const T*)q, (const T*)Kc, (const T*)Vc, (T*)o, a_seq, n, H, Hkv, scale);
+    };
+    if (hd == 32) go(attn_simt_few_kernel<T, 1>);
+    else if (hd == 64) go(attn_simt_few_kernel<T, 2>);
+    else if (hd == 96) go(attn_simt_few_kernel<T, 3>);
+    else go(attn_simt_few_kernel<T, 4>);
+  } else {
+    launch_k(L, attn_simt_kernel<T>, dim3((a_seq + TQ - 1) / TQ, H, B), dim3(128), 0, (const T*)q, (const T*)Kc,
+             (const T*)Vc, (T*)o, a_seq, n, H, Hkv, hd, scale);
+  }
+  L.count();
+}
+
 // ============================================================================
 // attn_mma_kernel (bf16): one CTA of 128 threads runs one attn_tile (see
 // attention_core.cuh): 64 (query, head-of-group) rows of one (sequence, KV
@@ -568,7 +699,7 @@ cudaError_t launch_attention(const Launch& L, int dtype, const void* q, const vo
                              int a_seq, int n, int H, int Hkv, int hd, float* scratch, size_t scratch_floats,
                              bool force_simt, int k_static, int v_static) {
   if (B <= 0 || a_seq <= 0) return cudaSuccess;
-  if (hd > HD_MAX || (hd & 31) || H % Hkv) return cudaErrorInvalidValue;
+  if (hd > HD_MAX || hd < 32 || (hd & 31) || H % Hkv) return cudaErrorInvalidValue;
   const bool tensor = dtype == 1 && !force_simt && (hd == 64 || hd == 128) && ((Hkv * hd) % 8 == 0);
   const AttnChoice ch = tensor ? choose_attention(B, a_seq, n, H, Hkv, scratch ? scratch_floats : 0) : AttnChoice{};
   if (tensor && ch.umma) {
@@ -598,16 +729,10 @@ cudaError_t launch_attention(const Launch& L, int dtype, const void* q, const vo
     return hd == 64 ? launch_mma<64>(L, tmK, tmV, q, o, scratch, B, a_seq, n, H, Hkv, S, kps, ks, vs)
                     : launch_mma<128>(L, tmK, tmV, q, o, scratch, B, a_seq, n, H, Hkv, S, kps, ks, vs);
   }
-  const float scale = 1.0f / sqrtf((float)hd);
-  dim3 grid((a_seq + TQ - 1) / TQ, H, B);
   if (dtype == 0)
-    launch_k(L, attn_simt_kernel<float>, dim3(grid), dim3(128), 0, (const float*)q, (const float*)Kc, (const float*)Vc,
-                                                        (float*)o, a_seq, n, H, Hkv, hd, scale);
+    launch_simt<float>(L, q, Kc, Vc, o, B, a_seq, n, H, Hkv, hd);
   else
-    launch_k(L, attn_simt_kernel<__nv_bfloat16>, dim3(grid), dim3(128), 0, (const __nv_bfloat16*)q, (const __nv_bfloat16*)Kc,
-                                                                (const __nv_bfloat16*)Vc, (__nv_bfloat16*)o, a_seq, n,
-                                                                H, Hkv, hd, scale);
-  L.count();
+    launch_simt<__nv_bfloat16>(L, q, Kc, Vc, o, B, a_seq, n, H, Hkv, hd);
   return cudaGetLastError();
 }
 

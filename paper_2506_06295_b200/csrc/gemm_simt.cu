@@ -1,66 +1,147 @@
 // C[M,N] (fp32) = A[M,K] * W[N,K]^T on the plain fp32 ALUs.
 //
-// This is the GEMM of the fp32 mode (the tiny configuration asks for 1e-4
-// relative error, which TF32 tensor cores do not give) and the independent
-// cross-check for the tensor-core kernel in tests.  64x64 output tile, 16x16
-// threads, 4x4 outputs per thread, K staged through shared memory 16 at a time.
+// This is the GEMM of the fp32 mode (the tiny configuration asks for 1e-4 relative error, which TF32 tensor cores do
+// not give) and the independent cross-check for the tensor-core kernels in tests.
+//
+// The fp32 models are small, so a product is bound by latency: a loop over the whole k range with two block barriers per
+// 16 k took 12 us at K = 256 and 30 us at K = 688 for 50 MFLOP.  Here the eight warps of a CTA take DIFFERENT 32-wide
+// k-chunks (warp w the chunks w, w + 8, ...) of a small output tile, each with a shared-memory buffer of its own and no
+// barrier in the loop: K = 256 is one chunk per warp, all of whose loads are in flight together, and the weight half of
+// the first chunk is requested ahead of the dependency wait.  The eight partial tiles are added in warp order at the end.
+// An element's sum does not depend on the tile (same chunks, same order), so rows are bit-identical whatever the number
+// of rows in the launch.
 #include "internal.h"
 
 namespace dllm {
 
+namespace {
+
+constexpr int SG_WARPS = 8, SG_K = 32, SG_LD = SG_K + 4;  // row stride in shared memory: 16-byte aligned, 4 banks apart
+
+// four consecutive elements from column k of a row (zero past K); vec: the row allows one vector load
 template <typename T>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ A, const T* __restrict__ W,
-                                                        float* __restrict__ C, int M, int N, int K) {
+__device__ __forceinline__ float4 load4(const T* row, bool in, int k, int K, bool vec) {
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (!in || k >= K) return v;
+  if (vec) {
+    if constexpr (sizeof(T) == 4) {
+      v = __ldcg(reinterpret_cast<const float4*>(row + k));
+    } else {
+      const uint2 u = __ldcg(reinterpret_cast<const uint2*>(row + k));
+      v = make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                      __uint_as_float(u.y & 0xFFFF0000u));
+    }
+  } else {
+    float t[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (k + j < K) t[j] = to_f32<T>(row[k + j]);
+    v = make_float4(t[0], t[1], t[2], t[3]);
+  }
+  return v;
+}
+
+// Tile of 4 TM rows x 8 TN columns; a lane holds TM x TN outputs (rows 4 i + lane / 8, columns 8 j + lane % 8).
+template <typename T, int TM, int TN>
+__global__ void __launch_bounds__(SG_WARPS * 32)
+    gemm_simt_kernel(const T* __restrict__ A, const T* __restrict__ W, float* __restrict__ C, int M, int N, int K, bool vec) {
+  constexpr int BM = 4 * TM, BN = 8 * TN;
+  extern __shared__ __align__(16) float sg_smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float* As = sg_smem + warp * (BM + BN) * SG_LD;
+  float* Ws = As + BM * SG_LD;
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const int lr = lane >> 3, lk = (lane & 7) * 4;            // loads: four rows per pass, 8 lanes x 4 k per row
+  const int chunks = (K + SG_K - 1) / SG_K;
+  float4 ra[TM], rw[2 * TN];
+  auto load_w = [&](int c) {
+#pragma unroll
+    for (int i = 0; i < 2 * TN; ++i)
+      rw[i] = load4(W + (size_t)(n0 + 4 * i + lr) * K, n0 + 4 * i + lr < N, c * SG_K + lk, K, vec);
+  };
+  auto load_a = [&](int c) {
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+      ra[i] = load4(A + (size_t)(m0 + 4 * i + lr) * K, m0 + 4 * i + lr < M, c * SG_K + lk, K, vec);
+  };
+  if (warp < chunks) load_w(warp);                          // weights are written by no kernel
   pdl_wait();
   pdl_trigger();
-  constexpr int BM = 64, BN = 64, BK = 16;
-  __shared__ float As[BK][BM + 4];
-  __shared__ float Ws[BK][BN + 4];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += BK) {
-    // 64 rows x 16 k per operand = 1024 elements, 4 per thread
-    for (int e = threadIdx.x; e < BM * BK; e += 256) {
-      const int r = e / BK, kk = e - r * BK;
-      const int gm = m0 + r, gn = n0 + r, gk = k0 + kk;
-      As[kk][r] = (gm < M && gk < K) ? to_f32<T>(A[(size_t)gm * K + gk]) : 0.f;
-      Ws[kk][r] = (gn < N && gk < K) ? to_f32<T>(W[(size_t)gn * K + gk]) : 0.f;
+  if (warp < chunks) load_a(warp);
+  float acc[TM][TN] = {};
+  const int ly = lane >> 3, lx = lane & 7;
+  for (int c = warp; c < chunks; c += SG_WARPS) {
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < TM; ++i) *reinterpret_cast<float4*>(As + (4 * i + lr) * SG_LD + lk) = ra[i];
+#pragma unroll
+    for (int i = 0; i < 2 * TN; ++i) *reinterpret_cast<float4*>(Ws + (4 * i + lr) * SG_LD + lk) = rw[i];
+    __syncwarp();
+    if (c + SG_WARPS < chunks) {                            // the warp's next chunk travels under this one's arithmetic
+      load_w(c + SG_WARPS);
+      load_a(c + SG_WARPS);
     }
-    __syncthreads();
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float a[4], w[4];
+    for (int k = 0; k < SG_K; k += 4) {
+      float4 a[TM], w[TN];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
+      for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const float4*>(As + (4 * i + ly) * SG_LD + k);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) w[j] = Ws[kk][tx * 4 + j];
+      for (int j = 0; j < TN; ++j) w[j] = *reinterpret_cast<const float4*>(Ws + (8 * j + lx) * SG_LD + k);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], w[j], acc[i][j]);
+        for (int j = 0; j < TN; ++j) {
+          acc[i][j] = fmaf(a[i].x, w[j].x, acc[i][j]);
+          acc[i][j] = fmaf(a[i].y, w[j].y, acc[i][j]);
+          acc[i][j] = fmaf(a[i].z, w[j].z, acc[i][j]);
+          acc[i][j] = fmaf(a[i].w, w[j].w, acc[i][j]);
+        }
     }
-    __syncthreads();
   }
+  // partial tiles through shared memory (every warp is done with the buffers), added in warp order
+  static_assert(BM * BN <= (BM + BN) * SG_LD, "a warp's partial tile must fit its buffer");
+  __syncwarp();
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gm = m0 + ty * 4 + i;
-    if (gm >= M) continue;
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gn = n0 + tx * 4 + j;
-      if (gn < N) C[(size_t)gm * N + gn] = acc[i][j];
-    }
+    for (int j = 0; j < TN; ++j) As[(4 * i + ly) * BN + 8 * j + lx] = acc[i][j];
+  __syncthreads();
+  for (int e = threadIdx.x; e < BM * BN; e += SG_WARPS * 32) {
+    const int m = m0 + e / BN, n = n0 + e % BN;
+    float s = 0.f;
+#pragma unroll
+    for (int w = 0; w < SG_WARPS; ++w) s += sg_smem[w * (BM + BN) * SG_LD + e];
+    if (m < M && n < N) C[(size_t)m * N + n] = s;
   }
 }
 
+template <typename T, int TM, int TN>
+void launch_tile(const Launch& L, const void* A, const void* W, float* C, int M, int N, int K) {
+  constexpr int BM = 4 * TM, BN = 8 * TN, SMEM = SG_WARPS * (BM + BN) * SG_LD * 4;
+  static DeviceOnce once;
+  if (once.run([] { return cudaFuncSetAttribute(gemm_simt_kernel<T, TM, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM); }) !=
+      cudaSuccess)
+    return;  // the error stays for the caller's cudaGetLastError
+  const bool vec = K % 4 == 0 && (((uintptr_t)A | (uintptr_t)W) & (4 * sizeof(T) - 1)) == 0;
+  launch_k(L, gemm_simt_kernel<T, TM, TN>, dim3((N + BN - 1) / BN, (M + BM - 1) / BM), dim3(SG_WARPS * 32), SMEM, (const T*)A,
+           (const T*)W, C, M, N, K, vec);
+}
+
+}  // namespace
+
 void launch_gemm_simt(const Launch& L, int dtype, const void* A, const void* W, float* C, int M, int N, int K) {
   if (M <= 0 || N <= 0) return;
-  dim3 grid((N + 63) / 64, (M + 63) / 64);
-  if (dtype == 0)
-    launch_k(L, gemm_simt_kernel<float>, dim3(grid), dim3(256), 0, (const float*)A, (const float*)W, C, M, N, K);
-  else
-    launch_k(L, gemm_simt_kernel<__nv_bfloat16>, dim3(grid), dim3(256), 0, (const __nv_bfloat16*)A, (const __nv_bfloat16*)W, C, M, N, K);
+  // 32 x 64 tiles (half the shared-memory reads per product) once they are two per SM, 16 x 32 below: more CTAs, and a
+  // shorter chain in each
+  const bool big = (long)((M + 31) / 32) * ((N + 63) / 64) >= 2L * sm_count();
+  if (dtype == 0) {
+    if (big) launch_tile<float, 8, 8>(L, A, W, C, M, N, K);
+    else launch_tile<float, 4, 4>(L, A, W, C, M, N, K);
+  } else {
+    if (big) launch_tile<__nv_bfloat16, 8, 8>(L, A, W, C, M, N, K);
+    else launch_tile<__nv_bfloat16, 4, 4>(L, A, W, C, M, N, K);
+  }
   L.count();
 }
 

@@ -158,6 +158,35 @@ def test_gemm_simt(env, dtype):
     assert rel_l2(got, want) < 2e-6
 
 
+@pytest.mark.parametrize("M,N,K", [(1, 7, 5), (16, 32, 32), (17, 33, 260), (95, 1376, 256), (33, 70, 31), (400, 3000, 688)])
+def test_gemm_simt_tiles(env, M, N, K):
+    """Edges of the plain-ALU GEMM: a single element row, whole and ragged tiles, a k range that is no multiple of a
+    vector or of the warps' chunks, and enough tiles for the larger tile; float32 sums of K products (2e-6 as above)."""
+    torch, dllm = env
+    A = synth.random_normal((M, K), seed=51)
+    W = synth.random_normal((N, K), seed=52, std=0.05)
+    got = dllm.gemm_simt(torch.from_numpy(A).cuda(), torch.from_numpy(W).cuda()).cpu().numpy()
+    assert rel_l2(got, A.astype(np.float64) @ W.astype(np.float64).T) < 2e-6
+    one = dllm.gemm_simt(torch.from_numpy(A[-1:]).cuda(), torch.from_numpy(W).cuda()).cpu().numpy()
+    assert np.array_equal(got[-1:], one)      # a row does not depend on how many others are in the launch
+
+
+@pytest.mark.parametrize("a,n,H,hd,dtype", [(1, 1, 2, 64, "fp32"), (5, 33, 3, 96, "fp32"), (4, 300, 2, 32, "fp32"),
+                                            (7, 257, 2, 96, "bf16"), (620, 64, 8, 32, "fp32")])
+def test_attention_plain_alu_forms(env, a, n, H, hd, dtype):
+    """The plain-ALU attention whose warps split the keys (one key, a ragged chunk, several rounds of the warps) and, at
+    620 rows x 8 heads, the form whose warps split the queries (tolerances of test_attention)."""
+    torch, dllm = env
+    q, k, v = (synth.random_normal(sh, seed=61 + i) for i, sh in enumerate(((a, H * hd), (1, n, H * hd), (1, n, H * hd))))
+    if dtype == "bf16":
+        q, k, v = (synth.round_to_bf16(t) for t in (q, k, v))
+    td = torch.bfloat16 if dtype == "bf16" else torch.float32
+    got = dllm.attention(*(torch.from_numpy(t).cuda().to(td) for t in (q, k, v)), 1, a, n, H, H, hd).float().cpu().numpy()
+    want = O.attention(q.astype(np.float64).reshape(a, H, hd), k[0].astype(np.float64).reshape(n, H, hd),
+                       v[0].astype(np.float64).reshape(n, H, hd), H)
+    assert rel_l2(got, want) < (1e-5 if dtype == "fp32" else 8e-3)
+
+
 ATT_CASES = [
     # B, a, n, H, Hkv, hd
     (1, 8, 96, 4, 4, 64),      # tiny configuration, partial step
