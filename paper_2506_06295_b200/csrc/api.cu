@@ -212,6 +212,49 @@ Workspace make_workspace(const dllm_config& c, int B, int P, int R, int flags) {
 
 }  // namespace
 
+// Page-locked host blocks for the small copies of a session (tokens, predictions): a copy from or to pageable memory is
+// staged by the driver with a synchronisation of its own (about 8 us each; reading a prediction took two and a stream
+// synchronisation).  Destroyed sessions leave up to PINNED_KEPT blocks for the next ones, since allocating one takes as
+// long as a small step; the blocks belong to no device or stream.
+namespace {
+struct PinnedBlock {
+  void* p = nullptr;
+  size_t bytes = 0;
+};
+constexpr size_t PINNED_KEPT = 8, PINNED_MAX_KEPT_BYTES = 1 << 20;
+std::mutex g_pinned_mu;
+std::vector<PinnedBlock> g_pinned_free;
+PinnedBlock take_pinned(size_t bytes) {
+  {
+    std::lock_guard<std::mutex> lock(g_pinned_mu);
+    for (size_t i = 0; i < g_pinned_free.size(); ++i)
+      if (g_pinned_free[i].bytes >= bytes) {
+        const PinnedBlock b = g_pinned_free[i];
+        g_pinned_free.erase(g_pinned_free.begin() + i);
+        return b;
+      }
+  }
+  PinnedBlock b;
+  b.bytes = align_up(bytes, 64 << 10);
+  if (cudaHostAlloc(&b.p, b.bytes, cudaHostAllocPortable) != cudaSuccess) {
+    cudaGetLastError();
+    return PinnedBlock{};  // the copies then go straight to the caller's memory
+  }
+  return b;
+}
+void give_pinned(PinnedBlock b) {
+  if (!b.p) return;
+  if (b.bytes <= PINNED_MAX_KEPT_BYTES) {
+    std::lock_guard<std::mutex> lock(g_pinned_mu);
+    if (g_pinned_free.size() < PINNED_KEPT) {
+      g_pinned_free.push_back(b);
+      return;
+    }
+  }
+  cudaFreeHost(b.p);
+}
+}  // namespace
+
 struct dllm_model {
   dllm_config cfg;
   WeightLayout lay;
@@ -256,6 +299,9 @@ struct dllm_session {
   bool use_pdl = true;
   int sel_strategy = DLLM_SELECT_V_VERIFY, sel_metric = DLLM_METRIC_COSINE, v_selected_only = 0;  // ablation variants
   bool block_head = false;     // dllm_generate predicts only the block each step works on
+  PinnedBlock pinned;          // staging of tokens and predictions; a call that uses it ends with a synchronisation
+  std::mutex pinned_mu;        // held from filling it to reading it
+  ~dllm_session() { give_pinned(pinned); }
   struct GraphEntry {
     cudaGraphExec_t exec;
     uint64_t kernels;
@@ -374,6 +420,45 @@ cudaError_t h2d(void* dst, const void* src, size_t bytes, cudaStream_t st) {
   cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return e;
   return cudaStreamSynchronize(st);
+}
+
+// The session's page-locked staging for n values, allocated on first use; nullptr if there is none.
+template <typename T>
+T* staging(dllm_session* s, size_t n) {
+  if (s->pinned.bytes < n * sizeof(T)) {
+    give_pinned(s->pinned);
+    s->pinned = take_pinned(std::max(n * sizeof(T), (size_t)s->B * s->n * 4));
+  }
+  return static_cast<T*>(s->pinned.p);
+}
+
+// Device -> host copies ordered on the stream and complete on return, through the staging where there is one.
+struct HostCopy {
+  void* h;
+  size_t ws_off, bytes;
+};
+cudaError_t d2h(dllm_session* s, const HostCopy* c, int n, cudaStream_t st) {
+  std::lock_guard<std::mutex> lock(s->pinned_mu);
+  size_t lo = SIZE_MAX, hi = 0;
+  for (int i = 0; i < n; ++i) {
+    if (!c[i].h) continue;
+    lo = std::min(lo, c[i].ws_off);
+    hi = std::max(hi, c[i].ws_off + c[i].bytes);
+  }
+  cudaError_t e;
+  uint8_t* tmp = lo < hi ? staging<uint8_t>(s, hi - lo) : nullptr;
+  if (!tmp) {
+    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+    for (int i = 0; i < n; ++i)
+      if (c[i].h && (e = cudaMemcpy(c[i].h, s->d_ws + c[i].ws_off, c[i].bytes, cudaMemcpyDeviceToHost)) != cudaSuccess) return e;
+    return cudaSuccess;
+  }
+  // (the tensors of one call lie next to each other in the workspace: one copy)
+  if ((e = cudaMemcpyAsync(tmp, s->d_ws + lo, hi - lo, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+  if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+  for (int i = 0; i < n; ++i)
+    if (c[i].h) memcpy(c[i].h, tmp + (c[i].ws_off - lo), c[i].bytes);
+  return cudaSuccess;
 }
 
 int k_selected(float rho, int R, dllm_kround kr) {
@@ -900,7 +985,13 @@ dllm_status dllm_session_set_prompt(dllm_session* s, const int32_t* h_prompt, vo
   if (!s) return fail(nullptr, DLLM_INVALID_ARG, "session is NULL");
   if (!h_prompt) return fail(&s->err, DLLM_INVALID_ARG, "h_prompt is NULL");
   const int V = s->m->cfg.vocab;
-  std::vector<int32_t> tok((size_t)s->B * s->n);
+  std::lock_guard<std::mutex> lock(s->pinned_mu);
+  std::vector<int32_t> own;
+  int32_t* tok = staging<int32_t>(s, (size_t)s->B * s->n);
+  if (!tok) {
+    own.resize((size_t)s->B * s->n);
+    tok = own.data();
+  }
   for (int b = 0; b < s->B; ++b) {
     for (int i = 0; i < s->P; ++i) {
       const int32_t t = h_prompt[(size_t)b * s->P + i];
@@ -909,9 +1000,7 @@ dllm_status dllm_session_set_prompt(dllm_session* s, const int32_t* h_prompt, vo
     }
     for (int j = 0; j < s->R; ++j) tok[(size_t)b * s->n + s->P + j] = s->m->cfg.mask_id;
   }
-  cudaStream_t st = (cudaStream_t)stream;
-  CU_TRY(&s->err, cudaStreamSynchronize(st));
-  CU_TRY(&s->err, h2d(s->d_ws + s->ws.tokens, tok.data(), tok.size() * 4, st));
+  CU_TRY(&s->err, h2d(s->d_ws + s->ws.tokens, tok, (size_t)s->B * s->n * 4, (cudaStream_t)stream));
   s->valid = false;
   s->have_pred = false;
   return DLLM_OK;
@@ -1051,8 +1140,8 @@ dllm_status dllm_debug_skip_one_load(int enable) {
 dllm_status dllm_get_tokens(dllm_session* s, int32_t* h_out, void* stream) {
   if (!s) return fail(nullptr, DLLM_INVALID_ARG, "session is NULL");
   if (!h_out) return fail(&s->err, DLLM_INVALID_ARG, "h_out is NULL");
-  CU_TRY(&s->err, cudaStreamSynchronize((cudaStream_t)stream));
-  CU_TRY(&s->err, cudaMemcpy(h_out, s->d_ws + s->ws.tokens, (size_t)s->B * s->n * 4, cudaMemcpyDeviceToHost));
+  const HostCopy c{h_out, s->ws.tokens, (size_t)s->B * s->n * 4};
+  CU_TRY(&s->err, d2h(s, &c, 1, (cudaStream_t)stream));
   return DLLM_OK;
 }
 
@@ -1083,10 +1172,9 @@ dllm_status dllm_get_hidden(dllm_session* s, float* h_out, void* stream) {
 dllm_status dllm_get_pred(dllm_session* s, int32_t* h_x0, float* h_conf, void* stream) {
   if (!s) return fail(nullptr, DLLM_INVALID_ARG, "session is NULL");
   if (!s->have_pred) return fail(&s->err, DLLM_BAD_STATE, "no step has run");
-  CU_TRY(&s->err, cudaStreamSynchronize((cudaStream_t)stream));
   const size_t BR = (size_t)s->B * s->R;
-  if (h_x0) CU_TRY(&s->err, cudaMemcpy(h_x0, s->d_ws + s->ws.x0, BR * 4, cudaMemcpyDeviceToHost));
-  if (h_conf) CU_TRY(&s->err, cudaMemcpy(h_conf, s->d_ws + s->ws.conf, BR * 4, cudaMemcpyDeviceToHost));
+  const HostCopy c[2] = {{h_x0, s->ws.x0, BR * 4}, {h_conf, s->ws.conf, BR * 4}};
+  CU_TRY(&s->err, d2h(s, c, 2, (cudaStream_t)stream));
   return DLLM_OK;
 }
 
