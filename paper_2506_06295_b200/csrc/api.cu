@@ -481,9 +481,11 @@ struct ProfScope {
   ProfScope& operator=(const ProfScope&) = delete;
 };
 
-// One GEMM of the step: out = A[M,K] * W[N,K]^T as split-K partial slabs.
+// One GEMM of the step: out = A[M,K] * W[N,K]^T as split-K partial slabs.  weights_again: another product of the step reads
+// the same weights soon.
 dllm_status run_gemm(dllm_session* s, const Launch& L, int cls, const void* A, const void* W, int M, int N, int K,
-                     Partials* out, void* swiglu_out = nullptr, bool* fused = nullptr, int estimate_mask_id = -1) {
+                     Partials* out, void* swiglu_out = nullptr, bool* fused = nullptr, int estimate_mask_id = -1,
+                     bool weights_again = false) {
   float* part = s->wsp<float>(s->ws.part);
   if (fused) *fused = false;
   *out = Partials{part, (size_t)M * N, 1, N};
@@ -567,7 +569,8 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
     const bool identity = rr && !rp && Ma > 0;
     if (rr || (adaptive && s->sel_strategy == DLLM_SELECT_V_VERIFY)) {
       // V for ALL response rows (the 2 r d^2 term of Sec. A.7), V-verify, V overwrite
-      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u, Wv, BR, dkv, d, &part)) != DLLM_OK) return st;
+      // (a prompt refresh reads W_v once more, for the prompt rows)
+      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u, Wv, BR, dkv, d, &part, nullptr, nullptr, -1, rp)) != DLLM_OK) return st;
       const IdentityLists id{sel, act, inv};
       {  // the projection's fp32 result in, the cached row in, the row out
         ProfScope ps(s, DLLM_PROF_VVERIFY, (double)BR * dkv * (4.0 + 2.0 * es), 6.0 * BR * dkv, stream);

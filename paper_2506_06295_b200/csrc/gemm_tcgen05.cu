@@ -218,7 +218,7 @@ __device__ __forceinline__ void gemm_epilogue(uint32_t tmem_d, float* ex, int tl
   }
 }
 
-template <int BN>
+template <int BN, bool ONCE>
 __global__ void __launch_bounds__(128) gemm_bf16_tcgen05_kernel(const __grid_constant__ CUtensorMap tmW,
                                                                 const __grid_constant__ CUtensorMap tmA,
                                                                 float* __restrict__ part, int M, int N, int num_kb,
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(128) gemm_bf16_tcgen05_kernel(const __grid_con
       for (int i = 0; i < pre; ++i) {  // weights are written by no kernel: stream them ahead of the dependency
         const uint32_t fb = smem_u32(&full_bar[i]);
         mbar_expect_tx(fb, SL::STAGE_BYTES);
-        tma_load_2d(tiles + i * SL::STAGE_BYTES, &tmW, fb, (kb0 + i) * TILE_K, n0);
+        tma_load_2d_weights<ONCE>(tiles + i * SL::STAGE_BYTES, &tmW, fb, (kb0 + i) * TILE_K, n0);
       }
     }
     __syncwarp();
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(128) gemm_bf16_tcgen05_kernel(const __grid_con
       if (elect_one()) {
         if (i >= pre) {
           mbar_expect_tx(fb, SL::STAGE_BYTES);
-          tma_load_2d(dstW, &tmW, fb, kc, n0);
+          tma_load_2d_weights<ONCE>(dstW, &tmW, fb, kc, n0);
         }
         if (!skip) tma_load_2d(dstW + W_STAGE_BYTES, &tmA, fb, kc, m0);
       }
@@ -415,7 +415,7 @@ __device__ __forceinline__ void pair_unit(int u, int m_tiles, int n_pairs, int& 
   mt = grp * RASTER + within - np * wide;
 }
 
-template <int BN>
+template <int BN, bool ONCE>
 __global__ void __launch_bounds__(PAIR_THREADS, 1)
     gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmA,
                           float* __restrict__ part, int M, int N, int num_kb, int kb_per_split, size_t split_stride,
@@ -477,8 +477,8 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1)
     if (elect_one())
       for (int i = 0; i < pre; ++i) {
         if (leader) mbar_expect_tx(smem_u32(&full_bar[i]), 2 * PL::STAGE_BYTES);
-        tma_load_2d_pair(tiles_s + i * PL::STAGE_BYTES, &tmW, cluster_addr(smem_u32(&full_bar[i]), 0),
-                         (kb0 + i) * TILE_K, (2 * np + rank) * TILE_W);
+        tma_load_2d_pair_weights<ONCE>(tiles_s + i * PL::STAGE_BYTES, &tmW, cluster_addr(smem_u32(&full_bar[i]), 0),
+                              (kb0 + i) * TILE_K, (2 * np + rank) * TILE_W);
       }
     __syncwarp();
   }
@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1)
           const uint32_t dst = tiles_s + s * PL::STAGE_BYTES;
           if (issued >= pre) {
             if (leader) mbar_expect_tx(smem_u32(&full_bar[s]), 2 * PL::STAGE_BYTES);
-            tma_load_2d_pair(dst, &tmW, fb, kb * TILE_K, n0);
+            tma_load_2d_pair_weights<ONCE>(dst, &tmW, fb, kb * TILE_K, n0);
           }
           tma_load_2d_pair(dst + W_STAGE_BYTES, &tmA, fb, kb * TILE_K, m0);
         }
@@ -676,32 +676,32 @@ constexpr int max_stages(int bn) {
   return fit < MAX_STAGES ? fit : MAX_STAGES;
 }
 
-template <int BN>
+template <int BN, bool ONCE>
 cudaError_t launch_one(const Launch& L, const CUtensorMap& tmW, const CUtensorMap& tmA, float* part, int M, int N,
                        int num_kb, const GemmPlan& plan, void* act_out, int m_ffn) {
   using SL = SmemLayout<BN>;
   static DeviceOnce once;
   cudaError_t e0 = once.run([] {
-    return cudaFuncSetAttribute(gemm_bf16_tcgen05_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(gemm_bf16_tcgen05_kernel<BN, ONCE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)SL::total(max_stages(BN)));
   });
   if (e0 != cudaSuccess) return e0;
   const int stages = plan.stages < 2 ? 2 : plan.stages > max_stages(BN) ? max_stages(BN) : plan.stages;
   dim3 grid((M + BN - 1) / BN, (N + TILE_W - 1) / TILE_W, plan.S_max);
-  cudaError_t e = launch_k(L, gemm_bf16_tcgen05_kernel<BN>, grid, dim3(128), SL::total(stages), tmW, tmA, part, M, N,
+  cudaError_t e = launch_k(L, gemm_bf16_tcgen05_kernel<BN, ONCE>, grid, dim3(128), SL::total(stages), tmW, tmA, part, M, N,
                            num_kb, plan.upc, (size_t)M * N, stages, (__nv_bfloat16*)act_out, m_ffn, L.d_status);
   L.count();
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <int BN>
+template <int BN, bool ONCE>
 cudaError_t launch_pair(const Launch& L, const CUtensorMap& tmW, const CUtensorMap& tmA, float* part, int M, int N,
                         int num_kb, const GemmPlan& plan, void* act_out, int m_ffn) {
   using PL = PairLayout<BN>;
   const bool staged = act_out != nullptr || m_ffn < 0;
   static DeviceOnce once;
   cudaError_t e0 = once.run([] {
-    return cudaFuncSetAttribute(gemm_bf16_pair_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(gemm_bf16_pair_kernel<BN, ONCE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 227 * 1024 - 512);
   });
   if (e0 != cudaSuccess) return e0;
@@ -709,7 +709,7 @@ cudaError_t launch_pair(const Launch& L, const CUtensorMap& tmW, const CUtensorM
   const int m_tiles = (M + BN - 1) / BN, n_pairs = (N + 2 * TILE_W - 1) / (2 * TILE_W);
   const int units = m_tiles * n_pairs * plan.S_max;
   const int pairs = std::min(units, sm_count() / 2);
-  cudaError_t e = launch_k_cluster(L, gemm_bf16_pair_kernel<BN>, dim3(2 * pairs), dim3(PAIR_THREADS),
+  cudaError_t e = launch_k_cluster(L, gemm_bf16_pair_kernel<BN, ONCE>, dim3(2 * pairs), dim3(PAIR_THREADS),
                                    PL::total(stages, staged), dim3(2, 1, 1), tmW, tmA, part, M, N, num_kb, plan.upc,
                                    (size_t)M * N, m_tiles, n_pairs, units, stages, (__nv_bfloat16*)act_out, m_ffn,
                                    L.d_status);
@@ -818,6 +818,8 @@ GemmPlan plan_gemm_bf16(int M, int N, int K, int force_split, int force_stages, 
     if (S < 1) S = 1;
   }
   if (force_split > 0) S = force_split < p.num_kb ? force_split : p.num_kb;
+  // weight matrices that no L2 keeps until the next step (smaller ones may: a small model's layers stay there)
+  p.w_stream = (long)N * K >= 8L << 20;
   p.upc = (p.num_kb + S - 1) / S;                 // k-blocks per split
   p.S_max = (p.num_kb + p.upc - 1) / p.upc;       // no empty split
   p.ctas = (int)tiles * p.S_max;
@@ -849,20 +851,26 @@ cudaError_t launch_gemm_bf16(const Launch& L, const void* A, const void* W, floa
     return cudaErrorInvalidValue;
   }
   const int num_kb = (K + TILE_K - 1) / TILE_K;
+  // evict-first weights where one activation tile reads them (128-row tiles of the one-CTA kernel gained nothing)
+  const bool once = plan.w_stream && plan.m_tiles == 1;
+#define DLLM_LAUNCH(kind, bn, may)                                                                        \
+  ((may) && once ? launch_##kind<bn, may>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn)          \
+                 : launch_##kind<bn, false>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn))
   if (plan.pair) {
     switch (plan.BN) {
-      case 64: return launch_pair<64>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);
-      case 128: return launch_pair<128>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);
-      case 192: return launch_pair<192>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);
-      default: return launch_pair<256>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);
+      case 64: return DLLM_LAUNCH(pair, 64, false);
+      case 128: return DLLM_LAUNCH(pair, 128, false);
+      case 192: return DLLM_LAUNCH(pair, 192, true);
+      default: return DLLM_LAUNCH(pair, 256, true);
     }
   }
   switch (plan.BN) {
-    case 32: return launch_one<32>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);
-    case 64: return launch_one<64>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);
-    case 128: return launch_one<128>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);
-    default: return launch_one<256>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn);
+    case 32: return DLLM_LAUNCH(one, 32, true);
+    case 64: return DLLM_LAUNCH(one, 64, true);
+    case 128: return DLLM_LAUNCH(one, 128, false);
+    default: return DLLM_LAUNCH(one, 256, false);
   }
+#undef DLLM_LAUNCH
 }
 
 }  // namespace dllm

@@ -192,6 +192,7 @@ struct GemmPlan {
   int upc;          // k-blocks per split
   int ctas;         // grid size
   int S_max;        // split-K factor: slabs per output element
+  bool w_stream = false;  // weights are marked evict-first (when one activation tile reads them)
   int pair = 0;     // 1: persistent CTA pairs (cta_group::2) on tiles of 256 weight rows x BN activation rows
 };
 // 0 = auto.  force_pair: 0 auto, 1 CTA pairs (BN >= 64).  force_persistent: 0 auto, 1 the pair kernel for unsplit

@@ -131,6 +131,37 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
       ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(bar_cluster), "r"(c0), "r"(c1)
       : "memory");
 }
+// Tile loads marked evict-first in L2 where ONCE: the weights of a product with one activation tile are read once per
+// step, and a layer's 436 MB of them push out what every launch needs again (activations, caches, partial sums).  Without
+// the mark the plain instruction is used (an explicit evict-normal policy measured 1 % slower), chosen at compile time (a
+// branch in the copying loop cost the 768-row step 2 %).
+__device__ __forceinline__ uint64_t evict_first_policy() {
+  uint64_t p;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+template <bool ONCE>
+__device__ __forceinline__ void tma_load_2d_weights(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1) {
+  if constexpr (ONCE)
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], "
+        "[%2], %5;" ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(bar), "r"(c0), "r"(c1), "l"(evict_first_policy())
+        : "memory");
+  else
+    tma_load_2d(dst, tm, bar, c0, c1);
+}
+template <bool ONCE>
+__device__ __forceinline__ void tma_load_2d_pair_weights(uint32_t dst, const CUtensorMap* tm, uint32_t bar_cluster, int c0,
+                                                         int c1) {
+  if constexpr (ONCE)
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, "
+        "{%3, %4}], [%2], %5;" ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(bar_cluster), "r"(c0), "r"(c1),
+        "l"(evict_first_policy())
+        : "memory");
+  else
+    tma_load_2d_pair(dst, tm, bar_cluster, c0, c1);
+}
 // Untiled bulk copy global -> shared: both addresses 16-byte aligned, bytes a multiple of 16; completes on `bar`.
 __device__ __forceinline__ void bulk_load_1d(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
