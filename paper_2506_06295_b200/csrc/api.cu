@@ -482,10 +482,10 @@ struct ProfScope {
 };
 
 // One GEMM of the step: out = A[M,K] * W[N,K]^T as split-K partial slabs.  weights_again: another product of the step reads
-// the same weights soon.
+// the same weights soon.  rows: what an unsplit product of many rows does with its result itself (*fused).
 dllm_status run_gemm(dllm_session* s, const Launch& L, int cls, const void* A, const void* W, int M, int N, int K,
                      Partials* out, void* swiglu_out = nullptr, bool* fused = nullptr, int estimate_mask_id = -1,
-                     bool weights_again = false) {
+                     bool weights_again = false, const RowOut* rows = nullptr) {
   float* part = s->wsp<float>(s->ws.part);
   if (fused) *fused = false;
   *out = Partials{part, (size_t)M * N, 1, N};
@@ -493,16 +493,20 @@ dllm_status run_gemm(dllm_session* s, const Launch& L, int cls, const void* A, c
   const double es = (double)s->es();
   const bool tensor = !(s->m->cfg.dtype == DLLM_FP32 || s->simt_gemm);
   // the LM head is never split (its consumers read logits or records), nor is a gate / up projection of more rows
-  // than stream the weights anyway: the SwiGLU epilogue saves a launch and a pass over the slabs
-  const bool whole = cls == DLLM_PROF_GEMM_HEAD || (swiglu_out && M > 128 && gu_interleaved(s->m->cfg));
-  const GemmPlan plan = tensor ? plan_gemm_bf16(M, N, K, whole ? 1 : 0) : GemmPlan{};
+  // than stream the weights anyway: the SwiGLU epilogue saves a launch and a pass over the slabs; nor Q, K and V in one
+  const bool whole = cls == DLLM_PROF_GEMM_HEAD || (swiglu_out && M > 128 && gu_interleaved(s->m->cfg)) || (rows && rows->v);
+  GemmPlan plan = tensor ? plan_gemm_bf16(M, N, K, whole ? 1 : 0) : GemmPlan{};
+  if (weights_again) plan.w_stream = false;
+  const bool to_rows = tensor && rows && plan.pair && plan.S_max == 1;
   // an unsplit gate / up projection of an interleaved weight finishes SwiGLU in its own epilogue, and an unsplit
   // LM head writes per-tile estimate records instead of logits
   const bool estimate = tensor && !swiglu_out && estimate_mask_id >= 0 && plan.S_max == 1;
   const bool fuse = estimate || (tensor && swiglu_out && plan.S_max == 1 && gu_interleaved(s->m->cfg));
   // algorithmic traffic of one projection: the weight matrix and the activation rows once in, one result out
   // (fp32, or what the fused epilogue writes; split-K slabs are overhead, not counted)
-  const double out_bytes = estimate ? (double)M * ((N + 127) / 128) * 16.0 : fuse ? (double)M * (N / 2) * 2.0 : (double)M * N * 4.0;
+  const double out_bytes = estimate ? (double)M * ((N + 127) / 128) * 16.0
+                           : fuse   ? (double)M * (N / 2) * 2.0
+                                    : (double)M * N * (to_rows ? 2.0 : 4.0);
   s->prof_begin(cls, ((double)N * K + (double)M * K) * es + out_bytes, 2.0 * M * N * K, L.stream);
   struct End {
     dllm_session* s;
@@ -511,6 +515,15 @@ dllm_status run_gemm(dllm_session* s, const Launch& L, int cls, const void* A, c
   } end_guard{s, L.stream};
   if (!tensor) {
     launch_gemm_simt(L, s->m->cfg.dtype, A, W, part, M, N, K);
+    return DLLM_OK;
+  }
+  if (to_rows) {
+    const char* why = nullptr;
+    cudaError_t e = launch_gemm_rows(L, A, W, M, N, K, plan, *rows, &why);
+    if (e != cudaSuccess)
+      return fail(&s->err, DLLM_CUDA_ERROR, "bf16 GEMM %dx%dx%d: %s", M, N, K, why ? why : cudaGetErrorString(e));
+    if (fused) *fused = true;
+    out->p = nullptr;  // the row-wise kernels read the caches
     return DLLM_OK;
   }
   if ((size_t)plan.S_max * M * N > s->ws.part_floats)
@@ -546,10 +559,35 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
   Partials part{nullptr, 0, 1, 0};
 
   int32_t* inv = s->wsp<int32_t>(s->ws.inv);
+  // Projections of many rows finish their own rows (gemm_rows.cu).  Where every carried row is recomputed (response
+  // refresh, full step), Q, K and V are ONE product over the stacked weight whose epilogue rotates and scatters: no
+  // V-verify (nothing reads its scores then), selection, gather, RoPE or V scatter launch in any layer, and the lists are
+  // written once.  While profiling, V and Q / K stay launches of their own, so that each class can be read.
+  const bool tensor = dt == DLLM_BF16 && !s->simt_gemm;
+  const bool rotate = tensor && (hd == 64 || hd == 128) && !s->profiling;
+  const bool qkv_whole = rr && rotate && plan_gemm_bf16(c1, dq + 2 * dkv, d, 1).pair;
+  RowOut qkv;
+  qkv.qkv = 1;
+  qkv.q = reinterpret_cast<__nv_bfloat16*>(s->wsp<uint8_t>(s->ws.qbuf));
+  qkv.rope_tab = s->wsp<float>(s->ws.rope);
+  qkv.dq = dq;
+  qkv.dkv = dkv;
+  qkv.hd = hd;
+  qkv.g = g;
+  auto rows_into = [&](OutRows t, int width, const int32_t* list, int base) {  // rows of a [.., width] cache tensor
+    RowOut o;
+    o.rows = t;
+    o.g = g;
+    o.g.d = width;
+    o.act = list;
+    o.base = base;
+    return o;
+  };
   {
     ProfScope ps(s, DLLM_PROF_EMBED, (double)(c1 - c0) * d * (4.0 + 2.0 * es), 4.0 * (c1 - c0) * d, stream);
     launch_embed_norm(L, dt, W + wl.embed, s->wsp<int32_t>(s->ws.tokens), x,
-                      reinterpret_cast<const float*>(W + wl.layers[0].norm1), u, g, c0, c1, c.rms_eps);
+                      reinterpret_cast<const float*>(W + wl.layers[0].norm1), u, g, c0, c1, c.rms_eps,
+                      qkv_whole ? act : nullptr, qkv_whole ? inv : nullptr);
   }
   for (int l = 0; l < c.n_layers; ++l) {
     const LayerOff& lo = wl.layers[l];
@@ -567,7 +605,16 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
     // A response refresh alone takes every response row in carried order: u itself is the operand of the
     // projections and V-verify writes the (identity) lists, so no selection or gather launch is needed.
     const bool identity = rr && !rp && Ma > 0;
-    if (rr || (adaptive && s->sel_strategy == DLLM_SELECT_V_VERIFY)) {
+    bool fused = false;
+    if (qkv_whole) {
+      RowOut o = qkv;
+      o.q_by_slot = rp;
+      o.k = reinterpret_cast<__nv_bfloat16*>(s->cache(l, DLLM_CACHE_K));
+      o.v = reinterpret_cast<__nv_bfloat16*>(s->cache(l, DLLM_CACHE_V));
+      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_QK, u, Wq, c1, dq + 2 * dkv, d, &part, nullptr, nullptr, -1, false, &o)) !=
+          DLLM_OK)
+        return st;
+    } else if (rr || (adaptive && s->sel_strategy == DLLM_SELECT_V_VERIFY)) {
       // V for ALL response rows (the 2 r d^2 term of Sec. A.7), V-verify, V overwrite
       // (a prompt refresh reads W_v once more, for the prompt rows)
       if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u, Wv, BR, dkv, d, &part, nullptr, nullptr, -1, rp)) != DLLM_OK) return st;
@@ -586,14 +633,22 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
     }  // random selection: the scores were set by dllm_set_scores
     // V of the active rows is still missing when the verify pass did not write it
     const bool v_for_active = adaptive && (s->sel_strategy != DLLM_SELECT_V_VERIFY || s->v_selected_only);
-    if (rp) {
-      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u + (size_t)BR * d * es, Wv, BP, dkv, d, &part)) != DLLM_OK) return st;
-      ProfScope ps(s, DLLM_PROF_SCATTER, (double)BP * dkv * (4.0 + es), 0.0, stream);
-      launch_scatter_rows(L, dt, part, nullptr, BR, s->cache(l, DLLM_CACHE_V), g, BP, dkv);
+    const OutRows v_rows{s->cache(l, DLLM_CACHE_V), nullptr, 0};
+    if (rp && !qkv_whole) {
+      const RowOut o = rows_into(v_rows, dkv, nullptr, BR);
+      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u + (size_t)BR * d * es, Wv, BP, dkv, d, &part, nullptr, &fused, -1, false,
+                         &o)) != DLLM_OK)
+        return st;
+      if (!fused) {
+        ProfScope ps(s, DLLM_PROF_SCATTER, (double)BP * dkv * (4.0 + es), 0.0, stream);
+        launch_scatter_rows(L, dt, part, nullptr, BR, s->cache(l, DLLM_CACHE_V), g, BP, dkv);
+      }
     }
     if (Ma > 0) {
       const uint8_t* ua = s->wsp<uint8_t>(s->ws.ua);
-      if (identity) {
+      if (qkv_whole) {
+        // projected above
+      } else if (identity) {
         ua = u;
       } else if (s->R <= 1024 && (long)Ma * s->R <= 64L * 1024) {
         // few active rows: every CTA of the gather repeats the selection rather than wait for a launch
@@ -606,13 +661,25 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
         launch_gather_rows(L, dt, u, act, s->wsp<uint8_t>(s->ws.ua), Ma, d);
       }
       if (v_for_active) {
-        if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, ua, Wv, Ma, dkv, d, &part)) != DLLM_OK) return st;
-        ProfScope ps(s, DLLM_PROF_SCATTER, (double)Ma * dkv * (4.0 + es), 0.0, stream);
-        launch_scatter_rows(L, dt, part, act, 0, s->cache(l, DLLM_CACHE_V), g, Ma, dkv);
+        const RowOut o = rows_into(v_rows, dkv, act, 0);
+        if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, ua, Wv, Ma, dkv, d, &part, nullptr, &fused, -1, false, &o)) != DLLM_OK)
+          return st;
+        if (!fused) {
+          ProfScope ps(s, DLLM_PROF_SCATTER, (double)Ma * dkv * (4.0 + es), 0.0, stream);
+          launch_scatter_rows(L, dt, part, act, 0, s->cache(l, DLLM_CACHE_V), g, Ma, dkv);
+        }
       }
       // Q and K of the active rows in one GEMM over the stacked [W_q; W_k]
-      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_QK, ua, Wq, Ma, dq + dkv, d, &part)) != DLLM_OK) return st;
-      {
+      bool rotated = qkv_whole;
+      if (!qkv_whole) {
+        RowOut o = qkv;
+        o.act = act;
+        o.k = reinterpret_cast<__nv_bfloat16*>(s->cache(l, DLLM_CACHE_K));
+        if ((st = run_gemm(s, L, DLLM_PROF_GEMM_QK, ua, Wq, Ma, dq + dkv, d, &part, nullptr, &rotated, -1, false,
+                           rotate ? &o : nullptr)) != DLLM_OK)
+          return st;
+      }
+      if (!rotated) {
         ProfScope ps(s, DLLM_PROF_ROPE, (double)Ma * (dq + dkv) * (4.0 + es), 6.0 * Ma * (dq + dkv), stream);
         launch_qk_rope(L, dt, part, act, s->wsp<float>(s->ws.rope), s->wsp<uint8_t>(s->ws.qbuf),
                        s->cache(l, DLLM_CACHE_K), g, Ma, H, Hkv, hd);
@@ -625,20 +692,22 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
       cudaError_t e = launch_attention(L, dt, s->wsp<uint8_t>(s->ws.qbuf), s->cache(l, DLLM_CACHE_K),
                                        s->cache(l, DLLM_CACHE_V), s->wsp<uint8_t>(s->ws.obuf), s->B, a_seq, s->n, H,
                                        Hkv, hd, s->wsp<float>(s->ws.attn), s->ws.attn_floats, s->simt_gemm,
-                                       // the launch before attention is RoPE + K scatter (after the Q / K projection):
+                                       // the launch before attention is RoPE + K scatter or the Q / K projection itself:
                                        // every V row of the layer and, unless the prompt is refreshed, the prompt's K
-                                       // rows were written at least two launches earlier
-                                       rp ? 0 : s->P, s->n);
+                                       // rows were written at least two launches earlier (with one product for Q, K
+                                       // and V only the prompt's V, when it is not refreshed)
+                                       rp ? 0 : s->P, !qkv_whole ? s->n : rp ? 0 : s->P);
       s->prof_end(stream);
       if (e != cudaSuccess) return fail(&s->err, DLLM_CUDA_ERROR, "attention: %s", cudaGetErrorString(e));
-      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_O, s->wsp<uint8_t>(s->ws.obuf), W + lo.wo, Ma, d, dq, &part)) != DLLM_OK)
+      const RowOut attn_out = rows_into(s->outs(l, DLLM_CACHE_ATTN), d, act, 0);
+      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_O, s->wsp<uint8_t>(s->ws.obuf), W + lo.wo, Ma, d, dq, &part, nullptr, nullptr, -1,
+                         false, &attn_out)) != DLLM_OK)
         return st;
       {  // projection result and x in, AttnOut row and the normalised row out
         ProfScope ps(s, DLLM_PROF_OEPI, (double)Ma * d * (8.0 + 2.0 * es), 6.0 * Ma * d, stream);
         launch_oproj_epilogue(L, dt, part, act, x, reinterpret_cast<const float*>(W + lo.norm2),
                               s->outs(l, DLLM_CACHE_ATTN), s->wsp<uint8_t>(s->ws.hn), g, Ma, c.rms_eps);
       }
-      bool fused = false;
       if ((st = run_gemm(s, L, DLLM_PROF_GEMM_GU, s->wsp<uint8_t>(s->ws.hn), W + lo.wgu, Ma, 2 * m, d, &part,
                          s->wsp<uint8_t>(s->ws.ffn), &fused)) != DLLM_OK)
         return st;
@@ -646,7 +715,9 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
         ProfScope ps(s, DLLM_PROF_SILU, (double)Ma * m * (8.0 + es), 8.0 * Ma * m, stream);
         launch_silu_mul(L, dt, part, s->wsp<uint8_t>(s->ws.ffn), Ma, m, gu_interleaved(c));
       }
-      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_D, s->wsp<uint8_t>(s->ws.ffn), W + lo.wd, Ma, d, m, &part)) != DLLM_OK)
+      const RowOut ffn_out = rows_into(s->outs(l, DLLM_CACHE_FFN), d, act, 0);
+      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_D, s->wsp<uint8_t>(s->ws.ffn), W + lo.wd, Ma, d, m, &part, nullptr, nullptr, -1,
+                         false, &ffn_out)) != DLLM_OK)
         return st;
     }
     // FFNOut rows -> cache, residual assembly for all carried rows, next norm
@@ -1127,6 +1198,7 @@ dllm_status dllm_kernel_status(void* stream) {
 dllm_status dllm_debug_set_wait_limit_ns(uint64_t ns) {
   CU_TRY(nullptr, cudaDeviceSynchronize());
   CU_TRY(nullptr, set_wait_limit_gemm_tcgen05(ns));
+  CU_TRY(nullptr, set_wait_limit_gemm_rows(ns));
   CU_TRY(nullptr, set_wait_limit_attention(ns));
   CU_TRY(nullptr, set_wait_limit_attention_umma(ns));
   CU_TRY(nullptr, cudaDeviceSynchronize());
@@ -1209,7 +1281,9 @@ dllm_status dllm_get_selected(dllm_session* s, int layer, int32_t* h_idx, float*
   const size_t BR = (size_t)s->B * s->R;
   const int k_l = layer < (int)s->last_ksel.size() ? s->last_ksel[layer] : 0;
   if (k_sel_out) *k_sel_out = k_l;
-  if (h_idx && k_l > 0)
+  if (h_idx && k_l == s->R)  // every row: nothing was selected (a response refresh writes no list)
+    for (size_t i = 0; i < BR; ++i) h_idx[i] = (int32_t)(i % s->R);
+  else if (h_idx && k_l > 0)
     CU_TRY(&s->err, cudaMemcpy2D(h_idx, (size_t)k_l * 4, s->d_ws + s->ws.sel + (size_t)layer * BR * 4,
                                  (size_t)s->R * 4, (size_t)k_l * 4, s->B, cudaMemcpyDeviceToHost));
   if (h_sim)

@@ -228,6 +228,11 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
   return warp_sum(t);
 }
 
+// Rotation of one pair (rotate-half pairing); the rounding of each step is spelled out so that every kernel that rotates
+// gives the same bits.
+__device__ __forceinline__ float rope_lo(float lo, float hi, float c, float s) { return __fmaf_rn(lo, c, -__fmul_rn(hi, s)); }
+__device__ __forceinline__ float rope_hi(float lo, float hi, float c, float s) { return __fmaf_rn(hi, c, __fmul_rn(lo, s)); }
+
 // Online (max, argmax, sum exp) for the greedy estimate and its confidence (Eq. 4).  Ties go to the lowest id.
 struct MaxSum {
   float m, s;

@@ -272,9 +272,9 @@ __global__ void __launch_bounds__(STREAM_THREADS, 1)
   }
 }
 
-// After the O projection, streaming: see oproj_epilogue_kernel.  Stage = [projected row fp32 | x row fp32] of
-// active row r (carried row act[r]).
-template <typename T>
+// After the O projection, streaming: see oproj_epilogue_kernel.  Stage = [projected row fp32 (DIRECT: the
+// AttnOut row, which the projection has written) | x row fp32] of active row r (carried row act[r]).
+template <typename T, bool DIRECT>
 __global__ void __launch_bounds__(STREAM_THREADS, 1)
     oproj_stream_kernel(const float* __restrict__ part, const int32_t* __restrict__ act, const float* __restrict__ x,
                         const float* __restrict__ gain2, OutRows Ac, T* __restrict__ hn, Geo g, int Ma, float eps,
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(STREAM_THREADS, 1)
   __shared__ int meta[STREAM_MAX_STAGES];
   __shared__ int abort_flag;
   const int d = g.d, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rb = (uint32_t)d * 4, stage_bytes = 2 * rb;
+  const uint32_t rb = (uint32_t)d * 4, pb = DIRECT ? (uint32_t)d * (uint32_t)sizeof(T) : rb, stage_bytes = pb + rb;
   const uint32_t base = (smem_u32(smem_raw) + 127u) & ~127u;
   uint8_t* base_gen = smem_raw + (base - smem_u32(smem_raw));
   if (threadIdx.x == 0) {
@@ -313,8 +313,11 @@ __global__ void __launch_bounds__(STREAM_THREADS, 1)
         meta[s] = c;
         const uint32_t dst = base + s * stage_bytes, bar = smem_u32(&full_bar[s]);
         mbar_expect_tx(bar, stage_bytes);
-        bulk_load_1d(dst, part + (size_t)r * d, rb, bar);
-        bulk_load_1d(dst + rb, x + (size_t)c * d, rb, bar);
+        if constexpr (DIRECT)
+          bulk_load_1d(dst, Ac.row<T>(c, g), pb, bar);
+        else
+          bulk_load_1d(dst, part + (size_t)r * d, pb, bar);
+        bulk_load_1d(dst + pb, x + (size_t)c * d, rb, bar);
       }
     }
   } else {
@@ -325,13 +328,16 @@ __global__ void __launch_bounds__(STREAM_THREADS, 1)
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       const int c = meta[s];
-      const float* ps = reinterpret_cast<const float*>(base_gen + (size_t)s * stage_bytes);
-      float* xs = reinterpret_cast<float*>(base_gen + (size_t)s * stage_bytes + rb);
+      const uint8_t* ps = base_gen + (size_t)s * stage_bytes;
+      float* xs = reinterpret_cast<float*>(base_gen + (size_t)s * stage_bytes + pb);
       T* arow = Ac.row<T>(c, g);
       float ss = 0.f;
       for (int j = lane * 8; j < d; j += 256) {
         float a[8], xv[8];
-        Vec8<float>::load(ps + j, a);
+        if constexpr (DIRECT)
+          Vec8<T>::load(reinterpret_cast<const T*>(ps) + j, a);
+        else
+          Vec8<float>::load(reinterpret_cast<const float*>(ps) + j, a);
         Vec8<float>::load(xs + j, xv);
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
@@ -339,7 +345,7 @@ __global__ void __launch_bounds__(STREAM_THREADS, 1)
           xv[t] += a[t];
           ss += xv[t] * xv[t];
         }
-        Vec8<T>::store(arow + j, a);
+        if constexpr (!DIRECT) Vec8<T>::store(arow + j, a);
         Vec8<float>::store(xs + j, xv);   // kept for the second pass
       }
       ss = warp_sum(ss);
@@ -439,8 +445,8 @@ __global__ void __launch_bounds__(STREAM_THREADS, 1)
         float o_lo[4], o_hi[4];
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-          o_lo[t] = lo[t] * cc[t] - hi[t] * ss[t];
-          o_hi[t] = hi[t] * cc[t] + lo[t] * ss[t];
+          o_lo[t] = rope_lo(lo[t], hi[t], cc[t], ss[t]);
+          o_hi[t] = rope_hi(lo[t], hi[t], cc[t], ss[t]);
         }
         T* dst = head < H ? qrow + head * hd : krow + (head - H) * hd;
         store4<T>(dst + i0, o_lo);
@@ -904,8 +910,8 @@ __global__ void qk_rope_kernel(Partials part, const int32_t* __restrict__ act, c
     float o_lo[4], o_hi[4];
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
-      o_lo[t] = lo[u][t] * cc[t] - hi[u][t] * ss[t];
-      o_hi[t] = hi[u][t] * cc[t] + lo[u][t] * ss[t];
+      o_lo[t] = rope_lo(lo[u][t], hi[u][t], cc[t], ss[t]);
+      o_hi[t] = rope_hi(lo[u][t], hi[u][t], cc[t], ss[t]);
     }
     store4<T>(dst + i0, o_lo);
     store4<T>(dst + i0 + half, o_hi);
@@ -976,12 +982,12 @@ void launch_scatter_rows(const Launch& L, int dtype, Partials part, const int32_
 // ------------------------------------------------------------------ O-proj epilogue
 // AttnOut row -> cache (rounded to the cache dtype); h = x + AttnOut (the
 // rounded value, so a later step that reads the cache sees the same h);
-// hn = rmsnorm(h) * gain2.
-template <typename T>
+// hn = rmsnorm(h) * gain2.  DIRECT: the projection has written the AttnOut rows.
+template <typename T, bool DIRECT>
 __global__ void oproj_epilogue_kernel(Partials part, const int32_t* __restrict__ act, const float* __restrict__ x,
                                       const float* __restrict__ gain2, OutRows Ac, T* __restrict__ hn, Geo g,
                                       float eps) {
-  // The launch before this one is the O projection, which writes nothing but `part`: the row's place (act), its x
+  // The launch before this one is the O projection, which writes nothing but `part` (or AttnOut): the row's place (act), its x
   // row and the gain are fetched before the dependency wait, while the projection still runs.
   extern __shared__ float hrow[];
   __shared__ float red[32];
@@ -1002,7 +1008,10 @@ __global__ void oproj_epilogue_kernel(Partials part, const int32_t* __restrict__
   float ss = 0.f;
   for (int i = i0; i < d; i += blockDim.x * 8) {
     float a[8], xv[8];
-    sum_partials8(part.p, part.split_stride, part.count(r, i), (size_t)r * part.N + i, a);
+    if constexpr (DIRECT)
+      Vec8<T>::load_cg(arow + i, a);
+    else
+      sum_partials8(part.p, part.split_stride, part.count(r, i), (size_t)r * part.N + i, a);
     if (one_trip) {
 #pragma unroll
       for (int t = 0; t < 8; ++t) xv[t] = x0[t];
@@ -1016,7 +1025,7 @@ __global__ void oproj_epilogue_kernel(Partials part, const int32_t* __restrict__
       ss += xv[t] * xv[t];
       hv[t] = xv[t];
     }
-    Vec8<T>::store(arow + i, a);
+    if constexpr (!DIRECT) Vec8<T>::store(arow + i, a);
     if (!one_trip) Vec8<float>::store(hrow + i, xv);
   }
   ss = block_sum(ss, red);
@@ -1043,28 +1052,36 @@ __global__ void oproj_epilogue_kernel(Partials part, const int32_t* __restrict__
 void launch_oproj_epilogue(const Launch& L, int dtype, Partials part, const int32_t* act, const float* x,
                            const float* gain2, OutRows Ac_layer, void* hn, Geo g, int Ma, float eps) {
   if (Ma <= 0) return;
-  const size_t stage = (size_t)g.d * 8;
+  const bool direct = part.p == nullptr;   // bf16 models only
+  const size_t stage = (size_t)g.d * (direct ? 6 : 8);
   if (g.B * g.R >= STREAM_MIN_ROWS && part.S == 1 && part.upc == 0 && (g.d & 7) == 0 &&
       stream_stages(stage) >= STREAM_CONSUMERS + 1) {
     const int stages = stream_stages(stage);
     const size_t smem = (size_t)stages * stage + 128;
     const int ctas = std::min(Ma, sm_count());
-    DLLM_DISPATCH(dtype, {
-      static DeviceOnce once;
-      cudaError_t e0 = once.run([] {
-        return cudaFuncSetAttribute(oproj_stream_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024);
+    auto go = [&](auto* kernel, auto* out, DeviceOnce& once) {
+      cudaError_t e0 = once.run([&] {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024);
       });
       if (e0 == cudaSuccess)
-        launch_k(L, oproj_stream_kernel<T>, dim3(ctas), dim3(STREAM_THREADS), smem, part.p, act, x, gain2, Ac_layer,
-                 (T*)hn, g, Ma, eps, stages, L.d_status);
-    });
+        launch_k(L, kernel, dim3(ctas), dim3(STREAM_THREADS), smem, part.p, act, x, gain2, Ac_layer, out, g, Ma, eps, stages,
+                 L.d_status);
+    };
+    static DeviceOnce once_direct, once_f32, once_bf16;
+    if (direct) go(oproj_stream_kernel<__nv_bfloat16, true>, (__nv_bfloat16*)hn, once_direct);
+    else if (dtype == 0) go(oproj_stream_kernel<float, false>, (float*)hn, once_f32);
+    else go(oproj_stream_kernel<__nv_bfloat16, false>, (__nv_bfloat16*)hn, once_bf16);
     L.count();
     return;
   }
   const int threads = row_threads(g.d);
   const size_t smem = g.d <= threads * 8 ? 0 : (size_t)g.d * sizeof(float);  // staging only if a row takes several passes
-  DLLM_DISPATCH(dtype, (launch_k(L, oproj_epilogue_kernel<T>, dim3(Ma), dim3(threads), smem, part, act, x, gain2, Ac_layer,
-                                 (T*)hn, g, eps)));
+  if (direct)
+    launch_k(L, oproj_epilogue_kernel<__nv_bfloat16, true>, dim3(Ma), dim3(threads), smem, part, act, x, gain2, Ac_layer,
+             (__nv_bfloat16*)hn, g, eps);
+  else
+    DLLM_DISPATCH(dtype, (launch_k(L, oproj_epilogue_kernel<T, false>, dim3(Ma), dim3(threads), smem, part, act, x, gain2,
+                                   Ac_layer, (T*)hn, g, eps)));
   L.count();
 }
 
@@ -1096,10 +1113,13 @@ void launch_silu_mul(const Launch& L, int dtype, Partials part, void* out, int M
 }
 
 // ------------------------------------------------------------------ embedding + first RMSNorm
-// x[c] = E[token(c)], u[c] = rmsnorm(x[c]) * gain for carried rows c0 <= c < c1.
+// x[c] = E[token(c)], u[c] = rmsnorm(x[c]) * gain for carried rows c0 <= c < c1.  act / inv (may be null): the lists of a
+// step whose active rows are all the carried ones, in the order attention wants: carried order for the response rows
+// alone, sequence by sequence when the prompt rows are carried too.
 template <typename T>
 __global__ void embed_norm_kernel(const T* __restrict__ E, const int32_t* __restrict__ tokens, float* __restrict__ x,
-                                  const float* __restrict__ gain, T* __restrict__ u, Geo g, int c0, float eps) {
+                                  const float* __restrict__ gain, T* __restrict__ u, Geo g, int c0, float eps,
+                                  int32_t* __restrict__ act, int32_t* __restrict__ inv) {
   pdl_wait();
   pdl_trigger();
   __shared__ float red[32];
@@ -1107,6 +1127,11 @@ __global__ void embed_norm_kernel(const T* __restrict__ E, const int32_t* __rest
   int b, pos;
   carried_to_pos(c, g, b, pos);
   const int tok = tokens[(size_t)b * g.n + pos];
+  if (act && threadIdx.x == 0) {
+    const int row = (int)gridDim.x > g.B * g.R ? b * g.n + pos : c;
+    act[row] = c;
+    inv[c] = row;
+  }
   const T* src = E + (size_t)tok * g.d;
   float* xr = x + (size_t)c * g.d;
   float ss = 0.f;
@@ -1131,10 +1156,10 @@ __global__ void embed_norm_kernel(const T* __restrict__ E, const int32_t* __rest
 }
 
 void launch_embed_norm(const Launch& L, int dtype, const void* E, const int32_t* tokens, float* x, const float* gain,
-                       void* u, Geo g, int c0, int c1, float eps) {
+                       void* u, Geo g, int c0, int c1, float eps, int32_t* act, int32_t* inv) {
   if (c1 <= c0) return;
   DLLM_DISPATCH(dtype, (launch_k(L, embed_norm_kernel<T>, dim3(c1 - c0), dim3(row_threads(g.d)), 0, (const T*)E, tokens, x, gain,
-                                 (T*)u, g, c0, eps)));
+                                 (T*)u, g, c0, eps, act, inv)));
   L.count();
 }
 
@@ -1149,7 +1174,8 @@ void launch_embed_norm(const Launch& L, int dtype, const void* E, const int32_t*
 // written by launches that had completed before that projection passed its own dependency wait.  A one-pass row
 // therefore fetches all of it BEFORE the wait, while the projection still runs, and only the projection result
 // (active rows) after it.
-template <typename T, bool EARLY>
+// DIRECT: the projection has written the active FFNOut rows, which are then read after the wait like the others.
+template <typename T, bool EARLY, bool DIRECT = false>
 __global__ void __launch_bounds__(512, 2) tail_kernel(Partials part, const int32_t* __restrict__ inv, float* __restrict__ x,
                             OutRows Ac, OutRows Fc, const float* __restrict__ gain,
                             T* __restrict__ u, Geo g, int c0, float eps) {
@@ -1166,18 +1192,19 @@ __global__ void __launch_bounds__(512, 2) tail_kernel(Partials part, const int32
   int r = -1;
   if constexpr (EARLY) {   // the host passes EARLY only with inv != nullptr and a one-pass row
     float ae[8], fe[8];
-    r = __ldcg(inv + c);
+    if constexpr (!DIRECT) r = __ldcg(inv + c);
     if (i0 < d) {
       Vec8<float>::load(gain + i0, gv);
       Vec8<float>::load_cg(xr + i0, hv);
       Vec8<T>::load_cg(arow + i0, ae);
-      if (r < 0) Vec8<T>::load_cg(frow + i0, fe);
+      if (!DIRECT && r < 0) Vec8<T>::load_cg(frow + i0, fe);
     }
     pdl_wait();
     pdl_trigger();
     float ss = 0.f;
     if (i0 < d) {
-      if (r >= 0) {
+      if (DIRECT) Vec8<T>::load_cg(frow + i0, fe);
+      if (!DIRECT && r >= 0) {
         sum_partials8(part.p, part.split_stride, part.count(r, i0), (size_t)r * part.N + i0, fe);
         Vec8<T>::store(frow + i0, fe);
 #pragma unroll
@@ -1249,6 +1276,8 @@ __global__ void __launch_bounds__(512, 2) tail_kernel(Partials part, const int32
 void launch_tail(const Launch& L, int dtype, Partials part, const int32_t* inv, float* x, OutRows Ac_layer,
                  OutRows Fc_layer, const float* gain, void* u, Geo g, int c0, int c1, float eps) {
   if (c1 <= c0) return;
+  const bool direct = inv != nullptr && part.p == nullptr;   // bf16 models only
+  if (direct) inv = nullptr;
   {
     const size_t es = dtype == 0 ? 4 : 2, stage = (size_t)g.d * (8 + es);
     if (g.B * g.R >= STREAM_MIN_ROWS && part.S == 1 && part.upc == 0 && stream_stages(stage) >= STREAM_CONSUMERS + 1) {
@@ -1270,7 +1299,10 @@ void launch_tail(const Launch& L, int dtype, Partials part, const int32_t* inv, 
   }
   const int threads = row_threads(g.d);
   const size_t smem = g.d <= threads * 8 ? 0 : (size_t)g.d * sizeof(float);  // staging only if a row takes several passes
-  if (inv != nullptr && smem == 0)
+  if (direct && smem == 0)
+    launch_k(L, tail_kernel<__nv_bfloat16, true, true>, dim3(c1 - c0), dim3(threads), smem, part, inv, x, Ac_layer, Fc_layer,
+             gain, (__nv_bfloat16*)u, g, c0, eps);
+  else if (inv != nullptr && smem == 0)
     DLLM_DISPATCH(dtype, (launch_k(L, tail_kernel<T, true>, dim3(c1 - c0), dim3(threads), smem, part, inv, x, Ac_layer,
                                    Fc_layer, gain, (T*)u, g, c0, eps)));
   else

@@ -137,14 +137,16 @@ cudaError_t launch_select(const Launch& L, const float* sim, const int32_t* forc
 void launch_select_gather(const Launch& L, int dtype, const float* sim, const int32_t* forced, int mode, int ksel,
                           int32_t* sel, int32_t* act, int32_t* inv, const void* u, void* ua, Geo g,
                           int refresh_prompt);
-// x[c] = E[token(c)], u[c] = rmsnorm(x[c]) * gain for carried rows c0 <= c < c1.
+// x[c] = E[token(c)], u[c] = rmsnorm(x[c]) * gain for carried rows c0 <= c < c1; act / inv: lists of a step that
+// recomputes all of them (see the kernel).
 void launch_embed_norm(const Launch& L, int dtype, const void* E, const int32_t* tokens, float* x, const float* gain,
-                       void* u, Geo g, int c0, int c1, float eps);
+                       void* u, Geo g, int c0, int c1, float eps, int32_t* act = nullptr, int32_t* inv = nullptr);
 // End of a layer for carried rows c0 <= c < c1: FFNOut rows of the active set
 // (slabs in `part`, row = inv[c]) -> cache; x <- (x + AttnOut) + FFNOut from the
 // caches; u = rmsnorm(x) * gain.  inv == nullptr: no active row.
 void launch_tail(const Launch& L, int dtype, Partials part, const int32_t* inv, float* x, OutRows Ac_layer,
                  OutRows Fc_layer, const float* gain, void* u, Geo g, int c0, int c1, float eps);
+// (launch_tail and launch_oproj_epilogue: part.p == nullptr with active rows: the projection has written their rows.)
 void launch_gather_rows(const Launch& L, int dtype, const void* src, const int32_t* act, void* dst, int rows, int d);
 // RoPE on Q and K of the active rows; Q -> qbuf [Ma, dq]; K -> K cache rows.
 void launch_qk_rope(const Launch& L, int dtype, Partials part, const int32_t* act, const float* rope_tab, void* qbuf,
@@ -207,6 +209,25 @@ Partials make_partials(const float* p, int M, int N, const GemmPlan& plan);
 // one {max, sum exp, argmax, -} record per row and weight tile, [M][ceil(N / 128)] float4 (see launch_estimate_merge).
 cudaError_t launch_gemm_bf16(const Launch& L, const void* A, const void* W, float* part, int M, int N, int K,
                              const GemmPlan& plan, const char** err, void* act_out = nullptr, int m_ffn = 0);
+
+// ---------------- gemm_rows.cu ----------------
+// Where the bf16 rows of a projection go.  qkv == 0: rows of a cache tensor (`rows`, g.d = N elements each); qkv == 1:
+// columns [Q | K] or [Q | K | V] -- Q rotated -> q [., dq], K rotated and V -> cache rows (hd 64 or 128).
+struct RowOut {
+  int qkv = 0;
+  const int32_t* act = nullptr;    // carried row of row m; nullptr: base + m
+  int base = 0;
+  OutRows rows{};
+  __nv_bfloat16 *q = nullptr, *k = nullptr, *v = nullptr;
+  int q_by_slot = 0;               // rows of q sequence by sequence (b * n + position) instead of row m
+  const float* rope_tab = nullptr;
+  int dq = 0, dkv = 0, hd = 0;
+  Geo g{};
+};
+// Needs an unsplit pair plan.
+cudaError_t launch_gemm_rows(const Launch& L, const void* A, const void* W, int M, int N, int K, const GemmPlan& plan,
+                             const RowOut& out, const char** err);
+cudaError_t set_wait_limit_gemm_rows(unsigned long long ns);
 
 // Test hooks of the bounded device-side waits (see dllm_debug_* in the C ABI): the wait limit of each
 // translation unit that waits on mbarriers (0 = the 2 s default), and the dropped activation load.

@@ -374,3 +374,35 @@ def test_error_paths_on_device(env):
     with pytest.raises(dllm.DllmError):
         ses.set_prompt(np.full((1, 64), 5000))
     ses.sync()
+
+
+@pytest.mark.parametrize("hd,H,Hkv,d,B,P,R,compact", [
+    (64, 7, 1, 4736, 1, 37, 131, False),    # 131 / 168 rows, the response rows start inside a tile
+    (128, 3, 3, 5504, 2, 70, 100, True),    # 200 / 340 rows; prompt AttnOut / FFNOut rows outside the cache
+])
+def test_bf16_projections_of_many_rows_place_their_rows(env, hd, H, Hkv, d, B, P, R, compact):
+    """Unsplit projections of more than 128 rows (a wide model with few k-blocks: none is split) round, rotate and place
+    their own rows: full step, response refresh, and a prompt refresh whose response rows are selected (row lists).  2e-2
+    as for every bf16 step; one misplaced row of 131 is 9e-2."""
+    torch, dllm = env
+    cfg = synth.ModelConfig(n_layers=2, d_model=d, n_heads=H, n_kv_heads=Hkv, head_dim=hd, d_ffn=448, vocab=304,
+                            mask_id=303, dtype="bf16")
+    w = synth.make_weights(cfg, synth.WEIGHT_SEED)
+    prompt = synth.make_prompt(cfg, B, P)
+    orc = O.DLLMOracle(cfg, w, B, P, R, dtype=np.float32, compact_prompt_outs=compact)
+    ses = dllm.Session(dllm.Model(cfg).load(w), B, P, R, compact_cache=compact)
+    orc.set_prompt(prompt)
+    ses.set_prompt(prompt)
+    r = orc.step(True, True)
+    ses.step_full()
+    compare_step(orc, ses, r, 2e-2, what="full")
+    for step, (rp, rr, rho) in enumerate(((False, True, 0.0), (True, False, 0.25), (False, False, 0.25)), 1):
+        unmask(orc, ses, step, 3)
+        r = orc.step(rp, rr, rho)
+        ses.step_cached(rp, rr, rho)
+        compare_step(orc, ses, r, 2e-2, check_sets=False, what=f"step {step}")
+    for l in range(cfg.n_layers):
+        for which, ref in ((dllm.CACHE_K, orc.Kc), (dllm.CACHE_V, orc.Vc)):
+            assert rel_l2(ses.get_cache(l, which), ref[l]) < 2e-2
+    if not compact:
+        compare_caches(dllm, orc, ses, 2e-2, "after")
