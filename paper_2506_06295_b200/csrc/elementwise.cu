@@ -979,6 +979,52 @@ void launch_scatter_rows(const Launch& L, int dtype, Partials part, const int32_
   L.count();
 }
 
+// ------------------------------------------------------------------ rows a projection has written itself
+// After a projection that wrote its rows into AttnOut (TAIL false: h = x + AttnOut of active row r, out[r] = rmsnorm(h) *
+// gain) or FFNOut (TAIL true: x = (x + AttnOut) + FFNOut of carried row c, out[c] = rmsnorm(x) * gain): the sums of
+// oproj_epilogue_kernel and tail_kernel, for rows that fit one pass (d <= 8 x threads).  Such a step has hundreds of rows,
+// several waves of 512-thread CTAs, each a chain of load latency, block sum and store; 32 registers put four on an SM
+// (packed bf16 operands, the gain fetched under the block sum) where the general kernels fit two.
+template <bool TAIL>
+__global__ void __launch_bounds__(512, 4) direct_row_kernel(const int32_t* __restrict__ act, float* __restrict__ x,
+                                                            const float* __restrict__ gain, OutRows Ac, OutRows Fc,
+                                                            __nv_bfloat16* __restrict__ out, Geo g, int c0, float eps) {
+  using T = __nv_bfloat16;
+  __shared__ float red[32];
+  const int r = blockIdx.x, c = TAIL ? c0 + r : __ldcg(act + r), i0 = threadIdx.x * 8;
+  const bool in = i0 < g.d;
+  float* xr = x + (size_t)c * g.d + i0;
+  float hv[8], ev[8];
+  if (in) {   // written at least two launches ago
+    Vec8<float>::load_cg(xr, hv);
+    if constexpr (TAIL) {
+      Vec8<T>::load_cg(Ac.row<T>(c, g) + i0, ev);
+#pragma unroll
+      for (int t = 0; t < 8; ++t) hv[t] += ev[t];
+    }
+  }
+  pdl_wait();
+  pdl_trigger();
+  float ss = 0.f;
+  if (in) {
+    Vec8<T>::load_cg((TAIL ? Fc : Ac).row<T>(c, g) + i0, ev);
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      hv[t] += ev[t];
+      ss += hv[t] * hv[t];
+    }
+    if constexpr (TAIL) Vec8<float>::store(xr, hv);
+    Vec8<float>::load(gain + i0, ev);
+  }
+  ss = block_sum(ss, red);
+  const float rs = rsqrtf(ss / (float)g.d + eps);
+  if (in) {
+#pragma unroll
+    for (int t = 0; t < 8; ++t) hv[t] = hv[t] * rs * ev[t];
+    Vec8<T>::store(out + (size_t)(TAIL ? c : r) * g.d + i0, hv);
+  }
+}
+
 // ------------------------------------------------------------------ O-proj epilogue
 // AttnOut row -> cache (rounded to the cache dtype); h = x + AttnOut (the
 // rounded value, so a later step that reads the cache sees the same h);
@@ -1076,7 +1122,10 @@ void launch_oproj_epilogue(const Launch& L, int dtype, Partials part, const int3
   }
   const int threads = row_threads(g.d);
   const size_t smem = g.d <= threads * 8 ? 0 : (size_t)g.d * sizeof(float);  // staging only if a row takes several passes
-  if (direct)
+  if (direct && smem == 0)
+    launch_k(L, direct_row_kernel<false>, dim3(Ma), dim3(threads), 0, act, (float*)x, gain2, Ac_layer, OutRows{}, (__nv_bfloat16*)hn,
+             g, 0, eps);
+  else if (direct)
     launch_k(L, oproj_epilogue_kernel<__nv_bfloat16, true>, dim3(Ma), dim3(threads), smem, part, act, x, gain2, Ac_layer,
              (__nv_bfloat16*)hn, g, eps);
   else
@@ -1174,8 +1223,7 @@ void launch_embed_norm(const Launch& L, int dtype, const void* E, const int32_t*
 // written by launches that had completed before that projection passed its own dependency wait.  A one-pass row
 // therefore fetches all of it BEFORE the wait, while the projection still runs, and only the projection result
 // (active rows) after it.
-// DIRECT: the projection has written the active FFNOut rows, which are then read after the wait like the others.
-template <typename T, bool EARLY, bool DIRECT = false>
+template <typename T, bool EARLY>
 __global__ void __launch_bounds__(512, 2) tail_kernel(Partials part, const int32_t* __restrict__ inv, float* __restrict__ x,
                             OutRows Ac, OutRows Fc, const float* __restrict__ gain,
                             T* __restrict__ u, Geo g, int c0, float eps) {
@@ -1192,19 +1240,18 @@ __global__ void __launch_bounds__(512, 2) tail_kernel(Partials part, const int32
   int r = -1;
   if constexpr (EARLY) {   // the host passes EARLY only with inv != nullptr and a one-pass row
     float ae[8], fe[8];
-    if constexpr (!DIRECT) r = __ldcg(inv + c);
+    r = __ldcg(inv + c);
     if (i0 < d) {
       Vec8<float>::load(gain + i0, gv);
       Vec8<float>::load_cg(xr + i0, hv);
       Vec8<T>::load_cg(arow + i0, ae);
-      if (!DIRECT && r < 0) Vec8<T>::load_cg(frow + i0, fe);
+      if (r < 0) Vec8<T>::load_cg(frow + i0, fe);
     }
     pdl_wait();
     pdl_trigger();
     float ss = 0.f;
     if (i0 < d) {
-      if (DIRECT) Vec8<T>::load_cg(frow + i0, fe);
-      if (!DIRECT && r >= 0) {
+      if (r >= 0) {
         sum_partials8(part.p, part.split_stride, part.count(r, i0), (size_t)r * part.N + i0, fe);
         Vec8<T>::store(frow + i0, fe);
 #pragma unroll
@@ -1300,8 +1347,8 @@ void launch_tail(const Launch& L, int dtype, Partials part, const int32_t* inv, 
   const int threads = row_threads(g.d);
   const size_t smem = g.d <= threads * 8 ? 0 : (size_t)g.d * sizeof(float);  // staging only if a row takes several passes
   if (direct && smem == 0)
-    launch_k(L, tail_kernel<__nv_bfloat16, true, true>, dim3(c1 - c0), dim3(threads), smem, part, inv, x, Ac_layer, Fc_layer,
-             gain, (__nv_bfloat16*)u, g, c0, eps);
+    launch_k(L, direct_row_kernel<true>, dim3(c1 - c0), dim3(threads), 0, (const int32_t*)nullptr, x, gain, Ac_layer, Fc_layer,
+             (__nv_bfloat16*)u, g, c0, eps);
   else if (inv != nullptr && smem == 0)
     DLLM_DISPATCH(dtype, (launch_k(L, tail_kernel<T, true>, dim3(c1 - c0), dim3(threads), smem, part, inv, x, Ac_layer,
                                    Fc_layer, gain, (T*)u, g, c0, eps)));

@@ -376,16 +376,17 @@ def test_error_paths_on_device(env):
     ses.sync()
 
 
-@pytest.mark.parametrize("hd,H,Hkv,d,B,P,R,compact", [
-    (64, 7, 1, 4736, 1, 37, 131, False),    # 131 / 168 rows, the response rows start inside a tile
-    (128, 3, 3, 5504, 2, 70, 100, True),    # 200 / 340 rows; prompt AttnOut / FFNOut rows outside the cache
+@pytest.mark.parametrize("hd,H,Hkv,d,m,B,P,R,compact", [
+    (64, 7, 1, 4736, 448, 1, 37, 131, False),   # 131 / 168 rows, the response rows start inside a tile
+    (128, 3, 3, 5504, 448, 2, 70, 100, True),   # 200 / 340 rows; prompt AttnOut / FFNOut rows outside the cache
+    (64, 8, 2, 4096, 512, 5, 79, 71, False),    # 750 rows that fit one pass of a CTA: more of them than are resident at once
 ])
-def test_bf16_projections_of_many_rows_place_their_rows(env, hd, H, Hkv, d, B, P, R, compact):
+def test_bf16_projections_of_many_rows_place_their_rows(env, hd, H, Hkv, d, m, B, P, R, compact):
     """Unsplit projections of more than 128 rows (a wide model with few k-blocks: none is split) round, rotate and place
     their own rows: full step, response refresh, and a prompt refresh whose response rows are selected (row lists).  2e-2
     as for every bf16 step; one misplaced row of 131 is 9e-2."""
     torch, dllm = env
-    cfg = synth.ModelConfig(n_layers=2, d_model=d, n_heads=H, n_kv_heads=Hkv, head_dim=hd, d_ffn=448, vocab=304,
+    cfg = synth.ModelConfig(n_layers=2, d_model=d, n_heads=H, n_kv_heads=Hkv, head_dim=hd, d_ffn=m, vocab=304,
                             mask_id=303, dtype="bf16")
     w = synth.make_weights(cfg, synth.WEIGHT_SEED)
     prompt = synth.make_prompt(cfg, B, P)
