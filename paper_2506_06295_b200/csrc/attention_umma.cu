@@ -4,10 +4,10 @@
 // their sequence (Sec. A.7), grouped KV heads packed along the row dimension.
 //
 // One CTA = TWO tiles of 128 "virtual rows" ((query, head-of-group) pairs) of
-// one (sequence, KV head) x one split of the key range, key tiles of 64, ten
+// one (sequence, KV head) x one split of the key range, key tiles of 64, eleven
 // warps with fixed roles:
-//   warp 9           TMA: K/V tiles into a six-stage ring (all that shared memory holds)
-//   warp 8           issues every tcgen05.mma of the CTA
+//   warp 10          TMA: K/V tiles into a six-stage ring (all that shared memory holds)
+//   warp 8           issues the tcgen05.mma (warp 9 those of group 1 when the groups share a row tile)
 //   warps 0-3, 4-7   the softmax group of row tile 0 resp. 1 (one row per thread)
 // Per key tile t and row tile i:
 //   S_i = Q_i K^T     tcgen05.mma, M = 128 rows, N = 64 keys, contraction HD; Q_i is
@@ -33,6 +33,8 @@
 // Key-range splits write unnormalised partials plus (max, sum) exactly like the
 // mma.sync kernel, and the same merge kernel finishes them.  Every mbarrier wait
 // is bounded.
+#include <type_traits>
+
 #include "attention_core.cuh"
 #include "internal.h"
 #include "tma.cuh"
@@ -46,7 +48,8 @@ constexpr int UA_ROWS = 128;   // virtual rows per row tile (UMMA M); a CTA work
 constexpr int UA_TILES = 2;
 constexpr int UA_KEYS = 64;    // keys per tile
 constexpr int UA_STAGES = 6;   // K/V ring
-constexpr int UA_THREADS = 320;  // two softmax groups of 128, one MMA warp, one TMA warp
+constexpr int UA_THREADS = 352;  // two softmax groups of 128, two MMA warps, one TMA warp
+constexpr int UA_TMA_WARP = 10;
 // key tiles from which a CTA with one live row tile shares them between its two softmax groups: the exchange and
 // merge of the two halves at the end cost about as much as the overlap saves on eight tiles (B200: 24 tiles per CTA
 // 135 -> 114 us at 16 x 128 rows x 1536 keys; 3-4 tiles per CTA 13.8 -> 15.0 us at 128 rows x 768 keys)
@@ -92,6 +95,24 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
 }
 
 
+// Two fp32 operations in one instruction, each rounded as the scalar one.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
+      "fma.rn.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tadd.rn.f32x2 rd, ra, rb;\n\t"
+      "mov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+
 template <int HD>
 struct UaSmem {
   static constexpr uint32_t KV_TILE = UA_KEYS * HD * 2;          // one K or V tile
@@ -99,8 +120,11 @@ struct UaSmem {
   static constexpr uint32_t TOTAL = UA_STAGES * STAGE + 1024;    // shared memory holds nothing but the K/V ring
   // Tensor memory, 128 lanes = the rows of a tile: Q_i as bf16 pairs (HD / 2 columns each), the scores S_i (64
   // fp32 columns each; the probabilities P_i overwrite the first 32 of them as bf16 pairs), the outputs O_i.
-  static constexpr uint32_t Q_COL = 0, S_COL = UA_TILES * (HD / 2), O_COL = S_COL + UA_TILES * UA_KEYS;
+  // One row tile shared by the groups: one Q, three score buffers that the key tiles take in turn, O per group.
+  static constexpr uint32_t Q_COL = 0, S_COL = UA_TILES * (HD / 2), O_COL = 64 + 3 * UA_KEYS;
+  static constexpr uint32_t KPAR_S_COL = 64;
   static constexpr uint32_t TMEM_COLS = 512;
+  static_assert(S_COL + UA_TILES * UA_KEYS <= O_COL, "scores and outputs must not overlap");
   static_assert(O_COL + UA_TILES * HD <= TMEM_COLS, "tensor memory holds 512 columns");
 };
 
@@ -115,7 +139,7 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
   constexpr int PANELS = HD / 64;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t kv_full[UA_STAGES], kv_empty[UA_STAGES];
-  __shared__ __align__(8) uint64_t s_full[UA_TILES], p_full[UA_TILES], o_full[UA_TILES], q_bar;
+  __shared__ __align__(8) uint64_t s_full[3], p_full[UA_TILES], o_full[UA_TILES], q_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
 
@@ -147,16 +171,16 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
       mbar_init(smem_u32(&kv_empty[i]), 1);
     }
     for (int i = 0; i < UA_TILES; ++i) {
-      mbar_init(smem_u32(&s_full[i]), 1);
       mbar_init(smem_u32(&p_full[i]), UA_ROWS / 32);  // one arrival per warp of the tile's softmax group
       mbar_init(smem_u32(&o_full[i]), 1);
     }
+    for (int i = 0; i < 3; ++i) mbar_init(smem_u32(&s_full[i]), 1);
     mbar_init(smem_u32(&q_bar), UA_TILES * UA_ROWS / 32);  // one arrival per softmax warp
     mbar_fence_init();
     prefetch_tensormap(&tmK);
     prefetch_tensormap(&tmV);
   }
-  if (warp == 9) {
+  if (warp == UA_TMA_WARP) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                  "r"(SM::TMEM_COLS)
                  : "memory");
@@ -170,7 +194,7 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
   pdl_trigger();
   bool ok = true;
 
-  if (warp == 9) {
+  if (warp == UA_TMA_WARP) {
     // ---------------- TMA producer: the K/V tiles of the key range ----------------
     for (int t = 0; t < n_tiles; ++t) {
       const int st = t % UA_STAGES;
@@ -191,97 +215,102 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
       }
       __syncwarp();
     }
-  } else if (warp == 8) {
-    // ---------------- MMA issuer ----------------
+  } else if (warp >= 8) {
+    // ---------------- MMA issuers: warp 8, and warp 9 for group 1 when the groups share a row tile ----------------
     // Per key tile t and row tile i:  S_i(t) = Q_i K(t)^T  ->  [softmax group i]  ->  O_i += P_i(t) V(t), and right
     // behind it S_i(t+1), so that the tensor pipe works on one row tile while the other is in its softmax.  Q_i
     // and P_i are A operands in tensor memory (P_i in the columns its scores came from), so shared memory is
-    // read for K and V only.  A commit covers every MMA issued before it, so when s_full[i] flips for tile t+1
-    // the product O_i += P_i V of tile t has completed too: the group may then rescale O_i.
-    {
-      constexpr uint32_t idesc_s = make_idesc(UA_ROWS, UA_KEYS);
-      constexpr uint32_t idesc_o = make_idesc(UA_ROWS, HD) | (1u << 16);  // B operand (V) is MN-major
-      auto issue_s = [&](int i, int st) {
-        const uint32_t k_s = kv_s + st * SM::STAGE;
-        if (elect_one()) {
+    // read for K and V only.  A commit covers every MMA its thread issued before it, so when s_full[i] flips for tile t+1
+    // the product O_i += P_i V of tile t has completed too: the group may then rescale O_i.  (With an issuing warp per row
+    // tile the MMAs of both interleave and both groups wait longer: 305 -> 409 us at 4128 x 4128 x 32 heads.)
+    constexpr uint32_t idesc_s = make_idesc(UA_ROWS, UA_KEYS);
+    constexpr uint32_t idesc_o = make_idesc(UA_ROWS, HD) | (1u << 16);  // B operand (V) is MN-major
+    auto issue_s = [&](uint32_t s_col, uint32_t q_col, int bar, int st) {
+      if (elect_one()) {
+        const uint64_t dk = make_smem_desc(kv_s + st * SM::STAGE);
 #pragma unroll
-          for (int ks = 0; ks < HD / 16; ++ks) {
-            const uint32_t koff = (ks >> 2) * (UA_KEYS * 128) + (ks & 3) * 32;  // panel, then 32 bytes per k-step
-            // A = 16 dimensions of Q_i from tensor memory (8 columns of bf16 pairs per k-step)
-            umma_bf16_ta(tmem + SM::S_COL + (uint32_t)(i * UA_KEYS), tmem + SM::Q_COL + (uint32_t)(i * (HD / 2) + ks * 8),
-                         make_smem_desc(k_s + koff), idesc_s, ks > 0 ? 1u : 0u);
-          }
-          umma_commit(smem_u32(&s_full[i]));
+        for (int ks = 0; ks < HD / 16; ++ks) {
+          const uint32_t koff = (ks >> 2) * (UA_KEYS * 128) + (ks & 3) * 32;  // panel, then 32 bytes per k-step
+          // A = 16 dimensions of Q_i from tensor memory (8 columns of bf16 pairs per k-step)
+          umma_bf16_ta(tmem + s_col, tmem + q_col + (uint32_t)(ks * 8), dk + (uint64_t)(koff >> 4), idesc_s, ks > 0 ? 1u : 0u);
         }
-        __syncwarp();
-      };
-      // O_i += P_i V: A = 16 keys of P_i from tensor memory; V: 16 key rows of 128 bytes
-      auto issue_o = [&](int i, uint32_t v_s, bool accumulate) {
-        if (elect_one()) {
-#pragma unroll
-          for (int ks = 0; ks < UA_KEYS / 16; ++ks)
-            umma_bf16_ta(tmem + SM::O_COL + (uint32_t)(i * HD), tmem + SM::S_COL + (uint32_t)(i * UA_KEYS + ks * 8),
-                         make_smem_desc_mn(v_s + ks * (16 * 128), UA_KEYS * 128, 1024), idesc_o,
-                         (accumulate || ks > 0) ? 1u : 0u);
-        }
-        __syncwarp();
-      };
-      ok = mbar_wait_warp(smem_u32(&q_bar), 0u, abortp) && mbar_wait_warp(smem_u32(&kv_full[0]), 0u, abortp);
-      if (ok && kpar) {
-        // group i owns key tiles i, i + 2, ...: S_0(0), S_1(1); then per tile t (group i = t % 2):
-        // O_i += P_i(t) V(t) and right behind it S_i(t + 2)
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        issue_s(0, 0);
-        ok = mbar_wait_warp(smem_u32(&kv_full[1]), 0u, abortp);
-        if (ok) {
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          issue_s(1, 1);
-        }
-        for (int t = 0; t < n_tiles && ok; ++t) {
-          const int i = t & 1, u = t >> 1;
-          const int st = t % UA_STAGES;
-          const uint32_t v_s = kv_s + st * SM::STAGE + SM::KV_TILE;
-          ok = mbar_wait_warp(smem_u32(&p_full[i]), (uint32_t)u & 1u, abortp);
-          if (!ok) break;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          issue_o(i, v_s, u > 0);
-          if (t + 2 < n_tiles) {
-            const int st2 = (t + 2) % UA_STAGES;
-            ok = mbar_wait_warp(smem_u32(&kv_full[st2]), (uint32_t)((t + 2) / UA_STAGES) & 1u, abortp);
-            if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            issue_s(i, st2);
-          } else {
-            if (elect_one()) umma_commit(smem_u32(&o_full[i]));  // the group's last tile: O_i is final when this fires
-          }
-          if (elect_one()) umma_commit(smem_u32(&kv_empty[st]));  // only group i reads tile t
-        }
-      } else if (ok) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        for (int i = 0; i < live; ++i) issue_s(i, 0);
+        umma_commit(smem_u32(&s_full[bar]));
       }
-      for (int t = 0; t < n_tiles && ok && !kpar; ++t) {
-        const int st = t % UA_STAGES, st_next = (t + 1) % UA_STAGES;
-        const uint32_t v_s = kv_s + st * SM::STAGE + SM::KV_TILE;
+      __syncwarp();
+    };
+    // O_i += P_i V: A = 16 keys of P_i from tensor memory; V: 16 key rows of 128 bytes
+    auto issue_o = [&](int i, uint32_t s_col, int st, bool accumulate) {
+      if (elect_one()) {
+        const uint64_t dv = make_smem_desc_mn(kv_s + st * SM::STAGE + SM::KV_TILE, UA_KEYS * 128, 1024);
+#pragma unroll
+        for (int ks = 0; ks < UA_KEYS / 16; ++ks)
+          umma_bf16_ta(tmem + SM::O_COL + (uint32_t)(i * HD), tmem + s_col + (uint32_t)(ks * 8),
+                       dv + (uint64_t)((ks * 16 * 128) >> 4), idesc_o, (accumulate || ks > 0) ? 1u : 0u);
+      }
+      __syncwarp();
+    };
+    auto tile_ready = [&](int t) {
+      const bool r = mbar_wait_warp(smem_u32(&kv_full[t % UA_STAGES]), (uint32_t)(t / UA_STAGES) & 1u, abortp);
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      return r;
+    };
+    ok = mbar_wait_warp(smem_u32(&q_bar), 0u, abortp);
+    if (kpar) {
+      // Group i owns key tiles i, i + 2, ... and issuer i its MMAs.  Tile t has score buffer t % 3: S(0), S(1), S(2); then
+      // per tile t O_i += P(t) V(t) and right behind it S(t + 3) over the same columns, so that a group finds its next
+      // scores complete when it is through with a tile.
+      const int i = warp - 8;
+      for (int t = i; t < 3 && ok; t += 2) {
+        ok = tile_ready(t);
+        if (ok) issue_s(SM::KPAR_S_COL + (uint32_t)(t * UA_KEYS), SM::Q_COL, t, t);
+      }
+      int buf = i;
+      for (int t = i, u = 0; t < n_tiles && ok; t += 2, ++u) {
+        const uint32_t s_col = SM::KPAR_S_COL + (uint32_t)(buf * UA_KEYS);
+        const int st = t % UA_STAGES;
+        ok = mbar_wait_warp(smem_u32(&p_full[i]), (uint32_t)u & 1u, abortp);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        issue_o(i, s_col, st, u > 0);
+        if (elect_one()) {
+          umma_commit(smem_u32(&o_full[i]));     // the group may rescale O_i, or it is final
+          umma_commit(smem_u32(&kv_empty[st]));  // only group i reads V(t), and S(t) completed before its softmax
+        }
+        __syncwarp();
+        if (t + 3 < n_tiles) {
+          ok = tile_ready(t + 3);
+          if (!ok) break;
+          issue_s(s_col, SM::Q_COL, buf, (t + 3) % UA_STAGES);
+        }
+        buf = buf == 0 ? 2 : buf - 1;   // (t + 2) % 3
+      }
+    } else if (warp == 8) {
+      if (ok) ok = tile_ready(0);
+      for (int i = 0; i < live && ok; ++i)
+        issue_s(SM::S_COL + (uint32_t)(i * UA_KEYS), SM::Q_COL + (uint32_t)(i * (HD / 2)), i, 0);
+      for (int t = 0; t < n_tiles && ok; ++t) {
+        const int st = t % UA_STAGES;
         bool next_ready = t + 1 >= n_tiles;
         for (int i = 0; i < live && ok; ++i) {
+          const uint32_t s_col = SM::S_COL + (uint32_t)(i * UA_KEYS);
           ok = mbar_wait_warp(smem_u32(&p_full[i]), (uint32_t)t & 1u, abortp);
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          issue_o(i, v_s, t > 0);
+          issue_o(i, s_col, st, t > 0);
           if (t + 1 < n_tiles) {
             if (!next_ready) {
-              ok = mbar_wait_warp(smem_u32(&kv_full[st_next]), (uint32_t)((t + 1) / UA_STAGES) & 1u, abortp);
+              ok = tile_ready(t + 1);
               if (!ok) break;
-              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
               next_ready = true;
             }
-            issue_s(i, st_next);
+            issue_s(s_col, SM::Q_COL + (uint32_t)(i * (HD / 2)), i, (t + 1) % UA_STAGES);
           } else {
             if (elect_one()) umma_commit(smem_u32(&o_full[i]));  // last tile: O_i is final when this fires
+            __syncwarp();
           }
         }
         if (ok && elect_one()) umma_commit(smem_u32(&kv_empty[st]));  // the stage may be refilled once these MMAs have read it
+        __syncwarp();
       }
     }
   } else {
@@ -289,32 +318,36 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
     const int i = warp >> 2;                                  // row tile
     const int row = (warp & 3) * 32 + lane;                   // row of the tile = TMEM lane
     const uint32_t row_lane = ((uint32_t)((warp & 3) * 32)) << 16;
-    const uint32_t s_col = SM::S_COL + (uint32_t)(i * UA_KEYS), o_col = SM::O_COL + (uint32_t)(i * HD);
+    const uint32_t o_col = SM::O_COL + (uint32_t)(i * HD);
     const int gtid = tid & 127;
     {
-      // Q_i: every thread fetches its own row (HD bf16 = HD / 8 16-byte words, zero past the last row) and
-      // writes it to its TMEM lane as bf16 pairs; all loads of a thread are in flight before the first use
+      // Q to tensor memory as bf16 pairs, TMEM lane = row: every thread fetches its own row (zeros past the last one), all
+      // loads in flight before the first use.  A group brings in the Q of its row tile, or its half of the one both work
+      // on.  (Eight lanes per row and a turn through shared memory: 2 us longer per CTA when several follow on an SM.)
       const int vr = row0 + (kpar ? 0 : i * UA_ROWS) + row;
+      const int p_lo = kpar ? (i * PANELS + 1) / 2 : 0, p_hi = kpar ? ((i + 1) * PANELS + 1) / 2 : i < live ? PANELS : 0;
       uint4 qv[HD / 8];
 #pragma unroll
       for (int w = 0; w < HD / 8; ++w) qv[w] = make_uint4(0, 0, 0, 0);
-      if (vr < n_rows && (i < live || kpar)) {
+      if (vr < n_rows) {
         const int qi = vr / G, g = vr - qi * G;
         const uint4* src = reinterpret_cast<const uint4*>(q + ((size_t)b * a_seq + qi) * dq + (kh * G + g) * HD);
 #pragma unroll
-        for (int w = 0; w < HD / 8; ++w) qv[w] = __ldcg(src + w);
+        for (int w = 0; w < HD / 8; ++w)
+          if (w / 8 >= p_lo && w / 8 < p_hi) qv[w] = __ldcg(src + w);
       }
 #pragma unroll
-      for (int c = 0; c < HD / 2; c += 32) {
+      for (int p = 0; p < PANELS; ++p) {
+        if (p < p_lo || p >= p_hi) continue;
         uint32_t r[32];
 #pragma unroll
         for (int w = 0; w < 8; ++w) {
-          r[4 * w] = qv[c / 4 + w].x;
-          r[4 * w + 1] = qv[c / 4 + w].y;
-          r[4 * w + 2] = qv[c / 4 + w].z;
-          r[4 * w + 3] = qv[c / 4 + w].w;
+          r[4 * w] = qv[p * 8 + w].x;
+          r[4 * w + 1] = qv[p * 8 + w].y;
+          r[4 * w + 2] = qv[p * 8 + w].z;
+          r[4 * w + 3] = qv[p * 8 + w].w;
         }
-        tmem_st32(tmem + row_lane + SM::Q_COL + (uint32_t)(i * (HD / 2) + c), r);  // waits for the store
+        tmem_st32(tmem + row_lane + SM::Q_COL + (uint32_t)((kpar ? 0 : i * (HD / 2)) + p * 32), r);  // waits for the store
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -327,12 +360,26 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
     // TMEM is only rescaled when the maximum has grown by more than RESCALE_STEP, which keeps every exponential
     // below 2^8)
     float m_ref = -INFINITY, l_run = 0.f;
-    if (i < live || kpar) {
-      // u counts this group's tiles; with kpar they are the key tiles i, i + 2, ...
-      const int t_step = kpar ? 2 : 1;
-      for (int t = kpar ? i : 0, u = 0; t < n_tiles; t += t_step, ++u) {
-        ok = mbar_wait(smem_u32(&s_full[i]), (uint32_t)u & 1u, abortp);
+    // u counts this group's tiles; with KPAR they are the key tiles i, i + 2, ...  (one instance per mode: what the loop
+    // spends on the other's bookkeeping shows in its time)
+    auto softmax_tiles = [&](auto mode) {
+      constexpr bool KPAR = decltype(mode)::value;
+      constexpr int t_step = KPAR ? 2 : 1;
+      const uint32_t s_first = tmem + row_lane + (KPAR ? SM::KPAR_S_COL : SM::S_COL);
+      int buf = i;               // score buffer of the tile, and the parity of its barrier
+      uint32_t par = 0;
+      for (int t = KPAR ? i : 0, u = 0; t < n_tiles; t += t_step, ++u) {
+        const uint32_t s_col = s_first + (uint32_t)(buf * UA_KEYS);
+        ok = mbar_wait(smem_u32(&s_full[buf]), par, abortp);
         if (!ok) break;
+        if (!KPAR) {
+          par ^= 1u;
+        } else if (buf == 0) {
+          buf = 2;
+        } else {
+          --buf;
+          par ^= 1u;
+        }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (gtid == 0 && i == 0) timeline_mark(2 + (u < 5 ? u : 5));  // scores of this group's tile u complete
         // ---- this thread's row of scores (raw: the scale is folded into the exponent's multiply-add)
@@ -341,8 +388,8 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
         float mx;
         {
           uint32_t r0[32], r1[32];  // both loads in flight, one wait
-          tmem_ld32(tmem + row_lane + s_col, r0);
-          tmem_ld32(tmem + row_lane + s_col + 32u, r1);
+          tmem_ld32(s_col, r0);
+          tmem_ld32(s_col + 32u, r1);
           tmem_ld_wait();
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
@@ -368,6 +415,11 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
             l_run *= corr;
           }
           if (u > 0) {
+            if (KPAR) {  // the group's previous product may still be running
+              ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&o_full[i]), (uint32_t)(u - 1) & 1u, abortp));
+              if (!ok) break;
+              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            }
 #pragma unroll
             for (int c = 0; c < HD; c += 32) {
               uint32_t r[32];
@@ -381,23 +433,34 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
         }
         // ---- probabilities -> tensor memory as bf16 pairs (the A operand of O_i += P_i V), over the first 32 of
         // the columns this thread has just read its scores from
-        float p_sum4[4] = {0.f, 0.f, 0.f, 0.f};
+        // (multiply-adds and sums two keys at a time: the issue slots of the two groups' warps are what the exponentials
+        // compete for)
+        float2 p_sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        const float2 scale2 = make_float2(scale_log2, scale_log2), ref2 = make_float2(-m_ref, -m_ref);
         uint32_t pk[UA_KEYS / 2];
 #pragma unroll
         for (int c2 = 0; c2 < UA_KEYS / 2; ++c2) {
-          const float p0 = fast_exp2(fmaf(sv[2 * c2], scale_log2, -m_ref));
-          const float p1 = fast_exp2(fmaf(sv[2 * c2 + 1], scale_log2, -m_ref));
-          p_sum4[c2 & 1] += p0;
-          p_sum4[2 + (c2 & 1)] += p1;
-          pk[c2] = pack_bf16(p0, p1);
+          const float2 e = fma2(make_float2(sv[2 * c2], sv[2 * c2 + 1]), scale2, ref2);
+          const float2 pp = make_float2(fast_exp2(e.x), fast_exp2(e.y));
+          p_sum[c2 & 1] = add2(p_sum[c2 & 1], pp);
+          pk[c2] = pack_bf16(pp.x, pp.y);
         }
-        l_run += (p_sum4[0] + p_sum4[1]) + (p_sum4[2] + p_sum4[3]);
-        tmem_st32(tmem + row_lane + s_col, pk);  // waits for the store
+        l_run += (p_sum[0].x + p_sum[1].x) + (p_sum[0].y + p_sum[1].y);
+        tmem_st32(s_col, pk);  // waits for the store
+        if (KPAR && u > 0) {  // the other group's issuer may be ahead of this one's: not two arrivals that it has not seen
+          ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&o_full[i]), (uint32_t)(u - 1) & 1u, abortp));
+          if (!ok) break;
+        }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&p_full[i]));
       }
-      if (ok) ok = mbar_wait(smem_u32(&o_full[i]), 0u, abortp);
+    };
+    if (i < live || kpar) {
+      if (kpar) softmax_tiles(std::true_type{});
+      else softmax_tiles(std::false_type{});
+      // O_i is final: one commit after the last tile, or one per tile of the group
+      if (ok) ok = mbar_wait(smem_u32(&o_full[i]), kpar ? (uint32_t)((n_tiles - i + 1) / 2 - 1) & 1u : 0u, abortp);
       ok = __all_sync(0xffffffffu, ok);  // the TMEM loads below are warp-collective
       // ---- one live row tile shared by the groups: group 1 hands its half (max, sum, unnormalised output) to
       // group 0 through the K/V ring, which nothing reads any more once both groups' last products are complete
@@ -500,7 +563,7 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 9) {
+  if (warp == UA_TMA_WARP) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(SM::TMEM_COLS) : "memory");
   }
 }
@@ -532,11 +595,10 @@ cudaError_t launch_umma(const Launch& L, const CUtensorMap& tmK, const CUtensorM
 
 // Key-range splits for CTAs of two 128-row tiles, whole 64-key tiles per split, no more splits than the scratch
 // holds.  A split shortens the key range a CTA walks through but adds a partial result per (row, head) pair that
-// the merge has to write and read, and a CTA with one row tile instead of two doubles the CTAs but loses the
-// overlap of the two softmax groups, so both are what a small cost model likes best (microseconds, fitted to
-// sweeps on B200: per key tile of a CTA 1.76 us with two row tiles, 1.36 us with one and 1.15 us with one whose
-// groups share the key tiles, one CTA per SM at a time, 4 us of fixed cost, and for a merge 2.5 us plus 1040 bytes
-// per pair and split at 5 TB/s).
+// the merge has to write and read, and CTAs of one row tile are twice as many, so both are what a small cost model likes
+// best (microseconds, fitted to sweeps on B200, one CTA per SM at a time: per CTA 10.6 us of fixed cost and 1.02 us per
+// key tile with two row tiles, 8.6 and 0.44 us with one that the groups share, 8.6 and 0.9 us with one that they do not;
+// for a merge 1.2 us plus 1040 bytes per pair and split at 10 TB/s).
 AttnPlan plan_attention_umma(int B, int a_seq, int n, int H, int Hkv, size_t scratch_floats) {
   AttnPlan p;
   const int G = H / Hkv, sms = sm_count();
@@ -551,12 +613,11 @@ AttnPlan plan_attention_umma(int B, int a_seq, int n, int H, int Hkv, size_t scr
     for (int S = 1; S <= key_tiles && S <= 16; ++S) {
       if (S > 1 && (size_t)S * per_split > scratch_floats) break;
       const int tps = (key_tiles + S - 1) / S;
-      // a key tile of a CTA, from 16 x 512 x 1536 and 16 x 128 x 1536 (the latter with and without the two groups
-      // sharing the key tiles)
-      const double tile_us = rt == 2 ? 1.76 : tps >= UA_KPAR_MIN_TILES ? 1.15 : 1.36;
+      const double fixed_us = rt == 2 ? 10.6 : 8.6;
+      const double tile_us = rt == 2 ? 1.02 : tps >= UA_KPAR_MIN_TILES ? 0.44 : 0.9;
       if (S > 1 && (key_tiles + tps - 1) / tps != S) continue;  // the same tiles per split as a smaller count
       const double waves = (double)((ctas * S + sms - 1) / sms);
-      const double us = 4.0 + waves * tps * tile_us + (S > 1 ? 2.5 + S * pairs * 1040.0 / 5.0e6 : 0.0);
+      const double us = waves * (fixed_us + tps * tile_us) + (S > 1 ? 1.2 + S * pairs * 1040.0 / 10.0e6 : 0.0);
       if (best_us < 0.0 || us < best_us) {
         best_s = S;
         best_rt = rt;

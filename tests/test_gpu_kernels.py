@@ -271,6 +271,26 @@ def test_attention_with_row_maxima_that_keep_growing(env, case, split):
         assert rel_l2(got[b * a:(b + 1) * a], want) < 8e-3
 
 
+@pytest.mark.parametrize("hd,n,ramp", [(128, 1536, 0.0), (128, 1500, 1.0), (64, 577, 1.0), (64, 512, 0.0)])
+def test_attention_shared_row_tiles_in_many_ctas(env, hd, n, ramp):
+    """One row tile per CTA shared by the softmax groups (three score buffers, an MMA issuer per group), several CTAs per
+    SM one after the other so that the groups drift apart: even and odd tile counts, a last tile of one key, and row maxima
+    that keep growing (ramp: every tile rescales).  Against attention in float32; 8e-3 as above."""
+    torch, dllm = env
+    B, a, H = 12, 128, 32
+    gen = torch.Generator(device="cuda").manual_seed(n + hd)
+    rnd = lambda *shape: torch.randn(*shape, device="cuda", generator=gen)
+    q = (rnd(B * a, H * hd) * (8.0 if ramp else 1.3)).bfloat16()
+    k = (rnd(B, n, H * hd) * (1.3 * (1 - ramp * torch.linspace(0.85, 0.0, n, device="cuda")))[None, :, None]).bfloat16()
+    v = rnd(B, n, H * hd).bfloat16()
+    got = dllm.attention(q, k, v, B, a, n, H, H, hd, split=False).float()
+    dllm.kernel_status()
+    heads = lambda t, rows: t.float().view(B, rows, H, hd).transpose(1, 2)
+    s = heads(q, a) @ heads(k, n).transpose(2, 3) / hd ** 0.5
+    want = (torch.softmax(s, -1) @ heads(v, n)).transpose(1, 2).reshape(B * a, H * hd)
+    assert rel_l2(got.cpu().numpy(), want.cpu().numpy()) < 8e-3
+
+
 @pytest.mark.parametrize("M,N,K", [(520, 7680, 320), (4400, 1280, 200), (300, 20000, 64)])
 def test_gemm_persistent_kernel_is_bit_identical_to_the_one_tile_kernel(env, M, N, K):
     """Unsplit products with more tiles than SMs run on the persistent kernel (one CTA per SM walks through the
