@@ -485,7 +485,7 @@ struct ProfScope {
 // the same weights soon.  rows: what an unsplit product of many rows does with its result itself (*fused).
 dllm_status run_gemm(dllm_session* s, const Launch& L, int cls, const void* A, const void* W, int M, int N, int K,
                      Partials* out, void* swiglu_out = nullptr, bool* fused = nullptr, int estimate_mask_id = -1,
-                     bool weights_again = false, const RowOut* rows = nullptr) {
+                     bool weights_again = false, const RowOut* rows = nullptr, bool unsplit = false) {
   float* part = s->wsp<float>(s->ws.part);
   if (fused) *fused = false;
   *out = Partials{part, (size_t)M * N, 1, N};
@@ -493,8 +493,8 @@ dllm_status run_gemm(dllm_session* s, const Launch& L, int cls, const void* A, c
   const double es = (double)s->es();
   const bool tensor = !(s->m->cfg.dtype == DLLM_FP32 || s->simt_gemm);
   // the LM head is never split (its consumers read logits or records), nor is a gate / up projection of more rows
-  // than stream the weights anyway: the SwiGLU epilogue saves a launch and a pass over the slabs; nor Q, K and V in one
-  const bool whole = cls == DLLM_PROF_GEMM_HEAD || (swiglu_out && M > 128 && gu_interleaved(s->m->cfg)) || (rows && rows->v);
+  // than stream the weights anyway: the SwiGLU epilogue saves a launch and a pass over the slabs
+  const bool whole = cls == DLLM_PROF_GEMM_HEAD || (swiglu_out && M > 128 && gu_interleaved(s->m->cfg)) || unsplit;
   GemmPlan plan = tensor ? plan_gemm_bf16(M, N, K, whole ? 1 : 0) : GemmPlan{};
   if (weights_again) plan.w_stream = false;
   const bool to_rows = tensor && rows && plan.pair && plan.S_max == 1;
@@ -563,9 +563,13 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
   // refresh, full step), Q, K and V are ONE product over the stacked weight whose epilogue rotates and scatters: no
   // V-verify (nothing reads its scores then), selection, gather, RoPE or V scatter launch in any layer, and the lists are
   // written once.  While profiling, V and Q / K stay launches of their own, so that each class can be read.
+  // An adaptive step that happens to recompute every row, and one that is profiled, add up in the same order: their Q, K
+  // and V products are not split either, so such a step equals a response refresh bit for bit.
   const bool tensor = dt == DLLM_BF16 && !s->simt_gemm;
-  const bool rotate = tensor && (hd == 64 || hd == 128) && !s->profiling;
-  const bool qkv_whole = rr && rotate && plan_gemm_bf16(c1, dq + 2 * dkv, d, 1).pair;
+  const bool heads = tensor && (hd == 64 || hd == 128), rotate = heads && !s->profiling;
+  const bool all_rows = rr || std::all_of(ksels.begin(), ksels.end(), [&](int k) { return k == s->R; });
+  const bool qkv_unsplit = all_rows && heads && plan_gemm_bf16(c1, dq + 2 * dkv, d, 1).pair;
+  const bool qkv_whole = qkv_unsplit && rr && rotate;
   RowOut qkv;
   qkv.qkv = 1;
   qkv.q = reinterpret_cast<__nv_bfloat16*>(s->wsp<uint8_t>(s->ws.qbuf));
@@ -611,13 +615,15 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
       o.q_by_slot = rp;
       o.k = reinterpret_cast<__nv_bfloat16*>(s->cache(l, DLLM_CACHE_K));
       o.v = reinterpret_cast<__nv_bfloat16*>(s->cache(l, DLLM_CACHE_V));
-      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_QK, u, Wq, c1, dq + 2 * dkv, d, &part, nullptr, nullptr, -1, false, &o)) !=
+      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_QK, u, Wq, c1, dq + 2 * dkv, d, &part, nullptr, nullptr, -1, false, &o, true)) !=
           DLLM_OK)
         return st;
     } else if (rr || (adaptive && s->sel_strategy == DLLM_SELECT_V_VERIFY)) {
       // V for ALL response rows (the 2 r d^2 term of Sec. A.7), V-verify, V overwrite
       // (a prompt refresh reads W_v once more, for the prompt rows)
-      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u, Wv, BR, dkv, d, &part, nullptr, nullptr, -1, rp)) != DLLM_OK) return st;
+      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u, Wv, BR, dkv, d, &part, nullptr, nullptr, -1, rp, nullptr, qkv_unsplit)) !=
+          DLLM_OK)
+        return st;
       const IdentityLists id{sel, act, inv};
       {  // the projection's fp32 result in, the cached row in, the row out
         ProfScope ps(s, DLLM_PROF_VVERIFY, (double)BR * dkv * (4.0 + 2.0 * es), 6.0 * BR * dkv, stream);
@@ -637,7 +643,7 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
     if (rp && !qkv_whole) {
       const RowOut o = rows_into(v_rows, dkv, nullptr, BR);
       if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u + (size_t)BR * d * es, Wv, BP, dkv, d, &part, nullptr, &fused, -1, false,
-                         &o)) != DLLM_OK)
+                         &o, qkv_unsplit)) != DLLM_OK)
         return st;
       if (!fused) {
         ProfScope ps(s, DLLM_PROF_SCATTER, (double)BP * dkv * (4.0 + es), 0.0, stream);
@@ -662,7 +668,8 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
       }
       if (v_for_active) {
         const RowOut o = rows_into(v_rows, dkv, act, 0);
-        if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, ua, Wv, Ma, dkv, d, &part, nullptr, &fused, -1, false, &o)) != DLLM_OK)
+        if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, ua, Wv, Ma, dkv, d, &part, nullptr, &fused, -1, false, &o, qkv_unsplit)) !=
+            DLLM_OK)
           return st;
         if (!fused) {
           ProfScope ps(s, DLLM_PROF_SCATTER, (double)Ma * dkv * (4.0 + es), 0.0, stream);
@@ -676,7 +683,7 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
         o.act = act;
         o.k = reinterpret_cast<__nv_bfloat16*>(s->cache(l, DLLM_CACHE_K));
         if ((st = run_gemm(s, L, DLLM_PROF_GEMM_QK, ua, Wq, Ma, dq + dkv, d, &part, nullptr, &rotated, -1, false,
-                           rotate ? &o : nullptr)) != DLLM_OK)
+                           rotate ? &o : nullptr, qkv_unsplit)) != DLLM_OK)
           return st;
       }
       if (!rotated) {
