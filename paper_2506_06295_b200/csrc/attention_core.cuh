@@ -1,6 +1,5 @@
-// Flash-style attention tile on the tensor cores (bf16, mma.sync), written as a
-// device function of 128 cooperating threads so that the stand-alone attention
-// kernel and the persistent layer kernel run the same code.
+// Flash-style attention tile on the tensor cores (bf16, mma.sync), a device
+// function of 128 cooperating threads.
 //
 // One call = 64 "virtual rows" of one (sequence, KV head) x one split of the key
 // range.  A virtual row is a (query, query-head-of-the-group) pair, so with

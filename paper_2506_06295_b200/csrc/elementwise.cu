@@ -40,7 +40,7 @@ __device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16* p, const fl
 }
 // Sum of the slabs of four consecutive columns, slab 0 first; up to four loads in flight.
 __device__ __forceinline__ void sum_partials4(const Partials& part, int row, int col, float (&v)[4]) {
-  const int n = part.count(row, col);
+  const int n = part.S;
   const float* base = part.p + (size_t)row * part.N + col;
   v[0] = v[1] = v[2] = v[3] = 0.f;
   for (int s = 0; s < n; s += 4) {
@@ -605,7 +605,7 @@ __global__ void __launch_bounds__(512, 2) vverify_kernel(Partials part, T* __res
   float dot = 0.f, na = 0.f, nb = 0.f;
   for (int i = threadIdx.x * 8; i < dkv; i += blockDim.x * 8) {
     float vn[8], vo[8];
-    sum_partials8(part.p, part.split_stride, part.count(c, i), (size_t)c * part.N + i, vn);
+    sum_partials8(part.p, part.split_stride, part.S, (size_t)c * part.N + i, vn);
     if (one_trip) {
 #pragma unroll
       for (int t = 0; t < 8; ++t) vo[t] = vo0[t];
@@ -641,7 +641,7 @@ void launch_vverify(const Launch& L, int dtype, Partials part, void* Vc_layer, f
   const int rows = g.B * g.R;
   const IdentityLists id = lists ? *lists : IdentityLists{};
   const size_t es = dtype == 0 ? 4 : 2, stage = (size_t)dkv * (4 + es);
-  if (rows >= STREAM_MIN_ROWS && part.S == 1 && part.upc == 0 && stream_stages(stage) >= STREAM_CONSUMERS + 1) {
+  if (rows >= STREAM_MIN_ROWS && part.S == 1 && stream_stages(stage) >= STREAM_CONSUMERS + 1) {
     const int stages = stream_stages(stage);
     const size_t smem = (size_t)stages * stage + 128;
     const int ctas = std::min(rows, sm_count());
@@ -924,7 +924,7 @@ void launch_qk_rope(const Launch& L, int dtype, Partials part, const int32_t* ac
   if (Ma <= 0) return;
   const size_t stage = (size_t)(H + Hkv) * hd * 4;
   // streaming form: unsplit slabs, a head size whose pairs a group of lanes covers exactly (a power of two, 32..256)
-  if (g.B * g.R >= STREAM_MIN_ROWS && part.S == 1 && part.upc == 0 && hd >= 32 && hd <= 256 && (hd & (hd - 1)) == 0 &&
+  if (g.B * g.R >= STREAM_MIN_ROWS && part.S == 1 && hd >= 32 && hd <= 256 && (hd & (hd - 1)) == 0 &&
       stream_stages(stage) >= STREAM_CONSUMERS + 1) {
     const int stages = stream_stages(stage);
     const size_t smem = (size_t)stages * stage + 128;
@@ -967,7 +967,7 @@ __global__ void scatter_rows_kernel(Partials part, const int32_t* __restrict__ a
   T* dst = cache + ((size_t)b * g.n + pos) * width;
   for (int i = threadIdx.x * 8; i < width; i += blockDim.x * 8) {
     float v[8];
-    sum_partials8(part.p, part.split_stride, part.count(r, i), (size_t)r * part.N + i, v);
+    sum_partials8(part.p, part.split_stride, part.S, (size_t)r * part.N + i, v);
     Vec8<T>::store(dst + i, v);
   }
 }
@@ -1058,7 +1058,7 @@ __global__ void oproj_epilogue_kernel(Partials part, const int32_t* __restrict__
     if constexpr (DIRECT)
       Vec8<T>::load_cg(arow + i, a);
     else
-      sum_partials8(part.p, part.split_stride, part.count(r, i), (size_t)r * part.N + i, a);
+      sum_partials8(part.p, part.split_stride, part.S, (size_t)r * part.N + i, a);
     if (one_trip) {
 #pragma unroll
       for (int t = 0; t < 8; ++t) xv[t] = x0[t];
@@ -1101,7 +1101,7 @@ void launch_oproj_epilogue(const Launch& L, int dtype, Partials part, const int3
   if (Ma <= 0) return;
   const bool direct = part.p == nullptr;   // bf16 models only
   const size_t stage = (size_t)g.d * (direct ? 6 : 8);
-  if (std::max(Ma, g.B * g.R) >= STREAM_MIN_ROWS && part.S == 1 && part.upc == 0 && (g.d & 7) == 0 &&
+  if (std::max(Ma, g.B * g.R) >= STREAM_MIN_ROWS && part.S == 1 && (g.d & 7) == 0 &&
       stream_stages(stage) >= STREAM_CONSUMERS + 1) {
     const int stages = stream_stages(stage);
     const size_t smem = (size_t)stages * stage + 128;
@@ -1146,8 +1146,8 @@ __global__ void silu_mul_kernel(Partials part, T* __restrict__ out, int Ma, int 
     const int r = (int)(idx / mv), j = (int)(idx - (size_t)r * mv) * 8;
     float gt[8], up[8];
     const int cg = interleaved ? (j >> 6) * 128 + (j & 63) : j, cu = interleaved ? cg + 64 : m + j;
-    sum_partials8(part.p, part.split_stride, part.count(r, cg), (size_t)r * part.N + cg, gt);
-    sum_partials8(part.p, part.split_stride, part.count(r, cu), (size_t)r * part.N + cu, up);
+    sum_partials8(part.p, part.split_stride, part.S, (size_t)r * part.N + cg, gt);
+    sum_partials8(part.p, part.split_stride, part.S, (size_t)r * part.N + cu, up);
 #pragma unroll
     for (int t = 0; t < 8; ++t) gt[t] = __fdividef(gt[t], 1.f + __expf(-gt[t])) * up[t];  // as in the GEMM epilogue
     Vec8<T>::store(out + (size_t)r * m + j, gt);
@@ -1253,7 +1253,7 @@ __global__ void __launch_bounds__(512, 2) tail_kernel(Partials part, const int32
     float ss = 0.f;
     if (i0 < d) {
       if (r >= 0) {
-        sum_partials8(part.p, part.split_stride, part.count(r, i0), (size_t)r * part.N + i0, fe);
+        sum_partials8(part.p, part.split_stride, part.S, (size_t)r * part.N + i0, fe);
         Vec8<T>::store(frow + i0, fe);
 #pragma unroll
         for (int t = 0; t < 8; ++t) fe[t] = Vec8<T>::round(fe[t]);
@@ -1284,7 +1284,7 @@ __global__ void __launch_bounds__(512, 2) tail_kernel(Partials part, const int32
     Vec8<float>::load(xr + i, xv);
     Vec8<T>::load(arow + i, a);
     if (r >= 0) {
-      sum_partials8(part.p, part.split_stride, part.count(r, i), (size_t)r * part.N + i, f);
+      sum_partials8(part.p, part.split_stride, part.S, (size_t)r * part.N + i, f);
       Vec8<T>::store(frow + i, f);
 #pragma unroll
       for (int t = 0; t < 8; ++t) f[t] = Vec8<T>::round(f[t]);
@@ -1328,7 +1328,7 @@ void launch_tail(const Launch& L, int dtype, Partials part, const int32_t* inv, 
   if (direct) inv = nullptr;
   {
     const size_t es = dtype == 0 ? 4 : 2, stage = (size_t)g.d * (8 + es);
-    if (std::max(c1 - c0, g.B * g.R) >= STREAM_MIN_ROWS && part.S == 1 && part.upc == 0 && stream_stages(stage) >= STREAM_CONSUMERS + 1) {
+    if (std::max(c1 - c0, g.B * g.R) >= STREAM_MIN_ROWS && part.S == 1 && stream_stages(stage) >= STREAM_CONSUMERS + 1) {
       const int stages = stream_stages(stage);
       const size_t smem_s = (size_t)stages * stage + 128;
       const int ctas = std::min(c1 - c0, sm_count());
@@ -1628,7 +1628,7 @@ __global__ void reduce_partials_kernel(Partials part, float* __restrict__ C, siz
   pdl_trigger();
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
     float v = part.p[i];
-    const int n_slabs = part.count((int)(i / part.N), (int)(i % part.N));
+    const int n_slabs = part.S;
     for (int s = 1; s < n_slabs; ++s) v += part.p[(size_t)s * part.split_stride + i];
     C[i] = v;
   }

@@ -584,8 +584,6 @@ GemmPlan plan_gemm_bf16(int M, int N, int K, int force_split, int force_stages, 
   p.w_stream = (long)N * K >= 8L << 20;
   p.upc = (p.num_kb + S - 1) / S;                 // k-blocks per split
   p.S_max = (p.num_kb + p.upc - 1) / p.upc;       // no empty split
-  p.ctas = (int)tiles * p.S_max;
-  p.total_units = (int)tiles * p.num_kb;
   return p;
 }
 

@@ -84,22 +84,12 @@ inline cudaError_t launch_k_cluster(const Launch& L, void (*kernel)(KArgs...), d
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// Partial sums of one GEMM: slabs of [M, N] fp32, slab stride in floats.  With
-// upc == 0 every element has S slabs; otherwise the tile that holds (row, col)
-// has as many slabs as CTAs of the persistent GEMM touched it (see
-// gemm_tcgen05.cu): units of a tile are [tile*num_kb, (tile+1)*num_kb) and CTA
-// i owns units [i*upc, (i+1)*upc).
+// Partial sums of one GEMM: S slabs of [M, N] fp32, slab stride in floats.
 struct Partials {
   const float* p;
   size_t split_stride;
   int S;
   int N;  // row length
-  int upc = 0, num_kb = 0, m_tiles = 1, BN = 256, TW = 128;
-  __host__ __device__ inline int count(int row, int col) const {
-    if (upc == 0) return S;
-    const int tile = (col / TW) * m_tiles + row / BN;
-    return ((tile + 1) * num_kb - 1) / upc - (tile * num_kb) / upc + 1;
-  }
 };
 
 // ---------------- api.cu ----------------
@@ -190,9 +180,7 @@ struct GemmPlan {
   int stages;       // depth of the TMA ring
   int num_kb;       // k-blocks of 64
   int m_tiles;      // activation tiles
-  int total_units;  // tiles * num_kb
   int upc;          // k-blocks per split
-  int ctas;         // grid size
   int S_max;        // split-K factor: slabs per output element
   bool w_stream = false;  // weights are marked evict-first (when one activation tile reads them)
   int pair = 0;     // 1: persistent CTA pairs (cta_group::2) on tiles of 256 weight rows x BN activation rows

@@ -1,5 +1,5 @@
-// tcgen05 (5th-generation tensor core) helpers shared by the GEMM kernel and
-// the persistent layer kernel: shared-memory and instruction descriptors for
+// tcgen05 (5th-generation tensor core) helpers of the GEMM and attention
+// kernels: shared-memory and instruction descriptors for
 // bf16 K-major operands with 128-byte swizzle, MMA issue, commit, TMEM loads.
 #pragma once
 #include <stdint.h>
