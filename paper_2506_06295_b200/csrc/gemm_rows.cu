@@ -3,7 +3,8 @@
 //
 // Without a split k range the fp32 result of a projection is final, and writing it for a row-wise kernel to round and
 // scatter costs 8 bytes per element of traffic and a launch.  Here the pair kernel's epilogue rounds it to what the cache
-// holds: the same bits.  The accumulator goes through shared memory 32 activation rows at a time; 16 threads per row take
+// holds: the same bits.  The accumulator goes through shared memory 16 activation rows at a time, the next
+// ones on their way out of tensor memory meanwhile; 16 threads per row take
 // the columns 4 q .. 4 q + 3 and the same 64 further, which are pairs of the rotation (32 further within a block of 64
 // columns for head_dim 64; a tile holds whole heads): 128 coalesced bytes per half warp.  Rows' places are worked out
 // before the accumulator is complete, and a trip's rotation values are requested one trip ahead (fetched where they were
@@ -16,8 +17,8 @@ namespace {
 
 struct RowForm {
   RowOut o;
-  static constexpr int CH = 32, EXS = 132;   // rows per trip; floats per staged row (16-byte aligned, rows 4 banks apart)
-  static constexpr uint32_t EX_BYTES = CH * EXS * 4;
+  static constexpr int CH = 16, EXS = 132;   // rows per trip; floats per staged row (16-byte aligned, rows 4 banks apart)
+  static constexpr uint32_t EX_BYTES = 2 * CH * EXS * 4;
   template <int BN>
   struct Shared {
     int2 row[BN];   // cache rows: {address}; Q / K / V: {row of the K / V caches, position}
@@ -53,6 +54,11 @@ struct RowForm {
     }
     const int nlo = n0 + lo, nhi = n0 + hi;
     const bool rot = o.qkv && nlo < o.dq + o.dkv, vlo = nlo < N, vhi = nhi < N;
+    // the two pieces of a rotated pair lie in one head; otherwise each has a place of its own
+    auto column = [&](int n) {
+      return n < o.dq ? o.q + n : n < o.dq + o.dkv ? o.k + (n - o.dq) : o.v + (n - o.dq - o.dkv);
+    };
+    __nv_bfloat16 *blo = column(nlo), *bhi = column(nhi);
     constexpr int U = CH / 8;
     float4 cs[U], sn[U];
     auto fetch = [&](int c0) {   // rotation values of this thread's rows c0 + rsub + 8 u
@@ -69,21 +75,25 @@ struct RowForm {
     };
     fetch(0);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    auto landed = [&](uint32_t (&r)[CH], float* stage) {   // the rows on their way out of tensor memory -> staging
+      asm volatile("tcgen05.wait::ld.sync.aligned;"
+                   : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
+                     "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])::"memory");
+#pragma unroll
+      for (int j = 0; j < CH; ++j) stage[j * EXS + tl] = __uint_as_float(r[j]);
+    };
+    uint32_t r[CH];
+    tmem_ld16(tmem_w, r);
+    landed(r, ex);
+    asm volatile("bar.sync 1, 128;" ::: "memory");
 #pragma unroll 1
     for (int c0 = 0; c0 < BN && m0 + c0 < M; c0 += CH) {
-#pragma unroll 1
-      for (int c = 0; c < CH; c += 16) {
-        uint32_t r[16];
-        tmem_ld16(tmem_w + (uint32_t)(c0 + c), r);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int j = 0; j < 16; ++j) ex[(c + j) * EXS + tl] = __uint_as_float(r[j]);
-      }
-      asm volatile("bar.sync 1, 128;" ::: "memory");
+      const float* cur = ex + (c0 & CH) / CH * (CH * EXS);
+      tmem_ld16(tmem_w + (uint32_t)min(c0 + CH, BN - CH), r);   // the next trip's rows (again the last ones in the last)
       uint2 plo[U], phi[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const float* row = ex + (rsub + 8 * u) * EXS;
+        const float* row = cur + (rsub + 8 * u) * EXS;
         float4 a = *reinterpret_cast<const float4*>(row + lo), b = *reinterpret_cast<const float4*>(row + hi);
         if (rot) {
           const float4 l = a, h = b, c = cs[u], t = sn[u];
@@ -95,7 +105,6 @@ struct RowForm {
         plo[u] = pack(a);
         phi[u] = pack(b);
       }
-      asm volatile("bar.sync 1, 128;" ::: "memory");   // the staging is free for the next trip
       fetch(c0 + CH);
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -104,14 +113,9 @@ struct RowForm {
         const int2 ri = s.row[row];
         __nv_bfloat16 *dlo, *dhi;
         if (o.qkv) {
-          // the two pieces of a rotated pair lie in one head; otherwise each is placed on its own
-          auto dst = [&](int n) {
-            return n < o.dq             ? o.q + (size_t)(o.q_by_slot ? ri.x : m0 + row) * o.dq + n
-                   : n < o.dq + o.dkv ? o.k + (size_t)ri.x * o.dkv + (n - o.dq)
-                                      : o.v + (size_t)ri.x * o.dkv + (n - o.dq - o.dkv);
-          };
-          dlo = dst(nlo);
-          dhi = dst(nhi);
+          const size_t at = (size_t)ri.x, ql = o.q_by_slot ? at : (size_t)(m0 + row);
+          dlo = blo + (nlo < o.dq ? ql * o.dq : at * o.dkv);
+          dhi = bhi + (nhi < o.dq ? ql * o.dq : at * o.dkv);
         } else {
           __nv_bfloat16* base =
               reinterpret_cast<__nv_bfloat16*>(((unsigned long long)(unsigned)ri.y << 32) | (unsigned)ri.x);
@@ -121,8 +125,9 @@ struct RowForm {
         if (vlo) *reinterpret_cast<uint2*>(dlo) = plo[u];
         if (vhi) *reinterpret_cast<uint2*>(dhi) = phi[u];
       }
+      landed(r, ex + ((c0 + CH) & CH) / CH * (CH * EXS));
+      asm volatile("bar.sync 1, 128;" ::: "memory");     // staged; behind the last trip: the rows' places are free
     }
-    asm volatile("bar.sync 1, 128;" ::: "memory");     // the rows' places are free for the next tile
   }
 };
 
