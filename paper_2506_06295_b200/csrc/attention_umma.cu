@@ -259,8 +259,13 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
       // Group i owns key tiles i, i + 2, ... and issuer i its MMAs.  Tile t has score buffer t % 3: S(0), S(1), S(2); then
       // per tile t O_i += P(t) V(t) and right behind it S(t + 3) over the same columns, so that a group finds its next
       // scores complete when it is through with a tile.
+      // A buffer's tiles belong to the groups in turn, and a wait by parity passes early when the barrier is a whole phase
+      // behind: a group may only wait for S(t) once S(t - 3), which it never waits for itself, is complete.  So issuer 0
+      // alone issues the first three, in order (a commit covers what its thread issued before): group 1, through with tile
+      // 1, knows S(0) complete when it waits for S(3), group 0 after tile 2 S(1).  S(2) precedes S(3) in issuer 0; from
+      // tile 6 on S(t - 3) precedes the product of tile t - 4 in the same issuer, which the group has waited for.
       const int i = warp - 8;
-      for (int t = i; t < 3 && ok; t += 2) {
+      for (int t = 0; t < 3 && ok && i == 0; ++t) {
         ok = tile_ready(t);
         if (ok) issue_s(SM::KPAR_S_COL + (uint32_t)(t * UA_KEYS), SM::Q_COL, t, t);
       }
