@@ -560,16 +560,24 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
 
   int32_t* inv = s->wsp<int32_t>(s->ws.inv);
   // Projections of many rows finish their own rows (gemm_rows.cu).  Where every carried row is recomputed (response
-  // refresh, full step), Q, K and V are ONE product over the stacked weight whose epilogue rotates and scatters: no
-  // V-verify (nothing reads its scores then), selection, gather, RoPE or V scatter launch in any layer, and the lists are
-  // written once.  While profiling, V and Q / K stay launches of their own, so that each class can be read.
-  // An adaptive step that happens to recompute every row, and one that is profiled, add up in the same order: their Q, K
-  // and V products are not split either, so such a step equals a response refresh bit for bit.
+  // refresh, full step) and the Q / K product is not split, it runs over the normalised rows as they lie and its epilogue
+  // rotates and scatters: no selection, gather or RoPE launch in any layer, and the lists are written once.  (Unsplit for
+  // that alone it loses: 256 x 8192 x 4096 30 us against two splits and a RoPE launch, the refresh 5788 against 5569 us.)
+  // V of the response rows is added up in the same order in every step kind, so that a row whose inputs did not change
+  // reproduces its cached V bit for bit (V-verify then scores exactly 1 or 0; against another order the L2 metric would
+  // rank rounding noise): it joins that product only where the product it has in adaptive steps is not split either.  V of
+  // the prompt rows always does.
+  // While profiling, V and Q / K stay launches of their own, so that each class can be read.
+  // An adaptive step that happens to recompute every row, and one that is profiled, equal a response refresh bit for bit:
+  // their products have the same plans, and V of the prompt rows is not split where that product has it.
   const bool tensor = dt == DLLM_BF16 && !s->simt_gemm;
   const bool heads = tensor && (hd == 64 || hd == 128), rotate = heads && !s->profiling;
   const bool all_rows = rr || std::all_of(ksels.begin(), ksels.end(), [&](int k) { return k == s->R; });
-  const bool qkv_unsplit = all_rows && heads && plan_gemm_bf16(c1, dq + 2 * dkv, d, 1).pair;
-  const bool qkv_whole = qkv_unsplit && rr && rotate;
+  const GemmPlan qk_plan = heads ? plan_gemm_bf16(c1, dq + dkv, d) : GemmPlan{};
+  const bool qk_unsplit = all_rows && heads && qk_plan.pair && qk_plan.S_max == 1;
+  const bool qk_whole = qk_unsplit && rr && rotate;
+  const bool v_whole = qk_whole && plan_gemm_bf16(BR, dkv, d).S_max == 1;   // V of the response rows too
+  const bool qkv_whole = v_whole || (qk_whole && rp);
   RowOut qkv;
   qkv.qkv = 1;
   qkv.q = reinterpret_cast<__nv_bfloat16*>(s->wsp<uint8_t>(s->ws.qbuf));
@@ -591,7 +599,7 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
     ProfScope ps(s, DLLM_PROF_EMBED, (double)(c1 - c0) * d * (4.0 + 2.0 * es), 4.0 * (c1 - c0) * d, stream);
     launch_embed_norm(L, dt, W + wl.embed, s->wsp<int32_t>(s->ws.tokens), x,
                       reinterpret_cast<const float*>(W + wl.layers[0].norm1), u, g, c0, c1, c.rms_eps,
-                      qkv_whole ? act : nullptr, qkv_whole ? inv : nullptr);
+                      qk_whole ? act : nullptr, qk_whole ? inv : nullptr);
   }
   for (int l = 0; l < c.n_layers; ++l) {
     const LayerOff& lo = wl.layers[l];
@@ -610,25 +618,17 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
     // projections and V-verify writes the (identity) lists, so no selection or gather launch is needed.
     const bool identity = rr && !rp && Ma > 0;
     bool fused = false;
-    if (qkv_whole) {
-      RowOut o = qkv;
-      o.q_by_slot = rp;
-      o.k = reinterpret_cast<__nv_bfloat16*>(s->cache(l, DLLM_CACHE_K));
-      o.v = reinterpret_cast<__nv_bfloat16*>(s->cache(l, DLLM_CACHE_V));
-      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_QK, u, Wq, c1, dq + 2 * dkv, d, &part, nullptr, nullptr, -1, false, &o, true)) !=
-          DLLM_OK)
-        return st;
+    if (v_whole) {
+      // projected with Q and K below
     } else if (rr || (adaptive && s->sel_strategy == DLLM_SELECT_V_VERIFY)) {
       // V for ALL response rows (the 2 r d^2 term of Sec. A.7), V-verify, V overwrite
       // (a prompt refresh reads W_v once more, for the prompt rows)
-      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u, Wv, BR, dkv, d, &part, nullptr, nullptr, -1, rp, nullptr, qkv_unsplit)) !=
-          DLLM_OK)
-        return st;
+      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u, Wv, BR, dkv, d, &part, nullptr, nullptr, -1, rp)) != DLLM_OK) return st;
       const IdentityLists id{sel, act, inv};
       {  // the projection's fp32 result in, the cached row in, the row out
         ProfScope ps(s, DLLM_PROF_VVERIFY, (double)BR * dkv * (4.0 + 2.0 * es), 6.0 * BR * dkv, stream);
         launch_vverify(L, dt, part, s->cache(l, DLLM_CACHE_V), sim, g, dkv, rr ? 0 : s->sel_metric,
-                       rr || !s->v_selected_only, identity ? &id : nullptr);
+                       rr || !s->v_selected_only, identity && !qk_whole ? &id : nullptr);
       }
     } else if (adaptive && s->sel_strategy == DLLM_SELECT_K_VERIFY) {
       // ablation: the same test on K; K of ALL response rows is projected, rotated and overwritten
@@ -643,7 +643,7 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
     if (rp && !qkv_whole) {
       const RowOut o = rows_into(v_rows, dkv, nullptr, BR);
       if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u + (size_t)BR * d * es, Wv, BP, dkv, d, &part, nullptr, &fused, -1, false,
-                         &o, qkv_unsplit)) != DLLM_OK)
+                         &o, qk_unsplit)) != DLLM_OK)
         return st;
       if (!fused) {
         ProfScope ps(s, DLLM_PROF_SCATTER, (double)BP * dkv * (4.0 + es), 0.0, stream);
@@ -652,9 +652,7 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
     }
     if (Ma > 0) {
       const uint8_t* ua = s->wsp<uint8_t>(s->ws.ua);
-      if (qkv_whole) {
-        // projected above
-      } else if (identity) {
+      if (qk_whole || identity) {
         ua = u;
       } else if (s->R <= 1024 && (long)Ma * s->R <= 64L * 1024) {
         // few active rows: every CTA of the gather repeats the selection rather than wait for a launch
@@ -668,24 +666,24 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
       }
       if (v_for_active) {
         const RowOut o = rows_into(v_rows, dkv, act, 0);
-        if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, ua, Wv, Ma, dkv, d, &part, nullptr, &fused, -1, false, &o, qkv_unsplit)) !=
-            DLLM_OK)
+        if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, ua, Wv, Ma, dkv, d, &part, nullptr, &fused, -1, false, &o)) != DLLM_OK)
           return st;
         if (!fused) {
           ProfScope ps(s, DLLM_PROF_SCATTER, (double)Ma * dkv * (4.0 + es), 0.0, stream);
           launch_scatter_rows(L, dt, part, act, 0, s->cache(l, DLLM_CACHE_V), g, Ma, dkv);
         }
       }
-      // Q and K of the active rows in one GEMM over the stacked [W_q; W_k]
-      bool rotated = qkv_whole;
-      if (!qkv_whole) {
-        RowOut o = qkv;
-        o.act = act;
-        o.k = reinterpret_cast<__nv_bfloat16*>(s->cache(l, DLLM_CACHE_K));
-        if ((st = run_gemm(s, L, DLLM_PROF_GEMM_QK, ua, Wq, Ma, dq + dkv, d, &part, nullptr, &rotated, -1, false,
-                           rotate ? &o : nullptr, qkv_unsplit)) != DLLM_OK)
-          return st;
-      }
+      // Q and K of the active rows in one GEMM over the stacked [W_q; W_k] (and W_v behind them)
+      bool rotated = false;
+      RowOut o = qkv;
+      if (!qk_whole) o.act = act;
+      o.q_by_slot = qk_whole && rp;
+      o.k = reinterpret_cast<__nv_bfloat16*>(s->cache(l, DLLM_CACHE_K));
+      o.v = reinterpret_cast<__nv_bfloat16*>(s->cache(l, DLLM_CACHE_V));
+      o.v_from = v_whole ? 0 : BR;
+      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_QK, ua, Wq, Ma, dq + (qkv_whole ? 2 : 1) * dkv, d, &part, nullptr, &rotated, -1,
+                         false, rotate ? &o : nullptr, qk_whole)) != DLLM_OK)
+        return st;
       if (!rotated) {
         ProfScope ps(s, DLLM_PROF_ROPE, (double)Ma * (dq + dkv) * (4.0 + es), 6.0 * Ma * (dq + dkv), stream);
         launch_qk_rope(L, dt, part, act, s->wsp<float>(s->ws.rope), s->wsp<uint8_t>(s->ws.qbuf),
@@ -701,8 +699,8 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
                                        Hkv, hd, s->wsp<float>(s->ws.attn), s->ws.attn_floats, s->simt_gemm,
                                        // the launch before attention is RoPE + K scatter or the Q / K projection itself:
                                        // every V row of the layer and, unless the prompt is refreshed, the prompt's K
-                                       // rows were written at least two launches earlier (with one product for Q, K
-                                       // and V only the prompt's V, when it is not refreshed)
+                                       // rows were written at least two launches earlier (with V in the product of Q
+                                       // and K only the prompt's V, when it is not refreshed)
                                        rp ? 0 : s->P, !qkv_whole ? s->n : rp ? 0 : s->P);
       s->prof_end(stream);
       if (e != cudaSuccess) return fail(&s->err, DLLM_CUDA_ERROR, "attention: %s", cudaGetErrorString(e));

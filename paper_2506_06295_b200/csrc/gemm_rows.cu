@@ -54,6 +54,7 @@ struct RowForm {
     }
     const int nlo = n0 + lo, nhi = n0 + hi;
     const bool rot = o.qkv && nlo < o.dq + o.dkv, vlo = nlo < N, vhi = nhi < N;
+    const int lo_from = o.qkv && nlo >= o.dq + o.dkv ? o.v_from : 0, hi_from = o.qkv && nhi >= o.dq + o.dkv ? o.v_from : 0;
     // the two pieces of a rotated pair lie in one head; otherwise each has a place of its own
     auto column = [&](int n) {
       return n < o.dq ? o.q + n : n < o.dq + o.dkv ? o.k + (n - o.dq) : o.v + (n - o.dq - o.dkv);
@@ -122,8 +123,8 @@ struct RowForm {
           dlo = base + nlo;
           dhi = base + nhi;
         }
-        if (vlo) *reinterpret_cast<uint2*>(dlo) = plo[u];
-        if (vhi) *reinterpret_cast<uint2*>(dhi) = phi[u];
+        if (vlo && m0 + row >= lo_from) *reinterpret_cast<uint2*>(dlo) = plo[u];
+        if (vhi && m0 + row >= hi_from) *reinterpret_cast<uint2*>(dhi) = phi[u];
       }
       landed(r, ex + ((c0 + CH) & CH) / CH * (CH * EXS));
       asm volatile("bar.sync 1, 128;" ::: "memory");     // staged; behind the last trip: the rows' places are free

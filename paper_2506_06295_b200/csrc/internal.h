@@ -207,6 +207,7 @@ struct RowOut {
   int base = 0;
   OutRows rows{};
   __nv_bfloat16 *q = nullptr, *k = nullptr, *v = nullptr;
+  int v_from = 0;                  // rows m from which on V is stored (those before it have theirs)
   int q_by_slot = 0;               // rows of q sequence by sequence (b * n + position) instead of row m
   const float* rope_tab = nullptr;
   int dq = 0, dkv = 0, hd = 0;
