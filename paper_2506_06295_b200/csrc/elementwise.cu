@@ -463,9 +463,10 @@ __global__ void __launch_bounds__(STREAM_THREADS, 1)
   }
 }
 
-// Rows from which the streaming forms are taken: the rows of the launch, or the session's response rows, so that with
-// many of those every step kind of the session reduces a row in the same order.  (One prompt of thousands of rows and a
-// few response rows: the full step's 4128 rows took 59.2 ms of step in the one-row-per-CTA kernels, 58.8 here.)
+// Rows from which the streaming forms are taken: a property of the session's response rows and not of the launch, since a
+// warp adds a row up in another order than a block.  (By the rows of the launch the full step of 4096 prompt and 32
+// response rows is 0.5 % faster, and its norms differ from an adaptive step's in the last bit: the next V-verify scored
+// unchanged rows by that.)
 constexpr int STREAM_MIN_ROWS = 1024;
 static int stream_stages(size_t stage_bytes) {
   const size_t fit = (227 * 1024 - 2048) / stage_bytes;
@@ -1101,7 +1102,7 @@ void launch_oproj_epilogue(const Launch& L, int dtype, Partials part, const int3
   if (Ma <= 0) return;
   const bool direct = part.p == nullptr;   // bf16 models only
   const size_t stage = (size_t)g.d * (direct ? 6 : 8);
-  if (std::max(Ma, g.B * g.R) >= STREAM_MIN_ROWS && part.S == 1 && (g.d & 7) == 0 &&
+  if (g.B * g.R >= STREAM_MIN_ROWS && part.S == 1 && (g.d & 7) == 0 &&
       stream_stages(stage) >= STREAM_CONSUMERS + 1) {
     const int stages = stream_stages(stage);
     const size_t smem = (size_t)stages * stage + 128;
@@ -1328,7 +1329,7 @@ void launch_tail(const Launch& L, int dtype, Partials part, const int32_t* inv, 
   if (direct) inv = nullptr;
   {
     const size_t es = dtype == 0 ? 4 : 2, stage = (size_t)g.d * (8 + es);
-    if (std::max(c1 - c0, g.B * g.R) >= STREAM_MIN_ROWS && part.S == 1 && stream_stages(stage) >= STREAM_CONSUMERS + 1) {
+    if (g.B * g.R >= STREAM_MIN_ROWS && part.S == 1 && stream_stages(stage) >= STREAM_CONSUMERS + 1) {
       const int stages = stream_stages(stage);
       const size_t smem_s = (size_t)stages * stage + 128;
       const int ctas = std::min(c1 - c0, sm_count());

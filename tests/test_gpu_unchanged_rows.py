@@ -26,8 +26,9 @@ def dllm():
     (WIDE, 1, 512, 256),       # V of the response is split over the k range in adaptive steps
     (GROUPED, 1, 256, 256),    # 512-wide V: many splits
     (WIDE, 2, 130, 150),       # ragged, two sequences
+    (WIDE, 1, 1100, 300),      # more than 1024 rows in a full step, 300 in the others
     (WIDE, 4, 200, 512),       # the V product of 2048 rows is not split: it joins Q and K
-], ids=["wide", "grouped", "ragged", "batched"])
+], ids=["wide", "grouped", "ragged", "long", "batched"])
 def test_unchanged_rows_score_exactly(dllm, cfg, B, P, R, metric):
     rng = np.random.default_rng(5)
     ses = dllm.Session(dllm.Model(cfg, "cuda:0").random_init_on_device(3), B, P, R)
