@@ -116,6 +116,17 @@ def test_invalid_arguments_are_rejected_without_a_gpu(dllm):
     assert dllm.lib.dllm_gemm_bf16_scratch_bytes(256, 126464, 4096) == 0      # enough tiles: no split
 
 
+@pytest.mark.parametrize("splits", [1, 2], ids=["unsplit", "split"])
+def test_gemm_without_an_output_is_rejected(dllm, splits):
+    """Whatever the plan: with a split k range the kernel itself writes to the scratch only."""
+    M, N, K = 300, 512, 256
+    p = C.c_void_p(256)                                   # never read: the arguments are rejected first
+    nbytes = dllm.lib.dllm_gemm_bf16_pair_scratch_bytes(M, N, K, 256, splits)
+    assert (nbytes > 0) == (splits > 1)
+    assert dllm.lib.dllm_gemm_bf16_pair(p, p, None, M, N, K, 256, splits, 0, p, nbytes, None) == dllm.INVALID_ARG
+    assert dllm.lib.dllm_gemm_bf16(p, p, None, 64 * splits, 4096 * splits, K, p, None) == dllm.INVALID_ARG
+
+
 def test_timeline_build_exports_its_hooks_and_the_product_library_has_none(dllm):
     """The timeline variant is a separate library with the same ABI plus one pair of hooks per kernel file; the
     product library carries no instrumentation."""
