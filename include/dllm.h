@@ -319,8 +319,9 @@ dllm_status dllm_debug_set_wait_limit_ns(uint64_t ns);
 /* Tuning / test hook: kernel choice of the bf16 projections, for every later
  * call in this process: 0 automatic (persistent CTA pairs above 128 activation
  * rows), 1 the pair kernel for every unsplit plan with 256-row activation tiles,
- * -1 always the one-tile-per-CTA kernel.  Unsplit plans give bit-identical
- * results on both. */
+ * -1 always the one-tile-per-CTA kernel, with the splits of the automatic plan.
+ * Results are bit-identical in all three, and so are a session's steps (whose
+ * row-wise kernels then place the rows that the pair kernel's epilogue places). */
 dllm_status dllm_debug_gemm_plan(int persistent);
 /* Tuning hook: overrides, for every later call in this process, the number of
  * key-range splits the tensor-core attention kernels take (0 = automatic); if

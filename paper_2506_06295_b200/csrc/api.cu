@@ -574,8 +574,8 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
   const bool heads = tensor && (hd == 64 || hd == 128), rotate = heads && !s->profiling;
   const bool all_rows = rr || std::all_of(ksels.begin(), ksels.end(), [&](int k) { return k == s->R; });
   const GemmPlan qk_plan = heads ? plan_gemm_bf16(c1, dq + dkv, d) : GemmPlan{};
-  const bool qk_unsplit = all_rows && heads && qk_plan.pair && qk_plan.S_max == 1;
-  const bool qk_whole = qk_unsplit && rr && rotate;
+  const bool qk_unsplit = all_rows && heads && qk_plan.wide && qk_plan.S_max == 1;
+  const bool qk_whole = qk_unsplit && qk_plan.pair && rr && rotate;
   const bool v_whole = qk_whole && plan_gemm_bf16(BR, dkv, d).S_max == 1;   // V of the response rows too
   const bool qkv_whole = v_whole || (qk_whole && rp);
   RowOut qkv;
@@ -807,7 +807,7 @@ dllm_status run_step(dllm_session* s, int rp, int rr, const float* rhos, int n_r
   if (!graph_ok) {
     st = enqueue_step(s, rp, rr, ksels, stream, head_start, head_len);
   } else {
-    StepKey key{rp, rr, ksels[0], forced_signature(s), s->sel_strategy * 4 + s->sel_metric * 2 + s->v_selected_only,
+    StepKey key{rp, rr, ksels[0], forced_signature(s), (s->sel_strategy * 4 + s->sel_metric * 2 + s->v_selected_only) * 3 + gemm_plan_mode() + 1,
                 uniform ? 0 : sig, head_start, head_len, s->profiling ? 1 : 0};
     auto it = s->graphs.find(key);
     if (it == s->graphs.end()) {

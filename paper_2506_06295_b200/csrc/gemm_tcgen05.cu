@@ -504,9 +504,11 @@ int sm_count() {
   return v;
 }
 
-// tuning / test override of the kernel choice for unsplit plans with 256-row tiles: 0 automatic, 1 always the
-// persistent pair kernel, -1 the one-tile kernel (see dllm_debug_gemm_plan)
+// tuning / test override of the kernel choice: 0 automatic, 1 the pair kernel for unsplit plans with 256-row tiles too,
+// -1 the one-tile kernel (see dllm_debug_gemm_plan)
 int g_gemm_force_persistent = 0;
+
+int gemm_plan_mode() { return g_gemm_force_persistent; }
 
 Partials make_partials(const float* p, int M, int N, const GemmPlan& plan) {
   return Partials{p, (size_t)M * N, plan.S_max, N};  // every element has S_max slabs
@@ -552,12 +554,14 @@ GemmPlan plan_gemm_bf16(int M, int N, int K, int force_split, int force_stages, 
   p.BN = M <= 32 ? 32 : M <= 64 ? 64 : M <= 256 ? 128 : 256;
   p.pair = 0;
   int S = 0;
-  if (force_pair == 0 && force_bn == 0 && force_split <= 1 && force_persistent >= 0 && M > 128 &&
+  if (force_pair == 0 && force_bn == 0 && force_split <= 1 && M > 128 &&
       (long)N * K >= 1L << 21) {
     // (a weight matrix of a few MB is over before a cluster launch pays: with the 448-wide test model's 144 rows the
     // step took 127 us on pairs, 121 us on the one-tile kernel)
-    p.pair = 1;
+    p.wide = true;
     plan_pair(M, N, K, force_split == 1 ? 1 : 16, &p.BN, &S);
+    p.pair = force_persistent >= 0;
+    if (!p.pair && p.BN == 192) p.BN = 128;   // the one-tile kernel on the same splits: the same sums, the same slabs
   } else if (force_pair == 0 && force_bn == 0 && force_split == 0 && M > 64 && M <= 128 && n_tiles * ((M + 63) / 64) <= sms) {
     // 65..128 rows against few weight tiles (the product will be split): two 64-row tiles per weight tile put
     // twice the CTAs on the weight stream (128 x 4096 x 4096: 14.9 against 17.8 us, 128 x 4096 x 3584: 10.0
@@ -565,7 +569,7 @@ GemmPlan plan_gemm_bf16(int M, int N, int K, int force_split, int force_stages, 
     p.BN = 64;
   }
   if (force_bn == 32 || force_bn == 64 || force_bn == 128 || force_bn == 192 || force_bn == 256) p.BN = force_bn;
-  if (force_pair > 0 || p.BN == 192 || (p.BN == 256 && force_persistent > 0 && force_split <= 1)) p.pair = p.BN >= 64;
+  if (force_pair > 0 || force_bn == 192 || (p.BN == 256 && force_persistent > 0 && force_split <= 1)) p.pair = p.BN >= 64;
   p.stages = force_stages > 0 ? force_stages : p.pair ? MAX_STAGES : (p.BN == 128 ? 3 : 4);
   p.m_tiles = (M + p.BN - 1) / p.BN;
   const long tiles = (long)p.m_tiles * n_tiles;

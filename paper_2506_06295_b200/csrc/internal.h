@@ -183,12 +183,14 @@ struct GemmPlan {
   int upc;          // k-blocks per split
   int S_max;        // split-K factor: slabs per output element
   bool w_stream = false;  // weights are marked evict-first (when one activation tile reads them)
+  bool wide = false;  // an automatic plan for pairs (also where dllm_debug_gemm_plan gives it to the one-tile kernel)
   int pair = 0;     // 1: persistent CTA pairs (cta_group::2) on tiles of 256 weight rows x BN activation rows
 };
 // 0 = auto.  force_pair: 0 auto, 1 CTA pairs (BN >= 64).  force_persistent: 0 auto, 1 the pair kernel for unsplit
-// plans with 256-row tiles, -1 the one-tile kernel for every automatic plan.
+// plans with 256-row tiles, -1 the one-tile kernel with the splits of the automatic plan.
 GemmPlan plan_gemm_bf16(int M, int N, int K, int force_split = 0, int force_stages = 0, int force_bn = 0,
                         int force_pair = 0, int force_persistent = 0);
+int gemm_plan_mode();  // what dllm_debug_gemm_plan set
 Partials make_partials(const float* p, int M, int N, const GemmPlan& plan);
 // Returns cudaSuccess or the failing error.  part must hold S*M*N floats.
 // act_out != nullptr (unsplit plan, W = gate / up rows interleaved in blocks of 64, N = 2 * m_ffn): instead of
