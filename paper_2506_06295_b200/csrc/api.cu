@@ -8,6 +8,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <new>
@@ -301,6 +302,17 @@ struct dllm_session {
   bool block_head = false;     // dllm_generate predicts only the block each step works on
   PinnedBlock pinned;          // staging of tokens and predictions; a call that uses it ends with a synchronisation
   std::mutex pinned_mu;        // held from filling it to reading it
+  // the stream that the session's work was enqueued on, or that there were several (see d2h)
+  std::atomic<void*> work_stream{nullptr};
+  std::atomic<int> work_streams{0};   // 0, 1, 2 = several
+  void enqueues_on(void* st) {
+    if (work_streams == 0) {
+      work_stream = st;
+      work_streams = 1;
+    } else if (work_stream != st) {
+      work_streams = 2;
+    }
+  }
   ~dllm_session() { give_pinned(pinned); }
   struct GraphEntry {
     cudaGraphExec_t exec;
@@ -432,7 +444,9 @@ T* staging(dllm_session* s, size_t n) {
   return static_cast<T*>(s->pinned.p);
 }
 
-// Device -> host copies ordered on the stream and complete on return, through the staging where there is one.
+// Device -> host copies ordered on the stream and complete on return, through the staging where there is one.  Where the
+// session's work is on another stream (or was on several), a copy on the legacy stream behind the synchronisation instead:
+// it waits for the work of every blocking stream, not only for this one's.
 struct HostCopy {
   void* h;
   size_t ws_off, bytes;
@@ -446,7 +460,8 @@ cudaError_t d2h(dllm_session* s, const HostCopy* c, int n, cudaStream_t st) {
     hi = std::max(hi, c[i].ws_off + c[i].bytes);
   }
   cudaError_t e;
-  uint8_t* tmp = lo < hi ? staging<uint8_t>(s, hi - lo) : nullptr;
+  const bool ordered = s->work_streams == 0 || (s->work_streams == 1 && s->work_stream == (void*)st);
+  uint8_t* tmp = ordered && lo < hi ? staging<uint8_t>(s, hi - lo) : nullptr;
   if (!tmp) {
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
     for (int i = 0; i < n; ++i)
@@ -799,6 +814,7 @@ dllm_status run_step(dllm_session* s, int rp, int rr, const float* rhos, int n_r
         return fail(&s->err, DLLM_INVALID_ARG, "forced selection of layer %d has %d rows, step selects %d", l,
                     s->forced_count[l], ksels[l]);
   cudaStream_t stream = (cudaStream_t)stream_v;
+  s->enqueues_on(stream_v);
   dllm_status st = DLLM_OK;
   const bool graph_ok = s->use_graphs && stream != nullptr && stream != cudaStreamLegacy;
   if (head_len < 0 || head_start < 0 || head_start + head_len > s->R)
@@ -1135,6 +1151,7 @@ dllm_status dllm_remask_low_confidence(dllm_session* s, int block_start, int blo
   if (block_len > 4096) return fail(&s->err, DLLM_UNSUPPORTED, "block_len > 4096");
   if (!s->have_pred) return fail(&s->err, DLLM_BAD_STATE, "no prediction yet: run a step first");
   Launch L{(cudaStream_t)stream, s->wsp<int>(s->ws.status), &s->launches};
+  s->enqueues_on(stream);
   launch_remask(L, s->wsp<int32_t>(s->ws.tokens), s->wsp<int32_t>(s->ws.x0), s->wsp<float>(s->ws.conf), s->geo(),
                 s->m->cfg.mask_id, block_start, block_len, n_transfer);
   CU_TRY(&s->err, cudaGetLastError());

@@ -407,3 +407,40 @@ def test_bf16_projections_of_many_rows_place_their_rows(env, hd, H, Hkv, d, m, B
             assert rel_l2(ses.get_cache(l, which), ref[l]) < 2e-2
     if not compact:
         compare_caches(dllm, orc, ses, 2e-2, "after")
+
+
+def test_prediction_read_through_another_blocking_stream(env):
+    """A read waits for the step even when it names another stream: both are blocking streams, and the copy behind a
+    synchronisation of its own stream is ordered with all of those."""
+    import ctypes
+    import dataclasses
+    from cuda.bindings import runtime
+    torch, dllm = env
+    cfg = dataclasses.replace(synth.LLADA_8B, n_layers=3, d_ffn=4096, vocab=1024, mask_id=1023)
+    B, P, R = 4, 500, 512                     # a step of milliseconds
+    ses = dllm.Session(dllm.Model(cfg, "cuda:0").random_init_on_device(3), B, P, R)
+    work, other = (runtime.cudaStreamCreate()[1] for _ in range(2))
+    rng = np.random.default_rng(6)
+    try:
+        ses.sp = ctypes.c_void_p(int(work))
+        ses.set_prompt(rng.integers(0, cfg.vocab - 1, size=(B, P), dtype=np.int32))
+        for _ in range(4):
+            ses.sp = ctypes.c_void_p(int(work))
+            ses.set_response_tokens(rng.integers(0, cfg.vocab - 1, size=(B, R), dtype=np.int32))
+            ses.step_full()
+            ses.sp = ctypes.c_void_p(int(other))
+            _, got = ses.pred()
+            ses.sp = ctypes.c_void_p(int(work))
+            ses.sync()
+            assert np.array_equal(got, ses.pred()[1])
+        ses.step_full()
+        ses.remask_low_confidence(0, R, R)
+        ses.sp = ctypes.c_void_p(int(other))
+        got = ses.tokens()
+        ses.sp = ctypes.c_void_p(int(work))
+        ses.sync()
+        assert np.array_equal(got, ses.tokens())
+    finally:
+        ses.close()
+        for s in (work, other):
+            runtime.cudaStreamDestroy(s)
