@@ -224,14 +224,14 @@ struct PinnedBlock {
 };
 constexpr size_t PINNED_KEPT = 8, PINNED_MAX_KEPT_BYTES = 1 << 20;
 std::mutex g_pinned_mu;
-std::vector<PinnedBlock> g_pinned_free;
+PinnedBlock g_pinned_free[PINNED_KEPT];   // p == nullptr: empty (a plain array: nothing to allocate when a session ends)
 PinnedBlock take_pinned(size_t bytes) {
   {
     std::lock_guard<std::mutex> lock(g_pinned_mu);
-    for (size_t i = 0; i < g_pinned_free.size(); ++i)
-      if (g_pinned_free[i].bytes >= bytes) {
-        const PinnedBlock b = g_pinned_free[i];
-        g_pinned_free.erase(g_pinned_free.begin() + i);
+    for (PinnedBlock& kept : g_pinned_free)
+      if (kept.p && kept.bytes >= bytes) {
+        const PinnedBlock b = kept;
+        kept = PinnedBlock{};
         return b;
       }
   }
@@ -247,10 +247,11 @@ void give_pinned(PinnedBlock b) {
   if (!b.p) return;
   if (b.bytes <= PINNED_MAX_KEPT_BYTES) {
     std::lock_guard<std::mutex> lock(g_pinned_mu);
-    if (g_pinned_free.size() < PINNED_KEPT) {
-      g_pinned_free.push_back(b);
-      return;
-    }
+    for (PinnedBlock& kept : g_pinned_free)
+      if (!kept.p) {
+        kept = b;
+        return;
+      }
   }
   cudaFreeHost(b.p);
 }
