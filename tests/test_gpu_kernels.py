@@ -171,6 +171,17 @@ def test_gemm_simt_tiles(env, M, N, K):
     assert np.array_equal(got[-1:], one)      # a row does not depend on how many others are in the launch
 
 
+def test_gemm_simt_more_rows_than_a_grid_is_high(env):
+    """2^21 + 33 rows: more 32-row tiles than one grid dimension may have (eight products per element, 2e-6 as above)."""
+    torch, dllm = env
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    A = torch.randn(2 ** 21 + 33, 8, device="cuda", generator=gen)
+    W = torch.randn(8, 8, device="cuda", generator=gen)
+    got, want = dllm.gemm_simt(A, W).double(), A.double() @ W.double().T
+    assert float((got - want).norm() / want.norm()) < 2e-6
+    assert float((got[-64:] - want[-64:]).norm() / want[-64:].norm()) < 2e-6
+
+
 @pytest.mark.parametrize("a,n,H,hd,dtype", [(1, 1, 2, 64, "fp32"), (5, 33, 3, 96, "fp32"), (4, 300, 2, 32, "fp32"),
                                             (7, 257, 2, 96, "bf16"), (620, 64, 8, 32, "fp32")])
 def test_attention_plain_alu_forms(env, a, n, H, hd, dtype):
