@@ -144,7 +144,10 @@ __global__ void __launch_bounds__(256, 1) attn_simt_few_kernel(const T* __restri
 #pragma unroll
       for (int j = 0; j < VB; ++j)
 #pragma unroll
-        for (int d = 0; d < ND; ++d) v[j][d] = to_f32<T>(Vb[(size_t)(k0 + min(j0 + j, keys - 1)) * dkv + lane + 32 * d]);
+        for (int d = 0; d < ND; ++d) {   // keys past the end: zero, whatever the last row holds (0 x inf)
+          const float x = to_f32<T>(Vb[(size_t)(k0 + min(j0 + j, keys - 1)) * dkv + lane + 32 * d]);
+          v[j][d] = j0 + j < keys ? x : 0.f;
+        }
     };
     if (keys > 0) {
       const T* krow = Kb + (size_t)(k0 + (valid ? lane : 0)) * dkv;
@@ -173,8 +176,10 @@ __global__ void __launch_bounds__(256, 1) attn_simt_few_kernel(const T* __restri
 #pragma unroll
     for (int t = 0; t < NQ; ++t) {
       const float sv = valid ? s[t] : -INFINITY;
-      const float m_new = fmaxf(m_run[t], warp_max(sv)), corr = expf(m_run[t] - m_new);  // first chunk: exp(-inf) = 0
-      p[t] = valid ? expf(sv - m_new) : 0.f;
+      const float m_new = fmaxf(m_run[t], warp_max(sv));
+      const float ref = m_new == -INFINITY ? 0.f : m_new;   // no score above -inf so far: weights 0, not exp(-inf + inf)
+      const float corr = expf(m_run[t] - ref);              // first chunk: exp(-inf) = 0
+      p[t] = valid ? expf(sv - ref) : 0.f;
       l_run[t] = l_run[t] * corr + warp_sum(p[t]);
       m_run[t] = m_new;
 #pragma unroll

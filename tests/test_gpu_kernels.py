@@ -198,6 +198,28 @@ def test_attention_plain_alu_forms(env, a, n, H, hd, dtype):
     assert rel_l2(got, want) < (1e-5 if dtype == "fp32" else 8e-3)
 
 
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("n", [300, 33])
+def test_attention_plain_alu_with_infinite_scores_and_values(env, n, dtype):
+    """Keys that overflow to a score of -inf weigh nothing, also where a warp has no others (keys 64..95 are a whole chunk);
+    an infinite value makes its own output column infinite and no other, also in a ragged last chunk.  Tolerances of
+    test_attention."""
+    torch, dllm = env
+    a, H, hd = 5, 2, 96
+    q, k, v = (synth.round_to_bf16(synth.random_normal(sh, seed=71 + i))
+               for i, sh in enumerate(((a, H * hd), (1, n, H * hd), (1, n, H * hd))))
+    q = synth.round_to_bf16(np.abs(q) + np.float32(0.5))
+    k[0, 64:96] = k[0, :3] = synth.round_to_bf16(np.full((1, H * hd), -3.0e38, np.float32))
+    td = torch.bfloat16 if dtype == "bf16" else torch.float32
+    want = O.attention(q.astype(np.float64).reshape(a, H, hd), k[0].astype(np.float64).reshape(n, H, hd),
+                       v[0].astype(np.float64).reshape(n, H, hd), H)
+    v[0, n - 1, 7] = np.inf
+    got = dllm.attention(*(torch.from_numpy(t).cuda().to(td) for t in (q, k, v)), 1, a, n, H, H, hd).float().cpu().numpy()
+    assert np.isposinf(got[:, 7]).all()
+    got[:, 7] = want[:, 7] = 0
+    assert rel_l2(got, want) < (1e-5 if dtype == "fp32" else 8e-3)
+
+
 ATT_CASES = [
     # B, a, n, H, Hkv, hd
     (1, 8, 96, 4, 4, 64),      # tiny configuration, partial step
