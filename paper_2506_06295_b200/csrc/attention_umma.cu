@@ -441,7 +441,8 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
         // (multiply-adds and sums two keys at a time: the issue slots of the two groups' warps are what the exponentials
         // compete for)
         float2 p_sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        const float2 scale2 = make_float2(scale_log2, scale_log2), ref2 = make_float2(-m_ref, -m_ref);
+        const float ref = m_ref == -INFINITY ? 0.f : m_ref;  // no score above -inf so far: weights 0, not exp2(-inf + inf)
+        const float2 scale2 = make_float2(scale_log2, scale_log2), ref2 = make_float2(-ref, -ref);
         uint32_t pk[UA_KEYS / 2];
 #pragma unroll
         for (int c2 = 0; c2 < UA_KEYS / 2; ++c2) {

@@ -324,6 +324,23 @@ def test_attention_shared_row_tiles_in_many_ctas(env, hd, n, ramp):
     assert rel_l2(got.cpu().numpy(), want.cpu().numpy()) < 8e-3
 
 
+@pytest.mark.parametrize("hd,split", [(64, False), (128, False), (128, True)])
+def test_attention_with_a_key_tile_of_infinite_scores(env, hd, split):
+    """Keys that overflow to -inf weigh nothing where they fill the first key tile of a softmax group or of a split (one row
+    tile per CTA, groups on alternate tiles of 64 keys); 8e-3 as above."""
+    torch, dllm = env
+    a, n, H = 300, 1040, 4
+    q, k, v = (synth.round_to_bf16(synth.random_normal(sh, seed=81 + i))
+               for i, sh in enumerate(((a, H * hd), (1, n, H * hd), (1, n, H * hd))))
+    q = synth.round_to_bf16(np.abs(q) + np.float32(0.5))
+    k[0, :128] = k[0, 512:576] = synth.round_to_bf16(np.full((1, H * hd), -3.0e38, np.float32))
+    got = dllm.attention(*(torch.from_numpy(t).cuda().to(torch.bfloat16) for t in (q, k, v)), 1, a, n, H, H, hd, split=split)
+    dllm.kernel_status()
+    want = O.attention(q.astype(np.float64).reshape(a, H, hd), k[0].astype(np.float64).reshape(n, H, hd),
+                       v[0].astype(np.float64).reshape(n, H, hd), H)
+    assert rel_l2(got.float().cpu().numpy(), want) < 8e-3
+
+
 @pytest.mark.parametrize("M,N,K", [(520, 7680, 320), (4400, 1280, 200), (300, 20000, 64)])
 def test_gemm_persistent_kernel_is_bit_identical_to_the_one_tile_kernel(env, M, N, K):
     """Unsplit products with more tiles than SMs run on the persistent kernel (one CTA per SM walks through the
