@@ -554,10 +554,14 @@ GemmPlan plan_gemm_bf16(int M, int N, int K, int force_split, int force_stages, 
   p.BN = M <= 32 ? 32 : M <= 64 ? 64 : M <= 256 ? 128 : 256;
   p.pair = 0;
   int S = 0;
-  if (force_pair == 0 && force_bn == 0 && force_split <= 1 && M > 128 &&
-      (long)N * K >= 1L << 21) {
-    // (a weight matrix of a few MB is over before a cluster launch pays: with the 448-wide test model's 144 rows the
-    // step took 127 us on pairs, 121 us on the one-tile kernel)
+  // Pairs, for weight matrices of 2 M elements or more: up to 128 rows they would take 0.99-1.25 of the one-tile kernel's
+  // time (B200, isolated, ten projections of 65 / 96 / 128 rows; only the LM head's 126464 x 4096 0.95-0.97).  Smaller
+  // weights are over before a cluster launch pays at few rows (144..256 rows: 5.9-9.4 us against 6.9-10.9 on pairs); pairs
+  // take them where the 256-row tiles need a second wave (8192 x 2560 x 448 35.6 -> 30.1 us, 12288 x 512 x 3584 53 -> 38)
+  // or where one wave of them would be split for many rows, whose slabs cost more (1024 x 1792 x 1024 19.1 -> 9.5,
+  // 4096 x 512 x 3584 30 -> 22; at 444 rows 11.3 against 11.5).
+  const bool many_rows = ((M + 255) / 256) * n_tiles > sms || (M >= 768 && K >= 1024);
+  if (force_pair == 0 && force_bn == 0 && force_split <= 1 && M > 128 && ((long)N * K >= 1L << 21 || many_rows)) {
     p.wide = true;
     plan_pair(M, N, K, force_split == 1 ? 1 : 16, &p.BN, &S);
     p.pair = force_persistent >= 0;

@@ -144,6 +144,29 @@ def test_gemm_bf16_pair_walk(env, M, N, K, act_tile, splits):
     assert rel_l2(got.cpu().numpy(), A.double().cpu().numpy() @ W.double().cpu().numpy().T) < 1e-5
 
 
+@pytest.mark.parametrize("M,N,K", [
+    (768, 512, 1216),     # the fewest rows of a small weight that pairs take; split
+    (1000, 328, 1032),    # ragged in every dimension
+    (2050, 2432, 448),    # more 256-row tiles than SMs, seven k-blocks
+    (19000, 250, 64),     # the same with two weight tiles and one k-block
+])
+def test_gemm_many_rows_against_a_small_weight(env, M, N, K):
+    """Tall products against weights of fewer than 2 M elements, on pairs: against the product in float64 (1e-5 as above),
+    and bit-identical to the one-tile kernel on the same splits."""
+    torch, dllm = env
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    A = torch.randn(M, K, device="cuda", generator=gen).bfloat16()
+    W = (torch.randn(N, K, device="cuda", generator=gen) * 0.05).bfloat16()
+    got = dllm.gemm_bf16(A, W)
+    dllm.kernel_status()
+    assert rel_l2(got.cpu().numpy(), (A.double() @ W.double().T).cpu().numpy()) < 1e-5
+    try:
+        dllm._check(dllm.lib.dllm_debug_gemm_plan(-1))
+        assert torch.equal(got, dllm.gemm_bf16(A, W))
+    finally:
+        dllm._check(dllm.lib.dllm_debug_gemm_plan(0))
+
+
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
 def test_gemm_simt(env, dtype):
     torch, dllm = env
