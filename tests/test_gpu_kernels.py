@@ -145,13 +145,15 @@ def test_gemm_bf16_pair_walk(env, M, N, K, act_tile, splits):
 
 
 @pytest.mark.parametrize("M,N,K", [
+    (131, 448, 448),      # 64-row tiles; the last one holds three rows
+    (577, 904, 448),      # 128-row tiles
     (768, 512, 1216),     # the fewest rows of a small weight that pairs take; split
     (1000, 328, 1032),    # ragged in every dimension
     (2050, 2432, 448),    # more 256-row tiles than SMs, seven k-blocks
     (19000, 250, 64),     # the same with two weight tiles and one k-block
 ])
 def test_gemm_many_rows_against_a_small_weight(env, M, N, K):
-    """Tall products against weights of fewer than 2 M elements, on pairs: against the product in float64 (1e-5 as above),
+    """Products of more than 128 rows against weights of fewer than 2 M elements, the tall ones on pairs: against the product in float64 (1e-5 as above),
     and bit-identical to the one-tile kernel on the same splits."""
     torch, dllm = env
     gen = torch.Generator(device="cuda").manual_seed(7)
