@@ -22,14 +22,16 @@
 //                     accumulates in TMEM and is rescaled (tcgen05.ld / st) only
 //                     when a row's maximum has grown by more than 2^8 since its
 //                     reference was set
-// The MMA warp issues O_i += P_i V of tile t and, right behind it, S_i of tile
+// One MMA warp issues O_i += P_i V of tile t and, right behind it, S_i of tile
 // t+1, alternating between the row tiles: while one group is in its softmax the
 // tensor pipe works for the other, and both row tiles read every K/V tile that
 // arrives once.  A CTA with ONE live row tile (at most 128 rows per KV head, the
-// odd last tile, or a plan of one-tile CTAs) gives both groups that tile's rows:
-// group 0 takes the even key tiles of the CTA's range and group 1 the odd ones,
-// each with its own scores, running maximum, sum and output accumulator, and the
-// two halves are merged through shared memory at the end (group 1's first).
+// odd last tile, or a plan of one-tile CTAs) and at least UA_KPAR_MIN_TILES key
+// tiles gives both groups that tile's rows: group 0 takes the even key tiles of
+// the CTA's range and group 1 the odd ones, each with its own MMA warp, running
+// maximum, sum and output accumulator; the tiles' scores take three buffers in
+// turn, and the two halves are merged through shared memory at the end (group
+// 1's first).
 // Key-range splits write unnormalised partials plus (max, sum) exactly like the
 // mma.sync kernel, and the same merge kernel finishes them.  Every mbarrier wait
 // is bounded.
@@ -50,10 +52,11 @@ constexpr int UA_KEYS = 64;    // keys per tile
 constexpr int UA_STAGES = 6;   // K/V ring
 constexpr int UA_THREADS = 352;  // two softmax groups of 128, two MMA warps, one TMA warp
 constexpr int UA_TMA_WARP = 10;
-// key tiles from which a CTA with one live row tile shares them between its two softmax groups: the exchange and
-// merge of the two halves at the end cost about as much as the overlap saves on eight tiles (B200: 24 tiles per CTA
-// 135 -> 114 us at 16 x 128 rows x 1536 keys; 3-4 tiles per CTA 13.8 -> 15.0 us at 128 rows x 768 keys)
-constexpr int UA_KPAR_MIN_TILES = 8;
+// key tiles from which a CTA with one live row tile shares them between its two softmax groups: the exchange and merge of
+// the two halves at the end cost 1.1 us, a shared tile takes 0.50 us instead of 0.93 (B200, 128 rows x 32 heads of 128, us
+// not shared -> shared: 4 tiles 10.0 -> 9.3, 5 11.0 -> 9.9, 6 12.2 -> 10.7, 7 13.0 -> 11.1, 8 13.9 -> 11.6, 16 21.1 ->
+// 15.4; heads of 64: 4 tiles 8.15 -> 7.3); the start takes three tiles at least
+constexpr int UA_KPAR_MIN_TILES = 4;
 
 // MN-major operand ([k][mn] rows of 64 mn-elements = 128 bytes, 128-byte swizzle,
 // panels of 64 mn-elements): lbo = bytes between panels along MN, sbo = bytes
@@ -151,8 +154,8 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
   const int G = H / Hkv;
   const int kh = blockIdx.y;
   const int b = blockIdx.z / S, split = blockIdx.z - b * S;
-  // row_tiles_per_cta = 1: every CTA takes one 128-row tile only (its second softmax group idles); the plan
-  // asks for that when two-tile CTAs would be too few to fill the GPU
+  // row_tiles_per_cta = 1: every CTA takes one 128-row tile only, which its softmax groups share where there are enough key
+  // tiles (else the second idles)
   const int row0 = blockIdx.x * (row_tiles_per_cta * UA_ROWS);
   const int n_rows = a_seq * G;
   const int live = (row_tiles_per_cta > 1 && row0 + UA_ROWS < n_rows) ? 2 : 1;  // row tiles of this CTA that hold rows
@@ -603,7 +606,7 @@ cudaError_t launch_umma(const Launch& L, const CUtensorMap& tmK, const CUtensorM
 // holds.  A split shortens the key range a CTA walks through but adds a partial result per (row, head) pair that
 // the merge has to write and read, and CTAs of one row tile are twice as many, so both are what a small cost model likes
 // best (microseconds, fitted to sweeps on B200, one CTA per SM at a time: per CTA 10.6 us of fixed cost and 1.02 us per
-// key tile with two row tiles, 8.6 and 0.44 us with one that the groups share, 8.6 and 0.9 us with one that they do not;
+// key tile with two row tiles, 8.6 and 0.44 us with one that the groups share, 8.6 and 0.9 us with one of fewer key tiles;
 // for a merge 1.2 us plus 1040 bytes per pair and split at 10 TB/s).
 AttnPlan plan_attention_umma(int B, int a_seq, int n, int H, int Hkv, size_t scratch_floats) {
   AttnPlan p;

@@ -349,6 +349,29 @@ def test_attention_shared_row_tiles_in_many_ctas(env, hd, n, ramp):
     assert rel_l2(got.cpu().numpy(), want.cpu().numpy()) < 8e-3
 
 
+@pytest.mark.parametrize("hd", [64, 128])
+@pytest.mark.parametrize("n", [193, 256, 257, 320, 384, 447])
+def test_attention_shared_row_tiles_with_few_keys(env, hd, n):
+    """Four to seven key tiles per CTA (the fewest that the softmax groups share) and ragged last tiles, grouped heads, one
+    CTA per row tile: 150 queries x 3 heads per KV head.  8e-3 as above."""
+    torch, dllm = env
+    B, a, H, Hkv = 2, 150, 6, 2
+    q, k, v = (synth.round_to_bf16(synth.random_normal(sh, seed=91 + i))
+               for i, sh in enumerate(((B * a, H * hd), (B, n, Hkv * hd), (B, n, Hkv * hd))))
+    try:
+        dllm._check(dllm.lib.dllm_debug_attention_plan(0, 0, 1, 1))
+        got = dllm.attention(*(torch.from_numpy(t).cuda().to(torch.bfloat16) for t in (q, k, v)), B, a, n, H, Hkv, hd,
+                             split=False)
+    finally:
+        dllm._check(dllm.lib.dllm_debug_attention_plan(0, 0, 1, 0))
+    dllm.kernel_status()
+    got = got.float().cpu().numpy()
+    for b in range(B):
+        want = O.attention(q[b * a:(b + 1) * a].astype(np.float64).reshape(a, H, hd),
+                           k[b].astype(np.float64).reshape(n, Hkv, hd), v[b].astype(np.float64).reshape(n, Hkv, hd), Hkv)
+        assert rel_l2(got[b * a:(b + 1) * a], want) < 8e-3
+
+
 @pytest.mark.parametrize("hd,split", [(64, False), (128, False), (128, True)])
 def test_attention_with_a_key_tile_of_infinite_scores(env, hd, split):
     """Keys that overflow to -inf weigh nothing where they fill the first key tile of a softmax group or of a split (one row
