@@ -24,16 +24,18 @@ constexpr int RASTER = 16;     // activation tiles per group of the launch-order
 
 // ---------------------------------------------------------------- persistent CTA-pair kernel
 // The product for more than 128 activation rows, with cta_group::2: two CTAs of a cluster work on one tile of 256
-// weight rows x BN activation rows.  Each stages its own 128 weight rows and HALF of the activation tile, one thread of the first CTA issues
-// MMAs that read both CTAs' shared memory, and each CTA ends with its own 128 x BN accumulator in its own TMEM.
-// What bounds a product from about 128 activation rows on is the L2 -> SM fabric (about 12.7 TB/s over all SMs on
-// B200): a 128 x 256 tile of one CTA moves 48 KB per k-block of 512 tensor cycles, the pair's share of 256 x 256
-// moves 32 KB.  One pair per two SMs walks through units p, p + pairs, ... (a unit = a tile, or a tile's share of
-// the k range) with fixed roles: warp 0 requests operands without a gap between units, warp 1 issues the MMAs into one
-// of TWO accumulators in tensor memory, and warps 2-5 drain one accumulator while the other fills.  The k loop of a
-// tile is the one-tile kernel's: results are bit-identical to it.  With a
-// split k range every split writes its own slab.  Loads carry no multicast: every byte is requested by the CTA
-// that stages it.
+// weight rows x BN activation rows.  Each stages its own 128 weight rows and HALF of the activation tile, one thread of
+// the first CTA issues MMAs that read both CTAs' shared memory, and each CTA ends with its own 128 x BN accumulator in
+// its own TMEM.  What bounds such a product is the L2 -> SM fabric (about 12 TB/s over all SMs on B200): a 128 x 256 tile
+// of one CTA moves 48 KB per k-block of 512 tensor cycles, the pair's share of 256 x 256 moves 32 KB.
+// One pair per two SMs walks through units p, p + pairs, ... (a unit = a tile, or a tile's share of the k range) with
+// fixed roles: warp 0 requests operands without a gap between units, warp 1 issues the MMAs into one of TWO accumulators
+// in tensor memory, and warps 2-5 drain one accumulator while the other fills.  The k loop of a tile is the one-tile
+// kernel's: results are bit-identical to it.  With a split k range every split writes its own slab.  Loads carry no
+// multicast: every byte is requested by the CTA that stages it.
+// (In the replayed response refresh of 256 rows, us from the release to the first stage / accumulators complete / rows
+// written: Q/K in two splits 1.9 / 12.8 / 15.6, down in two 1.7 / 18.5 / 21.2, gate / up with SwiGLU, two rounds, 2.4 /
+// 25.8-49.0 / 31.6-54.7: an epilogue of slabs takes 2.8 us, of SwiGLU 5.8, of placed and rotated rows 16.)
 constexpr int PAIR_THREADS = 192;
 template <int BN, typename FORM>
 struct PairLayout {
@@ -187,6 +189,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1)
             ok = false;
             break;
           }
+          if (j == 0 && kb == kb0 && lane == 0) timeline_mark(1);   // first stage complete
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t sW = tiles_s + s * PL::STAGE_BYTES, empty = smem_u32(&empty_bar[s]);
           if (++s == STAGES) {
@@ -236,10 +239,12 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1)
         ok = false;
         break;
       }
+      if (tl == 0) timeline_mark(3);                                // accumulator complete
       const int nt = 2 * np + rank;
       if (nt * TILE_W < N)  // the second CTA of the last pair has no rows when the weight tiles are odd in number
         form.template drain<BN>(fs, tmem_d + (uint32_t)a * ACC, ex, tl, mt * BN, nt * TILE_W, nt, M, N,
                                 part + (size_t)z * split_stride);
+      if (tl == 0) timeline_mark(4);                                // this thread's part of the epilogue written
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(cluster_addr(smem_u32(&acc_empty[a]), 0));
