@@ -62,7 +62,8 @@ __device__ __forceinline__ void sum_partials4(const Partials& part, int row, int
 // per SM for the whole launch: a producer thread fetches the rows of the CTA (blockIdx.x, + gridDim.x, ...) by
 // untiled bulk copies into a ring of shared-memory stages, ahead of four consumer warps that each take a whole
 // row (no block barrier: lane-local sums and one warp reduction per row) and write its results straight to
-// global memory.  Split-K slabs are not supported here (S = 1: with this many rows no projection is split).
+// global memory.  Split-K slabs are not supported here: behind a split product (few selected rows, or a narrow V) the
+// one-row kernels run.
 constexpr int STREAM_CONSUMERS = 4;                 // warps 1..4; warp 0 produces
 constexpr int STREAM_THREADS = 32 * (1 + STREAM_CONSUMERS);
 constexpr int STREAM_MAX_STAGES = 12;

@@ -391,8 +391,8 @@ def test_attention_with_a_key_tile_of_infinite_scores(env, hd, split):
 
 @pytest.mark.parametrize("M,N,K", [(520, 7680, 320), (4400, 1280, 200), (300, 20000, 64)])
 def test_gemm_persistent_kernel_is_bit_identical_to_the_one_tile_kernel(env, M, N, K):
-    """Unsplit products with more tiles than SMs run on the persistent kernel (one CTA per SM walks through the
-    tiles, two accumulators, epilogue under the next main loop).  Same k loop per tile: the same bits as the
+    """Products of many rows run on the persistent pair kernel (a CTA pair per two SMs walks through the tiles, two
+    accumulators, epilogue under the next main loop).  Same k loop per tile: the same bits as the
     one-tile-per-CTA kernel, for the plain epilogue and for the SwiGLU epilogue; ragged activation tiles, a ragged
     k block, more than 16 activation tiles (the launch-order remap), fewer tiles than SMs."""
     torch, dllm = env
@@ -417,7 +417,7 @@ def test_gemm_persistent_kernel_is_bit_identical_to_the_one_tile_kernel(env, M, 
 
 @pytest.mark.parametrize("M,N,K,forced", [(576, 20000, 320, 0), (530, 1280, 200, 192), (192, 384, 64, 192)])
 def test_gemm_192_row_tiles(env, M, N, K, forced):
-    """Activation tiles of 192 rows in the persistent kernel (the 576 rows of a mixed step are 3 x 192, not
+    """Activation tiles of 192 rows in the persistent pair kernel (the 576 rows of a mixed step are 3 x 192, not
     3 x 256): the default plan takes them for 576 rows against many weight tiles; ragged last tile, a ragged k
     block, a single tile.  The k loop per output element is the same: the same bits as with 256-row tiles, for
     the plain and for the SwiGLU epilogue."""

@@ -382,9 +382,9 @@ def test_error_paths_on_device(env):
     (64, 8, 2, 4096, 512, 5, 79, 71, False),    # 750 rows that fit one pass of a CTA: more of them than are resident at once
 ])
 def test_bf16_projections_of_many_rows_place_their_rows(env, hd, H, Hkv, d, m, B, P, R, compact):
-    """Unsplit projections of more than 128 rows (a wide model with few k-blocks: none is split) round, rotate and place
-    their own rows: full step, response refresh, and a prompt refresh whose response rows are selected (row lists).  2e-2
-    as for every bf16 step; one misplaced row of 131 is 9e-2."""
+    """Steps of wide models with few k-blocks per O and down product, whose rows the unsplit ones of more than 128 rows place
+    themselves (Q / K and V are split here: test_gpu_row_epilogue.py has them unsplit): full step, response refresh, and a
+    prompt refresh whose response rows are selected.  2e-2 as for every bf16 step; one misplaced row of 131 is 9e-2."""
     torch, dllm = env
     cfg = synth.ModelConfig(n_layers=2, d_model=d, n_heads=H, n_kv_heads=Hkv, head_dim=hd, d_ffn=m, vocab=304,
                             mask_id=303, dtype="bf16")
