@@ -643,7 +643,9 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
       const IdentityLists id{sel, act, inv};
       {  // the projection's fp32 result in, the cached row in, the row out
         ProfScope ps(s, DLLM_PROF_VVERIFY, (double)BR * dkv * (4.0 + 2.0 * es), 6.0 * BR * dkv, stream);
-        launch_vverify(L, dt, part, s->cache(l, DLLM_CACHE_V), sim, g, dkv, rr ? 0 : s->sel_metric,
+        // (with random selection the scores are the caller's and outlive a refresh)
+        launch_vverify(L, dt, part, s->cache(l, DLLM_CACHE_V),
+                       rr && s->sel_strategy == DLLM_SELECT_RANDOM ? nullptr : sim, g, dkv, rr ? 0 : s->sel_metric,
                        rr || !s->v_selected_only, identity && !qk_whole ? &id : nullptr);
       }
     } else if (adaptive && s->sel_strategy == DLLM_SELECT_K_VERIFY) {

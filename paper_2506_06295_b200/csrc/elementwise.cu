@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(STREAM_THREADS, 1)
       na = warp_sum(na);
       nb = warp_sum(nb);
       if (lane == 0) {
-        sim[c] = metric == 0 ? dot / fmaxf(sqrtf(na * nb), 1e-8f) : -sqrtf(dot);
+        if (sim) sim[c] = metric == 0 ? dot / fmaxf(sqrtf(na * nb), 1e-8f) : -sqrtf(dot);
         if (id.act) {  // a response refresh recomputes every response row, in carried order: identity lists
           id.sel[c] = c % g.R;
           id.act[c] = c;
@@ -589,7 +589,7 @@ __device__ __forceinline__ int32_t* select_sequence(unsigned long long* keys, co
 // ------------------------------------------------------------------ V-verify (Eq. 6) + V overwrite
 // metric 0: cosine (Eq. 6); 1: negated Euclidean distance (Sec. A.6), so that the
 // least similar rows have the lowest score either way.  write_v 0: the cache is
-// left as it is (the selected-only variant of Sec. A.5 writes the selected rows later).
+// left as it is (the selected-only variant of Sec. A.5 writes the selected rows later).  sim may be null: no scores.
 // The launch before this one is the V projection, which writes nothing but `part`: a row that fits one pass
 // fetches its cached V row before the dependency wait, while the projection still runs.
 template <typename T>
@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(512, 2) vverify_kernel(Partials part, T* __res
     if (write_v) Vec8<T>::store(vrow + i, vn);
   }
   block_sum3(dot, na, nb, red);
-  if (threadIdx.x == 0) sim[c] = metric == 0 ? dot / fmaxf(sqrtf(na * nb), 1e-8f) : -sqrtf(dot);
+  if (threadIdx.x == 0 && sim) sim[c] = metric == 0 ? dot / fmaxf(sqrtf(na * nb), 1e-8f) : -sqrtf(dot);
   // a response refresh recomputes every response row, in carried order: the lists are the identity
   if (id.act && threadIdx.x == 0) {
     id.sel[c] = j;

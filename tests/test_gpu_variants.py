@@ -91,3 +91,24 @@ def test_per_layer_update_ratio_matches_the_oracle(env, mode):
         compare_caches(dllm, orc, ses, tol, f"step {step}")
     with pytest.raises(dllm.DllmError):
         ses.step_cached_layers(False, False, [0.25])
+
+
+@pytest.mark.parametrize("mode", ["fp32", "bf16"])
+def test_random_selection_scores_outlive_a_refresh(env, mode):
+    """Scores stay in place until set again: a full step, a response refresh and a mixed step leave them alone."""
+    torch, dllm = env
+    cfg, B, P, R = (synth.TINY, 2, 64, 32) if mode == "fp32" else (synth.small_bf16_model(), 2, 150, 72)
+    _, ses, _ = make_pair(dllm, cfg, B, P, R)
+    ses.set_selection("random")
+    scores = synth.random_uniform((cfg.n_layers, B, R), 7)
+    for l in range(cfg.n_layers):
+        ses.set_scores(l, scores[l])
+    ses.step_full()
+    for rp, rr in ((False, False), (False, True), (False, False), (True, False), (True, True), (False, False)):
+        ses.step_cached(rp, rr, 0.25)
+        ses.sync()
+        for l in range(cfg.n_layers):
+            idx, _ = ses.selected(l)
+            for b in range(B):
+                want = np.arange(R) if rr else O.select_lowest(scores[l, b], R // 4)
+                assert np.array_equal(idx[b], want), f"({rp},{rr}) layer {l}"
