@@ -34,7 +34,7 @@ constexpr int RASTER = 16;     // activation tiles per group of the launch-order
 // kernel's: results are bit-identical to it.  With a split k range every split writes its own slab.  Loads carry no
 // multicast: every byte is requested by the CTA that stages it.
 // (In the replayed response refresh of 256 rows, us from the release to the first stage / accumulators complete / rows
-// written: Q/K in two splits 1.9 / 12.8 / 15.6, down in two 1.7 / 18.5 / 21.2, gate / up with SwiGLU, two rounds, 2.4 /
+// written: Q/K in two splits 1.9 / 12.8 / 15.6, down in four 1.7 / 18.5 / 21.2, gate / up with SwiGLU, two rounds, 2.4 /
 // 25.8-49.0 / 31.6-54.7: an epilogue of slabs takes 2.8 us, of SwiGLU 5.8, of placed and rotated rows 16.)
 constexpr int PAIR_THREADS = 192;
 template <int BN, typename FORM>
