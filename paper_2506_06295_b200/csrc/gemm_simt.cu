@@ -50,8 +50,7 @@ __global__ void __launch_bounds__(SG_WARPS * 32)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* As = sg_smem + warp * (BM + BN) * SG_LD;
   float* Ws = As + BM * SG_LD;
-  const int m0 = (blockIdx.y + blockIdx.z * gridDim.y) * BM, n0 = blockIdx.x * BN;
-  if (m0 >= M) return;                                      // the last layer of the grid
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   const int lr = lane >> 3, lk = (lane & 7) * 4;            // loads: four rows per pass, 8 lanes x 4 k per row
   const int chunks = (K + SG_K - 1) / SG_K;
   float4 ra[TM], rw[2 * TN];
@@ -125,10 +124,14 @@ void launch_tile(const Launch& L, const void* A, const void* W, float* C, int M,
       cudaSuccess)
     return;  // the error stays for the caller's cudaGetLastError
   const bool vec = K % 4 == 0 && (((uintptr_t)A | (uintptr_t)W) & (4 * sizeof(T) - 1)) == 0;
-  // a grid is at most 65535 high: millions of rows take several layers of it
-  const int m_tiles = (M + BM - 1) / BM, layers = (m_tiles + 65534) / 65535;
-  launch_k(L, gemm_simt_kernel<T, TM, TN>, dim3((N + BN - 1) / BN, (m_tiles + layers - 1) / layers, layers), dim3(SG_WARPS * 32),
-           SMEM, (const T*)A, (const T*)W, C, M, N, K, vec);
+  // a grid is at most 65535 high: millions of rows take several launches (a third grid dimension in the kernel's indices
+  // cost the tiny configuration's generations up to 3 %)
+  constexpr int MOST = 65535 * BM;
+  for (long r = 0; r < M; r += MOST) {
+    const int rows = (int)(M - r < MOST ? M - r : MOST);
+    launch_k(L, gemm_simt_kernel<T, TM, TN>, dim3((N + BN - 1) / BN, (rows + BM - 1) / BM), dim3(SG_WARPS * 32), SMEM,
+             (const T*)A + (size_t)r * K, (const T*)W, C + (size_t)r * N, rows, N, K, vec);
+  }
 }
 
 }  // namespace
