@@ -1,9 +1,14 @@
 // The persistent CTA-pair GEMM (tcgen05, cta_group::2), with the epilogue as a parameter.
 //
-// FORM: what happens to a finished tile (a kernel argument).  EX_BYTES of staging; Shared<BN> static shared memory; ahead()
-// runs before the accumulator is waited for, drain() behind it, both by the 128 epilogue threads (tl = 0..127 = TMEM lane,
-// meeting on named barrier 1).  One kernel instance holds one form's code: an epilogue runs once per launch from a cold
-// instruction cache, and a form's unused neighbours in the same body cost more than their branches.
+// FORM: what happens to a finished tile (a kernel argument), W = BN / GROUPS of its columns by each of GROUPS groups of 128
+// epilogue threads.  ex_bytes<W>() of staging and Shared<W> static shared memory per group; ahead() runs before the
+// accumulator is waited for, drain() behind it (tl = 0..127 = TMEM lane; a group meets on its named barrier).  One kernel
+// instance holds one form's code: an epilogue runs once per launch from a cold instruction cache, and a form's unused
+// neighbours in the same body cost more than their branches.
+// An epilogue is bound by the latency of its own instructions: one group puts one warp on each scheduler, which waits for
+// every result it needs next.  Two groups halve the staged forms: SwiGLU of 256 rows 5.8 -> 3.9 us, placed and rotated rows
+// 16 -> about 6 (with fewer instructions per row, see gemm_rows.cu).  Slabs take 2.8 us either way (their stores) and keep
+// one group, whose 192 small threads leave room for the next kernel's CTAs.
 #pragma once
 #include <algorithm>
 
@@ -22,6 +27,29 @@ constexpr uint32_t W_STAGE_BYTES = TILE_W * TILE_K * 2;
 constexpr int MAX_STAGES = 12;
 constexpr int RASTER = 16;     // activation tiles per group of the launch-order remap
 
+// A group of 128 epilogue threads meets on named barrier 1 or 2 (numbers in the code: a barrier named by a register would
+// reserve all sixteen).
+__device__ __forceinline__ void group_sync(int bar) {
+  if (bar == 1)
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+  else
+    asm volatile("bar.sync 2, 128;" ::: "memory");
+}
+template <int BAR>
+__device__ __forceinline__ bool group_all_on(bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 q, %1, 0;\n\t"
+      "bar.red.and.pred p, %2, 128, q;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)v), "n"(BAR)
+      : "memory");
+  return r != 0;
+}
+__device__ __forceinline__ bool group_all(int bar, bool v) { return bar == 1 ? group_all_on<1>(v) : group_all_on<2>(v); }
+
 // ---------------------------------------------------------------- persistent CTA-pair kernel
 // The product for more than 128 activation rows, with cta_group::2: two CTAs of a cluster work on one tile of 256
 // weight rows x BN activation rows.  Each stages its own 128 weight rows and HALF of the activation tile, one thread of
@@ -30,24 +58,27 @@ constexpr int RASTER = 16;     // activation tiles per group of the launch-order
 // of one CTA moves 48 KB per k-block of 512 tensor cycles, the pair's share of 256 x 256 moves 32 KB.
 // One pair per two SMs walks through units p, p + pairs, ... (a unit = a tile, or a tile's share of the k range) with
 // fixed roles: warp 0 requests operands without a gap between units, warp 1 issues the MMAs into one of TWO accumulators
-// in tensor memory, and warps 2-5 drain one accumulator while the other fills.  The k loop of a tile is the one-tile
+// in tensor memory, and the other warps drain one accumulator while the other fills.  The k loop of a tile is the one-tile
 // kernel's: results are bit-identical to it.  With a split k range every split writes its own slab.  Loads carry no
 // multicast: every byte is requested by the CTA that stages it.
 // (In the replayed response refresh of 256 rows, us from the release to the first stage / accumulators complete / rows
 // written: Q/K in two splits 1.9 / 12.8 / 15.6, down in four 1.7 / 18.5 / 21.2, gate / up with SwiGLU, two rounds, 2.4 /
-// 25.8-49.0 / 31.6-54.7: an epilogue of slabs takes 2.8 us, of SwiGLU 5.8, of placed and rotated rows 16.)
-constexpr int PAIR_THREADS = 192;
+// 25.8-49.0 / 30-53.)
+template <typename FORM>
+constexpr int PAIR_THREADS = 64 + 128 * FORM::GROUPS;
 template <int BN, typename FORM>
 struct PairLayout {
   static constexpr uint32_t A_HALF_BYTES = (BN / 2) * TILE_K * 2;
   static constexpr uint32_t STAGE_BYTES = W_STAGE_BYTES + A_HALF_BYTES;
-  static constexpr uint32_t EX_BYTES = FORM::EX_BYTES;  // staging of the forms that go through shared memory
+  static constexpr int W = BN / FORM::GROUPS;
+  // staging of the forms that go through shared memory, all groups'
+  static constexpr uint32_t EX_GROUP = FORM::template ex_bytes<W>(), EX_BYTES = FORM::GROUPS * EX_GROUP;
   static constexpr uint32_t total(int stages, bool staged) {
     return (uint32_t)stages * STAGE_BYTES + (staged ? EX_BYTES : 0) + 1024;
   }
   static constexpr int most(bool staged) {
-    const int fit = (227 * 1024 - 1024 - 512 - (int)sizeof(typename FORM::template Shared<BN>) - (staged ? (int)EX_BYTES : 0)) /
-                    (int)STAGE_BYTES;
+    const int shared = FORM::GROUPS * (int)sizeof(typename FORM::template Shared<W>);
+    const int fit = (227 * 1024 - 1024 - 512 - shared - (staged ? (int)EX_BYTES : 0)) / (int)STAGE_BYTES;
     return fit < MAX_STAGES ? fit : MAX_STAGES;
   }
 };
@@ -65,7 +96,7 @@ __device__ __forceinline__ void pair_unit(int u, int m_tiles, int n_pairs, int& 
 }
 
 template <int BN, bool ONCE, typename FORM>
-__global__ void __launch_bounds__(PAIR_THREADS, 1)
+__global__ void __launch_bounds__(PAIR_THREADS<FORM>, 2)
     gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmA,
                           float* __restrict__ part, int M, int N, int num_kb, int kb_per_split, size_t split_stride,
                           int m_tiles, int n_pairs, int units, int STAGES, const __grid_constant__ FORM form,
@@ -78,7 +109,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1)
   __shared__ __align__(8) uint64_t empty_bar[MAX_STAGES];  // in each CTA: its stage may be refilled
   __shared__ __align__(8) uint64_t acc_full[2];            // in each CTA: accumulator complete
   __shared__ __align__(8) uint64_t acc_empty[2];           // used in the first CTA: both CTAs' epilogues have read it
-  __shared__ typename FORM::template Shared<BN> fs;
+  __shared__ typename FORM::template Shared<PL::W> fs[FORM::GROUPS];
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
 
@@ -99,7 +130,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(smem_u32(&acc_full[a]), 1);
-      mbar_init(smem_u32(&acc_empty[a]), 2 * 4);  // one arrival per epilogue warp of both CTAs
+      mbar_init(smem_u32(&acc_empty[a]), 2 * 4 * FORM::GROUPS);  // one arrival per epilogue warp of both CTAs
     }
     mbar_fence_init();
     prefetch_tensormap(&tmW);
@@ -212,39 +243,32 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1)
       }
     }
   } else {
-    // ---------------- epilogue warps 2..5 of both CTAs: own 128 weight rows, TMEM lanes 32 * (warp % 4) .. + 31 ----
-    const int tl = (warp & 3) * 32 + lane;
+    // ---------------- epilogue warps of both CTAs: own 128 weight rows, TMEM lanes 32 * (warp % 4) .. + 31; warps 2-5 the
+    // first W activation rows, warps 6-9 (where there are two groups) the others ----
+    constexpr int W = PL::W;
+    const int tl = (warp & 3) * 32 + lane, group = FORM::GROUPS == 1 ? 0 : (warp - 2) >> 2, bar = 1 + group;
     int j = 0;
     for (int u = pair; u < units; u += pairs, ++j) {
       const int a = j & 1;
       int mt, np, z;
       pair_unit(u, m_tiles, n_pairs, mt, np, z);
-      form.template ahead<BN>(fs, tl, mt * BN, M);
+      const int m0 = mt * BN + group * W;
+      form.template ahead<W>(fs[group], tl, m0, M);
       bool have = mbar_wait(smem_u32(&acc_full[a]), (uint32_t)(j >> 1) & 1u, abortp);
-      // the 128 epilogue threads agree (the TMEM loads are warp-collective and the staged forms exchange data)
-      {
-        uint32_t r;
-        asm volatile(
-            "{\n\t.reg .pred p, q;\n\t"
-            "setp.ne.u32 q, %1, 0;\n\t"
-            "bar.red.and.pred p, 1, 128, q;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(r)
-            : "r"((uint32_t)have)
-            : "memory");
-        have = r != 0;
-      }
+      // the 128 threads of the group agree (the TMEM loads are warp-collective and the staged forms exchange data)
+      have = group_all(bar, have);
       if (!have) {
         if (tl == 0 && status) atomicCAS(status, ST_OK, ST_TIMEOUT_EPI);
         ok = false;
         break;
       }
-      if (tl == 0) timeline_mark(3);                                // accumulator complete
+      if (tl == 0 && group == 0) timeline_mark(3);                   // accumulator complete
       const int nt = 2 * np + rank;
       if (nt * TILE_W < N)  // the second CTA of the last pair has no rows when the weight tiles are odd in number
-        form.template drain<BN>(fs, tmem_d + (uint32_t)a * ACC, ex, tl, mt * BN, nt * TILE_W, nt, M, N,
-                                part + (size_t)z * split_stride);
-      if (tl == 0) timeline_mark(4);                                // this thread's part of the epilogue written
+        form.template drain<W>(fs[group], tmem_d + (uint32_t)(a * ACC + group * W),
+                               ex + group * (PL::EX_GROUP / 4), tl, bar, m0, nt * TILE_W, nt, M, N,
+                               part + (size_t)z * split_stride);
+      if (tl == 0 && group == 0) timeline_mark(4);                         // this thread's part of the epilogue written
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(cluster_addr(smem_u32(&acc_empty[a]), 0));
@@ -267,14 +291,14 @@ cudaError_t launch_pair_form(const Launch& L, const CUtensorMap& tmW, const CUte
   static DeviceOnce once;
   cudaError_t e0 = once.run([] {
     return cudaFuncSetAttribute(gemm_bf16_pair_kernel<BN, ONCE, FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                227 * 1024 - 512 - (int)sizeof(typename FORM::template Shared<BN>));
+                                227 * 1024 - 512 - FORM::GROUPS * (int)sizeof(typename FORM::template Shared<BN / FORM::GROUPS>));
   });
   if (e0 != cudaSuccess) return e0;
   const int most = PL::most(staged), stages = plan.stages < 2 ? 2 : plan.stages > most ? most : plan.stages;
   const int m_tiles = (M + BN - 1) / BN, n_pairs = (N + 2 * TILE_W - 1) / (2 * TILE_W);
   const int units = m_tiles * n_pairs * plan.S_max;
   const int pairs = std::min(units, sm_count() / 2);
-  cudaError_t e = launch_k_cluster(L, gemm_bf16_pair_kernel<BN, ONCE, FORM>, dim3(2 * pairs), dim3(PAIR_THREADS),
+  cudaError_t e = launch_k_cluster(L, gemm_bf16_pair_kernel<BN, ONCE, FORM>, dim3(2 * pairs), dim3(PAIR_THREADS<FORM>),
                                    PL::total(stages, staged), dim3(2, 1, 1), tmW, tmA, part, M, N, num_kb, plan.upc,
                                    (size_t)M * N, m_tiles, n_pairs, units, stages, form, L.d_status);
   L.count();

@@ -56,55 +56,73 @@ struct SmemLayout {
   static constexpr uint32_t total(int stages) { return (uint32_t)stages * STAGE_BYTES + 1024; }  // + slack to align the base to 1024
 };
 
-// Epilogue of one tile by 128 threads: the accumulator, TMEM lanes = 128 weight rows from n0 (tile number
-// tile_y), columns = BN activation rows from m0, goes to the fp32 slab (coalesced: lane = output column) or,
-// with act_out, through the SwiGLU combination.  `ex`: at least min(BN, 64) * 528 bytes of shared memory that
-// nothing else uses meanwhile.  tl = 0..127 identifies the thread: it works on TMEM lane tl, so its warp must be
-// the one allowed to touch lanes 32 * (tl / 32) .. + 31 (warp index % 4 == tl / 32).  NAMED_BAR == 0: the 128
-// threads are the whole CTA (__syncthreads); otherwise they meet on that named barrier.
-template <int NAMED_BAR>
-__device__ __forceinline__ void epilogue_sync() {
-  if constexpr (NAMED_BAR == 0)
-    __syncthreads();
-  else
-    asm volatile("bar.sync %0, 128;" ::"n"(NAMED_BAR) : "memory");
+// Epilogue of W columns of a tile by a group of 128 threads: the accumulator, TMEM lanes = 128 weight rows from n0 (tile
+// number tile_y), columns = W activation rows from m0, goes to the fp32 slab (coalesced: lane = output column), through
+// the SwiGLU combination (act_out) or into estimate records (m_ffn < 0).  `ex`: PlainStage<W>::BYTES of shared memory that
+// nothing else uses meanwhile.  tl = 0..127 identifies the thread: it works on TMEM lane tl, so its warp must be the one
+// allowed to touch lanes 32 * (tl / 32) .. + 31 (warp index % 4 == tl / 32).  The group meets on named barrier `bar` (1 or 2).
+// Two groups share a tile, half of its columns each: one group of four warps spends most of the epilogue waiting for
+// tensor memory and for its stores to issue.
+template <int W>
+struct PlainStage {
+  static constexpr int CH = W < 32 ? W : 32;   // activation rows staged at a time
+  static constexpr int EXS = 132;              // floats per staged row: 16-byte aligned, rows 4 banks apart
+  static constexpr uint32_t BYTES = CH * EXS * 4;
+};
+// CH columns of tensor memory on their way into registers; landed: they are there and go to staging.
+template <int CH>
+__device__ __forceinline__ void tmem_fetch(uint32_t taddr, uint32_t (&r)[CH / 16][16]) {
+#pragma unroll
+  for (int i = 0; i < CH / 16; ++i) tmem_ld16(taddr + 16u * i, r[i]);
 }
-template <int BN, int NAMED_BAR = 0>
-__device__ __forceinline__ void gemm_epilogue(uint32_t tmem_d, float* ex, int tl, int m0, int n0, int tile_y, int M,
+template <int CH>
+__device__ __forceinline__ void tmem_last(uint32_t (&r)[CH / 16][16]) {
+#pragma unroll
+  for (int i = 0; i < CH / 16; ++i) tmem_ld16_wait(r[i]);
+}
+template <int CH, int EXS>
+__device__ __forceinline__ void tmem_landed(uint32_t (&r)[CH / 16][16], float* ex, int tl) {
+  tmem_last<CH>(r);
+#pragma unroll
+  for (int i = 0; i < CH / 16; ++i)
+#pragma unroll
+    for (int j = 0; j < 16; ++j) ex[(16 * i + j) * EXS + tl] = __uint_as_float(r[i][j]);
+}
+enum PlainKind { SLABS, SWIGLU, ESTIMATE };
+template <int W, PlainKind KIND>
+__device__ __forceinline__ void gemm_epilogue(uint32_t tmem_d, float* ex, int tl, int bar, int m0, int n0, int tile_y, int M,
                                               int N, float* __restrict__ slab, __nv_bfloat16* __restrict__ act_out,
                                               int m_ffn) {
-  const int warp = tl >> 5, lane = tl & 31;
-  if (m_ffn < 0) {
+  const int lane = tl & 31;
+  const uint32_t tmem_w = tmem_d + ((uint32_t)(tl >> 5) << 21);
+  constexpr int CH = PlainStage<W>::CH, EXS = PlainStage<W>::EXS;
+  auto sync = [&] { group_sync(bar); };
+  if (m0 >= M) return;  // uniform across the group
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if constexpr (KIND == ESTIMATE) {
     // Estimate epilogue of the LM head (no split-K, act_out == nullptr, m_ffn = -1 - mask id): instead of 128
     // logits per row the CTA writes one record per activation row, {max, sum exp(v - max), argmax, -} over its
     // 128 vocabulary columns (Eq. 4; the mask id and columns past N are skipped); a merge over the tiles
-    // follows.  Staged like the SwiGLU epilogue; two threads share a row, 64 columns each.
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    constexpr int EXS = 132;
-    constexpr int CH = BN < 64 ? BN : 64;
+    // follows.  Staged like the SwiGLU epilogue; four threads share a row, 32 columns each (the same sums in every tile
+    // width).
     const int mask_id = -1 - m_ffn, n_tiles = (N + TILE_W - 1) / TILE_W;
     float4* rec = reinterpret_cast<float4*>(slab);
-    const int rr = tl >> 1, half = tl & 1;
+    const int rr = tl >> 2, part = tl & 3;
+    uint32_t r[CH / 16][16];
+    tmem_fetch<CH>(tmem_w, r);
 #pragma unroll 1
-    for (int c0 = 0; c0 < BN; c0 += CH) {
-      if (m0 + c0 >= M) break;  // uniform across the CTA
-#pragma unroll 1
-      for (int c = 0; c < CH; c += 16) {
-        uint32_t r[16];
-        tmem_ld16(tmem_d + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c0 + c), r);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int j = 0; j < 16; ++j) ex[(c + j) * EXS + tl] = __uint_as_float(r[j]);
-      }
-      epilogue_sync<NAMED_BAR>();
+    for (int c0 = 0; c0 < W && m0 + c0 < M; c0 += CH) {
+      tmem_landed<CH, EXS>(r, ex, tl);
+      sync();
+      tmem_fetch<CH>(tmem_w + (uint32_t)min(c0 + CH, W - CH), r);   // the next rows (again the last ones in the last trip)
       MaxSum t{-INFINITY, 0.f, 0x7fffffff};
       if (rr < CH) {
-        // two passes over the thread's 64 columns: maximum and its first index, then the exponentials as four
+        // two passes over the thread's 32 columns: maximum and its first index, then the exponentials as four
         // independent sums (one serial chain of dependent exponentials would dominate the epilogue)
-        const float* row = ex + rr * EXS + half * 64;
-        const int nb = n0 + half * 64;
+        const float* row = ex + rr * EXS + part * 32;
+        const int nb = n0 + part * 32;
 #pragma unroll 4
-        for (int j = 0; j < 64; j += 4) {
+        for (int j = 0; j < 32; j += 4) {
           const float4 v = *reinterpret_cast<const float4*>(row + j);
           const float e[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -119,7 +137,7 @@ __device__ __forceinline__ void gemm_epilogue(uint32_t tmem_d, float* ex, int tl
         if (t.m > -INFINITY) {
           float s4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
-          for (int j = 0; j < 64; j += 4) {
+          for (int j = 0; j < 32; j += 4) {
             const float4 v = *reinterpret_cast<const float4*>(row + j);
             const float e[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -131,38 +149,35 @@ __device__ __forceinline__ void gemm_epilogue(uint32_t tmem_d, float* ex, int tl
           t.s = (s4[0] + s4[1]) + (s4[2] + s4[3]);
         }
       }
-      MaxSum o;
-      o.m = __shfl_xor_sync(0xffffffffu, t.m, 1);
-      o.s = __shfl_xor_sync(0xffffffffu, t.s, 1);
-      o.a = __shfl_xor_sync(0xffffffffu, t.a, 1);
-      t = merge(t, o);
+#pragma unroll
+      for (int x = 1; x <= 2; x <<= 1) {
+        MaxSum o;
+        o.m = __shfl_xor_sync(0xffffffffu, t.m, x);
+        o.s = __shfl_xor_sync(0xffffffffu, t.s, x);
+        o.a = __shfl_xor_sync(0xffffffffu, t.a, x);
+        t = merge(t, o);
+      }
       const int m = m0 + c0 + rr;
-      if (rr < CH && half == 0 && m < M)
+      if (rr < CH && part == 0 && m < M)
         rec[(size_t)m * n_tiles + tile_y] = make_float4(t.m, t.s, __int_as_float(t.a), 0.f);
-      epilogue_sync<NAMED_BAR>();
+      sync();
     }
-  } else if (act_out) {
+    tmem_last<CH>(r);
+  } else if constexpr (KIND == SWIGLU) {
     // SwiGLU epilogue (no split-K): the tile's 128 weight rows are 64 gate rows followed by the 64 up rows
     // of the same FFN columns, so TMEM lanes 0..63 hold gate and 64..127 hold up.  The accumulator goes
-    // through shared memory (every MMA has completed) 64 activation rows at a time, transposed to
-    // [row][weight row], and comes back as silu(gate) * up in bf16, 8 bytes per thread.
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    constexpr int EXS = 132;   // floats per staged row: 16-byte aligned, rows 4 banks apart
-    constexpr int CH = BN < 64 ? BN : 64;
+    // through shared memory (every MMA has completed) CH activation rows at a time, transposed to
+    // [row][weight row], the next ones on their way out of tensor memory meanwhile, and comes back as silu(gate) * up in
+    // bf16, 8 bytes per thread.
     const int q = tl & 15, rsub = tl >> 4;  // 4 FFN columns, 8 rows per pass
     const int col = tile_y * 64 + 4 * q;
+    uint32_t r[CH / 16][16];
+    tmem_fetch<CH>(tmem_w, r);
 #pragma unroll 1
-    for (int c0 = 0; c0 < BN; c0 += CH) {
-      if (m0 + c0 >= M) break;  // uniform across the CTA
-#pragma unroll 1
-      for (int c = 0; c < CH; c += 16) {
-        uint32_t r[16];
-        tmem_ld16(tmem_d + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c0 + c), r);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int j = 0; j < 16; ++j) ex[(c + j) * EXS + tl] = __uint_as_float(r[j]);
-      }
-      epilogue_sync<NAMED_BAR>();
+    for (int c0 = 0; c0 < W && m0 + c0 < M; c0 += CH) {
+      tmem_landed<CH, EXS>(r, ex, tl);
+      sync();
+      tmem_fetch<CH>(tmem_w + (uint32_t)min(c0 + CH, W - CH), r);   // the next rows (again the last ones in the last trip)
 #pragma unroll 2
       for (int rr = rsub; rr < CH; rr += 8) {
         const int m = m0 + c0 + rr;
@@ -181,19 +196,19 @@ __device__ __forceinline__ void gemm_epilogue(uint32_t tmem_d, float* ex, int tl
           *reinterpret_cast<uint2*>(act_out + (size_t)m * m_ffn + col) = pk;
         }
       }
-      epilogue_sync<NAMED_BAR>();
+      sync();
     }
+    tmem_last<CH>(r);
   } else {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const int n = n0 + warp * 32 + lane;
+    const int n = n0 + (tl >> 5) * 32 + lane;
     float* out = slab + n;
     // (16 columns per trip and little code: an epilogue runs once per launch from a cold instruction cache, and 64 columns
     // unrolled took 0.5 to 1.5 us longer per projection)
 #pragma unroll 1
-    for (int c0 = 0; c0 < BN; c0 += 16) {
-      if (m0 + c0 >= M) break;  // uniform across the CTA
+    for (int c0 = 0; c0 < W; c0 += 16) {
+      if (m0 + c0 >= M) break;  // uniform across the group
       uint32_t r[16];
-      tmem_ld16(tmem_d + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, r);
+      tmem_ld16(tmem_w + (uint32_t)c0, r);
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
       if (n < N) {
         float* row = out + (size_t)(m0 + c0) * N;
@@ -210,8 +225,11 @@ __device__ __forceinline__ void gemm_epilogue(uint32_t tmem_d, float* ex, int tl
   }
 }
 
+// One-tile kernel: warp 0 requests operands, warp 1 issues the MMAs, and all eight drain the accumulator, two per quarter
+// of the TMEM lanes with half of the activation rows each.
+constexpr int ONE_THREADS = 256;
 template <int BN, bool ONCE>
-__global__ void __launch_bounds__(128) gemm_bf16_tcgen05_kernel(const __grid_constant__ CUtensorMap tmW,
+__global__ void __launch_bounds__(ONE_THREADS) gemm_bf16_tcgen05_kernel(const __grid_constant__ CUtensorMap tmW,
                                                                 const __grid_constant__ CUtensorMap tmA,
                                                                 float* __restrict__ part, int M, int N, int num_kb,
                                                                 int kb_per_split, size_t split_stride, int STAGES,
@@ -346,7 +364,7 @@ __global__ void __launch_bounds__(128) gemm_bf16_tcgen05_kernel(const __grid_con
   }
   __syncwarp();
 
-  // ---------------- epilogue: TMEM -> registers -> global (all four warps) ----------------
+  // ---------------- epilogue: TMEM -> registers -> global (all eight warps) ----------------
   const bool have = mbar_wait(smem_u32(&accum_bar), 0u, abortp);
   if (!have && threadIdx.x == 0 && status) atomicCAS(status, ST_OK, ST_TIMEOUT_EPI);
   if (threadIdx.x == 0) timeline_mark(3);              // accumulator complete
@@ -354,9 +372,17 @@ __global__ void __launch_bounds__(128) gemm_bf16_tcgen05_kernel(const __grid_con
   bool warp_ok = __all_sync(0xffffffffu, have);
   if (act_out || m_ffn < 0) warp_ok = __syncthreads_and(warp_ok);  // these epilogues exchange data between warps
   if (warp_ok) {
-    float* ex = reinterpret_cast<float*>(smem_raw + (tiles - smem_u32(smem_raw)));  // the drained ring
-    gemm_epilogue<BN>(tmem_d, ex, (int)threadIdx.x, m0, n0, nt, M, N, part + (size_t)blockIdx.z * split_stride, act_out,
-                      m_ffn);
+    constexpr int W = BN / 2;
+    const int half = (int)threadIdx.x >> 7;
+    float* ex = reinterpret_cast<float*>(smem_raw + (tiles - smem_u32(smem_raw)) + half * PlainStage<W>::BYTES);  // the drained ring
+    const uint32_t tmem_h = tmem_d + (uint32_t)(half * W);
+    const int tl = (int)threadIdx.x & 127, bar = 1 + half, m0h = m0 + half * W;
+    if (m_ffn < 0)
+      gemm_epilogue<W, ESTIMATE>(tmem_h, ex, tl, bar, m0h, n0, nt, M, N, part, act_out, m_ffn);
+    else if (act_out)
+      gemm_epilogue<W, SWIGLU>(tmem_h, ex, tl, bar, m0h, n0, nt, M, N, part, act_out, m_ffn);
+    else
+      gemm_epilogue<W, SLABS>(tmem_h, ex, tl, bar, m0h, n0, nt, M, N, part + (size_t)blockIdx.z * split_stride, act_out, m_ffn);
     if (threadIdx.x == 0) timeline_mark(4);            // this thread's part of the epilogue written
   } else {
     drain_delay();  // gave up: let copies in flight land before shared memory is released
@@ -368,19 +394,23 @@ __global__ void __launch_bounds__(128) gemm_bf16_tcgen05_kernel(const __grid_con
   }
 }
 
-// The pair kernel's plain forms (fp32 slabs, SwiGLU, estimate records).
+// The pair kernel's plain forms.  Slabs leave at the rate of the stores with one group of epilogue warps already (2.8 us for
+// 256 rows either way); the staged ones take two.
+template <PlainKind KIND>
 struct PlainForm {
   __nv_bfloat16* act_out;
   int m_ffn;
-  static constexpr uint32_t EX_BYTES = 64 * 132 * 4;
-  template <int BN>
+  static constexpr int GROUPS = KIND == SLABS ? 1 : 2;
+  template <int W>
+  static constexpr uint32_t ex_bytes() { return KIND == SLABS ? 0 : PlainStage<W>::BYTES; }
+  template <int W>
   struct Shared {};
-  template <int BN>
-  __device__ __forceinline__ void ahead(Shared<BN>&, int, int, int) const {}
-  template <int BN>
-  __device__ __forceinline__ void drain(Shared<BN>&, uint32_t tmem_d, float* ex, int tl, int m0, int n0, int tile_y, int M,
-                                        int N, float* slab) const {
-    gemm_epilogue<BN, 1>(tmem_d, ex, tl, m0, n0, tile_y, M, N, slab, act_out, m_ffn);
+  template <int W>
+  __device__ __forceinline__ void ahead(Shared<W>&, int, int, int) const {}
+  template <int W>
+  __device__ __forceinline__ void drain(Shared<W>&, uint32_t tmem_d, float* ex, int tl, int bar, int m0, int n0, int tile_y,
+                                        int M, int N, float* slab) const {
+    gemm_epilogue<W, KIND>(tmem_d, ex, tl, bar, m0, n0, tile_y, M, N, slab, act_out, m_ffn);
   }
 };
 
@@ -466,7 +496,7 @@ cudaError_t launch_one(const Launch& L, const CUtensorMap& tmW, const CUtensorMa
   if (e0 != cudaSuccess) return e0;
   const int stages = plan.stages < 2 ? 2 : plan.stages > max_stages(BN) ? max_stages(BN) : plan.stages;
   dim3 grid((M + BN - 1) / BN, (N + TILE_W - 1) / TILE_W, plan.S_max);
-  cudaError_t e = launch_k(L, gemm_bf16_tcgen05_kernel<BN, ONCE>, grid, dim3(128), SL::total(stages), tmW, tmA, part, M, N,
+  cudaError_t e = launch_k(L, gemm_bf16_tcgen05_kernel<BN, ONCE>, grid, dim3(ONE_THREADS), SL::total(stages), tmW, tmA, part, M, N,
                            num_kb, plan.upc, (size_t)M * N, stages, (__nv_bfloat16*)act_out, m_ffn, L.d_status);
   L.count();
   return e != cudaSuccess ? e : cudaGetLastError();
@@ -475,8 +505,13 @@ cudaError_t launch_one(const Launch& L, const CUtensorMap& tmW, const CUtensorMa
 template <int BN, bool ONCE>
 cudaError_t launch_pair(const Launch& L, const CUtensorMap& tmW, const CUtensorMap& tmA, float* part, int M, int N,
                         int num_kb, const GemmPlan& plan, void* act_out, int m_ffn) {
-  return launch_pair_form<BN, ONCE>(L, tmW, tmA, part, M, N, num_kb, plan, PlainForm{(__nv_bfloat16*)act_out, m_ffn},
-                                    act_out != nullptr || m_ffn < 0);
+  auto go = [&](auto form, bool staged) {
+    return launch_pair_form<BN, ONCE>(L, tmW, tmA, part, M, N, num_kb, plan, form, staged);
+  };
+  __nv_bfloat16* const act = (__nv_bfloat16*)act_out;
+  return m_ffn < 0 ? go(PlainForm<ESTIMATE>{act, m_ffn}, true)
+         : act     ? go(PlainForm<SWIGLU>{act, m_ffn}, true)
+                   : go(PlainForm<SLABS>{act, m_ffn}, false);
 }
 
 }  // namespace
