@@ -146,6 +146,28 @@ struct Workspace {
   size_t part_floats, attn_floats;
 };
 
+// Sessions whose Q, K and V of ALL response rows come from one product, in adaptive steps too: it streams the weights hardly
+// slower than the products of V (all rows) and of Q / K (the selected ones) one after the other, selection needs no launch and
+// no gather in front of it, and in a refresh V-verify and RoPE launches go.  Up to the arithmetic that takes as long as
+// streaming its weights does in the largest model (16 us): 256 rows of the LLaDA-8B shape, 780 of Dream-7B, all of a small
+// one.  B200, us, separate -> one: LLaDA-8B partial / refresh / full step, 256 rows 4187 / 5580 / 11205 -> 4194 / 5296 /
+// 10652, 128 rows partial 3699 -> 3654, 32 rows 3848 -> 3741; 300 rows (eight layers) 1111 / 1474 -> 1253 / 1528, beyond the
+// line; Dream-7B partial 256 rows 4168 -> 4053, (eight layers) 400 rows 1251 -> 1194, 512 rows 1342 -> 1293; 320-wide model
+// with 500 rows, full step 120 -> 93.  (1024 rows and more belong to the streaming row kernels.)
+constexpr double QKV_WORK = 256.0 * 12288 * 4096;
+bool qkv_in_one(const dllm_config& c, int B, int R) {
+  const double rows = (double)B * R, width = (double)(c.n_heads + 2 * c.n_kv_heads) * c.head_dim;
+  return c.dtype == DLLM_BF16 && rows < 1024 && rows * width * c.d_model <= QKV_WORK;
+}
+// Whether a full step of such a session takes Q, K and V of all `rows` carried rows from one product with the response rows'
+// splits: where its own plan has as many, or where their slabs stay small beside the launches they replace (V, V-verify,
+// the prompt's V and its scatter, selection, gather: 25 us and more against 8 us for 40 MB written and read).
+constexpr size_t QKV_SLAB_BYTES = 40 << 20;
+bool qkv_all_rows(const dllm_config& c, size_t rows, int split) {
+  const size_t width = (size_t)(c.n_heads + 2 * c.n_kv_heads) * c.head_dim;
+  return plan_gemm_bf16((int)rows, (int)width, c.d_model).S_max == split || split * rows * width * 4 <= QKV_SLAB_BYTES;
+}
+
 Workspace make_workspace(const dllm_config& c, int B, int P, int R, int flags) {
   Workspace w;
   const size_t es = esize(c), d = c.d_model, dq = (size_t)c.n_heads * c.head_dim,
@@ -193,6 +215,11 @@ Workspace make_workspace(const dllm_config& c, int B, int P, int R, int flags) {
       mn = std::max(mn, (size_t)p.S_max * M * N);
     };
     slabs(BR, dkv, d);
+    if (qkv_in_one(c, B, R)) {  // [Q | K | V] of all response rows, or of all carried rows with as many splits
+      const int split = plan_gemm_bf16((int)BR, (int)(dq + 2 * dkv), (int)d).S_max;
+      slabs(BR, dq + 2 * dkv, d);
+      mn = std::max(mn, (size_t)split * rows * (qkv_all_rows(c, rows, split) ? dq + 2 * dkv : dkv));
+    }
     slabs(BR, V, d);
     slabs((size_t)B * P, dkv, d);
     for (size_t Ma = 1; Ma <= rows; ++Ma) {
@@ -498,10 +525,11 @@ struct ProfScope {
 };
 
 // One GEMM of the step: out = A[M,K] * W[N,K]^T as split-K partial slabs.  weights_again: another product of the step reads
-// the same weights soon.  rows: what an unsplit product of many rows does with its result itself (*fused).
+// the same weights soon.  rows: what an unsplit product of many rows does with its result itself (*fused).  split: exactly so
+// many splits of the k range (0: the plan's choice).
 dllm_status run_gemm(dllm_session* s, const Launch& L, int cls, const void* A, const void* W, int M, int N, int K,
                      Partials* out, void* swiglu_out = nullptr, bool* fused = nullptr, int estimate_mask_id = -1,
-                     bool weights_again = false, const RowOut* rows = nullptr, bool unsplit = false) {
+                     bool weights_again = false, const RowOut* rows = nullptr, int split = 0) {
   float* part = s->wsp<float>(s->ws.part);
   if (fused) *fused = false;
   *out = Partials{part, (size_t)M * N, 1, N};
@@ -510,8 +538,8 @@ dllm_status run_gemm(dllm_session* s, const Launch& L, int cls, const void* A, c
   const bool tensor = !(s->m->cfg.dtype == DLLM_FP32 || s->simt_gemm);
   // the LM head is never split (its consumers read logits or records), nor is a gate / up projection of more rows
   // than stream the weights anyway: the SwiGLU epilogue saves a launch and a pass over the slabs
-  const bool whole = cls == DLLM_PROF_GEMM_HEAD || (swiglu_out && M > 128 && gu_interleaved(s->m->cfg)) || unsplit;
-  GemmPlan plan = tensor ? plan_gemm_bf16(M, N, K, whole ? 1 : 0) : GemmPlan{};
+  const bool whole = cls == DLLM_PROF_GEMM_HEAD || (swiglu_out && M > 128 && gu_interleaved(s->m->cfg));
+  GemmPlan plan = tensor ? plan_gemm_bf16(M, N, K, whole ? 1 : -split) : GemmPlan{};
   if (weights_again) plan.w_stream = false;
   const bool to_rows = tensor && rows && plan.pair && plan.S_max == 1;
   // an unsplit gate / up projection of an interleaved weight finishes SwiGLU in its own epilogue, and an unsplit
@@ -586,14 +614,22 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
   // While profiling, V and Q / K stay launches of their own, so that each class can be read.
   // An adaptive step that happens to recompute every row, and one that is profiled, equal a response refresh bit for bit:
   // their products have the same plans, and V of the prompt rows is not split where that product has it.
+  // In a session of not too many response rows (in_one) their V has the splits of the one product for Q, K and V (v_split) wherever it
+  // is computed.  Every row of a step comes from that product where it has these splits over all carried rows (all_in_one).
   const bool tensor = dt == DLLM_BF16 && !s->simt_gemm;
   const bool heads = tensor && (hd == 64 || hd == 128), rotate = heads && !s->profiling;
   const bool all_rows = rr || std::all_of(ksels.begin(), ksels.end(), [&](int k) { return k == s->R; });
+  const bool in_one = tensor && qkv_in_one(c, s->B, s->R);
+  const int v_split = in_one ? plan_gemm_bf16(BR, dq + 2 * dkv, d).S_max : 0;
+  const bool all_in_one = in_one && all_rows && (!rp || qkv_all_rows(c, c1, v_split));
   const GemmPlan qk_plan = heads ? plan_gemm_bf16(c1, dq + dkv, d) : GemmPlan{};
-  const bool qk_unsplit = all_rows && heads && qk_plan.wide && qk_plan.S_max == 1;
-  const bool qk_whole = qk_unsplit && qk_plan.pair && rr && rotate;
-  const bool v_whole = qk_whole && plan_gemm_bf16(BR, dkv, d).S_max == 1;   // V of the response rows too
+  const bool qk_unsplit = !all_in_one && all_rows && heads && qk_plan.wide && qk_plan.S_max == 1;
+  const bool qk_whole = all_in_one ? rr && !s->profiling : qk_unsplit && qk_plan.pair && rr && rotate;
+  // V of the response rows too
+  const bool v_whole = qk_whole && (all_in_one || (in_one ? v_split : plan_gemm_bf16(BR, dkv, d).S_max) == 1);
   const bool qkv_whole = v_whole || (qk_whole && rp);
+  // splits of Q / K and of the prompt's V in such a step (0: their own plans')
+  const int all_split = all_in_one ? v_split : 0, prompt_v_split = all_in_one ? v_split : qk_unsplit ? 1 : 0;
   RowOut qkv;
   qkv.qkv = 1;
   qkv.q = reinterpret_cast<__nv_bfloat16*>(s->wsp<uint8_t>(s->ws.qbuf));
@@ -634,12 +670,45 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
     // projections and V-verify writes the (identity) lists, so no selection or gather launch is needed.
     const bool identity = rr && !rp && Ma > 0;
     bool fused = false;
+    const bool verify_v = adaptive && s->sel_strategy == DLLM_SELECT_V_VERIFY;
+    // Adaptive step of such a session: one product of all response rows, V-verify, and a launch that selects among the rows and
+    // rotates the selected ones (not where the product of Q / K would place its own rows).  Profiled, the same sums in
+    // launches of their own.
+    bool one_product = in_one && !rp && verify_v;
+    if (one_product && heads) {
+      const GemmPlan p = plan_gemm_bf16(Ma, dq + dkv, d);
+      one_product = !(p.wide && p.S_max == 1);
+    }
+    const int qk_split = one_product ? v_split : all_split;
+    const bool selected_rows = one_product && !s->profiling;   // Q, K and V are there before the selection
+    // Mixed step: one product for V of the response rows (as it comes, for V-verify) and of the prompt rows behind them, which
+    // an unsplit product of many rows places itself; split, only up to a thousand rows (a long prompt's slabs would cost more
+    // than the launch)
+    const bool v_together = in_one && rp && !rr && verify_v && (!all_rows || prompt_v_split == v_split) &&
+                            (c1 <= 1024 || (v_split == 1 && plan_gemm_bf16(c1, dkv, d, -1).wide));
+    const bool v_one = v_together && !s->profiling;
     if (v_whole) {
       // projected with Q and K below
-    } else if (rr || (adaptive && s->sel_strategy == DLLM_SELECT_V_VERIFY)) {
+    } else if (selected_rows) {
+      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_QK, u, Wq, BR, dq + 2 * dkv, d, &part, nullptr, nullptr, -1, false, nullptr,
+                         v_split)) != DLLM_OK)
+        return st;
+      Partials v_part = part;
+      v_part.p += dq + dkv;
+      launch_vverify(L, dt, v_part, s->cache(l, DLLM_CACHE_V), sim, g, dkv, s->sel_metric, !s->v_selected_only);
+      launch_select_rope(L, dt, part, sim, forced, mode, ksel, sel, act, inv, s->wsp<float>(s->ws.rope),
+                         s->wsp<uint8_t>(s->ws.qbuf), s->cache(l, DLLM_CACHE_K),
+                         s->v_selected_only ? s->cache(l, DLLM_CACHE_V) : nullptr, g, H, Hkv, hd);
+    } else if (rr || verify_v) {
       // V for ALL response rows (the 2 r d^2 term of Sec. A.7), V-verify, V overwrite
       // (a prompt refresh reads W_v once more, for the prompt rows)
-      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u, Wv, BR, dkv, d, &part, nullptr, nullptr, -1, rp)) != DLLM_OK) return st;
+      RowOut o = rows_into({s->cache(l, DLLM_CACHE_V), nullptr, 0}, dkv, nullptr, 0);
+      o.slab = s->wsp<float>(s->ws.part);
+      o.slab_rows = BR;
+      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u, Wv, v_one ? c1 : BR, dkv, d, &part, nullptr, &fused, -1, rp && !v_one,
+                         v_one ? &o : nullptr, v_split)) != DLLM_OK)
+        return st;
+      if (fused) part = Partials{o.slab, (size_t)BR * dkv, 1, dkv};
       const IdentityLists id{sel, act, inv};
       {  // the projection's fp32 result in, the cached row in, the row out
         ProfScope ps(s, DLLM_PROF_VVERIFY, (double)BR * dkv * (4.0 + 2.0 * es), 6.0 * BR * dkv, stream);
@@ -656,12 +725,14 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
                      s->sel_metric);
     }  // random selection: the scores were set by dllm_set_scores
     // V of the active rows is still missing when the verify pass did not write it
-    const bool v_for_active = adaptive && (s->sel_strategy != DLLM_SELECT_V_VERIFY || s->v_selected_only);
+    const bool v_for_active = adaptive && !selected_rows && (!verify_v || s->v_selected_only);
     const OutRows v_rows{s->cache(l, DLLM_CACHE_V), nullptr, 0};
     if (rp && !qkv_whole) {
       const RowOut o = rows_into(v_rows, dkv, nullptr, BR);
-      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u + (size_t)BR * d * es, Wv, BP, dkv, d, &part, nullptr, &fused, -1, false,
-                         &o, qk_unsplit)) != DLLM_OK)
+      if (v_one)
+        part.p += (size_t)BR * dkv;   // (behind the response rows' in every slab, if the product has not placed them)
+      else if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u + (size_t)BR * d * es, Wv, BP, dkv, d, &part, nullptr, &fused, -1, false,
+                              &o, v_together ? v_split : prompt_v_split)) != DLLM_OK)
         return st;
       if (!fused) {
         ProfScope ps(s, DLLM_PROF_SCATTER, (double)BP * dkv * (4.0 + es), 0.0, stream);
@@ -670,7 +741,9 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
     }
     if (Ma > 0) {
       const uint8_t* ua = s->wsp<uint8_t>(s->ws.ua);
-      if (qk_whole || identity) {
+      if (selected_rows) {
+        // selected, rotated and placed above
+      } else if (qk_whole || identity) {
         ua = u;
       } else if (s->R <= 1024 && (long)Ma * s->R <= 64L * 1024) {
         // few active rows: every CTA of the gather repeats the selection rather than wait for a launch
@@ -684,7 +757,7 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
       }
       if (v_for_active) {
         const RowOut o = rows_into(v_rows, dkv, act, 0);
-        if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, ua, Wv, Ma, dkv, d, &part, nullptr, &fused, -1, false, &o)) != DLLM_OK)
+        if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, ua, Wv, Ma, dkv, d, &part, nullptr, &fused, -1, false, &o, qk_split)) != DLLM_OK)
           return st;
         if (!fused) {
           ProfScope ps(s, DLLM_PROF_SCATTER, (double)Ma * dkv * (4.0 + es), 0.0, stream);
@@ -692,20 +765,22 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
         }
       }
       // Q and K of the active rows in one GEMM over the stacked [W_q; W_k] (and W_v behind them)
-      bool rotated = false;
+      bool rotated = selected_rows;
       RowOut o = qkv;
       if (!qk_whole) o.act = act;
       o.q_by_slot = qk_whole && rp;
       o.k = reinterpret_cast<__nv_bfloat16*>(s->cache(l, DLLM_CACHE_K));
       o.v = reinterpret_cast<__nv_bfloat16*>(s->cache(l, DLLM_CACHE_V));
       o.v_from = v_whole ? 0 : BR;
-      if ((st = run_gemm(s, L, DLLM_PROF_GEMM_QK, ua, Wq, Ma, dq + (qkv_whole ? 2 : 1) * dkv, d, &part, nullptr, &rotated, -1,
-                         false, rotate ? &o : nullptr, qk_whole)) != DLLM_OK)
+      if (!selected_rows &&
+          (st = run_gemm(s, L, DLLM_PROF_GEMM_QK, ua, Wq, Ma, dq + (qkv_whole ? 2 : 1) * dkv, d, &part, nullptr, &rotated, -1,
+                         false, rotate ? &o : nullptr, qk_whole && !all_in_one ? 1 : qk_split)) != DLLM_OK)
         return st;
       if (!rotated) {
         ProfScope ps(s, DLLM_PROF_ROPE, (double)Ma * (dq + dkv) * (4.0 + es), 6.0 * Ma * (dq + dkv), stream);
         launch_qk_rope(L, dt, part, act, s->wsp<float>(s->ws.rope), s->wsp<uint8_t>(s->ws.qbuf),
-                       s->cache(l, DLLM_CACHE_K), g, Ma, H, Hkv, hd);
+                       s->cache(l, DLLM_CACHE_K), g, Ma, H, Hkv, hd, v_whole ? s->cache(l, DLLM_CACHE_V) : nullptr,
+                       v_whole && rp);
       }
       // algorithmic traffic: K and V of every sequence once, Q in, O out (the merge of split key ranges runs
       // inside the same pair).  Class by the kernel the shape takes: 64-row mma.sync or 128-row tcgen05.
@@ -718,8 +793,9 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
                                        // the launch before attention is RoPE + K scatter or the Q / K projection itself:
                                        // every V row of the layer and, unless the prompt is refreshed, the prompt's K
                                        // rows were written at least two launches earlier (with V in the product of Q
-                                       // and K only the prompt's V, when it is not refreshed)
-                                       rp ? 0 : s->P, !qkv_whole ? s->n : rp ? 0 : s->P);
+                                       // and K, or written with the selected rows' Q and K, only the prompt's V, when it is
+                                       // not refreshed)
+                                       rp ? 0 : s->P, !qkv_whole && !(selected_rows && s->v_selected_only) ? s->n : rp ? 0 : s->P);
       s->prof_end(stream);
       if (e != cudaSuccess) return fail(&s->err, DLLM_CUDA_ERROR, "attention: %s", cudaGetErrorString(e));
       const RowOut attn_out = rows_into(s->outs(l, DLLM_CACHE_ATTN), d, act, 0);
@@ -1311,6 +1387,8 @@ dllm_status dllm_get_selected(dllm_session* s, int layer, int32_t* h_idx, float*
   else if (h_idx && k_l > 0)
     CU_TRY(&s->err, cudaMemcpy2D(h_idx, (size_t)k_l * 4, s->d_ws + s->ws.sel + (size_t)layer * BR * 4,
                                  (size_t)s->R * 4, (size_t)k_l * 4, s->B, cudaMemcpyDeviceToHost));
+  if (h_idx && k_l > 0 && k_l < s->R)  // a step lists the rows in the order it works on them
+    for (int b = 0; b < s->B; ++b) std::sort(h_idx + (size_t)b * k_l, h_idx + (size_t)(b + 1) * k_l);
   if (h_sim)
     CU_TRY(&s->err, cudaMemcpy(h_sim, s->d_ws + s->ws.sim + (size_t)layer * BR * 4, BR * 4, cudaMemcpyDeviceToHost));
   return DLLM_OK;

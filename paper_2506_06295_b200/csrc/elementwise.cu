@@ -511,6 +511,13 @@ void launch_rmsnorm(const Launch& L, int dtype, const float* x, const float* gai
 }
 
 // ------------------------------------------------------------------ selection inside a kernel
+// Sortable score of row j: round(s * 2^20), offset into 1 .. 2^32 - 1 (scores beyond +-2047 saturate), NaN first; ties go
+// to the lower index.
+__device__ __forceinline__ unsigned long long select_key(float s, int j) {
+  const float qf = fminf(fmaxf(rintf(s * 1048576.0f), -2147483520.0f), 2147483520.0f);
+  const long long q = (s == s) ? (long long)qf + (1ll << 31) : 0ll;
+  return ((unsigned long long)q << 32) | (unsigned)j;
+}
 // Bottom-k selection of sequence b by the whole CTA (R <= 1024: R^2 comparisons out of shared memory, 13 R + 16
 // bytes at `keys`).  Fills slot[j] = position of response row j among the selected rows, or -1; with `write` the
 // CTA also writes the index list, the active list (np prompt rows first) and its inverse.
@@ -531,11 +538,7 @@ __device__ __forceinline__ int32_t* select_sequence(unsigned long long* keys, co
     for (int r = threadIdx.x; r < ksel; r += blockDim.x) slot[forced[(size_t)b * R + r]] = r;
   } else {
     for (int j = threadIdx.x; j < R; j += blockDim.x) {
-      const float s = __ldcg(sim + (size_t)b * R + j);
-      // key = round(s * 2^20), offset into 1 .. 2^32 - 1 (scores beyond +-2047 saturate); NaN sorts first
-      const float qf = fminf(fmaxf(rintf(s * 1048576.0f), -2147483520.0f), 2147483520.0f);
-      const long long q = (s == s) ? (long long)qf + (1ll << 31) : 0ll;
-      keys[j] = ((unsigned long long)q << 32) | (unsigned)j;
+      keys[j] = select_key(__ldcg(sim + (size_t)b * R + j), j);
     }
     __syncthreads();
     // rank of every key (two keys per shared-memory load); a row is selected iff its rank is below ksel
@@ -805,11 +808,7 @@ __global__ void select_kernel(const float* __restrict__ sim, const int32_t* __re
     return;
   }
   for (int j = threadIdx.x; j < R; j += blockDim.x) {
-    const float s = sim[(size_t)b * R + j];
-    // key = round(s * 2^20), offset into 1 .. 2^32 - 1 (scores beyond +-2047 saturate); NaN sorts first
-    const float qf = fminf(fmaxf(rintf(s * 1048576.0f), -2147483520.0f), 2147483520.0f);
-    const long long q = (s == s) ? (long long)qf + (1ll << 31) : 0ll;
-    keys[j] = ((unsigned long long)q << 32) | (unsigned)j;
+    keys[j] = select_key(sim[(size_t)b * R + j], j);
     flag[j] = 0;
   }
   __syncthreads();
@@ -874,20 +873,22 @@ void launch_gather_rows(const Launch& L, int dtype, const void* src, const int32
 // element i with i + hd/2, angle pos * theta^(-2i/hd) from a table built on the host.  HP = 2 (the heads of a
 // thread share the row's position and rotation values) halves the CTAs when there are several per SM slot, so
 // that all of them are resident, and have fetched those values, before the projection ahead of them ends.
+// Vc: V heads follow the K heads in `part`, whose rows are the carried rows in their order; they are rounded and stored.
 template <typename T, int HP>
 __global__ void qk_rope_kernel(Partials part, const int32_t* __restrict__ act, const float* __restrict__ rope_tab,
-                               T* __restrict__ qbuf, T* __restrict__ Kc, Geo g, int Ma, int H, int Hkv, int hd) {
+                               T* __restrict__ qbuf, T* __restrict__ Kc, T* __restrict__ Vc, int q_by_slot, Geo g, int Ma,
+                               int H, int Hkv, int hd) {
   // The launch before this one is the Q / K projection, which writes nothing but `part`: the row's position and
   // its cos / sin values are fetched before the dependency wait, while the projection still runs.
   const int half = hd >> 1, q4 = half >> 2;
-  const int heads = H + Hkv, hgroups = (heads + HP - 1) / HP;
+  const int heads = H + (Vc ? 2 : 1) * Hkv, hgroups = (heads + HP - 1) / HP;
   const int groups = hgroups * q4;
   const long w = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const bool live = w < (long)Ma * groups;
   const int r = live ? (int)(w / groups) : 0, gidx = live ? (int)(w - (long)r * groups) : 0;
   const int hg = gidx / q4, i0 = (gidx - hg * q4) * 4;
   int b, pos;
-  carried_to_pos(__ldcg(act + r), g, b, pos);
+  carried_to_pos(Vc ? r : __ldcg(act + r), g, b, pos);
   const int dq = H * hd, dkv = Hkv * hd;
   const float* tab = rope_tab + (size_t)pos * hd;  // [cos(half) | sin(half)]
   const float4 cs = *reinterpret_cast<const float4*>(tab + i0);
@@ -901,20 +902,23 @@ __global__ void qk_rope_kernel(Partials part, const int32_t* __restrict__ act, c
   for (int u = 0; u < HP; ++u) {
     const int head = hg * HP + u;
     if (head >= heads) break;
-    const int col0 = head < H ? head * hd : dq + (head - H) * hd;
-    sum_partials4(part, r, col0 + i0, lo[u]);
-    sum_partials4(part, r, col0 + i0 + half, hi[u]);
+    sum_partials4(part, r, head * hd + i0, lo[u]);   // the heads of Q, K (and V) lie side by side
+    sum_partials4(part, r, head * hd + i0 + half, hi[u]);
   }
 #pragma unroll
   for (int u = 0; u < HP; ++u) {
     const int head = hg * HP + u;
     if (head >= heads) break;
-    T* dst = head < H ? qbuf + (size_t)r * dq + head * hd : Kc + ((size_t)b * g.n + pos) * dkv + (head - H) * hd;
+    const size_t at = (size_t)b * g.n + pos;
+    T* dst = head < H         ? qbuf + (q_by_slot ? at : (size_t)r) * dq + head * hd
+             : head < H + Hkv ? Kc + at * dkv + (head - H) * hd
+                              : Vc + at * dkv + (head - H - Hkv) * hd;
     float o_lo[4], o_hi[4];
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
-      o_lo[t] = rope_lo(lo[u][t], hi[u][t], cc[t], ss[t]);
-      o_hi[t] = rope_hi(lo[u][t], hi[u][t], cc[t], ss[t]);
+      const bool rotate = head < H + Hkv;
+      o_lo[t] = rotate ? rope_lo(lo[u][t], hi[u][t], cc[t], ss[t]) : lo[u][t];
+      o_hi[t] = rotate ? rope_hi(lo[u][t], hi[u][t], cc[t], ss[t]) : hi[u][t];
     }
     store4<T>(dst + i0, o_lo);
     store4<T>(dst + i0 + half, o_hi);
@@ -922,11 +926,11 @@ __global__ void qk_rope_kernel(Partials part, const int32_t* __restrict__ act, c
 }
 
 void launch_qk_rope(const Launch& L, int dtype, Partials part, const int32_t* act, const float* rope_tab, void* qbuf,
-                    void* Kc_layer, Geo g, int Ma, int H, int Hkv, int hd) {
+                    void* Kc_layer, Geo g, int Ma, int H, int Hkv, int hd, void* Vc_layer, int q_by_slot) {
   if (Ma <= 0) return;
   const size_t stage = (size_t)(H + Hkv) * hd * 4;
   // streaming form: unsplit slabs, a head size whose pairs a group of lanes covers exactly (a power of two, 32..256)
-  if (g.B * g.R >= STREAM_MIN_ROWS && part.S == 1 && hd >= 32 && hd <= 256 && (hd & (hd - 1)) == 0 &&
+  if (!Vc_layer && g.B * g.R >= STREAM_MIN_ROWS && part.S == 1 && hd >= 32 && hd <= 256 && (hd & (hd - 1)) == 0 &&
       stream_stages(stage) >= STREAM_CONSUMERS + 1) {
     const int stages = stream_stages(stage);
     const size_t smem = (size_t)stages * stage + 128;
@@ -943,16 +947,104 @@ void launch_qk_rope(const Launch& L, int dtype, Partials part, const int32_t* ac
     L.count();
     return;
   }
-  const long total = (long)Ma * (H + Hkv) * (hd >> 3);
+  const int heads = H + (Vc_layer ? 2 : 1) * Hkv;
+  const long total = (long)Ma * heads * (hd >> 3);
   const long blocks1 = (total + 255) / 256;
   if (blocks1 > 2L * sm_count()) {   // two heads per thread: half the CTAs
-    const long total2 = (long)Ma * ((H + Hkv + 1) / 2) * (hd >> 3);
+    const long total2 = (long)Ma * ((heads + 1) / 2) * (hd >> 3);
     DLLM_DISPATCH(dtype, (launch_k(L, qk_rope_kernel<T, 2>, dim3((unsigned)((total2 + 255) / 256)), dim3(256), 0, part, act,
-                                   rope_tab, (T*)qbuf, (T*)Kc_layer, g, Ma, H, Hkv, hd)));
+                                   rope_tab, (T*)qbuf, (T*)Kc_layer, (T*)Vc_layer, q_by_slot, g, Ma, H, Hkv, hd)));
   } else {
     DLLM_DISPATCH(dtype, (launch_k(L, qk_rope_kernel<T, 1>, dim3((unsigned)blocks1), dim3(256), 0, part, act, rope_tab,
-                                   (T*)qbuf, (T*)Kc_layer, g, Ma, H, Hkv, hd)));
+                                   (T*)qbuf, (T*)Kc_layer, (T*)Vc_layer, q_by_slot, g, Ma, H, Hkv, hd)));
   }
+  L.count();
+}
+
+// ------------------------------------------------------------------ selection + RoPE of the selected rows
+// Grid (response rows, column chunks of SELECT_ROPE_IT * 256 groups of four rotation pairs).  The projections of ALL
+// response rows are in `part`.  A row is selected iff fewer than ksel rows of its sequence have a lower key, and that count is
+// its place in the active list (the order of the active rows is free: every row's result is independent of its neighbours);
+// the CTAs of the other rows are done then.  (Slabs requested ahead of the dependency wait, before the selection is known,
+// are four times as many and slow V-verify down, beside which they travel: the launch took 4.8 us.)
+constexpr int SELECT_ROPE_IT = 2;
+template <typename T>
+__global__ void __launch_bounds__(256) select_rope_kernel(Partials part, const float* __restrict__ sim,
+                                                          const int32_t* __restrict__ forced, int mode, int ksel,
+                                                          int32_t* __restrict__ sel, int32_t* __restrict__ act,
+                                                          int32_t* __restrict__ inv, const float* __restrict__ rope_tab,
+                                                          T* __restrict__ qbuf, T* __restrict__ Kc, T* __restrict__ Vc, Geo g,
+                                                          int H, int Hkv, int hd) {
+  __shared__ int slot_s;
+  const int c = blockIdx.x, R = g.R, b = c / R, j = c - b * R, pos = g.P + j;
+  const int half = hd >> 1, q4 = half >> 2, dq = H * hd, dkv = Hkv * hd;
+  const int items = (H + (Vc ? 2 : 1) * Hkv) * q4;
+  const int first = blockIdx.y * (SELECT_ROPE_IT * 256) + threadIdx.x;
+  const float* tab = rope_tab + (size_t)pos * hd;  // [cos(half) | sin(half)]
+  pdl_wait();
+  pdl_trigger();
+  int slot = -1;
+  if (mode == 2) {
+    if (threadIdx.x == 0) slot_s = -1;
+    __syncthreads();
+    for (int r = threadIdx.x; r < ksel; r += 256)
+      if (forced[(size_t)b * R + r] == j) slot_s = r;
+    __syncthreads();
+    slot = slot_s;
+  } else {
+    const unsigned long long own = select_key(__ldcg(sim + c), j);
+    int rank = 0;
+    for (int i0 = 0; i0 < R; i0 += 256) {
+      const int i = i0 + threadIdx.x;
+      rank += __syncthreads_count(i < R && select_key(__ldcg(sim + (size_t)b * R + min(i, R - 1)), i) < own);
+    }
+    if (rank < ksel) slot = rank;
+  }
+  if (blockIdx.y == 0 && threadIdx.x == 0) {
+    inv[c] = slot >= 0 ? b * ksel + slot : -1;
+    if (slot >= 0) {
+      sel[(size_t)b * R + slot] = j;
+      act[(size_t)b * ksel + slot] = c;
+    }
+  }
+  if (slot < 0) return;
+  T* qrow = qbuf + ((size_t)b * ksel + slot) * dq;
+  const size_t at = ((size_t)b * g.n + pos) * dkv;
+  float lo[SELECT_ROPE_IT][4], hi[SELECT_ROPE_IT][4];
+#pragma unroll
+  for (int u = 0; u < SELECT_ROPE_IT; ++u) {
+    const int idx = min(first + u * 256, items - 1), head = idx / q4, i0 = (idx - head * q4) * 4;
+    sum_partials4(part, c, head * hd + i0, lo[u]);
+    sum_partials4(part, c, head * hd + i0 + half, hi[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < SELECT_ROPE_IT; ++u) {
+    const int idx = first + u * 256;
+    if (idx >= items) break;
+    const int head = idx / q4, i0 = (idx - head * q4) * 4;
+    T* dst = head < H ? qrow + head * hd : head < H + Hkv ? Kc + at + (head - H) * hd : Vc + at + (head - H - Hkv) * hd;
+    if (head < H + Hkv) {
+      const float4 cs = *reinterpret_cast<const float4*>(tab + i0), sn = *reinterpret_cast<const float4*>(tab + half + i0);
+      const float cc[4] = {cs.x, cs.y, cs.z, cs.w}, ss[4] = {sn.x, sn.y, sn.z, sn.w};
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const float l = lo[u][t], h = hi[u][t];
+        lo[u][t] = rope_lo(l, h, cc[t], ss[t]);
+        hi[u][t] = rope_hi(l, h, cc[t], ss[t]);
+      }
+    }
+    store4<T>(dst + i0, lo[u]);
+    store4<T>(dst + i0 + half, hi[u]);
+  }
+}
+
+void launch_select_rope(const Launch& L, int dtype, Partials part, const float* sim, const int32_t* forced, int mode, int ksel,
+                        int32_t* sel, int32_t* act, int32_t* inv, const float* rope_tab, void* qbuf, void* Kc_layer,
+                        void* Vc_layer, Geo g, int H, int Hkv, int hd) {
+  const int items = (H + (Vc_layer ? 2 : 1) * Hkv) * (hd >> 3), per = SELECT_ROPE_IT * 256;
+  DLLM_DISPATCH(dtype, (launch_k(L, select_rope_kernel<T>, dim3(g.B * g.R, (items + per - 1) / per), dim3(256), 0, part, sim,
+                                 forced, mode, ksel, sel, act, inv, rope_tab, (T*)qbuf, (T*)Kc_layer, (T*)Vc_layer, g, H, Hkv,
+                                 hd)));
   L.count();
 }
 

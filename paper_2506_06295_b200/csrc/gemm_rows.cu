@@ -43,7 +43,8 @@ struct RowForm {
         const int at = b * o.g.n + pos;
         s.row[i] = make_int4(o.q_by_slot ? at : m0 + i, at, pos, 0);
       } else {
-        s.row[i] = reinterpret_cast<unsigned long long>(o.rows.row<__nv_bfloat16>(c, o.g));
+        s.row[i] = m0 + i < o.slab_rows ? reinterpret_cast<unsigned long long>(o.slab + (size_t)(m0 + i) * o.g.d)
+                                        : reinterpret_cast<unsigned long long>(o.rows.row<__nv_bfloat16>(c, o.g));
       }
     }
   }
@@ -122,6 +123,7 @@ struct RowForm {
       sync();                                                  // read: the staging is free for the next trip
       uint2 plo[U], phi[U];
       __nv_bfloat16 *dlo[U], *dhi[U];
+      unsigned long long raw_at[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         plo[u] = pack(rot ? lo4(a[u], b[u], cs[u], sn[u]) : a[u]);
@@ -130,6 +132,7 @@ struct RowForm {
           dlo[u] = blo + (unsigned long long)(unsigned)(qlo ? at[u].x : at[u].y) * slo;
           dhi[u] = bhi + (unsigned long long)(unsigned)(qhi ? at[u].x : at[u].y) * shi;
         } else {
+          raw_at[u] = at[u];
           dlo[u] = reinterpret_cast<__nv_bfloat16*>(at[u]) + nlo;
           dhi[u] = reinterpret_cast<__nv_bfloat16*>(at[u]) + nhi;
         }
@@ -138,6 +141,14 @@ struct RowForm {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int row = c0 + rsub + 8 * u;
+        if constexpr (!QKV) {
+          if (m0 + row < o.slab_rows) {   // (their columns 4 q .. and 64 further, as the others')
+            float* const raw = reinterpret_cast<float*>(raw_at[u]);
+            if (vlo && row < rows) *reinterpret_cast<float4*>(raw + nlo) = a[u];
+            if (vhi && row < rows) *reinterpret_cast<float4*>(raw + nhi) = b[u];
+            continue;
+          }
+        }
         if (vlo && row < rows && row >= lo_from) *reinterpret_cast<uint2*>(dlo[u]) = plo[u];
         if (vhi && row < rows && row >= hi_from) *reinterpret_cast<uint2*>(dhi[u]) = phi[u];
       }

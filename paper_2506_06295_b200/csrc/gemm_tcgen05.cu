@@ -556,14 +556,15 @@ Partials make_partials(const float* p, int M, int N, const GemmPlan& plan) {
 // slabs, 5.8 for SwiGLU, 16 for rotated and placed rows of a 256-row tile).  Measured with it, B200, us
 // (before -> now): 768 x 4096 x 12288 77 -> 63, 768 x 24576 x 4096 120 -> 110, 4096 x 24576 x 4096 614 -> 583, 4096 x
 // 4096 x 12288 362 -> 306, 24576 x 4096 x 4096 711 -> 646, 256 x 126464 x 4096 258 -> 221.
-static void plan_pair(int M, int N, int K, int max_split, int* bn, int* splits) {
+static void plan_pair(int M, int N, int K, int max_split, int exact_split, int* bn, int* splits) {
   const int pairs = sm_count() / 2, num_kb = (K + TILE_K - 1) / TILE_K;
   const long n_pairs = (N + 2 * TILE_W - 1) / (2 * TILE_W);
   double best = -1.0;
   for (int BN : {256, 192, 128}) {
     const long tiles = n_pairs * ((M + BN - 1) / BN);
     const double issue = BN == 256 ? 0.33 : BN == 192 ? 0.27 : 0.25, bytes = (TILE_W + BN / 2) * TILE_K * 2.0;
-    for (int S = 1; S == 1 || (S <= max_split && S * tiles <= pairs && S <= num_kb / 4); ++S) {
+    const int S0 = exact_split > 0 ? exact_split : 1;
+    for (int S = S0; S == S0 || (exact_split == 0 && S <= max_split && S * tiles <= pairs && S <= num_kb / 4); ++S) {
       const long units = tiles * S, rounds = (units + pairs - 1) / pairs;
       const double ctas = 2.0 * (units < pairs ? units : pairs), fabric = bytes * ctas / 12.0e6;
       const double us = (double)rounds * ((num_kb + S - 1) / S) * (issue > fabric ? issue : fabric) +
@@ -585,6 +586,8 @@ GemmPlan plan_gemm_bf16(int M, int N, int K, int force_split, int force_stages, 
   GemmPlan p;
   const int sms = sm_count();
   const long n_tiles = (N + TILE_W - 1) / TILE_W;
+  const int exact = force_split < 0 ? -force_split : 0;
+  if (exact) force_split = 0;
   if (force_persistent == 0) force_persistent = g_gemm_force_persistent;
   p.num_kb = (K + TILE_K - 1) / TILE_K;
   p.BN = M <= 32 ? 32 : M <= 64 ? 64 : M <= 256 ? 128 : 256;
@@ -599,7 +602,7 @@ GemmPlan plan_gemm_bf16(int M, int N, int K, int force_split, int force_stages, 
   const bool many_rows = ((M + 255) / 256) * n_tiles > sms || (M >= 768 && K >= 1024);
   if (force_pair == 0 && force_bn == 0 && force_split <= 1 && M > 128 && ((long)N * K >= 1L << 21 || many_rows)) {
     p.wide = true;
-    plan_pair(M, N, K, force_split == 1 ? 1 : 16, &p.BN, &S);
+    plan_pair(M, N, K, force_split == 1 ? 1 : 16, exact, &p.BN, &S);
     p.pair = force_persistent >= 0;
     if (!p.pair && p.BN == 192) p.BN = 128;   // the one-tile kernel on the same splits: the same sums, the same slabs
   } else if (force_pair == 0 && force_bn == 0 && force_split == 0 && M > 64 && M <= 128 && n_tiles * ((M + 63) / 64) <= sms) {
@@ -628,7 +631,7 @@ GemmPlan plan_gemm_bf16(int M, int N, int K, int force_split, int force_stages, 
     if (S > max_s) S = max_s;
     if (S < 1) S = 1;
   }
-  if (force_split > 0) S = force_split < p.num_kb ? force_split : p.num_kb;
+  if (exact || force_split > 0) S = std::min(exact ? exact : force_split, p.num_kb);
   // weight matrices that no L2 keeps until the next step (smaller ones may: a small model's layers stay there)
   p.w_stream = (long)N * K >= 8L << 20;
   p.upc = (p.num_kb + S - 1) / S;                 // k-blocks per split

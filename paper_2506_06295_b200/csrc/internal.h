@@ -138,9 +138,15 @@ void launch_tail(const Launch& L, int dtype, Partials part, const int32_t* inv, 
                  OutRows Fc_layer, const float* gain, void* u, Geo g, int c0, int c1, float eps);
 // (launch_tail and launch_oproj_epilogue: part.p == nullptr with active rows: the projection has written their rows.)
 void launch_gather_rows(const Launch& L, int dtype, const void* src, const int32_t* act, void* dst, int rows, int d);
-// RoPE on Q and K of the active rows; Q -> qbuf [Ma, dq]; K -> K cache rows.
+// RoPE on Q and K of the active rows; Q -> qbuf [Ma, dq]; K -> K cache rows.  Vc_layer: `part` is the [Q | K | V] product of
+// all carried rows in their order (act is not read); V -> cache rows too, q_by_slot: Q rows sequence by sequence.
 void launch_qk_rope(const Launch& L, int dtype, Partials part, const int32_t* act, const float* rope_tab, void* qbuf,
-                    void* Kc_layer, Geo g, int Ma, int H, int Hkv, int hd);
+                    void* Kc_layer, Geo g, int Ma, int H, int Hkv, int hd, void* Vc_layer = nullptr, int q_by_slot = 0);
+// Selection among the response rows and RoPE of the selected ones, out of the [Q | K | V] product of all of them (R <= 1024).
+// Q -> qbuf and the lists in the order of the scores; Vc_layer (may be null): V of the selected rows -> cache.
+void launch_select_rope(const Launch& L, int dtype, Partials part, const float* sim, const int32_t* forced, int mode, int ksel,
+                        int32_t* sel, int32_t* act, int32_t* inv, const float* rope_tab, void* qbuf, void* Kc_layer,
+                        void* Vc_layer, Geo g, int H, int Hkv, int hd);
 // rows of `part` -> cache rows (model dtype).  act == nullptr: rows are the
 // carried ids c_base + i; otherwise act[i].
 void launch_scatter_rows(const Launch& L, int dtype, Partials part, const int32_t* act, int c_base, void* cache_layer,
@@ -186,7 +192,7 @@ struct GemmPlan {
   bool wide = false;  // an automatic plan for pairs (also where dllm_debug_gemm_plan gives it to the one-tile kernel)
   int pair = 0;     // 1: persistent CTA pairs (cta_group::2) on tiles of 256 weight rows x BN activation rows
 };
-// 0 = auto.  force_pair: 0 auto, 1 CTA pairs (BN >= 64).  force_persistent: 0 auto, 1 the pair kernel for unsplit
+// 0 = auto; force_split < 0: the automatic tile with exactly -force_split splits.  force_pair: 0 auto, 1 CTA pairs (BN >= 64).  force_persistent: 0 auto, 1 the pair kernel for unsplit
 // plans with 256-row tiles, -1 the one-tile kernel with the splits of the automatic plan.
 GemmPlan plan_gemm_bf16(int M, int N, int K, int force_split = 0, int force_stages = 0, int force_bn = 0,
                         int force_pair = 0, int force_persistent = 0);
@@ -208,6 +214,8 @@ struct RowOut {
   const int32_t* act = nullptr;    // carried row of row m; nullptr: base + m
   int base = 0;
   OutRows rows{};
+  float* slab = nullptr;           // qkv == 0: rows m < slab_rows as they are, fp32, here instead
+  int slab_rows = 0;
   __nv_bfloat16 *q = nullptr, *k = nullptr, *v = nullptr;
   int v_from = 0;                  // rows m from which on V is stored (those before it have theirs)
   int q_by_slot = 0;               // rows of q sequence by sequence (b * n + position) instead of row m
