@@ -230,7 +230,7 @@ Workspace make_workspace(const dllm_config& c, int B, int P, int R, int flags) {
       slabs(Ma, d, m);
     }
   } else {
-    mn = std::max(mn, rows * std::max(std::max(dq + dkv, d), 2 * m));
+    mn = std::max(mn, rows * std::max(std::max(dq + 2 * dkv, d), 2 * m));
   }
   w.part_floats = mn + 4096;
   w.part = take(w.part_floats * 4);
@@ -621,7 +621,9 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
   const bool all_rows = rr || std::all_of(ksels.begin(), ksels.end(), [&](int k) { return k == s->R; });
   const bool in_one = tensor && qkv_in_one(c, s->B, s->R);
   const int v_split = in_one ? plan_gemm_bf16(BR, dq + 2 * dkv, d).S_max : 0;
-  const bool all_in_one = in_one && all_rows && (!rp || qkv_all_rows(c, c1, v_split));
+  const bool all_in_one = tensor ? in_one && all_rows && (!rp || qkv_all_rows(c, c1, v_split))
+                                 // the plain-ALU product adds up alike whatever it is stacked with: one product wherever it fits
+                                 : rr && (size_t)c1 * (dq + 2 * dkv) <= s->ws.part_floats;
   const GemmPlan qk_plan = heads ? plan_gemm_bf16(c1, dq + dkv, d) : GemmPlan{};
   const bool qk_unsplit = !all_in_one && all_rows && heads && qk_plan.wide && qk_plan.S_max == 1;
   const bool qk_whole = all_in_one ? rr && !s->profiling : qk_unsplit && qk_plan.pair && rr && rotate;
@@ -684,8 +686,9 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
     // Mixed step: one product for V of the response rows (as it comes, for V-verify) and of the prompt rows behind them, which
     // an unsplit product of many rows places itself; split, only up to a thousand rows (a long prompt's slabs would cost more
     // than the launch)
-    const bool v_together = in_one && rp && !rr && verify_v && (!all_rows || prompt_v_split == v_split) &&
-                            (c1 <= 1024 || (v_split == 1 && plan_gemm_bf16(c1, dkv, d, -1).wide));
+    const bool v_together = rp && !rr && verify_v &&
+                            (!tensor || (in_one && (!all_rows || prompt_v_split == v_split) &&
+                                         (c1 <= 1024 || (v_split == 1 && plan_gemm_bf16(c1, dkv, d, -1).wide))));
     const bool v_one = v_together && !s->profiling;
     if (v_whole) {
       // projected with Q and K below
