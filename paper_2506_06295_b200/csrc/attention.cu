@@ -112,15 +112,15 @@ __global__ void __launch_bounds__(128) attn_simt_kernel(const T* __restrict__ q,
 
 
 // The same arithmetic where the grid of attn_simt_kernel would leave the chip empty (few rows: the step of a small
-// model): a CTA takes four queries of one head and its eight warps take DIFFERENT chunks of 32 keys (warp w the chunks
+// model): a CTA takes NQ queries of one head and its eight warps take DIFFERENT chunks of 32 keys (warp w the chunks
 // w, w + 8, ...), so 96 keys are one chunk deep instead of three with a block barrier each; the warps' results are merged
 // in warp order.  lane = key for the scores (K straight from memory, q broadcast from shared memory), lane = output
 // column for P V.
-template <typename T, int ND>
+template <typename T, int ND, int NQ>
 __global__ void __launch_bounds__(256, 1) attn_simt_few_kernel(const T* __restrict__ q, const T* __restrict__ Kc,
                                                             const T* __restrict__ Vc, T* __restrict__ o, int a_seq, int n,
                                                             int H, int Hkv, float scale) {
-  constexpr int HD = 32 * ND, NQ = 4, NW = 8;
+  constexpr int HD = 32 * ND, NW = 8;
   __shared__ __align__(16) float qs[NQ][HD];
   __shared__ float part[NW][NQ][HD], pm[NW][NQ], pl[NW][NQ];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -228,18 +228,20 @@ void launch_simt(const Launch& L, const void* q, const void* Kc, const void* Vc,
                  int Hkv, int hd) {
   const float scale = 1.0f / sqrtf((float)hd);
   const long ctas = (long)((a_seq + TQ - 1) / TQ) * H * B;
-  // below two CTAs of 16 queries per SM the warps share the keys instead of the queries (four times the CTAs); above, the
-  // 16 queries of a CTA share each key's trip into shared memory
+  // below two CTAs of 16 queries per SM the warps share the keys instead of the queries (four times the CTAs, or sixteen times
+  // while one query per CTA still is one wave: a warp's chain of products is as long as its queries are many: 8 rows x 4 heads against
+  // 96 keys 5.0 -> 4.0 us); above, the 16 queries of a CTA share each key's trip into shared memory
   const bool aligned = (((uintptr_t)Kc) & 15) == 0 && (Hkv * hd * sizeof(T)) % 16 == 0;
   if (ctas < 2L * sm_count() && aligned) {
-    const dim3 grid((a_seq + 3) / 4, H, B);
+    const bool one = (long)a_seq * H * B <= sm_count();
+    const dim3 grid(one ? a_seq : (a_seq + 3) / 4, H, B);
     auto go = [&](auto* kernel) {
       launch_k(L, kernel, grid, dim3(256), 0, (const T*)q, (const T*)Kc, (const T*)Vc, (T*)o, a_seq, n, H, Hkv, scale);
     };
-    if (hd == 32) go(attn_simt_few_kernel<T, 1>);
-    else if (hd == 64) go(attn_simt_few_kernel<T, 2>);
-    else if (hd == 96) go(attn_simt_few_kernel<T, 3>);
-    else go(attn_simt_few_kernel<T, 4>);
+    if (hd == 32) one ? go(attn_simt_few_kernel<T, 1, 1>) : go(attn_simt_few_kernel<T, 1, 4>);
+    else if (hd == 64) one ? go(attn_simt_few_kernel<T, 2, 1>) : go(attn_simt_few_kernel<T, 2, 4>);
+    else if (hd == 96) one ? go(attn_simt_few_kernel<T, 3, 1>) : go(attn_simt_few_kernel<T, 3, 4>);
+    else one ? go(attn_simt_few_kernel<T, 4, 1>) : go(attn_simt_few_kernel<T, 4, 4>);
   } else {
     launch_k(L, attn_simt_kernel<T>, dim3((a_seq + TQ - 1) / TQ, H, B), dim3(128), 0, (const T*)q, (const T*)Kc,
              (const T*)Vc, (T*)o, a_seq, n, H, Hkv, hd, scale);
