@@ -53,50 +53,62 @@ __global__ void __launch_bounds__(SG_WARPS * 32)
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   const int lr = lane >> 3, lk = (lane & 7) * 4;            // loads: four rows per pass, 8 lanes x 4 k per row
   const int chunks = (K + SG_K - 1) / SG_K;
-  float4 ra[TM], rw[2 * TN];
-  auto load_w = [&](int c) {
+  // chunks of a warp whose operands are on their way at once: small tiles have the registers for three, and less arithmetic
+  // per chunk than a load takes (K = 688 is three chunks of most warps: the tiny configuration's generation 516 -> 499 us)
+  constexpr int DEPTH = TM * TN <= 4 ? 3 : 1;
+  float4 ra[DEPTH][TM], rw[DEPTH][2 * TN];
+  auto load_w = [&](int d, int c) {
 #pragma unroll
     for (int i = 0; i < 2 * TN; ++i)
-      rw[i] = load4(W + (size_t)(n0 + 4 * i + lr) * K, n0 + 4 * i + lr < N, c * SG_K + lk, K, vec);
+      rw[d][i] = load4(W + (size_t)(n0 + 4 * i + lr) * K, n0 + 4 * i + lr < N, c * SG_K + lk, K, vec);
   };
-  auto load_a = [&](int c) {
+  auto load_a = [&](int d, int c) {
 #pragma unroll
     for (int i = 0; i < TM; ++i)
-      ra[i] = load4(A + (size_t)(m0 + 4 * i + lr) * K, m0 + 4 * i + lr < M, c * SG_K + lk, K, vec);
+      ra[d][i] = load4(A + (size_t)(m0 + 4 * i + lr) * K, m0 + 4 * i + lr < M, c * SG_K + lk, K, vec);
   };
-  if (warp < chunks) load_w(warp);                          // weights are written by no kernel
+#pragma unroll
+  for (int d = 0; d < DEPTH; ++d)
+    if (warp + d * SG_WARPS < chunks) load_w(d, warp + d * SG_WARPS);   // weights are written by no kernel
   pdl_wait();
   pdl_trigger();
-  if (warp < chunks) load_a(warp);
+#pragma unroll
+  for (int d = 0; d < DEPTH; ++d)
+    if (warp + d * SG_WARPS < chunks) load_a(d, warp + d * SG_WARPS);
   float acc[TM][TN] = {};
   const int ly = lane >> 3, lx = lane & 7;
-  for (int c = warp; c < chunks; c += SG_WARPS) {
-    __syncwarp();
+  for (int c0 = warp; c0 < chunks; c0 += DEPTH * SG_WARPS) {
 #pragma unroll
-    for (int i = 0; i < TM; ++i) *reinterpret_cast<float4*>(As + (4 * i + lr) * SG_LD + lk) = ra[i];
+    for (int d = 0; d < DEPTH; ++d) {
+      const int c = c0 + d * SG_WARPS;
+      if (c >= chunks) break;
+      __syncwarp();
 #pragma unroll
-    for (int i = 0; i < 2 * TN; ++i) *reinterpret_cast<float4*>(Ws + (4 * i + lr) * SG_LD + lk) = rw[i];
-    __syncwarp();
-    if (c + SG_WARPS < chunks) {                            // the warp's next chunk travels under this one's arithmetic
-      load_w(c + SG_WARPS);
-      load_a(c + SG_WARPS);
-    }
+      for (int i = 0; i < TM; ++i) *reinterpret_cast<float4*>(As + (4 * i + lr) * SG_LD + lk) = ra[d][i];
 #pragma unroll
-    for (int k = 0; k < SG_K; k += 4) {
-      float4 a[TM], w[TN];
+      for (int i = 0; i < 2 * TN; ++i) *reinterpret_cast<float4*>(Ws + (4 * i + lr) * SG_LD + lk) = rw[d][i];
+      __syncwarp();
+      if (c + DEPTH * SG_WARPS < chunks) {                    // the warp's next chunk travels under this one's arithmetic
+        load_w(d, c + DEPTH * SG_WARPS);
+        load_a(d, c + DEPTH * SG_WARPS);
+      }
 #pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const float4*>(As + (4 * i + ly) * SG_LD + k);
+      for (int k = 0; k < SG_K; k += 4) {
+        float4 a[TM], w[TN];
 #pragma unroll
-      for (int j = 0; j < TN; ++j) w[j] = *reinterpret_cast<const float4*>(Ws + (8 * j + lx) * SG_LD + k);
+        for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const float4*>(As + (4 * i + ly) * SG_LD + k);
 #pragma unroll
-      for (int i = 0; i < TM; ++i)
+        for (int j = 0; j < TN; ++j) w[j] = *reinterpret_cast<const float4*>(Ws + (8 * j + lx) * SG_LD + k);
 #pragma unroll
-        for (int j = 0; j < TN; ++j) {
-          acc[i][j] = fmaf(a[i].x, w[j].x, acc[i][j]);
-          acc[i][j] = fmaf(a[i].y, w[j].y, acc[i][j]);
-          acc[i][j] = fmaf(a[i].z, w[j].z, acc[i][j]);
-          acc[i][j] = fmaf(a[i].w, w[j].w, acc[i][j]);
-        }
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < TN; ++j) {
+            acc[i][j] = fmaf(a[i].x, w[j].x, acc[i][j]);
+            acc[i][j] = fmaf(a[i].y, w[j].y, acc[i][j]);
+            acc[i][j] = fmaf(a[i].z, w[j].z, acc[i][j]);
+            acc[i][j] = fmaf(a[i].w, w[j].w, acc[i][j]);
+          }
+      }
     }
   }
   // partial tiles through shared memory (every warp is done with the buffers), added in warp order
