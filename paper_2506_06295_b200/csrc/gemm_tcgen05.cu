@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(ONE_THREADS) gemm_bf16_tcgen05_kernel(const __
                                                                 const __grid_constant__ CUtensorMap tmA,
                                                                 float* __restrict__ part, int M, int N, int num_kb,
                                                                 int kb_per_split, size_t split_stride, int STAGES,
-                                                                __nv_bfloat16* __restrict__ act_out, int m_ffn,
+                                                                __nv_bfloat16* __restrict__ act_out, int m_ffn, int turned,
                                                                 int* __restrict__ status) {
   using SL = SmemLayout<BN>;
   extern __shared__ uint8_t smem_raw[];
@@ -260,6 +260,11 @@ __global__ void __launch_bounds__(ONE_THREADS) gemm_bf16_tcgen05_kernel(const __
   const int kb0 = blockIdx.z * kb_per_split;
   const int kb1 = min(num_kb, kb0 + kb_per_split);
   const int nkb = kb1 - kb0;            // >= 1 by construction of the plan
+  const int turn = turned && ((nt >> 1) & 1) ? nkb / 2 : 0;   // see run_gemm
+  auto k_block = [&](int i) {           // the i-th k-block of the walk
+    const int j = i + turn;
+    return kb0 + (j < nkb ? j : j - nkb);
+  };
 
   const uint32_t tiles = (smem_u32(smem_raw) + 1023u) & ~1023u;
 
@@ -280,7 +285,7 @@ __global__ void __launch_bounds__(ONE_THREADS) gemm_bf16_tcgen05_kernel(const __
       for (int i = 0; i < pre; ++i) {  // weights are written by no kernel: stream them ahead of the dependency
         const uint32_t fb = smem_u32(&full_bar[i]);
         mbar_expect_tx(fb, SL::STAGE_BYTES);
-        tma_load_2d_weights<ONCE>(tiles + i * SL::STAGE_BYTES, &tmW, fb, (kb0 + i) * TILE_K, n0);
+        tma_load_2d_weights<ONCE>(tiles + i * SL::STAGE_BYTES, &tmW, fb, k_block(i) * TILE_K, n0);
       }
     }
     __syncwarp();
@@ -306,7 +311,7 @@ __global__ void __launch_bounds__(ONE_THREADS) gemm_bf16_tcgen05_kernel(const __
     for (int i = 0; i < nkb; ++i) {
       const uint32_t fb = smem_u32(&full_bar[s]);
       const uint32_t dstW = tiles + s * SL::STAGE_BYTES;
-      const int kc = (kb0 + i) * TILE_K;
+      const int kc = k_block(i) * TILE_K;
       const bool skip = i == 0 && dbg_skip != 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0;
       if (i >= pre && !mbar_wait_warp(smem_u32(&empty_bar[s]), ph ^ 1u, abortp)) {
         if (status && lane == 0) atomicCAS(status, ST_OK, ST_TIMEOUT_TMA);
@@ -497,7 +502,7 @@ cudaError_t launch_one(const Launch& L, const CUtensorMap& tmW, const CUtensorMa
   const int stages = plan.stages < 2 ? 2 : plan.stages > max_stages(BN) ? max_stages(BN) : plan.stages;
   dim3 grid((M + BN - 1) / BN, (N + TILE_W - 1) / TILE_W, plan.S_max);
   cudaError_t e = launch_k(L, gemm_bf16_tcgen05_kernel<BN, ONCE>, grid, dim3(ONE_THREADS), SL::total(stages), tmW, tmA, part, M, N,
-                           num_kb, plan.upc, (size_t)M * N, stages, (__nv_bfloat16*)act_out, m_ffn, L.d_status);
+                           num_kb, plan.upc, (size_t)M * N, stages, (__nv_bfloat16*)act_out, m_ffn, (int)plan.turned, L.d_status);
   L.count();
   return e != cudaSuccess ? e : cudaGetLastError();
 }
