@@ -32,6 +32,8 @@
 // maximum, sum and output accumulator; the tiles' scores take three buffers in
 // turn, and the two halves are merged through shared memory at the end (group
 // 1's first).
+// With many row tiles a CTA takes one of them with one softmax group, half of the ring and half of the tensor memory, and two
+// CTAs share an SM.
 // Key-range splits write unnormalised partials plus (max, sum) exactly like the
 // mma.sync kernel, and the same merge kernel finishes them.  Every mbarrier wait
 // is bounded.
@@ -49,9 +51,6 @@ namespace {
 constexpr int UA_ROWS = 128;   // virtual rows per row tile (UMMA M); a CTA works on two row tiles
 constexpr int UA_TILES = 2;
 constexpr int UA_KEYS = 64;    // keys per tile
-constexpr int UA_STAGES = 6;   // K/V ring
-constexpr int UA_THREADS = 352;  // two softmax groups of 128, two MMA warps, one TMA warp
-constexpr int UA_TMA_WARP = 10;
 // key tiles from which a CTA with one live row tile shares them between its two softmax groups: the exchange and merge of
 // the two halves at the end cost 1.1 us, a shared tile takes 0.50 us instead of 0.93 (B200, 128 rows x 32 heads of 128, us
 // not shared -> shared: 4 tiles 10.0 -> 9.3, 5 11.0 -> 9.9, 6 12.2 -> 10.7, 7 13.0 -> 11.1, 8 13.9 -> 11.6, 16 21.1 ->
@@ -116,33 +115,37 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
   return d;
 }
 
-template <int HD>
+// TILES = 2: one CTA per SM, two softmax groups; 1: two CTAs per SM, each with one row tile, one softmax group, one MMA and
+// one TMA warp, half of the shared memory and of the tensor memory.
+template <int HD, int TILES>
 struct UaSmem {
+  static constexpr int STAGES = TILES == 2 ? 6 : HD == 64 ? 6 : 3;              // K/V ring
+  static constexpr int THREADS = TILES == 2 ? 352 : 192, MMA_WARP = 4 * TILES, TMA_WARP = TILES == 2 ? 10 : 5;
   static constexpr uint32_t KV_TILE = UA_KEYS * HD * 2;          // one K or V tile
   static constexpr uint32_t STAGE = 2 * KV_TILE;                 // K then V
-  static constexpr uint32_t TOTAL = UA_STAGES * STAGE + 1024;    // shared memory holds nothing but the K/V ring
+  static constexpr uint32_t TOTAL = STAGES * STAGE + 1024;    // shared memory holds nothing but the K/V ring
   // Tensor memory, 128 lanes = the rows of a tile: Q_i as bf16 pairs (HD / 2 columns each), the scores S_i (64
   // fp32 columns each; the probabilities P_i overwrite the first 32 of them as bf16 pairs), the outputs O_i.
   // One row tile shared by the groups: one Q, three score buffers that the key tiles take in turn, O per group.
-  static constexpr uint32_t Q_COL = 0, S_COL = UA_TILES * (HD / 2), O_COL = 64 + 3 * UA_KEYS;
+  static constexpr uint32_t Q_COL = 0, S_COL = TILES * (HD / 2), O_COL = TILES == 2 ? 64 + 3 * UA_KEYS : 64 + UA_KEYS;
   static constexpr uint32_t KPAR_S_COL = 64;
-  static constexpr uint32_t TMEM_COLS = 512;
-  static_assert(S_COL + UA_TILES * UA_KEYS <= O_COL, "scores and outputs must not overlap");
-  static_assert(O_COL + UA_TILES * HD <= TMEM_COLS, "tensor memory holds 512 columns");
+  static constexpr uint32_t TMEM_COLS = 256 * TILES;
+  static_assert(S_COL + TILES * UA_KEYS <= O_COL, "scores and outputs must not overlap");
+  static_assert(O_COL + TILES * HD <= TMEM_COLS, "tensor memory holds 512 columns");
 };
 
-template <int HD>
-__global__ void __launch_bounds__(UA_THREADS, 1)
+template <int HD, int TILES>
+__global__ void __launch_bounds__((UaSmem<HD, TILES>::THREADS), 3 - TILES)
     attn_umma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                      const __nv_bfloat16* __restrict__ q,
                      __nv_bfloat16* __restrict__ o, float* __restrict__ o_part, float* __restrict__ ml_part, int a_seq,
                      int n, int H, int Hkv, int S, int keys_per_split, int row_tiles_per_cta, float scale_log2,
                      int* __restrict__ status) {
-  using SM = UaSmem<HD>;
-  constexpr int PANELS = HD / 64;
+  using SM = UaSmem<HD, TILES>;
+  constexpr int PANELS = HD / 64, UA_STAGES = SM::STAGES, UA_TMA_WARP = SM::TMA_WARP;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t kv_full[UA_STAGES], kv_empty[UA_STAGES];
-  __shared__ __align__(8) uint64_t s_full[3], p_full[UA_TILES], o_full[UA_TILES], q_bar;
+  __shared__ __align__(8) uint64_t s_full[3], p_full[TILES], o_full[TILES], q_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
 
@@ -165,7 +168,7 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
   const int dq = H * HD;
   // one live row tile and enough key tiles: both softmax groups work on that tile's rows, group i on the key
   // tiles t with t % 2 == i
-  const bool kpar = live == 1 && n_tiles >= UA_KPAR_MIN_TILES;
+  const bool kpar = TILES == 2 && live == 1 && n_tiles >= UA_KPAR_MIN_TILES;
 
   if (tid == 0) {
     abort_flag = 0;
@@ -173,12 +176,12 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
       mbar_init(smem_u32(&kv_full[i]), 1);
       mbar_init(smem_u32(&kv_empty[i]), 1);
     }
-    for (int i = 0; i < UA_TILES; ++i) {
+    for (int i = 0; i < TILES; ++i) {
       mbar_init(smem_u32(&p_full[i]), UA_ROWS / 32);  // one arrival per warp of the tile's softmax group
       mbar_init(smem_u32(&o_full[i]), 1);
     }
     for (int i = 0; i < 3; ++i) mbar_init(smem_u32(&s_full[i]), 1);
-    mbar_init(smem_u32(&q_bar), UA_TILES * UA_ROWS / 32);  // one arrival per softmax warp
+    mbar_init(smem_u32(&q_bar), TILES * UA_ROWS / 32);  // one arrival per softmax warp
     mbar_fence_init();
     prefetch_tensormap(&tmK);
     prefetch_tensormap(&tmV);
@@ -218,7 +221,7 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
       }
       __syncwarp();
     }
-  } else if (warp >= 8) {
+  } else if (warp >= SM::MMA_WARP) {
     // ---------------- MMA issuers: warp 8, and warp 9 for group 1 when the groups share a row tile ----------------
     // Per key tile t and row tile i:  S_i(t) = Q_i K(t)^T  ->  [softmax group i]  ->  O_i += P_i(t) V(t), and right
     // behind it S_i(t+1), so that the tensor pipe works on one row tile while the other is in its softmax.  Q_i
@@ -267,7 +270,7 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
       // alone issues the first three, in order (a commit covers what its thread issued before): group 1, through with tile
       // 1, knows S(0) complete when it waits for S(3), group 0 after tile 2 S(1).  S(2) precedes S(3) in issuer 0; from
       // tile 6 on S(t - 3) precedes the product of tile t - 4 in the same issuer, which the group has waited for.
-      const int i = warp - 8;
+      const int i = warp - SM::MMA_WARP;
       for (int t = 0; t < 3 && ok && i == 0; ++t) {
         ok = tile_ready(t);
         if (ok) issue_s(SM::KPAR_S_COL + (uint32_t)(t * UA_KEYS), SM::Q_COL, t, t);
@@ -292,7 +295,7 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
         }
         buf = buf == 0 ? 2 : buf - 1;   // (t + 2) % 3
       }
-    } else if (warp == 8) {
+    } else if (warp == SM::MMA_WARP) {
       if (ok) ok = tile_ready(0);
       for (int i = 0; i < live && ok; ++i)
         issue_s(SM::S_COL + (uint32_t)(i * UA_KEYS), SM::Q_COL + (uint32_t)(i * (HD / 2)), i, 0);
@@ -479,7 +482,7 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
       float w_self = 1.f, w_peer = 0.f;  // weights of this group's and the other group's half in the merged row
       bool peer = false, write_out = ok;
       if (kpar) {
-        static_assert((UA_ROWS * XS + 2 * UA_ROWS) * 4 <= UA_STAGES * SM::STAGE, "the exchange area must fit the ring");
+        static_assert(TILES == 1 || (UA_ROWS * XS + 2 * UA_ROWS) * 4 <= UA_STAGES * SM::STAGE, "the exchange area must fit the ring");
         {  // both groups are past their last product (or gave up): all 256 threads agree
           uint32_t r;
           asm volatile(
@@ -577,14 +580,14 @@ __global__ void __launch_bounds__(UA_THREADS, 1)
   }
 }
 
-template <int HD>
+template <int HD, int TILES>
 cudaError_t launch_umma(const Launch& L, const CUtensorMap& tmK, const CUtensorMap& tmV, const void* q, void* o,
                         float* scratch, int B, int a_seq, int n, int H, int Hkv, int S, int keys_per_split,
                         int row_tiles_per_cta) {
-  constexpr int SMEM = (int)UaSmem<HD>::TOTAL;
+  constexpr int SMEM = (int)UaSmem<HD, TILES>::TOTAL;
   static DeviceOnce once;
   cudaError_t e0 = once.run(
-      [] { return cudaFuncSetAttribute(attn_umma_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM); });
+      [] { return cudaFuncSetAttribute(attn_umma_kernel<HD, TILES>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM); });
   if (e0 != cudaSuccess) return e0;
   const int G = H / Hkv;
   const size_t total = (size_t)B * a_seq * H;
@@ -593,7 +596,7 @@ cudaError_t launch_umma(const Launch& L, const CUtensorMap& tmK, const CUtensorM
   const int rows_per_cta = row_tiles_per_cta * UA_ROWS;
   dim3 grid((a_seq * G + rows_per_cta - 1) / rows_per_cta, Hkv, B * S);
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)HD);
-  cudaError_t e = launch_k(L, attn_umma_kernel<HD>, grid, dim3(UA_THREADS), SMEM, tmK, tmV, (const __nv_bfloat16*)q,
+  cudaError_t e = launch_k(L, attn_umma_kernel<HD, TILES>, grid, dim3(UaSmem<HD, TILES>::THREADS), SMEM, tmK, tmV, (const __nv_bfloat16*)q,
                            (__nv_bfloat16*)o, o_part, ml_part, a_seq, n, H, Hkv, S, keys_per_split, row_tiles_per_cta,
                            scale_log2, L.d_status);
   L.count();
@@ -643,6 +646,15 @@ AttnPlan plan_attention_umma(int B, int a_seq, int n, int H, int Hkv, size_t scr
   p.S = (key_tiles + tiles_per_split - 1) / tiles_per_split;
   p.scratch_floats = p.S > 1 ? (size_t)p.S * per_split : 0;
   p.row_tiles = a_seq * G <= UA_ROWS ? 1 : best_rt;
+  // Three CTAs of one row tile per SM or more: two at a time, so that one's start and end (8 to 10 us of loads, merges and
+  // stores) run beside the other's products.  B200, us, one CTA per SM -> two: 16 x 128 x 1536 x 32 heads 99 -> 86, 16 x 128 x
+  // 768 69 -> 57, 8 x 300 x 700 75 -> 63, 4 x 1536 x 1536 209 -> 189, 4128 x 4128 301 -> 293; below, where a CTA's own chain is
+  // what counts and two row tiles share each K / V tile: 1024 x 1024 30.5 -> 32.7, 4 x 128 x 1536 28 -> 34.
+  const long tiles = (long)((a_seq * G + UA_ROWS - 1) / UA_ROWS) * Hkv * B;
+  if (p.S == 1 && tiles >= 3L * sms && g_attn_umma_row_tiles == 0 && g_attn_force_splits == 0) {
+    p.row_tiles = 1;
+    p.two_per_sm = true;
+  }
   return p;
 }
 
@@ -655,9 +667,9 @@ cudaError_t launch_attention_umma(const Launch& L, const void* q, const void* Kc
       !get_tensor_map_3d(Vc, (uint64_t)B, (uint64_t)n, (uint64_t)Hkv * hd, 64, &tmV))
     return cudaErrorInvalidValue;
   if (S_out) *S_out = p.S;
-  return hd == 64
-             ? launch_umma<64>(L, tmK, tmV, q, o, scratch, B, a_seq, n, H, Hkv, p.S, p.keys_per_split, p.row_tiles)
-             : launch_umma<128>(L, tmK, tmV, q, o, scratch, B, a_seq, n, H, Hkv, p.S, p.keys_per_split, p.row_tiles);
+  auto go = [&](auto launch) { return launch(L, tmK, tmV, q, o, scratch, B, a_seq, n, H, Hkv, p.S, p.keys_per_split, p.row_tiles); };
+  if (p.two_per_sm) return hd == 64 ? go(launch_umma<64, 1>) : go(launch_umma<128, 1>);
+  return hd == 64 ? go(launch_umma<64, 2>) : go(launch_umma<128, 2>);
 }
 
 }  // namespace dllm

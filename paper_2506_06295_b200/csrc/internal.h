@@ -243,6 +243,7 @@ struct AttnPlan {
   size_t scratch_floats;
   int few_rg = 0;      // 64-row kernel family: 0 = the 64-row kernel, 1 / 2 = the few-rows kernel with 16 / 32 rows per CTA
   int row_tiles = 2;   // tcgen05 kernel: 128-row tiles per CTA (2, or 1 when two-tile CTAs would be too few)
+  bool two_per_sm = false;  // tcgen05 kernel: one row tile per CTA and two CTAs per SM
 };
 AttnPlan plan_attention(int B, int a_seq, int n, int H, int Hkv);
 // Plan of the 128-row tcgen05 kernel (attention_umma.cu) with at most scratch_floats floats for split partials.
