@@ -637,6 +637,9 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
   // V of the response rows too
   const bool v_whole = qk_whole && (all_in_one || (in_one ? v_split : plan_gemm_bf16(BR, dkv, d).S_max) == 1);
   const bool qkv_whole = v_whole || (qk_whole && rp);
+  // Many response rows, V unsplit: its product verifies (and overwrites) the rows itself, profiled too
+  const GemmPlan v_plan = tensor && !in_one ? plan_gemm_bf16(BR, dkv, d) : GemmPlan{};
+  const bool verify_in_product = tensor && !in_one && v_plan.pair && v_plan.S_max == 1 && dkv % 4 == 0;
   // splits of Q / K and of the prompt's V in such a step (0: their own plans')
   const int all_split = all_in_one ? v_split : 0, prompt_v_split = all_in_one ? v_split : qk_unsplit ? 1 : 0;
   RowOut qkv;
@@ -713,19 +716,32 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
       // V for ALL response rows (the 2 r d^2 term of Sec. A.7), V-verify, V overwrite
       // (a prompt refresh reads W_v once more, for the prompt rows)
       RowOut o = rows_into({s->cache(l, DLLM_CACHE_V), nullptr, 0}, dkv, nullptr, 0);
-      o.slab = s->wsp<float>(s->ws.part);
-      o.slab_rows = BR;
+      const bool verify = verify_in_product && !rr;
+      if (verify) {
+        o.verify = s->wsp<float4>(s->ws.part);
+        o.metric = s->sel_metric;
+        o.keep_rows = s->v_selected_only;
+      } else {
+        o.slab = s->wsp<float>(s->ws.part);
+        o.slab_rows = BR;
+      }
       if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, u, Wv, v_one ? c1 : BR, dkv, d, &part, nullptr, &fused, -1, rp && !v_one,
-                         v_one ? &o : nullptr, v_split)) != DLLM_OK)
+                         v_one || verify ? &o : nullptr, v_split)) != DLLM_OK)
         return st;
-      if (fused) part = Partials{o.slab, (size_t)BR * dkv, 1, dkv};
-      const IdentityLists id{sel, act, inv};
-      {  // the projection's fp32 result in, the cached row in, the row out
-        ProfScope ps(s, DLLM_PROF_VVERIFY, (double)BR * dkv * (4.0 + 2.0 * es), 6.0 * BR * dkv, stream);
-        // (with random selection the scores are the caller's and outlive a refresh)
-        launch_vverify(L, dt, part, s->cache(l, DLLM_CACHE_V),
-                       rr && s->sel_strategy == DLLM_SELECT_RANDOM ? nullptr : sim, g, dkv, rr ? 0 : s->sel_metric,
-                       rr || !s->v_selected_only, identity && !qk_whole ? &id : nullptr);
+      if (fused && !verify) part = Partials{o.slab, (size_t)BR * dkv, 1, dkv};
+      if (verify) {  // the product has compared and overwritten the rows
+        ProfScope ps(s, DLLM_PROF_VVERIFY, (double)BR * ((dkv + 127) / 128) * 16.0 + BR * 4.0, 3.0 * BR * ((dkv + 127) / 128), stream);
+        launch_verify_merge(L, o.verify, sim, BR, (dkv + 127) / 128, s->sel_metric);
+        fused = false;
+      } else {
+        const IdentityLists id{sel, act, inv};
+        {  // the projection's fp32 result in, the cached row in, the row out
+          ProfScope ps(s, DLLM_PROF_VVERIFY, (double)BR * dkv * (4.0 + 2.0 * es), 6.0 * BR * dkv, stream);
+          // (with random selection the scores are the caller's and outlive a refresh)
+          launch_vverify(L, dt, part, s->cache(l, DLLM_CACHE_V),
+                         rr && s->sel_strategy == DLLM_SELECT_RANDOM ? nullptr : sim, g, dkv, rr ? 0 : s->sel_metric,
+                         rr || !s->v_selected_only, identity && !qk_whole ? &id : nullptr);
+        }
       }
     } else if (adaptive && s->sel_strategy == DLLM_SELECT_K_VERIFY) {
       // ablation: the same test on K; K of ALL response rows is projected, rotated and overwritten

@@ -667,6 +667,31 @@ void launch_vverify(const Launch& L, int dtype, Partials part, void* Vc_layer, f
   L.count();
 }
 
+// One warp per row adds up the sums that the V projection's epilogue has left per 128 columns.
+__global__ void __launch_bounds__(256) verify_merge_kernel(const float4* __restrict__ sums, float* __restrict__ sim, int rows,
+                                                           int n_tiles, int metric) {
+  pdl_wait();
+  pdl_trigger();
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (row >= rows) return;
+  float dot = 0.f, na = 0.f, nb = 0.f;
+  for (int t = lane; t < n_tiles; t += 32) {
+    const float4 v = __ldcg(sums + (size_t)row * n_tiles + t);
+    dot += v.x;
+    na += v.y;
+    nb += v.z;
+  }
+  dot = warp_sum(dot);
+  na = warp_sum(na);
+  nb = warp_sum(nb);
+  if (lane == 0) sim[row] = metric == 0 ? dot / fmaxf(sqrtf(na * nb), 1e-8f) : -sqrtf(dot);
+}
+
+void launch_verify_merge(const Launch& L, const float4* sums, float* sim, int rows, int n_tiles, int metric) {
+  launch_k(L, verify_merge_kernel, dim3((rows + 7) / 8), dim3(256), 0, sums, sim, rows, n_tiles, metric);
+  L.count();
+}
+
 // ------------------------------------------------------------------ K-verify: the same test on the post-RoPE K
 // One block per response row: slab sum of the K projection, RoPE at the row's
 // position, rounding to the cache dtype, score against the cached K row, and

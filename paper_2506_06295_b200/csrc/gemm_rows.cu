@@ -10,6 +10,10 @@
 // before the accumulator is complete, and a trip's rotation values are requested one trip ahead (fetched where they were
 // used they came from L2 or memory eight times behind the main loop: 12 us for a 256-row tile).  LLaDA-8B shape, full step
 // 11579 -> 11243 us with two groups of epilogue warps and the per-row arithmetic reduced to one multiply-add per pointer.
+//
+// VERIFY: V of all response rows of an adaptive step, compared (Eq. 6) with the rows it overwrites: a thread's eight columns,
+// the sixteen threads of a row, one triple of sums per row and 128 columns for a small merge.  Without it the fp32 result
+// went to memory and back for a kernel that read it beside the old rows (8192 rows of the LLaDA-8B shape: 54 us per layer).
 #include <type_traits>
 
 #include "gemm_pair.cuh"
@@ -18,9 +22,11 @@ namespace dllm {
 
 namespace {
 
-template <bool QKV>
+enum RowKind { PLACE, HEADS, VERIFY };
+template <RowKind KIND>
 struct RowForm {
   RowOut o;
+  static constexpr bool QKV = KIND == HEADS;
   static constexpr int GROUPS = 2;
   // rows per trip; floats per staged row (no padding: a quarter warp's 16-byte reads lie in one row)
   static constexpr int CH = 16, EXS = 128;
@@ -61,8 +67,8 @@ struct RowForm {
                        rope_hi(l.w, h.w, c.w, t.w));
   }
   template <int W>
-  __device__ __forceinline__ void drain(Shared<W>& s, uint32_t tmem_d, float* ex, int tl, int bar, int m0, int n0, int, int M,
-                                        int N, float*) const {
+  __device__ __forceinline__ void drain(Shared<W>& s, uint32_t tmem_d, float* ex, int tl, int bar, int m0, int n0, int tile_y,
+                                        int M, int N, float*) const {
     if (m0 >= M) return;   // uniform across the group
     const int rows = min(W, M - m0);
     const uint32_t tmem_w = tmem_d + ((uint32_t)(tl >> 5) << 21);
@@ -87,6 +93,7 @@ struct RowForm {
     const float* const tab = QKV ? o.rope_tab + nlo % o.hd : nullptr;
     constexpr int U = CH / 8;
     float4 cs[U], sn[U];
+    uint2 olo[U], ohi[U];   // V-verify: the rows' old values
     Place at[U];
     auto fetch = [&](int c0) {   // places and rotation values of this thread's rows c0 + rsub + 8 u (the last one past the end)
 #pragma unroll
@@ -98,6 +105,11 @@ struct RowForm {
             cs[u] = *reinterpret_cast<const float4*>(t);
             sn[u] = *reinterpret_cast<const float4*>(t + (o.hd >> 1));
           }
+        }
+        if constexpr (KIND == VERIFY) {
+          const __nv_bfloat16* p = reinterpret_cast<const __nv_bfloat16*>(at[u]);
+          olo[u] = vlo ? __ldcg(reinterpret_cast<const uint2*>(p + nlo)) : make_uint2(0, 0);
+          ohi[u] = vhi ? __ldcg(reinterpret_cast<const uint2*>(p + nhi)) : make_uint2(0, 0);
         }
       }
     };
@@ -137,11 +149,42 @@ struct RowForm {
           dhi[u] = reinterpret_cast<__nv_bfloat16*>(at[u]) + nhi;
         }
       }
+      if constexpr (KIND == VERIFY) {
+        // Eq. 6 on what the cache will hold: this thread's eight columns, then the row's sixteen threads
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const uint32_t nw[4] = {plo[u].x, plo[u].y, phi[u].x, phi[u].y}, od[4] = {olo[u].x, olo[u].y, ohi[u].x, ohi[u].y};
+          float dot = 0.f, na = 0.f, nb = 0.f;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const bool used = i < 4 ? vlo : vhi;
+            const float x = used ? __uint_as_float(i & 1 ? nw[i >> 1] & 0xFFFF0000u : nw[i >> 1] << 16) : 0.f;
+            const float y = __uint_as_float(i & 1 ? od[i >> 1] & 0xFFFF0000u : od[i >> 1] << 16);
+            if (o.metric == 0) {
+              dot += x * y;
+              na += x * x;
+              nb += y * y;
+            } else {
+              const float df = x - y;
+              dot += df * df;
+            }
+          }
+#pragma unroll
+          for (int x = 8; x > 0; x >>= 1) {
+            dot += __shfl_xor_sync(0xffffffffu, dot, x);
+            na += __shfl_xor_sync(0xffffffffu, na, x);
+            nb += __shfl_xor_sync(0xffffffffu, nb, x);
+          }
+          const int row = c0 + rsub + 8 * u;
+          if (q == 0 && row < rows) o.verify[(size_t)(m0 + row) * ((N + TILE_W - 1) / TILE_W) + tile_y] = make_float4(dot, na, nb, 0.f);
+        }
+      }
       fetch(c0 + CH);
+      if (KIND == VERIFY && o.keep_rows) continue;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int row = c0 + rsub + 8 * u;
-        if constexpr (!QKV) {
+        if constexpr (KIND == PLACE) {
           if (m0 + row < o.slab_rows) {   // (their columns 4 q .. and 64 further, as the others')
             float* const raw = reinterpret_cast<float*>(raw_at[u]);
             if (vlo && row < rows) *reinterpret_cast<float4*>(raw + nlo) = a[u];
@@ -185,7 +228,7 @@ cudaError_t launch_gemm_rows(const Launch& L, const void* A, const void* W, int 
       default: return cudaErrorInvalidValue;
     }
   };
-  return out.qkv ? go(RowForm<true>{out}) : go(RowForm<false>{out});
+  return out.qkv ? go(RowForm<HEADS>{out}) : out.verify ? go(RowForm<VERIFY>{out}) : go(RowForm<PLACE>{out});
 }
 
 }  // namespace dllm

@@ -113,6 +113,8 @@ struct IdentityLists {
 };
 void launch_vverify(const Launch& L, int dtype, Partials part, void* Vc_layer, float* sim, Geo g, int dkv,
                     int metric = 0, int write_v = 1, const IdentityLists* lists = nullptr);
+// The scores of rows whose sums over 128 columns each a projection has left (RowOut::verify).
+void launch_verify_merge(const Launch& L, const float4* sums, float* sim, int rows, int n_tiles, int metric);
 // The same test on K (ablation of Sec. 4.3): slab sum of the K projection of all
 // response rows, RoPE, score against the cached (post-RoPE) K, whole-K overwrite.
 void launch_kverify(const Launch& L, int dtype, Partials part, void* Kc_layer, float* sim, const float* rope_tab, Geo g,
@@ -217,6 +219,8 @@ struct RowOut {
   OutRows rows{};
   float* slab = nullptr;           // qkv == 0: rows m < slab_rows as they are, fp32, here instead
   int slab_rows = 0;
+  float4* verify = nullptr;        // qkv == 0: V-verify against the rows' old values, [M][ceil(N / 128)] sums per tile
+  int metric = 0, keep_rows = 0;   // as launch_vverify's; keep_rows: the cache rows stay as they are
   __nv_bfloat16 *q = nullptr, *k = nullptr, *v = nullptr;
   int v_from = 0;                  // rows m from which on V is stored (those before it have theirs)
   int q_by_slot = 0;               // rows of q sequence by sequence (b * n + position) instead of row m
