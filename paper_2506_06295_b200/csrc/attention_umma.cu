@@ -270,7 +270,7 @@ __global__ void __launch_bounds__((UaSmem<HD, TILES>::THREADS), 3 - TILES)
       // alone issues the first three, in order (a commit covers what its thread issued before): group 1, through with tile
       // 1, knows S(0) complete when it waits for S(3), group 0 after tile 2 S(1).  S(2) precedes S(3) in issuer 0; from
       // tile 6 on S(t - 3) precedes the product of tile t - 4 in the same issuer, which the group has waited for.
-      const int i = warp - SM::MMA_WARP;
+      const int i = warp - 8;   // two row tiles' worth of warps: the MMA warps are 8 and 9
       for (int t = 0; t < 3 && ok && i == 0; ++t) {
         ok = tile_ready(t);
         if (ok) issue_s(SM::KPAR_S_COL + (uint32_t)(t * UA_KEYS), SM::Q_COL, t, t);
