@@ -771,15 +771,13 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
         // selected, rotated and placed above
       } else if (qk_whole || identity) {
         ua = u;
-      } else if (s->R <= 1024 && (long)Ma * s->R <= 64L * 1024) {
-        // few active rows: every CTA of the gather repeats the selection rather than wait for a launch
-        ProfScope ps(s, DLLM_PROF_SELECT, (double)Ma * d * 2.0 * es + (double)BR * 4.0, 0.0, stream);
-        launch_select_gather(L, dt, sim, forced, mode, ksel, sel, act, inv, u, s->wsp<uint8_t>(s->ws.ua), g, rp);
       } else {
         ProfScope ps(s, DLLM_PROF_SELECT, (double)Ma * d * 2.0 * es + (double)BR * 4.0, 0.0, stream);
-        cudaError_t se = launch_select(L, sim, forced, mode, ksel, sel, s->R, act, inv, g, rp);
+        // u is the last layer's tail's; the launch before this one is V-verify (or a product behind it), unless the scores were
+        // given
+        cudaError_t se = launch_select_gather(L, dt, sim, forced, mode, ksel, sel, act, inv, u, s->wsp<uint8_t>(s->ws.ua), g, rp,
+                                              s->sel_strategy != DLLM_SELECT_RANDOM && adaptive);
         if (se != cudaSuccess) return fail(&s->err, DLLM_CUDA_ERROR, "selection: %s", cudaGetErrorString(se));
-        launch_gather_rows(L, dt, u, act, s->wsp<uint8_t>(s->ws.ua), Ma, d);
       }
       if (v_for_active) {
         const RowOut o = rows_into(v_rows, dkv, act, 0);
@@ -1707,7 +1705,7 @@ dllm_status dllm_vverify_select(const void* d_vnew, void* d_vcache, float* d_sim
   if (width % 8 || R > 8192) return fail(nullptr, DLLM_UNSUPPORTED, "width must be a multiple of 8 and R <= 8192");
   Launch L{(cudaStream_t)stream, kernel_status_word(), nullptr};
   launch_vverify_rows(L, dtype, d_vnew, d_vcache, d_sim, B * R, width);
-  if (k > 0) CU_TRY(nullptr, launch_select(L, d_sim, nullptr, 1, k, d_idx, k, nullptr, nullptr, Geo{B, 0, R, R, width}, 0));
+  if (k > 0) CU_TRY(nullptr, launch_select(L, d_sim, k, d_idx, B, R));
   CU_TRY(nullptr, cudaGetLastError());
   return DLLM_OK;
 }

@@ -518,77 +518,6 @@ __device__ __forceinline__ unsigned long long select_key(float s, int j) {
   const long long q = (s == s) ? (long long)qf + (1ll << 31) : 0ll;
   return ((unsigned long long)q << 32) | (unsigned)j;
 }
-// Bottom-k selection of sequence b by the whole CTA (R <= 1024: R^2 comparisons out of shared memory, 13 R + 16
-// bytes at `keys`).  Fills slot[j] = position of response row j among the selected rows, or -1; with `write` the
-// CTA also writes the index list, the active list (np prompt rows first) and its inverse.
-// mode 0: every row; 1: the ksel lowest scores (Sec. 3.2.2); 2: the forced list.  Ends with a barrier.
-__device__ __forceinline__ int32_t* select_sequence(unsigned long long* keys, const float* __restrict__ sim,
-                                                    const int32_t* __restrict__ forced, int mode, int ksel,
-                                                    int32_t* __restrict__ sel, int32_t* __restrict__ act,
-                                                    int32_t* __restrict__ inv, const Geo& g, int np, int b, bool write) {
-  const int R = g.R;
-  int32_t* slot = reinterpret_cast<int32_t*>(keys + R);
-  uint32_t* words = reinterpret_cast<uint32_t*>(slot + R);  // one ballot word per 32 rows
-  const int a_seq = np + ksel;
-  if (mode == 0) {
-    for (int j = threadIdx.x; j < R; j += blockDim.x) slot[j] = j;
-  } else if (mode == 2) {
-    for (int j = threadIdx.x; j < R; j += blockDim.x) slot[j] = -1;
-    __syncthreads();
-    for (int r = threadIdx.x; r < ksel; r += blockDim.x) slot[forced[(size_t)b * R + r]] = r;
-  } else {
-    for (int j = threadIdx.x; j < R; j += blockDim.x) {
-      keys[j] = select_key(__ldcg(sim + (size_t)b * R + j), j);
-    }
-    __syncthreads();
-    // rank of every key (two keys per shared-memory load); a row is selected iff its rank is below ksel
-    const int Rw = (R + 31) & ~31;
-    for (int j = threadIdx.x; j < Rw; j += blockDim.x) {
-      bool f = false;
-      if (j < R) {
-        const unsigned long long kj = keys[j];
-        int rank = 0;
-#pragma unroll 4
-        for (int i = 0; i + 1 < R; i += 2) {
-          const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(keys + i);
-          rank += (kk.x < kj) + (kk.y < kj);
-        }
-        if (R & 1) rank += (keys[R - 1] < kj);
-        f = rank < ksel;
-      }
-      const unsigned bal = __ballot_sync(0xffffffffu, f);
-      if ((threadIdx.x & 31) == 0) words[j >> 5] = bal;
-    }
-    __syncthreads();
-    for (int j = threadIdx.x; j < R; j += blockDim.x) {
-      const unsigned wj = words[j >> 5];
-      int r = -1;
-      if ((wj >> (j & 31)) & 1u) {
-        r = __popc(wj & ((1u << (j & 31)) - 1u));
-        for (int w = 0; w < (j >> 5); ++w) r += __popc(words[w]);
-      }
-      slot[j] = r;
-    }
-  }
-  __syncthreads();
-  if (write) {
-    for (int j = threadIdx.x; j < R; j += blockDim.x) {
-      const int r = slot[j];
-      inv[(size_t)b * R + j] = r >= 0 ? b * a_seq + np + r : -1;
-      if (r >= 0) {
-        sel[(size_t)b * R + r] = j;
-        act[(size_t)b * a_seq + np + r] = b * R + j;
-      }
-    }
-    for (int i = threadIdx.x; i < np; i += blockDim.x) {
-      act[(size_t)b * a_seq + i] = g.B * R + b * g.P + i;
-      inv[(size_t)g.B * R + (size_t)b * g.P + i] = b * a_seq + i;
-    }
-  }
-  __syncthreads();
-  return slot;
-}
-
 // ------------------------------------------------------------------ V-verify (Eq. 6) + V overwrite
 // metric 0: cosine (Eq. 6); 1: negated Euclidean distance (Sec. A.6), so that the
 // least similar rows have the lowest score either way.  write_v 0: the cache is
@@ -789,53 +718,17 @@ void launch_vverify_rows(const Launch& L, int dtype, const void* vnew, void* vca
 }
 
 // ------------------------------------------------------------------ bottom-k selection
-// One block per sequence.  Keys are unique (the index is part of the key), so
-// the rank of a key among all R keys is its position in sorted order; a row is
-// selected iff rank < k.  R^2 comparisons out of shared memory: R <= 8192.
-__global__ void select_kernel(const float* __restrict__ sim, const int32_t* __restrict__ forced, int mode, int ksel,
-                              int32_t* __restrict__ sel, int sel_stride, int32_t* __restrict__ act,
-                              int32_t* __restrict__ inv, Geo g, int refresh_prompt) {
+constexpr int SELECT_MAX_R = 8192;
+// The selected rows in ascending order (the kernel-level entry point).  One block per sequence.  Keys are unique (the index is
+// part of the key), so the rank of a key among all R keys is its position in sorted order; a row is selected iff rank < k.
+// R^2 comparisons out of shared memory: R <= 8192.
+__global__ void select_kernel(const float* __restrict__ sim, int ksel, int32_t* __restrict__ sel, int R) {
   pdl_wait();
   pdl_trigger();
   extern __shared__ unsigned long long keys[];  // R keys, then R flags (as bytes)
-  unsigned char* flag = reinterpret_cast<unsigned char*>(keys + g.R);
+  unsigned char* flag = reinterpret_cast<unsigned char*>(keys + R);
   const int b = blockIdx.x;
-  const int R = g.R;
-  const int a_seq = (refresh_prompt ? g.P : 0) + ksel;
-  int32_t* act_b = act ? act + (size_t)b * a_seq : nullptr;
-  int32_t* sel_b = sel + (size_t)b * sel_stride;
-  const int np = refresh_prompt ? g.P : 0;
-  if (refresh_prompt && act)
-    for (int i = threadIdx.x; i < g.P; i += blockDim.x) {
-      act_b[i] = g.B * R + b * g.P + i;
-      if (inv) inv[(size_t)g.B * R + (size_t)b * g.P + i] = b * a_seq + i;
-    }
-  int32_t* act_r = act ? act_b + np : nullptr;
-  if (mode == 0) {
-    for (int j = threadIdx.x; j < R; j += blockDim.x) {
-      sel_b[j] = j;
-      if (act_r) act_r[j] = b * R + j;
-      if (inv) inv[(size_t)b * R + j] = b * a_seq + np + j;
-    }
-    return;
-  }
-  if (mode == 2) {
-    if (inv) {
-      for (int j = threadIdx.x; j < R; j += blockDim.x) inv[(size_t)b * R + j] = -1;
-      __syncthreads();
-    }
-    for (int r = threadIdx.x; r < ksel; r += blockDim.x) {
-      const int j = forced[(size_t)b * R + r];
-      sel_b[r] = j;
-      if (act_r) act_r[r] = b * R + j;
-      if (inv) inv[(size_t)b * R + j] = b * a_seq + np + r;
-    }
-    return;
-  }
-  for (int j = threadIdx.x; j < R; j += blockDim.x) {
-    keys[j] = select_key(sim[(size_t)b * R + j], j);
-    flag[j] = 0;
-  }
+  for (int j = threadIdx.x; j < R; j += blockDim.x) keys[j] = select_key(sim[(size_t)b * R + j], j);
   __syncthreads();
   for (int j = threadIdx.x; j < R; j += blockDim.x) {
     const unsigned long long kj = keys[j];
@@ -845,52 +738,26 @@ __global__ void select_kernel(const float* __restrict__ sim, const int32_t* __re
   }
   __syncthreads();
   for (int j = threadIdx.x; j < R; j += blockDim.x) {
-    if (!flag[j]) {
-      if (inv) inv[(size_t)b * R + j] = -1;
-      continue;
-    }
+    if (!flag[j]) continue;
     int r = 0;
     for (int i = 0; i < j; ++i) r += flag[i];
-    sel_b[r] = j;
-    if (act_r) act_r[r] = b * R + j;
-    if (inv) inv[(size_t)b * R + j] = b * a_seq + np + r;
+    sel[(size_t)b * ksel + r] = j;
   }
 }
 
-cudaError_t launch_select(const Launch& L, const float* sim, const int32_t* forced, int mode, int ksel, int32_t* sel,
-                          int sel_stride, int32_t* act, int32_t* inv, Geo g, int refresh_prompt) {
+cudaError_t launch_select(const Launch& L, const float* sim, int ksel, int32_t* sel, int B, int R) {
   // 9 bytes per response row: beyond 48 KB (R > 5459) the kernel needs the opt-in for large dynamic shared memory
-  constexpr int MAX_R = 8192;
-  if (g.R > MAX_R) return cudaErrorInvalidValue;
+  if (R > SELECT_MAX_R) return cudaErrorInvalidValue;
   static DeviceOnce once;
   cudaError_t e = once.run([] {
-    return cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_R * 9 + 16);
+    return cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SELECT_MAX_R * 9 + 16);
   });
   if (e != cudaSuccess) return e;
-  const size_t smem = (size_t)g.R * 9 + 16;
   // one key per thread up to 1024 response rows (the rank of a key costs R comparisons of its thread)
-  const int threads = g.R <= 256 ? 256 : g.R >= 1024 ? 1024 : (g.R + 31) / 32 * 32;
-  e = launch_k(L, select_kernel, dim3(g.B), dim3(threads), smem, sim, forced, mode, ksel, sel, sel_stride, act, inv, g,
-               refresh_prompt);
+  const int threads = R <= 256 ? 256 : R >= 1024 ? 1024 : (R + 31) / 32 * 32;
+  e = launch_k(L, select_kernel, dim3(B), dim3(threads), (size_t)R * 9 + 16, sim, ksel, sel, R);
   L.count();
   return e;
-}
-
-// ------------------------------------------------------------------ gather
-template <typename T>
-__global__ void gather_rows_kernel(const T* __restrict__ src, const int32_t* __restrict__ act, T* __restrict__ dst,
-                                   int d) {
-  pdl_wait();
-  pdl_trigger();
-  const size_t r = blockIdx.x;
-  copy_row16(reinterpret_cast<const uint4*>(src + (size_t)act[r] * d), reinterpret_cast<uint4*>(dst + r * d),
-             d * (int)sizeof(T) / 16);
-}
-
-void launch_gather_rows(const Launch& L, int dtype, const void* src, const int32_t* act, void* dst, int rows, int d) {
-  if (rows <= 0) return;
-  DLLM_DISPATCH(dtype, (launch_k(L, gather_rows_kernel<T>, dim3(rows), dim3(128), 0, (const T*)src, act, (T*)dst, d)));
-  L.count();
 }
 
 // ------------------------------------------------------------------ RoPE + K scatter
@@ -1478,94 +1345,97 @@ void launch_tail(const Launch& L, int dtype, Partials part, const int32_t* inv, 
   L.count();
 }
 
-// ------------------------------------------------------------------ selection + gather in one launch
-// grid (a_seq, B): CTA (i, b) produces row i of sequence b's active list and
-// copies that row of u into ua.  Rows below the prompt length (on a prompt
-// refresh) are the prompt rows; the others are the selected response rows, for
-// which every CTA repeats the bottom-k selection of its sequence instead of
-// waiting for another launch.  CTA (0, b) writes the index list, the active
-// list and its inverse.
+// ------------------------------------------------------------------ selection + gather
+// One CTA per carried row: a response row is selected iff fewer than ksel rows of its sequence have a lower key, and that
+// count is its place among them (the order of the active rows is free: every row's result is independent of its neighbours);
+// prompt rows come first.  An active row copies itself.  R comparisons per row spread over the chip, where every gather CTA
+// ranked all rows against all, or one CTA per sequence did ahead of a gather launch (partial steps of eight layers of the LLaDA-8B
+// shape: 300 rows 1127 -> 1035 us, 400 rows 1255 -> 1176, 2 x 256 rows 1359 -> 1314; 16 x 512 rows even, 21 us in one launch
+// for 20 in two).
+// `early`: u is older than the launch before this one and its rows are few: the row travels while the scores are made.
+constexpr int SG_THREADS = 128, SG_VEC = 4;
 template <typename T>
-__global__ void select_gather_kernel(const float* __restrict__ sim, const int32_t* __restrict__ forced, int mode,
-                                     int ksel, int32_t* __restrict__ sel, int32_t* __restrict__ act,
-                                     int32_t* __restrict__ inv, const T* __restrict__ u, T* __restrict__ ua, Geo g,
-                                     int refresh_prompt) {
+__global__ void __launch_bounds__(SG_THREADS) select_gather_kernel(const float* __restrict__ sim, const int32_t* __restrict__ forced,
+                                                                   int mode, int ksel, int32_t* __restrict__ sel,
+                                                                   int32_t* __restrict__ act, int32_t* __restrict__ inv,
+                                                                   const T* __restrict__ u, T* __restrict__ ua, Geo g, int np,
+                                                                   bool early) {
+  __shared__ int slot_s;
+  const int c = blockIdx.x, R = g.R, BR = g.B * R, a_seq = np + ksel, nvec = g.d * (int)sizeof(T) / 16;
+  const uint4* const src = reinterpret_cast<const uint4*>(u + (size_t)c * g.d);
+  uint4 row[SG_VEC];
+  if (early)   // (a row fits the registers)
+#pragma unroll
+    for (int k = 0; k < SG_VEC; ++k)
+      if (k * SG_THREADS + (int)threadIdx.x < nvec) row[k] = __ldcg(src + k * SG_THREADS + threadIdx.x);
   pdl_wait();
   pdl_trigger();
-  extern __shared__ unsigned long long keys[];  // R keys, R slots (int), R / 8 bytes of ballot words
-  const int R = g.R, b = blockIdx.y, ridx = blockIdx.x;
-  __shared__ int my_j;
-  const int np = refresh_prompt ? g.P : 0;
-  const int a_seq = np + ksel;
-  const bool leader = ridx == 0;
-  if (mode == 1 && R <= (int)blockDim.x && (ridx >= np || leader)) {
-    // One key per thread (the usual case, R <= 256): key -> shared memory, rank against all keys, one ballot
-    // word per warp, position among the selected rows from the ballot words: three barriers in all.
-    uint32_t* words = reinterpret_cast<uint32_t*>(keys + R);
-    const int j = threadIdx.x;
-    unsigned long long kj = ~0ull;
-    if (j < R) {
-      const float s = __ldcg(sim + (size_t)b * R + j);
-      const float qf = fminf(fmaxf(rintf(s * 1048576.0f), -2147483520.0f), 2147483520.0f);
-      const long long q = (s == s) ? (long long)qf + (1ll << 31) : 0ll;
-      kj = ((unsigned long long)q << 32) | (unsigned)j;
-      keys[j] = kj;
-    }
-    __syncthreads();
-    int rank = 0;
-    if (j < R) {
-#pragma unroll 8
-      for (int i = 0; i + 1 < R; i += 2) {
-        const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(keys + i);
-        rank += (kk.x < kj) + (kk.y < kj);
-      }
-      if (R & 1) rank += (keys[R - 1] < kj);
-    }
-    const bool f = j < R && rank < ksel;
-    const unsigned bal = __ballot_sync(0xffffffffu, f);
-    if ((j & 31) == 0) words[j >> 5] = bal;
-    __syncthreads();
-    int r = -1;
-    if (f) {
-      r = __popc(bal & ((1u << (j & 31)) - 1u));
-      for (int w = 0; w < (j >> 5); ++w) r += __popc(words[w]);
-      if (r == ridx - np) my_j = j;
-    }
-    if (leader) {
-      if (j < R) {
-        inv[(size_t)b * R + j] = r >= 0 ? b * a_seq + np + r : -1;
-        if (r >= 0) {
-          sel[(size_t)b * R + r] = j;
-          act[(size_t)b * a_seq + np + r] = b * R + j;
+  int b, slot;   // sequence, and the row's place among its active rows
+  if (c >= BR) {
+    b = (c - BR) / g.P;
+    slot = c - BR - b * g.P;
+  } else {
+    b = c / R;
+    const int j = c - b * R;
+    slot = -1;
+    if (mode == 0) {
+      slot = j;
+    } else if (mode == 2) {
+      if (threadIdx.x == 0) slot_s = -1;
+      __syncthreads();
+      for (int r = threadIdx.x; r < ksel; r += SG_THREADS)
+        if (forced[(size_t)b * R + r] == j) slot_s = r;
+      __syncthreads();
+      slot = slot_s;
+    } else {
+      const unsigned long long own = select_key(__ldcg(sim + c), j);
+      int rank = 0;
+      for (int i0 = 0; i0 < R; i0 += 4 * SG_THREADS) {
+        int lower = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int i = i0 + k * SG_THREADS + threadIdx.x;
+          if (i0 + k * SG_THREADS < R) lower += i < R && select_key(__ldcg(sim + (size_t)b * R + min(i, R - 1)), i) < own;
         }
+        rank += lower;
       }
-      for (int i = threadIdx.x; i < np; i += blockDim.x) {
-        act[(size_t)b * a_seq + i] = g.B * R + b * g.P + i;
-        inv[(size_t)g.B * R + (size_t)b * g.P + i] = b * a_seq + i;
-      }
+      rank = __reduce_add_sync(0xffffffffu, rank);
+      __shared__ int ranks[SG_THREADS / 32];
+      if ((threadIdx.x & 31) == 0) ranks[threadIdx.x >> 5] = rank;
+      __syncthreads();
+      rank = 0;
+#pragma unroll
+      for (int w = 0; w < SG_THREADS / 32; ++w) rank += ranks[w];
+      if (rank < ksel) slot = rank;
     }
-    __syncthreads();
-  } else if (ridx >= np || leader) {
-    const int32_t* slot = select_sequence(keys, sim, forced, mode, ksel, sel, act, inv, g, np, b, leader);
-    if (ridx >= np)
-      for (int j = threadIdx.x; j < R; j += blockDim.x)
-        if (slot[j] == ridx - np) my_j = j;
-    __syncthreads();
+    if (threadIdx.x == 0 && slot >= 0) sel[(size_t)b * R + slot] = j;
+    if (slot >= 0) slot += np;
   }
-  const int c = ridx < np ? g.B * R + b * g.P + ridx : b * R + my_j;
-  copy_row16(reinterpret_cast<const uint4*>(u + (size_t)c * g.d),
-             reinterpret_cast<uint4*>(ua + ((size_t)b * a_seq + ridx) * g.d), g.d * (int)sizeof(T) / 16);
+  if (threadIdx.x == 0) {
+    inv[c] = slot >= 0 ? b * a_seq + slot : -1;
+    if (slot >= 0) act[(size_t)b * a_seq + slot] = c;
+  }
+  if (slot < 0) return;
+  uint4* const dst = reinterpret_cast<uint4*>(ua + ((size_t)b * a_seq + slot) * g.d);
+  if (early) {
+#pragma unroll
+    for (int k = 0; k < SG_VEC; ++k)
+      if (k * SG_THREADS + (int)threadIdx.x < nvec) dst[k * SG_THREADS + threadIdx.x] = row[k];
+  } else {
+    copy_row16(src, dst, nvec);
+  }
 }
-
-void launch_select_gather(const Launch& L, int dtype, const float* sim, const int32_t* forced, int mode, int ksel,
-                          int32_t* sel, int32_t* act, int32_t* inv, const void* u, void* ua, Geo g,
-                          int refresh_prompt) {
-  const int a_seq = (refresh_prompt ? g.P : 0) + ksel;
-  if (a_seq <= 0) return;
-  const size_t smem = (size_t)g.R * 13 + 16;
-  DLLM_DISPATCH(dtype, (launch_k(L, select_gather_kernel<T>, dim3(a_seq, g.B), dim3(256), smem, sim, forced, mode, ksel,
-                                 sel, act, inv, (const T*)u, (T*)ua, g, refresh_prompt)));
+cudaError_t launch_select_gather(const Launch& L, int dtype, const float* sim, const int32_t* forced, int mode, int ksel,
+                                 int32_t* sel, int32_t* act, int32_t* inv, const void* u, void* ua, Geo g,
+                                 int refresh_prompt, bool u_static) {
+  if (g.R > SELECT_MAX_R) return cudaErrorInvalidValue;
+  const int np = refresh_prompt ? g.P : 0, rows = g.B * (g.R + np);
+  // few rows: all CTAs are resident before the launch ahead ends, and the rows that nobody selects cost nothing
+  const bool early = u_static && rows <= 1024 && g.d * (dtype == 0 ? 4 : 2) <= SG_VEC * SG_THREADS * 16;
+  DLLM_DISPATCH(dtype, (launch_k(L, select_gather_kernel<T>, dim3(rows), dim3(SG_THREADS), 0, sim, forced, mode, ksel, sel, act,
+                                 inv, (const T*)u, (T*)ua, g, np, early)));
   L.count();
+  return cudaSuccess;
 }
 
 // ------------------------------------------------------------------ greedy estimate + confidence (Eq. 4)

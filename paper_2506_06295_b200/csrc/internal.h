@@ -119,16 +119,15 @@ void launch_verify_merge(const Launch& L, const float4* sums, float* sim, int ro
 // response rows, RoPE, score against the cached (post-RoPE) K, whole-K overwrite.
 void launch_kverify(const Launch& L, int dtype, Partials part, void* Kc_layer, float* sim, const float* rope_tab, Geo g,
                     int Hkv, int hd, int metric);
-// Bottom-k selection per sequence + active-row list.  mode 0: all R rows,
-// 1: bottom-k by (round(sim*2^20), index), 2: forced list.
-// inv (may be null): for every carried row its position in the active list, or -1.
-cudaError_t launch_select(const Launch& L, const float* sim, const int32_t* forced, int mode, int ksel, int32_t* sel,
-                          int sel_stride, int32_t* act, int32_t* inv, Geo g, int refresh_prompt);
-// Selection, active list, inverse list and the gather of the active rows of u
-// into ua in one launch (R <= 1024; sel rows have stride R).
-void launch_select_gather(const Launch& L, int dtype, const float* sim, const int32_t* forced, int mode, int ksel,
-                          int32_t* sel, int32_t* act, int32_t* inv, const void* u, void* ua, Geo g,
-                          int refresh_prompt);
+// Bottom-k selection per sequence by (round(sim*2^20), index): sel[b, 0 .. ksel), ascending.
+cudaError_t launch_select(const Launch& L, const float* sim, int ksel, int32_t* sel, int B, int R);
+// (launch_select_gather) mode 0: all R rows, 1: bottom-k, 2: forced list.
+// inv: for every carried row its position in the active list, or -1.
+// Selection, active list, inverse list and the gather of the active rows of u into ua in one launch (sel rows have stride R;
+// the selected rows in the order of their scores).  u_static: u is older than the launch before this one.
+cudaError_t launch_select_gather(const Launch& L, int dtype, const float* sim, const int32_t* forced, int mode, int ksel,
+                                 int32_t* sel, int32_t* act, int32_t* inv, const void* u, void* ua, Geo g,
+                                 int refresh_prompt, bool u_static);
 // x[c] = E[token(c)], u[c] = rmsnorm(x[c]) * gain for carried rows c0 <= c < c1; act / inv: lists of a step that
 // recomputes all of them (see the kernel).
 void launch_embed_norm(const Launch& L, int dtype, const void* E, const int32_t* tokens, float* x, const float* gain,
@@ -139,7 +138,6 @@ void launch_embed_norm(const Launch& L, int dtype, const void* E, const int32_t*
 void launch_tail(const Launch& L, int dtype, Partials part, const int32_t* inv, float* x, OutRows Ac_layer,
                  OutRows Fc_layer, const float* gain, void* u, Geo g, int c0, int c1, float eps);
 // (launch_tail and launch_oproj_epilogue: part.p == nullptr with active rows: the projection has written their rows.)
-void launch_gather_rows(const Launch& L, int dtype, const void* src, const int32_t* act, void* dst, int rows, int d);
 // RoPE on Q and K of the active rows; Q -> qbuf [Ma, dq]; K -> K cache rows.  Vc_layer: `part` is the [Q | K | V] product of
 // all carried rows in their order (act is not read); V -> cache rows too, q_by_slot: Q rows sequence by sequence.
 void launch_qk_rope(const Launch& L, int dtype, Partials part, const int32_t* act, const float* rope_tab, void* qbuf,
