@@ -149,15 +149,17 @@ struct Workspace {
 // Sessions whose Q, K and V of ALL response rows come from one product, in adaptive steps too: it streams the weights hardly
 // slower than the products of V (all rows) and of Q / K (the selected ones) one after the other, selection needs no launch and
 // no gather in front of it, and in a refresh V-verify and RoPE launches go.  Up to the arithmetic that takes as long as
-// streaming its weights does in the largest model (16 us): 256 rows of the LLaDA-8B shape, 780 of Dream-7B, all of a small
-// one.  B200, us, separate -> one: LLaDA-8B partial / refresh / full step, 256 rows 4187 / 5580 / 11205 -> 4194 / 5296 /
-// 10652, 128 rows partial 3699 -> 3654, 32 rows 3848 -> 3741; 300 rows (eight layers) 1111 / 1474 -> 1253 / 1528, beyond the
-// line; Dream-7B partial 256 rows 4168 -> 4053, (eight layers) 400 rows 1251 -> 1194, 512 rows 1342 -> 1293; 320-wide model
-// with 500 rows, full step 120 -> 93.  (1024 rows and more belong to the streaming row kernels.)
+// streaming its weights does in the largest model (16 us: 256 rows of the LLaDA-8B shape) and to 512 rows, where a few selected
+// rows of narrow heads begin to cost less than all of them; small weights up to 1023.  B200, us, separate -> one: LLaDA-8B
+// partial / refresh / full step, 256 rows 4187 / 5580 / 11205 -> 4194 / 5296 / 10652, 128 rows partial 3699 -> 3654, 32 rows
+// 3848 -> 3741; 300 rows (eight layers) 1111 / 1474 -> 1253 / 1528, beyond the line; Dream-7B partial 256 rows 4168 -> 4053,
+// (eight layers) 400 rows 1251 -> 1194, 512 rows 1342 -> 1293, 715 rows (all layers, 143 selected) 5063 -> 5172, beyond; 320-wide
+// model with 500 rows, full step 120 -> 93.  (1024 rows and more belong to the streaming row kernels.)
 constexpr double QKV_WORK = 256.0 * 12288 * 4096;
 bool qkv_in_one(const dllm_config& c, int B, int R) {
   const double rows = (double)B * R, width = (double)(c.n_heads + 2 * c.n_kv_heads) * c.head_dim;
-  return c.dtype == DLLM_BF16 && rows < 1024 && rows * width * c.d_model <= QKV_WORK;
+  return c.dtype == DLLM_BF16 && rows * width * c.d_model <= QKV_WORK &&
+         (rows <= 512 || (rows < 1024 && width * c.d_model < 1 << 21));
 }
 // Whether a full step of such a session takes Q, K and V of all `rows` carried rows from one product with the response rows'
 // splits: where its own plan has as many, or where their slabs stay small beside the launches they replace (V, V-verify,
