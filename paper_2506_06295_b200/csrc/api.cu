@@ -783,7 +783,8 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
       }
       if (v_for_active) {
         const RowOut o = rows_into(v_rows, dkv, act, 0);
-        if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, ua, Wv, Ma, dkv, d, &part, nullptr, &fused, -1, false, &o, qk_split)) != DLLM_OK)
+        if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, ua, Wv, Ma, dkv, d, &part, nullptr, &fused, -1, false, &o,
+                           in_one && verify_v ? v_split : qk_split)) != DLLM_OK)
           return st;
         if (!fused) {
           ProfScope ps(s, DLLM_PROF_SCATTER, (double)Ma * dkv * (4.0 + es), 0.0, stream);

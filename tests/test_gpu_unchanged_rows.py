@@ -52,3 +52,27 @@ def test_unchanged_rows_score_exactly(dllm, cfg, B, P, R, metric):
             assert (idx == np.arange(k)).all(), f"after {kind}, layer {l}: {np.setdiff1d(idx, np.arange(k))}"
             assert (sim[:, k:] == exact).all(), f"after {kind}, layer {l}: {np.abs(sim[:, k:] - exact).max()}"
             assert np.array_equal(ses.get_cache(l, dllm.CACHE_V)[:, P + k:], before[l][:, k:]), f"after {kind}, layer {l}"
+
+
+@pytest.mark.parametrize("metric", ["cosine", "l2"])
+@pytest.mark.parametrize("cfg,B,P,R,rho", [(GROUPED, 1, 256, 256, 0.5), (GROUPED, 2, 90, 70, 0.3), (WIDE, 1, 130, 200, 0.25)],
+                         ids=["grouped", "two sequences", "wide"])
+def test_rows_written_one_by_one_score_exactly(dllm, cfg, B, P, R, rho, metric):
+    """The same where only the selected rows' V is written (another product in a mixed step): in the first layer, whose V
+    depends on the tokens alone, every row keeps its bits."""
+    rng = np.random.default_rng(5)
+    ses = dllm.Session(dllm.Model(cfg, "cuda:0").random_init_on_device(3), B, P, R)
+    ses.set_selection("v_verify", metric=metric, v_update="selected")
+    ses.set_prompt(rng.integers(0, cfg.vocab - 1, size=(B, P), dtype=np.int32))
+    ses.set_response_tokens(rng.integers(0, cfg.vocab - 1, size=(B, R), dtype=np.int32))
+    exact = 1.0 if metric == "cosine" else 0.0
+    ses.step_full()
+    before = ses.get_cache(0, dllm.CACHE_V)[:, P:]
+    for kind, (rp, rr) in (("refresh", (False, True)), ("mixed", (True, False)), ("partial", (False, False))):
+        ses.step_cached(rp, rr, rho)
+        assert np.array_equal(ses.get_cache(0, dllm.CACHE_V)[:, P:], before), kind
+        ses.step_cached(False, False, rho)
+        ses.sync()
+        _, sim = ses.selected(0)
+        assert (sim == exact).all(), f"after {kind}: {np.abs(sim - exact).max()}"
+        assert np.array_equal(ses.get_cache(0, dllm.CACHE_V)[:, P:], before), f"after {kind}"
