@@ -373,20 +373,23 @@ __global__ void __launch_bounds__(STREAM_THREADS, 1)
   }
 }
 
-// RoPE + K scatter, streaming: see qk_rope_kernel.  Stage = the projected [Q | K] row (fp32) of active row r.  A
-// consumer warp rotates a whole row: hd / 8 lanes cover the hd / 2 pairs of a head four at a time (element i with
-// i + hd / 2), so a warp takes 256 / hd heads per trip; the row's cos / sin values are read once.
+// RoPE + K scatter, streaming: see qk_rope_kernel.  Stage = the projected [Q | K] row (fp32) of active row r, or [Q | K | V]
+// of carried row r (Vc).  A consumer warp rotates a whole row: hd / 8 lanes cover the hd / 2 pairs of a head four at a time (element i with
+// i + hd / 2), so a warp takes 256 / hd heads per trip; the row's cos / sin values are read once.  (fp32 models of two layers,
+// refresh of 4 x 1024 rows, [Q | K | V] through the kernel below -> through this one: 256 wide 1082 -> 1058 us per layer, 512
+// wide 2222 -> 2184; of 1024 rows 512 wide 706 -> 689, 256 wide 278 -> 281.)
 template <typename T>
 __global__ void __launch_bounds__(STREAM_THREADS, 1)
     qk_rope_stream_kernel(const float* __restrict__ part, const int32_t* __restrict__ act,
-                          const float* __restrict__ rope_tab, T* __restrict__ qbuf, T* __restrict__ Kc, Geo g, int Ma,
-                          int H, int Hkv, int hd, int stages, int* __restrict__ status) {
+                          const float* __restrict__ rope_tab, T* __restrict__ qbuf, T* __restrict__ Kc,
+                          T* __restrict__ Vc, int q_by_slot, Geo g, int Ma, int H, int Hkv, int hd, int stages,
+                          int* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[STREAM_MAX_STAGES], empty_bar[STREAM_MAX_STAGES];
   __shared__ int meta[STREAM_MAX_STAGES];
   __shared__ int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int dq = H * hd, dkv = Hkv * hd, width = dq + dkv, half = hd >> 1;
+  const int heads = H + (Vc ? 2 : 1) * Hkv, dq = H * hd, dkv = Hkv * hd, width = heads * hd, half = hd >> 1;
   const uint32_t stage_bytes = (uint32_t)width * 4;
   const uint32_t base = (smem_u32(smem_raw) + 127u) & ~127u;
   uint8_t* base_gen = smem_raw + (base - smem_u32(smem_raw));
@@ -412,7 +415,7 @@ __global__ void __launch_bounds__(STREAM_THREADS, 1)
           ok = false;
           break;
         }
-        meta[s] = act[r];
+        meta[s] = Vc ? r : act[r];
         const uint32_t bar = smem_u32(&full_bar[s]);
         mbar_expect_tx(bar, stage_bytes);
         bulk_load_1d(base + s * stage_bytes, part + (size_t)r * width, stage_bytes, bar);
@@ -435,21 +438,23 @@ __global__ void __launch_bounds__(STREAM_THREADS, 1)
       const float4 cs = *reinterpret_cast<const float4*>(tab + i0);
       const float4 sn = *reinterpret_cast<const float4*>(tab + half + i0);
       const float cc[4] = {cs.x, cs.y, cs.z, cs.w}, ss[4] = {sn.x, sn.y, sn.z, sn.w};
-      T* qrow = qbuf + (size_t)r * dq;
-      T* krow = Kc + ((size_t)b * g.n + pos) * dkv;
-      for (int h0 = 0; h0 < H + Hkv; h0 += hpt) {
+      const size_t at = (size_t)b * g.n + pos;
+      T* qrow = qbuf + (q_by_slot ? at : (size_t)r) * dq;
+      T* krow = Kc + at * dkv;
+      for (int h0 = 0; h0 < heads; h0 += hpt) {
         const int head = h0 + hl;
-        if (head >= H + Hkv) break;          // the last trip may be partly empty
+        if (head >= heads) break;            // the last trip may be partly empty
         const float4 lo4 = *reinterpret_cast<const float4*>(row + head * hd + i0);
         const float4 hi4 = *reinterpret_cast<const float4*>(row + head * hd + half + i0);
         const float lo[4] = {lo4.x, lo4.y, lo4.z, lo4.w}, hi[4] = {hi4.x, hi4.y, hi4.z, hi4.w};
         float o_lo[4], o_hi[4];
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-          o_lo[t] = rope_lo(lo[t], hi[t], cc[t], ss[t]);
-          o_hi[t] = rope_hi(lo[t], hi[t], cc[t], ss[t]);
+          const bool rotate = head < H + Hkv;
+          o_lo[t] = rotate ? rope_lo(lo[t], hi[t], cc[t], ss[t]) : lo[t];
+          o_hi[t] = rotate ? rope_hi(lo[t], hi[t], cc[t], ss[t]) : hi[t];
         }
-        T* dst = head < H ? qrow + head * hd : krow + (head - H) * hd;
+        T* dst = head < H ? qrow + head * hd : head < H + Hkv ? krow + (head - H) * hd : Vc + at * dkv + (head - H - Hkv) * hd;
         store4<T>(dst + i0, o_lo);
         store4<T>(dst + i0 + half, o_hi);
       }
@@ -820,9 +825,10 @@ __global__ void qk_rope_kernel(Partials part, const int32_t* __restrict__ act, c
 void launch_qk_rope(const Launch& L, int dtype, Partials part, const int32_t* act, const float* rope_tab, void* qbuf,
                     void* Kc_layer, Geo g, int Ma, int H, int Hkv, int hd, void* Vc_layer, int q_by_slot) {
   if (Ma <= 0) return;
-  const size_t stage = (size_t)(H + Hkv) * hd * 4;
+  const int heads = H + (Vc_layer ? 2 : 1) * Hkv;
+  const size_t stage = (size_t)heads * hd * 4;
   // streaming form: unsplit slabs, a head size whose pairs a group of lanes covers exactly (a power of two, 32..256)
-  if (!Vc_layer && g.B * g.R >= STREAM_MIN_ROWS && part.S == 1 && hd >= 32 && hd <= 256 && (hd & (hd - 1)) == 0 &&
+  if (g.B * g.R >= STREAM_MIN_ROWS && part.S == 1 && hd >= 32 && hd <= 256 && (hd & (hd - 1)) == 0 &&
       stream_stages(stage) >= STREAM_CONSUMERS + 1) {
     const int stages = stream_stages(stage);
     const size_t smem = (size_t)stages * stage + 128;
@@ -834,12 +840,11 @@ void launch_qk_rope(const Launch& L, int dtype, Partials part, const int32_t* ac
       });
       if (e0 == cudaSuccess)
         launch_k(L, qk_rope_stream_kernel<T>, dim3(ctas), dim3(STREAM_THREADS), smem, part.p, act, rope_tab, (T*)qbuf,
-                 (T*)Kc_layer, g, Ma, H, Hkv, hd, stages, L.d_status);
+                 (T*)Kc_layer, (T*)Vc_layer, q_by_slot, g, Ma, H, Hkv, hd, stages, L.d_status);
     });
     L.count();
     return;
   }
-  const int heads = H + (Vc_layer ? 2 : 1) * Hkv;
   const long total = (long)Ma * heads * (hd >> 3);
   const long blocks1 = (total + 255) / 256;
   if (blocks1 > 2L * sm_count()) {   // two heads per thread: half the CTAs

@@ -15,6 +15,9 @@ WIDE = dataclasses.replace(synth.LLADA_8B, n_layers=2, d_ffn=1024, vocab=1024, m
 GROUPED = dataclasses.replace(synth.DREAM_7B, n_layers=2, d_ffn=1024, vocab=1024, mask_id=1023)
 ODD = synth.small_bf16_model()                 # widths that are no multiples of 128, small weights
 
+PLAIN = dataclasses.replace(synth.TINY, n_kv_heads=2)                    # plain ALUs
+PLAIN96 = dataclasses.replace(PLAIN, n_heads=3, n_kv_heads=3, head_dim=96)   # heads that the streaming RoPE does not take
+
 
 @pytest.fixture(scope="module")
 def dllm():
@@ -43,7 +46,8 @@ CASES = [(cfg, B, P, R, rho, variant) for cfg, B, P, R, rho, variant in [
     (WIDE, 1, 64, 257, 0.25, "v_verify"),                       # one row too many: separate products
     (GROUPED, 1, 256, 256, 0.5, "v_verify"), (GROUPED, 3, 60, 259, 0.5, "v_verify"), (GROUPED, 3, 50, 85, 0.2, "selected_v"), (GROUPED, 1, 1500, 100, 0.3, "v_verify"),
     (ODD, 2, 150, 72, 0.25, "v_verify"), (ODD, 1, 90, 1023, 0.25, "selected_v"), (ODD, 16, 20, 16, 1.0, "v_verify"), (ODD, 2, 150, 72, 0.25, "k_verify"),
-    (ODD, 2, 150, 72, 0.25, "random")]]
+    (ODD, 2, 150, 72, 0.25, "random"),
+    (PLAIN, 1, 60, 1030, 0.25, "v_verify"), (PLAIN, 3, 40, 350, 0.25, "v_verify"), (PLAIN96, 2, 40, 520, 0.25, "v_verify")]]
 
 
 @pytest.mark.parametrize("cfg,B,P,R,rho,variant", CASES,
