@@ -1,3 +1,4 @@
+import gc
 import os
 import sys
 
@@ -10,6 +11,13 @@ if ROOT not in sys.path:
 
 def pytest_configure(config):
     config.addinivalue_line("markers", "gpu: needs a CUDA device (B200); run with -m gpu")
+
+
+@pytest.fixture(autouse=True, scope="module")
+def collect_garbage():
+    """What a module's tests leave in reference cycles (tensors in a traceback's frames) goes before the next module's."""
+    yield
+    gc.collect()
 
 
 def pytest_collection_modifyitems(config, items):
