@@ -156,8 +156,10 @@ dllm_status dllm_step_full(dllm_session* s, void* stream);
  *   s_j = cos(V_new[j], V_cached[j]) (Eq. 6), the k_sel = floor(rho*R) rows with
  *   the lowest s_j are selected per sequence and per layer (ties: lower
  *   round(s*2^20) first, then lower index), the whole response V cache is
- *   overwritten, and Q/K/attention/O-proj/FFN run only for the selected rows
+ *   overwritten, and attention/O-proj/FFN run only for the selected rows
  *   over the full cached K/V; their K, AttnOut, FFNOut rows are scattered back.
+ *   Only the selected rows' Q and K are used; where one product for Q, K and V of
+ *   all rows takes no longer, those of the other rows are projected and dropped.
  *   rho in [0,1]; k_sel = 0 leaves all caches untouched.
  * Returns DLLM_BAD_STATE before the first full step. */
 dllm_status dllm_step_cached(dllm_session* s, int refresh_prompt, int refresh_response, float rho,

@@ -148,18 +148,35 @@ struct Workspace {
 
 // Sessions whose Q, K and V of ALL response rows come from one product, in adaptive steps too: it streams the weights hardly
 // slower than the products of V (all rows) and of Q / K (the selected ones) one after the other, selection needs no launch and
-// no gather in front of it, and in a refresh V-verify and RoPE launches go.  Up to the arithmetic that takes as long as
-// streaming its weights does in the largest model (16 us: 256 rows of the LLaDA-8B shape) and to 512 rows, where a few selected
-// rows of narrow heads begin to cost less than all of them; small weights up to 1023.  B200, us, separate -> one: LLaDA-8B
-// partial / refresh / full step, 256 rows 4187 / 5580 / 11205 -> 4194 / 5296 / 10652, 128 rows partial 3699 -> 3654, 32 rows
-// 3848 -> 3741; 300 rows (eight layers) 1111 / 1474 -> 1253 / 1528, beyond the line; Dream-7B partial 256 rows 4168 -> 4053,
-// (eight layers) 400 rows 1251 -> 1194, 512 rows 1342 -> 1293, 715 rows (all layers, 143 selected) 5063 -> 5172, beyond; 320-wide
-// model with 500 rows, full step 120 -> 93.  (1024 rows and more belong to the streaming row kernels.)
-constexpr double QKV_WORK = 256.0 * 12288 * 4096;
+// no gather in front of it, and in a refresh V-verify and RoPE launches go.
+//   - Small weights: as long as the streaming row kernels do not take the session (1024 rows).
+//   - Otherwise up to 256 rows, one activation tile: beyond, every weight tile crosses the L2 -> SM fabric twice for rows of
+//     which an adaptive step wants few.
+//   - Up to 128 rows the one-tile kernel streams the weights at any width.  Beyond, CTA pairs may be too few to: the product
+//     may take QKV_EXCESS_US longer than its weights, about what the launches that go take.
+// The number of selected rows is not in it: V has the splits of this product in every kind of step, and with them the separate
+// launches are slower at any ratio (3 % to 50 % selected, 88 shapes: 0.92 .. 1.04 of the one product's speed).
+// B200, us per layer of partial steps with 5 / 25 / 50 % selected, refresh; separate launches with splits of their own -> one
+// product:
+//   4096 wide, 32 heads       192 rows  112.3 / 116.2 / 133.1, 149 -> 111.4 / 115.4 / 129.2, 141   (1.8 us above its weights)
+//                             256 rows  116.6 / 121.3 / 144.8, 166 -> 117.2 / 122.9 / 144.6, 158   (5.6 us)
+//                             264 rows  117.2 / 134.0 / 153.6, 196 -> 128.1 / 147.0 / 162.1, 195   beyond
+//   5120 wide, 40 heads       256 rows  173.7 / 180.5 / 207.3, 238 -> 171.5 / 180.6 / 205.1, 225   (2.2 us)
+//   8192 wide, 64 heads on 8  144 rows  319.7 / 341.6 / 398, 415 -> 326.3 / 346.6 / 399, 411       (8.7 us) beyond
+//                             256 rows  332.5 / 357.0 / 430, 494 -> 348.3 / 368.2 / 436, 494       (16 us) beyond
+//   3584 wide, 28 heads on 4  256 rows  112.4 / 121.3 / 140.9, 158 -> 110.7 / 118.1 / 139.1, 152   (4.0 us)
+//                             400 rows of four sequences  120.7 / 140.8 / 162.0, 249 -> 122.7 / 143.6 / 159.9, 242   beyond
+//   4096 wide, 32 heads on 8  256 rows  111.8 / 119.1 / 138.8, 162 -> 111.8 / 117.8 / 137.3, 154   (4.7 us)
+//                             400 rows of four sequences  120.0 / 138.8 / 166.5, 249 -> 127.1 / 145.7 / 168.9, 242   beyond
+// (256 rows of 32 heads are where a partial step has stopped gaining and a refresh, every sixth to eighth step, still does.  Full
+// steps gain too: 2 to 7 % at 264 .. 320 rows of 32 heads.)  320-wide model with 500 rows, full step 120 -> 93 us.
+constexpr double QKV_EXCESS_US = 7.0, WEIGHT_BYTES_PER_US = 6.5e6;
 bool qkv_in_one(const dllm_config& c, int B, int R) {
-  const double rows = (double)B * R, width = (double)(c.n_heads + 2 * c.n_kv_heads) * c.head_dim;
-  return c.dtype == DLLM_BF16 && rows * width * c.d_model <= QKV_WORK &&
-         (rows <= 512 || (rows < 1024 && width * c.d_model < 1 << 21));
+  const long rows = (long)B * R, width = (long)(c.n_heads + 2 * c.n_kv_heads) * c.head_dim;
+  if (c.dtype != DLLM_BF16) return false;
+  if (rows <= 128 || (rows < 1024 && width * c.d_model < 1L << 21)) return true;
+  return rows <= 256 &&
+         gemm_pair_us((int)rows, (int)width, c.d_model) <= width * c.d_model * 2.0 / WEIGHT_BYTES_PER_US + QKV_EXCESS_US;
 }
 // Whether a full step of such a session takes Q, K and V of all `rows` carried rows from one product with the response rows'
 // splits: where its own plan has as many, or where their slabs stay small beside the launches they replace (V, V-verify,

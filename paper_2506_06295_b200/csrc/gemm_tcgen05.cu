@@ -561,7 +561,7 @@ Partials make_partials(const float* p, int M, int N, const GemmPlan& plan) {
 // slabs, 5.8 for SwiGLU, 16 for rotated and placed rows of a 256-row tile).  Measured with it, B200, us
 // (before -> now): 768 x 4096 x 12288 77 -> 63, 768 x 24576 x 4096 120 -> 110, 4096 x 24576 x 4096 614 -> 583, 4096 x
 // 4096 x 12288 362 -> 306, 24576 x 4096 x 4096 711 -> 646, 256 x 126464 x 4096 258 -> 221.
-static void plan_pair(int M, int N, int K, int max_split, int exact_split, int* bn, int* splits) {
+static double plan_pair(int M, int N, int K, int max_split, int exact_split, int* bn, int* splits) {
   const int pairs = sm_count() / 2, num_kb = (K + TILE_K - 1) / TILE_K;
   const long n_pairs = (N + 2 * TILE_W - 1) / (2 * TILE_W);
   double best = -1.0;
@@ -581,6 +581,12 @@ static void plan_pair(int M, int N, int K, int max_split, int exact_split, int* 
       }
     }
   }
+  return best;
+}
+
+double gemm_pair_us(int M, int N, int K) {
+  int bn, splits;
+  return plan_pair(M, N, K, 16, 0, &bn, &splits);
 }
 
 // Tile shape, ring depth and split-K factor, from sweeps on B200.  Up to 128 activation rows the product is bound by

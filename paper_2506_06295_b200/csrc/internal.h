@@ -197,6 +197,8 @@ struct GemmPlan {
 // plans with 256-row tiles, -1 the one-tile kernel with the splits of the automatic plan.
 GemmPlan plan_gemm_bf16(int M, int N, int K, int force_split = 0, int force_stages = 0, int force_bn = 0,
                         int force_pair = 0, int force_persistent = 0);
+// Estimated time of the CTA-pair kernel's plan for that product, us.
+double gemm_pair_us(int M, int N, int K);
 int gemm_plan_mode();  // what dllm_debug_gemm_plan set
 Partials make_partials(const float* p, int M, int N, const GemmPlan& plan);
 // Returns cudaSuccess or the failing error.  part must hold S*M*N floats.

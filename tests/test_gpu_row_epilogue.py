@@ -33,9 +33,9 @@ def dllm():
     dllm._check(dllm.lib.dllm_debug_gemm_plan(0))
 
 
-def steps(dllm, m, B, P, R, compact, variant, rho, plan, profiled=False):
+def steps(dllm, m, B, P, R, compact, variant, rho, plan, profiled=False, lists=False):
     """(launches, bytes of the O and down products if profiled, outputs) of a full, an adaptive, a refresh, a mixed and
-    another adaptive step."""
+    another adaptive step; lists: with what the steps selected."""
     dllm._check(dllm.lib.dllm_debug_gemm_plan(plan))
     cfg = m.cfg
     rng = np.random.default_rng(9)
@@ -56,6 +56,9 @@ def steps(dllm, m, B, P, R, compact, variant, rho, plan, profiled=False):
         nbytes = [ses.profile_read(dllm.PROF_CLASSES.index(c))["bytes"] for c in ("gemm_o", "gemm_down")]
         out.append((launches, nbytes, [ses.hidden(), ses.pred()[1]] + [ses.get_cache(l, w) for l in range(cfg.n_layers)
                                                                for w in range(4)]))
+        for l in range(cfg.n_layers if lists else 0):
+            idx, scores = ses.selected(l)
+            out[-1][2].extend([idx] if rr else [idx, scores])   # (scores mean something after an adaptive step)
     return out
 
 
