@@ -560,13 +560,6 @@ dllm_status run_gemm(dllm_session* s, const Launch& L, int cls, const void* A, c
   const bool whole = cls == DLLM_PROF_GEMM_HEAD || (swiglu_out && M > 128 && gu_interleaved(s->m->cfg));
   GemmPlan plan = tensor ? plan_gemm_bf16(M, N, K, whole ? 1 : -split) : GemmPlan{};
   if (weights_again) plan.w_stream = false;
-  // Weights whose rows lie a multiple of 8 KB apart, streamed by one-tile CTAs: all CTAs in step read the same few address
-  // bits of every row, and every other pair of tiles half a row ahead spreads them (B200, LLaDA-8B shape, adaptive steps of
-  // 64 / 32 / 3 rows 4212 -> 4188, 3663 -> 3613, 3733 -> 3690 us; with rows of 7 KB the same turn cost 1.5 %, on CTA pairs
-  // 2 %; other turns and four or eight starting points gave less).  Not for V and Q / K, whose sums are the same in every
-  // kind of step, nor the LM head, whose are in every block.
-  plan.turned = !plan.wide && plan.w_stream && K % 4096 == 0 &&
-                (cls == DLLM_PROF_GEMM_O || cls == DLLM_PROF_GEMM_GU || cls == DLLM_PROF_GEMM_D);
   const bool to_rows = tensor && rows && plan.pair && plan.S_max == 1;
   // an unsplit gate / up projection of an interleaved weight finishes SwiGLU in its own epilogue, and an unsplit
   // LM head writes per-tile estimate records instead of logits

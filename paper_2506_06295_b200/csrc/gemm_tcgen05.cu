@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(ONE_THREADS) gemm_bf16_tcgen05_kernel(const __
   const int kb0 = blockIdx.z * kb_per_split;
   const int kb1 = min(num_kb, kb0 + kb_per_split);
   const int nkb = kb1 - kb0;            // >= 1 by construction of the plan
-  const int turn = turned && ((nt >> 1) & 1) ? nkb / 2 : 0;   // see run_gemm
+  const int turn = turned && ((nt >> 1) & 1) ? nkb / 2 : 0;   // see launch_gemm_bf16
   auto k_block = [&](int i) {           // the i-th k-block of the walk
     const int j = i + turn;
     return kb0 + (j < nkb ? j : j - nkb);
@@ -491,7 +491,7 @@ constexpr int max_stages(int bn) {
 
 template <int BN, bool ONCE>
 cudaError_t launch_one(const Launch& L, const CUtensorMap& tmW, const CUtensorMap& tmA, float* part, int M, int N,
-                       int num_kb, const GemmPlan& plan, void* act_out, int m_ffn) {
+                       int num_kb, const GemmPlan& plan, void* act_out, int m_ffn, bool turned) {
   using SL = SmemLayout<BN>;
   static DeviceOnce once;
   cudaError_t e0 = once.run([] {
@@ -502,14 +502,14 @@ cudaError_t launch_one(const Launch& L, const CUtensorMap& tmW, const CUtensorMa
   const int stages = plan.stages < 2 ? 2 : plan.stages > max_stages(BN) ? max_stages(BN) : plan.stages;
   dim3 grid((M + BN - 1) / BN, (N + TILE_W - 1) / TILE_W, plan.S_max);
   cudaError_t e = launch_k(L, gemm_bf16_tcgen05_kernel<BN, ONCE>, grid, dim3(ONE_THREADS), SL::total(stages), tmW, tmA, part, M, N,
-                           num_kb, plan.upc, (size_t)M * N, stages, (__nv_bfloat16*)act_out, m_ffn, (int)plan.turned, L.d_status);
+                           num_kb, plan.upc, (size_t)M * N, stages, (__nv_bfloat16*)act_out, m_ffn, (int)turned, L.d_status);
   L.count();
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <int BN, bool ONCE>
 cudaError_t launch_pair(const Launch& L, const CUtensorMap& tmW, const CUtensorMap& tmA, float* part, int M, int N,
-                        int num_kb, const GemmPlan& plan, void* act_out, int m_ffn) {
+                        int num_kb, const GemmPlan& plan, void* act_out, int m_ffn, bool) {
   auto go = [&](auto form, bool staged) {
     return launch_pair_form<BN, ONCE>(L, tmW, tmA, part, M, N, num_kb, plan, form, staged);
   };
@@ -676,9 +676,17 @@ cudaError_t launch_gemm_bf16(const Launch& L, const void* A, const void* W, floa
   const int num_kb = (K + TILE_K - 1) / TILE_K;
   // evict-first weights where one activation tile reads them (128-row tiles of the one-CTA kernel gained nothing)
   const bool once = plan.w_stream && plan.m_tiles == 1;
-#define DLLM_LAUNCH(kind, bn, may)                                                                        \
-  ((may) && once ? launch_##kind<bn, may>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn)          \
-                 : launch_##kind<bn, false>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn))
+  // Gate / up weights whose rows lie a multiple of 8 KB apart, streamed once by unsplit one-tile CTAs: all CTAs in step read
+  // the same few address bits of every row, and every other pair of tiles half a row ahead spreads them.  B200, us per layer
+  // of adaptive steps of 3 / 32 / 64 / 115 rows: 4096 wide, d_ffn 12288 102.1 / 105.9 / 116.4 / 126.9 -> 100.3 / 103.9 / 114.4 /
+  // 124.8, d_ffn 14336 103.8 / 104.9 / 113.6 / 122.0 -> 99.1 / 102.6 / 111.2 / 120.2, d_ffn 16384 2 % faster; 8192 wide (16 KB
+  // rows) even.  Not where the product is split or has other row lengths (O and down of the same models even, a down product of
+  // 20480 long rows 1.5 % slower, gate / up of 7 KB rows 1.5 % slower), nor on CTA pairs (2 % slower); other turns and
+  // four or eight starting points gave less.  Not for products whose sums are the same in every kind of step.
+  const bool turned = act_out && !plan.pair && !plan.wide && plan.m_tiles == 1 && plan.BN <= 128 && plan.w_stream && K % 4096 == 0;
+#define DLLM_LAUNCH(kind, bn, may)                                                                          \
+  ((may) && once ? launch_##kind<bn, may>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn, turned)    \
+                 : launch_##kind<bn, false>(L, tmW, tmA, part, M, N, num_kb, plan, act_out, m_ffn, turned))
   if (plan.pair) {
     switch (plan.BN) {
       case 64: return DLLM_LAUNCH(pair, 64, false);

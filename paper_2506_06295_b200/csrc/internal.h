@@ -190,7 +190,6 @@ struct GemmPlan {
   int S_max;        // split-K factor: slabs per output element
   bool w_stream = false;  // weights are marked evict-first (when one activation tile reads them)
   bool wide = false;  // an automatic plan for pairs (also where dllm_debug_gemm_plan gives it to the one-tile kernel)
-  bool turned = false;  // one-tile kernel: every other pair of weight tiles starts in the middle of its k range
   int pair = 0;     // 1: persistent CTA pairs (cta_group::2) on tiles of 256 weight rows x BN activation rows
 };
 // 0 = auto; force_split < 0: the automatic tile with exactly -force_split splits.  force_pair: 0 auto, 1 CTA pairs (BN >= 64).  force_persistent: 0 auto, 1 the pair kernel for unsplit
