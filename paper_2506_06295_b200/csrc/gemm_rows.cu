@@ -118,9 +118,9 @@ struct RowForm {
     auto sync = [&] { group_sync(bar); };
     uint32_t r[CH];
     tmem_ld16(tmem_w, r);
+    tmem_ld16_wait(r);
 #pragma unroll 1
     for (int c0 = 0; c0 < rows; c0 += CH) {
-      tmem_ld16_wait(r);
 #pragma unroll
       for (int j = 0; j < CH; ++j) ex[j * EXS + tl] = __uint_as_float(r[j]);
       sync();
@@ -180,23 +180,23 @@ struct RowForm {
         }
       }
       fetch(c0 + CH);
-      if (KIND == VERIFY && o.keep_rows) continue;
+      const int stored = KIND == VERIFY && o.keep_rows ? 0 : rows;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int row = c0 + rsub + 8 * u;
         if constexpr (KIND == PLACE) {
           if (m0 + row < o.slab_rows) {   // (their columns 4 q .. and 64 further, as the others')
             float* const raw = reinterpret_cast<float*>(raw_at[u]);
-            if (vlo && row < rows) *reinterpret_cast<float4*>(raw + nlo) = a[u];
-            if (vhi && row < rows) *reinterpret_cast<float4*>(raw + nhi) = b[u];
+            if (vlo && row < stored) *reinterpret_cast<float4*>(raw + nlo) = a[u];
+            if (vhi && row < stored) *reinterpret_cast<float4*>(raw + nhi) = b[u];
             continue;
           }
         }
-        if (vlo && row < rows && row >= lo_from) *reinterpret_cast<uint2*>(dlo[u]) = plo[u];
-        if (vhi && row < rows && row >= hi_from) *reinterpret_cast<uint2*>(dhi[u]) = phi[u];
+        if (vlo && row < stored && row >= lo_from) *reinterpret_cast<uint2*>(dlo[u]) = plo[u];
+        if (vhi && row < stored && row >= hi_from) *reinterpret_cast<uint2*>(dhi[u]) = phi[u];
       }
+      tmem_ld16_wait(r);   // in the trip that requested them: the compiler may move what it carries round the loop
     }
-    tmem_ld16_wait(r);
     sync();   // the rows' places are free
   }
 };

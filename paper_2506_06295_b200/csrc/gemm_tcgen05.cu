@@ -69,20 +69,21 @@ struct PlainStage {
   static constexpr int EXS = 132;              // floats per staged row: 16-byte aligned, rows 4 banks apart
   static constexpr uint32_t BYTES = CH * EXS * 4;
 };
-// CH columns of tensor memory on their way into registers; landed: they are there and go to staging.
+// CH columns of tensor memory on their way into registers; landed: they are there; then they go to staging.  The loops below
+// wait for what they have requested in the same trip: between a load and its wait nothing may read or move the registers, and
+// the compiler may move what a loop carries round its edge.
 template <int CH>
 __device__ __forceinline__ void tmem_fetch(uint32_t taddr, uint32_t (&r)[CH / 16][16]) {
 #pragma unroll
   for (int i = 0; i < CH / 16; ++i) tmem_ld16(taddr + 16u * i, r[i]);
 }
 template <int CH>
-__device__ __forceinline__ void tmem_last(uint32_t (&r)[CH / 16][16]) {
+__device__ __forceinline__ void tmem_landed(uint32_t (&r)[CH / 16][16]) {
 #pragma unroll
   for (int i = 0; i < CH / 16; ++i) tmem_ld16_wait(r[i]);
 }
 template <int CH, int EXS>
-__device__ __forceinline__ void tmem_landed(uint32_t (&r)[CH / 16][16], float* ex, int tl) {
-  tmem_last<CH>(r);
+__device__ __forceinline__ void tmem_stage(const uint32_t (&r)[CH / 16][16], float* ex, int tl) {
 #pragma unroll
   for (int i = 0; i < CH / 16; ++i)
 #pragma unroll
@@ -110,9 +111,10 @@ __device__ __forceinline__ void gemm_epilogue(uint32_t tmem_d, float* ex, int tl
     const int rr = tl >> 2, part = tl & 3;
     uint32_t r[CH / 16][16];
     tmem_fetch<CH>(tmem_w, r);
+    tmem_landed<CH>(r);
 #pragma unroll 1
     for (int c0 = 0; c0 < W && m0 + c0 < M; c0 += CH) {
-      tmem_landed<CH, EXS>(r, ex, tl);
+      tmem_stage<CH, EXS>(r, ex, tl);
       sync();
       tmem_fetch<CH>(tmem_w + (uint32_t)min(c0 + CH, W - CH), r);   // the next rows (again the last ones in the last trip)
       MaxSum t{-INFINITY, 0.f, 0x7fffffff};
@@ -160,9 +162,9 @@ __device__ __forceinline__ void gemm_epilogue(uint32_t tmem_d, float* ex, int tl
       const int m = m0 + c0 + rr;
       if (rr < CH && part == 0 && m < M)
         rec[(size_t)m * n_tiles + tile_y] = make_float4(t.m, t.s, __int_as_float(t.a), 0.f);
+      tmem_landed<CH>(r);
       sync();
     }
-    tmem_last<CH>(r);
   } else if constexpr (KIND == SWIGLU) {
     // SwiGLU epilogue (no split-K): the tile's 128 weight rows are 64 gate rows followed by the 64 up rows
     // of the same FFN columns, so TMEM lanes 0..63 hold gate and 64..127 hold up.  The accumulator goes
@@ -173,9 +175,10 @@ __device__ __forceinline__ void gemm_epilogue(uint32_t tmem_d, float* ex, int tl
     const int col = tile_y * 64 + 4 * q;
     uint32_t r[CH / 16][16];
     tmem_fetch<CH>(tmem_w, r);
+    tmem_landed<CH>(r);
 #pragma unroll 1
     for (int c0 = 0; c0 < W && m0 + c0 < M; c0 += CH) {
-      tmem_landed<CH, EXS>(r, ex, tl);
+      tmem_stage<CH, EXS>(r, ex, tl);
       sync();
       tmem_fetch<CH>(tmem_w + (uint32_t)min(c0 + CH, W - CH), r);   // the next rows (again the last ones in the last trip)
 #pragma unroll 2
@@ -196,9 +199,9 @@ __device__ __forceinline__ void gemm_epilogue(uint32_t tmem_d, float* ex, int tl
           *reinterpret_cast<uint2*>(act_out + (size_t)m * m_ffn + col) = pk;
         }
       }
+      tmem_landed<CH>(r);
       sync();
     }
-    tmem_last<CH>(r);
   } else {
     const int n = n0 + (tl >> 5) * 32 + lane;
     float* out = slab + n;
