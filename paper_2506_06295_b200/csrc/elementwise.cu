@@ -1437,10 +1437,11 @@ cudaError_t launch_select_gather(const Launch& L, int dtype, const float* sim, c
   const int np = refresh_prompt ? g.P : 0, rows = g.B * (g.R + np);
   // few rows: all CTAs are resident before the launch ahead ends, and the rows that nobody selects cost nothing
   const bool early = u_static && rows <= 1024 && g.d * (dtype == 0 ? 4 : 2) <= SG_VEC * SG_THREADS * 16;
-  DLLM_DISPATCH(dtype, (launch_k(L, select_gather_kernel<T>, dim3(rows), dim3(SG_THREADS), 0, sim, forced, mode, ksel, sel, act,
+  cudaError_t e;
+  DLLM_DISPATCH(dtype, (e = launch_k(L, select_gather_kernel<T>, dim3(rows), dim3(SG_THREADS), 0, sim, forced, mode, ksel, sel, act,
                                  inv, (const T*)u, (T*)ua, g, np, early)));
   L.count();
-  return cudaSuccess;
+  return e;
 }
 
 // ------------------------------------------------------------------ greedy estimate + confidence (Eq. 4)
