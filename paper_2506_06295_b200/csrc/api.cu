@@ -633,8 +633,19 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
   // While profiling, V and Q / K stay launches of their own, so that each class can be read.
   // An adaptive step that happens to recompute every row, and one that is profiled, equal a response refresh bit for bit:
   // their products have the same plans, and V of the prompt rows is not split where that product has it.
-  // In a session of not too many response rows (in_one) their V has the splits of the one product for Q, K and V (v_split) wherever it
-  // is computed.  Every row of a step comes from that product where it has these splits over all carried rows (all_in_one).
+  // In a session of not too many response rows (in_one) their V has the splits of the one product for Q, K and V (v_split) wherever
+  // V-verify scores or writes it.  Alone V would like more of them (32 response rows of a 4096-wide model: 17.9 us in two
+  // splits, 12.2 in five; 0.3 % of the full step of a 4096-token prompt, whose partial steps the one product makes 5 % faster).
+  // Every row of a step comes from that product where it has these splits over all carried rows (all_in_one).
+  // The products of a step, by kind:
+  //   refresh, full   all_in_one: [Q | K | V] of all rows (qk_whole = v_whole = true; profiled: the same sums one by one)
+  //                   otherwise V of the response rows (into Q / K's product too where both are unsplit: v_whole), V of the prompt
+  //                   rows (into it as well where it places its rows: qkv_whole), [Q | K] (qk_whole: of the rows as they lie)
+  //   partial         one_product: [Q | K | V] of all response rows, the selected ones rotated (selected_rows; profiled: one by one)
+  //                   otherwise V of all response rows (verify_in_product: which compares them), [Q | K] of the selected ones,
+  //                   and V of those alone where the strategy has not written it (v_for_active)
+  //   mixed           V of the response rows and V of the prompt rows, in one launch where both have the same splits (v_together,
+  //                   v_one), then [Q | K] of prompt and selected rows, V of those alone as above
   const bool tensor = dt == DLLM_BF16 && !s->simt_gemm;
   const bool heads = tensor && (hd == 64 || hd == 128), rotate = heads && !s->profiling;
   const bool all_rows = rr || std::all_of(ksels.begin(), ksels.end(), [&](int k) { return k == s->R; });

@@ -9,6 +9,7 @@
 //   warp 10          TMA: K/V tiles into a six-stage ring (all that shared memory holds)
 //   warp 8           issues the tcgen05.mma (warp 9 those of group 1 when the groups share a row tile)
 //   warps 0-3, 4-7   the softmax group of row tile 0 resp. 1 (one row per thread)
+// (a CTA of ONE row tile, two to an SM: warp 5 copies, warp 4 issues, warps 0-3 are its softmax group)
 // Per key tile t and row tile i:
 //   S_i = Q_i K^T     tcgen05.mma, M = 128 rows, N = 64 keys, contraction HD; Q_i is
 //                     the A operand in tensor memory (written there once by its
@@ -131,7 +132,7 @@ struct UaSmem {
   static constexpr uint32_t KPAR_S_COL = 64;
   static constexpr uint32_t TMEM_COLS = 256 * TILES;
   static_assert(S_COL + TILES * UA_KEYS <= O_COL, "scores and outputs must not overlap");
-  static_assert(O_COL + TILES * HD <= TMEM_COLS, "tensor memory holds 512 columns");
+  static_assert(O_COL + TILES * HD <= TMEM_COLS, "tensor memory holds 512 columns, 256 for each of two CTAs");
 };
 
 template <int HD, int TILES>
@@ -222,7 +223,7 @@ __global__ void __launch_bounds__((UaSmem<HD, TILES>::THREADS), 3 - TILES)
       __syncwarp();
     }
   } else if (warp >= SM::MMA_WARP) {
-    // ---------------- MMA issuers: warp 8, and warp 9 for group 1 when the groups share a row tile ----------------
+    // ---------------- MMA issuers: the first MMA warp, and the second for group 1 when the groups share a row tile ------
     // Per key tile t and row tile i:  S_i(t) = Q_i K(t)^T  ->  [softmax group i]  ->  O_i += P_i(t) V(t), and right
     // behind it S_i(t+1), so that the tensor pipe works on one row tile while the other is in its softmax.  Q_i
     // and P_i are A operands in tensor memory (P_i in the columns its scores came from), so shared memory is
@@ -270,7 +271,7 @@ __global__ void __launch_bounds__((UaSmem<HD, TILES>::THREADS), 3 - TILES)
       // alone issues the first three, in order (a commit covers what its thread issued before): group 1, through with tile
       // 1, knows S(0) complete when it waits for S(3), group 0 after tile 2 S(1).  S(2) precedes S(3) in issuer 0; from
       // tile 6 on S(t - 3) precedes the product of tile t - 4 in the same issuer, which the group has waited for.
-      const int i = warp - 8;   // two row tiles' worth of warps: the MMA warps are 8 and 9
+      const int i = warp - SM::MMA_WARP;
       for (int t = 0; t < 3 && ok && i == 0; ++t) {
         ok = tile_ready(t);
         if (ok) issue_s(SM::KPAR_S_COL + (uint32_t)(t * UA_KEYS), SM::Q_COL, t, t);

@@ -561,7 +561,7 @@ Partials make_partials(const float* p, int M, int N, const GemmPlan& plan) {
 // units, a k-block of a unit takes the larger of the issue / tensor time of its tile (0.33 / 0.27 / 0.25 us for 256 /
 // 192 / 128 rows) and its bytes' share of the L2 -> SM fabric (12 TB/s over all SMs: 0.40 / 0.35 / 0.30 us when every
 // SM is busy), and a split adds slabs that are written and read once more (10 TB/s); epilogues are not in it (2.8 us for
-// slabs, 5.8 for SwiGLU, 16 for rotated and placed rows of a 256-row tile).  Measured with it, B200, us
+// slabs, 3.9 for SwiGLU, about 6 for rotated and placed rows of a 256-row tile).  Measured with it, B200, us
 // (before -> now): 768 x 4096 x 12288 77 -> 63, 768 x 24576 x 4096 120 -> 110, 4096 x 24576 x 4096 614 -> 583, 4096 x
 // 4096 x 12288 362 -> 306, 24576 x 4096 x 4096 711 -> 646, 256 x 126464 x 4096 258 -> 221.
 static double plan_pair(int M, int N, int K, int max_split, int exact_split, int* bn, int* splits) {

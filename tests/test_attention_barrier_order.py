@@ -91,7 +91,7 @@ def test_the_model_finds_a_start_shared_by_the_issuers():
 
 def test_the_kernel_starts_with_one_issuer():
     src = open(os.path.join(CSRC, "attention_umma.cu")).read()
-    begin = src.index("const int i = warp - 8;")
-    startup = re.sub(r"//[^\n]*", "", src[begin:src.index("int buf = i;", begin)])
+    end = src.index("int buf = ")                              # the issuers' walk over the tiles; their start precedes it
+    startup = re.sub(r"//[^\n]*", "", src[src.rindex("if (kpar)", 0, end):end])
     assert re.search(r"for \(int t = 0; t < 3 && ok && i == 0; \+\+t\)", startup)
     assert startup.count("issue_s(") == 1 and "tile_ready(t)" in startup

@@ -46,14 +46,27 @@ def test_scores_and_rows(dllm, cfg, B, P, R, v_update, metric):
         ses.step_cached(False, False, 0.25)
         ses.sync()
         out.append((ses.selected(0), before, ses.get_cache(0, dllm.CACHE_V)))
+        # which kernel verified: the merge reads 16 bytes per row and 128 columns, the other the fp32 row and the cached one
+        ses.profile(True)
+        ses.step_cached(False, False, 0.25)
+        read = ses.profile_read(dllm.PROF_CLASSES.index("vverify"))
+        assert read["bytes"] == B * R * (-(-cfg.dkv // 128) * 16 + 4 if plan == 0 else cfg.dkv * 8)
     ((idx0, sim0), b0, v0), ((idx1, sim1), b1, v1) = out
     assert np.array_equal(b0, b1)
     same = first == then
     exact = 1.0 if metric == "cosine" else 0.0
     assert (sim0[same] == exact).all() and (sim1[same] == exact).all()      # rows whose input did not change
-    assert (sim0[~same] < exact).all() or metric == "cosine"
+    assert (sim0[~same] < (0.9 if metric == "cosine" else 0.0)).all()       # another token: another random row
     # sums of thousands of fp32 products in another order: a few ulp of each
     np.testing.assert_allclose(sim0, sim1, rtol=2e-6, atol=2e-6)
-    if np.array_equal(idx0, idx1) or v_update == "whole":
+    if v_update == "whole":
         assert np.array_equal(v0, v1)
-    assert (np.sort(idx0, 1) == idx0).all()
+    else:   # rows whose scores differ in the last bits may change places at the threshold
+        taken = np.zeros((2, B, R), bool)
+        for i, idx in enumerate((idx0, idx1)):
+            np.put_along_axis(taken[i], idx, True, 1)
+        assert taken.sum() == 2 * B * (R // 4) and (taken[0] != taken[1]).sum() <= 4
+        for v, t in zip((v0, v1), taken):
+            assert np.array_equal(v[:, P:][~t], b0[:, P:][~t])
+        assert np.array_equal(v0[:, P:][taken.all(0)], v1[:, P:][taken.all(0)])
+        assert (v0[:, P:] != b0[:, P:]).any(2)[taken[0] & ~same].all()
