@@ -61,9 +61,9 @@ __device__ __forceinline__ bool group_all(int bar, bool v) { return bar == 1 ? g
 // in tensor memory, and the other warps drain one accumulator while the other fills.  The k loop of a tile is the one-tile
 // kernel's: results are bit-identical to it.  With a split k range every split writes its own slab.  Loads carry no
 // multicast: every byte is requested by the CTA that stages it.
-// (In the replayed response refresh of 256 rows, us from the release to the first stage / accumulators complete / rows
-// written: Q/K in two splits 1.9 / 12.8 / 15.6, down in four 1.7 / 18.5 / 21.2, gate / up with SwiGLU, two rounds, 2.4 /
-// 25.8-49.0 / 30-53.)
+// (In the replayed response refresh of 256 rows of a 4096-wide model, us from the release to the first stage / accumulators
+// complete / rows written: Q / K / V, placed and rotated, 1.9 / 23.9 / 30.0; O in four splits 2.5 / 8.7 / 11.8; gate / up with
+// SwiGLU, two rounds, 3.1 / 27.8-51.6 / 31.5-55.2; down in four 1.9 / 19.8 / 22.8.)
 template <typename FORM>
 constexpr int PAIR_THREADS = 64 + 128 * FORM::GROUPS;
 template <int BN, typename FORM>
