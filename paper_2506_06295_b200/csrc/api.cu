@@ -234,6 +234,7 @@ Workspace make_workspace(const dllm_config& c, int B, int P, int R, int flags) {
       mn = std::max(mn, (size_t)p.S_max * M * N);
     };
     slabs(BR, dkv, d);
+    mn = std::max(mn, (size_t)plan_gemm_bf16((int)BR, (int)dkv, (int)d).S_max * rows * dkv);   // V of selected rows alone
     if (qkv_in_one(c, B, R)) {  // [Q | K | V] of all response rows, or of all carried rows with as many splits
       const int split = plan_gemm_bf16((int)BR, (int)(dq + 2 * dkv), (int)d).S_max;
       slabs(BR, dq + 2 * dkv, d);
@@ -663,6 +664,9 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
   // Many response rows, V unsplit: its product verifies (and overwrites) the rows itself, profiled too
   const GemmPlan v_plan = tensor && !in_one ? plan_gemm_bf16(BR, dkv, d) : GemmPlan{};
   const bool verify_in_product = tensor && !in_one && v_plan.pair && v_plan.S_max == 1 && dkv % 4 == 0;
+  // splits of V wherever V-verify scores or writes response rows, all or the selected ones alone (for a few hundred rows, where few
+  // selected ones would be split further, this costs up to 2 % of a partial step that writes only their V)
+  const int v_rows_split = in_one ? v_split : tensor ? v_plan.S_max : 0;
   // splits of Q / K and of the prompt's V in such a step (0: their own plans')
   const int all_split = all_in_one ? v_split : 0, prompt_v_split = all_in_one ? v_split : qk_unsplit ? 1 : 0;
   RowOut qkv;
@@ -805,7 +809,7 @@ dllm_status enqueue_step(dllm_session* s, int rp, int rr, const std::vector<int>
       if (v_for_active) {
         const RowOut o = rows_into(v_rows, dkv, act, 0);
         if ((st = run_gemm(s, L, DLLM_PROF_GEMM_V, ua, Wv, Ma, dkv, d, &part, nullptr, &fused, -1, false, &o,
-                           in_one && verify_v ? v_split : qk_split)) != DLLM_OK)
+                           verify_v ? v_rows_split : qk_split)) != DLLM_OK)
           return st;
         if (!fused) {
           ProfScope ps(s, DLLM_PROF_SCATTER, (double)Ma * dkv * (4.0 + es), 0.0, stream);

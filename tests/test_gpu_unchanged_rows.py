@@ -55,8 +55,9 @@ def test_unchanged_rows_score_exactly(dllm, cfg, B, P, R, metric):
 
 
 @pytest.mark.parametrize("metric", ["cosine", "l2"])
-@pytest.mark.parametrize("cfg,B,P,R,rho", [(GROUPED, 1, 256, 256, 0.5), (GROUPED, 2, 90, 70, 0.3), (WIDE, 1, 130, 200, 0.25)],
-                         ids=["grouped", "two sequences", "wide"])
+@pytest.mark.parametrize("cfg,B,P,R,rho", [(GROUPED, 1, 256, 256, 0.5), (GROUPED, 2, 90, 70, 0.3), (WIDE, 1, 130, 200, 0.25),
+                                               (GROUPED, 1, 200, 400, 0.25), (WIDE, 1, 100, 300, 0.25), (WIDE, 4, 60, 300, 0.25)],
+                         ids=["grouped", "two sequences", "wide", "grouped separate", "wide separate", "verified in the product"])
 def test_rows_written_one_by_one_score_exactly(dllm, cfg, B, P, R, rho, metric):
     """The same where only the selected rows' V is written (another product in a mixed step): in the first layer, whose V
     depends on the tokens alone, every row keeps its bits."""
